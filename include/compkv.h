@@ -197,10 +197,12 @@ int ckv_prefill(ckv_ctx *ctx, void *k_pool, void *v_pool, const int32_t *page_ta
 /* One decode step in one call: the results, the cache, the summaries, the lengths and the errors are those of
  * ckv_append(k_new, v_new) followed by ckv_decode(q, ...), bit for bit (Sec. 4.3: the new token enters the cache
  * and the summaries before blocks are selected; seq_lens holds N on entry and N + 1 once the step has run;
- * max_seq_len_host bounds the lengths after the append).  It is three launches, not four: a step can only change
- * the last block of a sequence, so a few CTAs of the scan launch write the new rows and redo that block's summary
- * while the other CTAs stream the summaries of all the other blocks; seq_lens is updated inside that launch, after
- * every CTA has read it.  (Batches above 1024 sequences take the two-call route.)  The decode arguments are
+ * max_seq_len_host bounds the lengths after the append).  Where a unit's blocks fit a thread-block cluster (bf16 pages,
+ * caches of 1536 tokens and more, as many units as clusters run at once) the whole step is ONE launch, and ckv_decode is
+ * the same launch without a new token.  Otherwise it is three launches on long scans: a step can only change the last
+ * block of a sequence, so a few CTAs of the scan launch write the new rows and redo that block's summary while the other
+ * CTAs stream the summaries of all the other blocks; seq_lens is updated inside that launch, after every CTA has read
+ * it.  (Short scans and batches above 1024 sequences take the two-call route.)  The decode arguments are
  * validated before anything is appended. */
 int ckv_step(ckv_ctx *ctx, const void *q, const void *k_new, const void *v_new, void *k_pool, void *v_pool,
              const int32_t *page_table, int32_t *seq_lens, int batch, int max_seq_len_host, int budget_tokens,
@@ -271,7 +273,8 @@ int ckv_read_status(ckv_ctx *ctx, int32_t *host_status, ckv_stream stream);
  * same launch -- while the other CTAs stream the remaining summaries; otherwise the scan covers every block and
  * ckv_step appends in a launch of its own.  The results agree to rounding (the last block's two per-head terms are
  * computed by different code); tail mode is the faster one once the scan runs for tens of microseconds.
- * mode: CKV_TAIL_AUTO (default: chosen per call from the batch and max_seq_len_host), CKV_TAIL_OFF, CKV_TAIL_ON
+ * mode: CKV_TAIL_AUTO (default: chosen per call from the batch and max_seq_len_host, the one-launch step included),
+ * CKV_TAIL_OFF, CKV_TAIL_ON (separate launches)
  * (honoured up to 1024 sequences).  Returns CKV_ERR_INVALID_ARG for a null context or an unknown mode. */
 enum ckv_tail_mode { CKV_TAIL_AUTO = 0, CKV_TAIL_OFF = 1, CKV_TAIL_ON = 2 };
 int ckv_set_tail_mode(ckv_ctx *ctx, int mode);

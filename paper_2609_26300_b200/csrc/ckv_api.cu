@@ -184,6 +184,7 @@ int ckv_create(const ckv_layout *layout, void *stats_dev, size_t stats_bytes, vo
   if (e == cudaSuccess) e = ckv_configure_scan(c);
   if (e == cudaSuccess) e = ckv_configure_attn(c);
   if (e == cudaSuccess) e = ckv_configure_attn_mma(c);
+  if (e == cudaSuccess) e = ckv_configure_unit_step(c);
   int dev_id = 0;
   if (e == cudaSuccess) e = cudaGetDevice(&dev_id);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, dev_id);
@@ -323,6 +324,11 @@ int decode_impl(ckv_ctx *c, const void *q, const void *k_pool, const void *v_poo
   if (budget_tokens <= 0 || kcap <= 0) return CKV_ERR_BUDGET_TOO_SMALL;
   if (kcap < L.sink_blocks + L.recent_blocks && (long long)kcap * L.block_size < max_seq_len_host)
     return CKV_ERR_BUDGET_TOO_SMALL;
+  CkvStepPlan plan;
+  if (ev == nullptr && ckv_unit_step_plan(c, batch, max_seq_len_host, kcap, &plan)) {
+    CKV_CUDA(ckv_launch_unit_step(c, plan, q, k_pool, v_pool, page_table, seq_lens, fresh, batch, kcap, sel_ids, sel_cnt, out, lse, s));
+    return CKV_OK;
+  }
   int scan_grid = 0, n_splits = 0;
   c->dev.tail = (fresh != nullptr || ckv_scan_wants_tail(c, batch, max_seq_len_host)) ? 1 : 0;   // one mode for the step's launches
   if (ev) CKV_CUDA(cudaEventRecord(ev[0], s));
@@ -361,7 +367,9 @@ int ckv_step(ckv_ctx *c, const void *q, const void *k_new, const void *v_new, vo
   if (kcap < L.sink_blocks + L.recent_blocks && (long long)kcap * L.block_size < max_seq_len_host)
     return CKV_ERR_BUDGET_TOO_SMALL;
   if (!k_pool || !v_pool || !page_table || !seq_lens || !k_new || !v_new) return CKV_ERR_INVALID_ARG;
-  if (ckv_scan_wants_tail(c, batch, max_seq_len_host)) {   // the append rides in the scan launch: three launches per step
+  CkvStepPlan plan;
+  // the append rides in the step's only launch, or in the scan launch (three launches per step)
+  if (ckv_unit_step_plan(c, batch, max_seq_len_host, kcap, &plan) || ckv_scan_wants_tail(c, batch, max_seq_len_host)) {
     const CkvNewToken fresh = {k_pool, v_pool, page_table, seq_lens, k_new, v_new};
     return decode_impl(c, q, k_pool, v_pool, page_table, seq_lens, batch, max_seq_len_host, budget_tokens, out, lse,
                        sel_ids, sel_cnt, (cudaStream_t)stream, nullptr, &fresh);

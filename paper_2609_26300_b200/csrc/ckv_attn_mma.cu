@@ -34,12 +34,10 @@
 #include "ckv_internal.cuh"
 #include "ckv_mma.cuh"
 #include "ckv_cluster.cuh"
+#include "ckv_attnpage.cuh"
 
 namespace {
 
-constexpr int kTileBytes = CKV_PAGE * CKV_D * 2;      // one head's K (or V) page in bf16: 4 KB
-constexpr int kPageBytes = 2 * kTileBytes;            // K tile | V tile
-constexpr int kRowBytes = CKV_D * 2;                  // 256
 constexpr int kMeanSlots = 4;                         // mean-value rows (512 B each) a warp can hold
 constexpr int kMeanFlush = 3;                         // ... of which at most 3 wait for removal while one is in flight
 constexpr int kZeroRow = kMeanSlots * 512;            // offset of the row of zeros inside the aux area
@@ -49,16 +47,6 @@ constexpr int kMaxEntries = 32;                       // partials a CTA folds pe
 constexpr int kPartBytes = CKV_PART_STRIDE * 4;       // one head's partial
 
 template <int W> constexpr size_t dyn_smem() { return (size_t)W * (2 * kPageBytes + kAuxBytes); }
-
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, bool valid) {
-  // valid == false copies nothing and zero-fills the 16 bytes
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(valid ? 16 : 0) : "memory");
-}
-__device__ __forceinline__ void cp_async4(uint32_t dst, const void *src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
 constexpr int kMaxCluster = 8;    // splits of a unit that can be one cluster (the portable size; 13 measured far slower)
 
@@ -261,15 +249,7 @@ ckv_attn_mma_kernel(CkvDev P, const __nv_bfloat16 *__restrict__ q, const __nv_bf
       const size_t src = ((size_t)r.phys * P.Hkv + h) * (CKV_PAGE * CKV_D);
       const uint32_t kb = wtiles_u32 + buf * kPageBytes;
       const uint32_t vb = kb + kTileBytes;
-#pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        const int idx = lane + 32 * k, row = idx >> 4, c = idx & 15;
-        const uint32_t off = (uint32_t)(row * kRowBytes + ((c ^ (row & 7)) << 4));
-        const bool valid = row < r.ntok;
-        const size_t so = src + (size_t)(valid ? row : 0) * CKV_D + 8 * c;
-        cp_async16(kb + off, k_pool + so, valid);
-        cp_async16(vb + off, v_pool + so, valid);
-      }
+      issue_page(kb, vb, k_pool + src, v_pool + src, r.ntok, lane);
       if (row_rm && r.first) {   // verbatim: hi halves then lo halves, swizzled by block index
         if (mean_lo || lane < 16)
           cp_async16(aux_u32 + 512 * slot + 16 * lane, vmean + (size_t)r.blk * P.row_elems + 8 * lane, true);
@@ -392,76 +372,11 @@ ckv_attn_mma_kernel(CkvDev P, const __nv_bfloat16 *__restrict__ q, const __nv_bf
     if (cur.phys >= 0) {
       const uint32_t kb = wtiles_u32 + buf * kPageBytes;
       const uint32_t vb = kb + kTileBytes;
-      // ---- S^T = Q K^T: heads x 16 tokens (two n-tiles of 8 tokens) ----
-      float sv[2][2] = {{0.f, 0.f}, {0.f, 0.f}}, sv2[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
-      {
-        const int lrow = lane & 7, lmat = lane >> 3;
-#pragma unroll
-        for (int nt = 0; nt < 2; ++nt) {
-          const int r = nt * 8 + lrow;
-          const uint32_t rowaddr = kb + r * kRowBytes;
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {   // two 16-coordinate steps per ldmatrix.x4
-            uint32_t b[4];
-            ldmatrix_x4(b, rowaddr + (uint32_t)(((4 * j + lmat) ^ (r & 7)) << 4));
-            mma_rows8(sv[nt][0], sv[nt][1], qa[2 * j][0], qa[2 * j][1], b[0], b[1]);
-            mma_rows8(sv2[nt][0], sv2[nt][1], qa[2 * j + 1][0], qa[2 * j + 1][1], b[2], b[3]);
-          }
-          sv[nt][0] += sv2[nt][0]; sv[nt][1] += sv2[nt][1];
-        }
-      }
-      // ---- softmax weights for this thread's head and its four tokens ----
-      float tmax = -CUDART_INF_F;
-#pragma unroll
-      for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          const bool ok = hv && nt * 8 + 2 * qd + e < cur.ntok;
-          sv[nt][e] = ok ? sv[nt][e] * sl2 : -CUDART_INF_F;
-          tmax = fmaxf(tmax, sv[nt][e]);
-        }
       // log2 of e^{zbar} of the page's block for this lane's head (token-weight removal)
       float lzt = -CUDART_INF_F;
       if (tok_rm && hv)
         lzt = *reinterpret_cast<const float *>(waux + kLsOff + (buf * G + head) * 4) - (cur.blk == X - 1 ? lg_last : lg_bs);
-      tmax = fmaxf(tmax, lzt);
-      tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, 1));
-      tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, 2));
-      if (tmax > m_ref + CKV_RESCALE_SLACK) {
-        const float sc = exp2_diff(m_ref, tmax);
-        m_ref = tmax;
-        l_acc *= sc;
-#pragma unroll
-        for (int t = 0; t < 16; ++t) { acc[t][0] *= sc; acc[t][1] *= sc; }
-      }
-      const float wtok = lzt == -CUDART_INF_F ? 0.f : fast_exp2(lzt - m_ref);
-      uint32_t ph[2], pl[2];
-#pragma unroll
-      for (int nt = 0; nt < 2; ++nt) {
-        float p[2];
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          p[e] = sv[nt][e] == -CUDART_INF_F ? 0.f : fast_exp2(sv[nt][e] - m_ref) - wtok;
-          l_acc += p[e];
-        }
-        ph[nt] = pack_bf16(p[0], p[1]);
-        pl[nt] = pack_bf16(p[0] - bf16_round(p[0]), p[1] - bf16_round(p[1]));
-      }
-      // ---- O += P V ----
-      {
-        const int r = ((lane >> 3) & 1) * 8 + (lane & 7);
-        const uint32_t rowaddr = vb + r * kRowBytes;
-        const int cpar = lane >> 4;
-#pragma unroll
-        for (int t2 = 0; t2 < 8; ++t2) {   // two 8-coordinate n-tiles per ldmatrix.x4
-          uint32_t v[4];
-          ldmatrix_x4_trans(v, rowaddr + (uint32_t)(((2 * t2 + cpar) ^ (r & 7)) << 4));
-          mma_rows8(acc[2 * t2][0], acc[2 * t2][1], ph[0], ph[1], v[0], v[1]);
-          mma_rows8(acc[2 * t2][0], acc[2 * t2][1], pl[0], pl[1], v[0], v[1]);
-          mma_rows8(acc[2 * t2 + 1][0], acc[2 * t2 + 1][1], ph[0], ph[1], v[2], v[3]);
-          mma_rows8(acc[2 * t2 + 1][0], acc[2 * t2 + 1][1], pl[0], pl[1], v[2], v[3]);
-        }
-      }
+      attn_page<false>(kb, vb, qa, cur.ntok, hv, lane, sl2, lzt, acc, m_ref, l_acc);
       if (row_rm && cur.first) {   // its mean-value row sits in aux slot cur_slot
 #pragma unroll
         for (int j = 0; j < kMeanFlush; ++j)

@@ -11,13 +11,23 @@
 #define CKV_BLOCKSTATS_CUH_
 #include "ckv_internal.cuh"
 
+// What a caller may keep of a block's fresh summary, as a reader of the stored rows would see it: the lane's eight entries
+// of the mean key (lower half warp) or of the mean value (upper), and of the variance of their groups.
+struct BlockRow { float x[8], dvar[8]; };
+
+// A stored mean entry as its readers see it: bf16(x), plus the rounded remainder when the row has lo halves.
+__device__ __forceinline__ float split_value(float x, bool lo_half) {
+  const float hi = __bfloat162float(__float2bfloat16_rn(x));
+  return lo_half ? hi + __bfloat162float(__float2bfloat16_rn(x - hi)) : hi;
+}
+
 // Second half of the block routine, shared by its variants: the half warps' squared deviations are combined, the
 // three summary rows are written (hw 0: mean key and variances, hw 1: mean value).  km: mean key, vs: value sums,
 // sq: this half warp's squared deviations, all for the lane's 8 coordinates.
 __device__ __forceinline__ void block_stats_finish(const CkvDev &P, int b, float fc, const float (&km)[8],
                                                    const float (&vs)[8], float (&sq)[8], float *sq_smem,
                                                    __nv_bfloat16 *kmean_row, float *dbar_row,
-                                                   __nv_bfloat16 *vmean_row, int lane, bool bad) {
+                                                   __nv_bfloat16 *vmean_row, int lane, bool bad, BlockRow *keep = nullptr) {
   const int hw = lane >> 4, li = lane & 15;
   const float inv = 1.0f / fc;
 #pragma unroll
@@ -28,6 +38,10 @@ __device__ __forceinline__ void block_stats_finish(const CkvDev &P, int b, float
 #pragma unroll
     for (int i = 0; i < 8; ++i) rowv[i] = hw == 0 ? km[i] : vs[i] * inv;
     store_split8(hw == 0 ? kmean_row : vmean_row, li, b, rowv, P.row_elems == CKV_ROW_ELEMS);
+    if (keep != nullptr) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) keep->x[i] = split_value(rowv[i], P.row_elems == CKV_ROW_ELEMS && !(hw == 1 && P.vhi));
+    }
   }
   const int gs = CKV_D / P.r;
   const int run = P.glayout == 0 ? gs : gs / 2;   // consecutive coordinates of a group (two runs, 64 apart, in layout 1)
@@ -40,6 +54,10 @@ __device__ __forceinline__ void block_stats_finish(const CkvDev &P, int b, float
       for (int i = 0; i < 8; ++i) dv[i] = sq[i] * inv;
       store_split8(reinterpret_cast<__nv_bfloat16 *>(dbar_row), li, b, dv);
     }
+    if (keep != nullptr) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) keep->dvar[i] = split_value(sq[i] * inv, true);
+    }
   } else if (run >= 8) {
     // grouped variance: average of the per-coordinate population variances of each group (Eq. 8).  A run is a
     // whole number of lanes: the lane's eight coordinates first, then the lanes of the run, then the second run.
@@ -48,7 +66,12 @@ __device__ __forceinline__ void block_stats_finish(const CkvDev &P, int b, float
     for (int o = 1; o < w; o <<= 1) ps += __shfl_xor_sync(0xffffffffu, ps, o);
     if (P.glayout != 0) ps += __shfl_xor_sync(0xffffffffu, ps, 8);
     const int lg = P.glayout == 0 ? li : (li & 7);
-    if (hw == 0 && (lg & (w - 1)) == 0 && (P.glayout == 0 || li < 8)) dbar_row[lg / w] = ps / (fc * (float)gs);
+    const float var = ps / (fc * (float)gs);
+    if (hw == 0 && (lg & (w - 1)) == 0 && (P.glayout == 0 || li < 8)) dbar_row[lg / w] = var;
+    if (keep != nullptr) {   // the lane's eight coordinates are of one group, and all lanes of a group hold its sum
+#pragma unroll
+      for (int i = 0; i < 8; ++i) keep->dvar[i] = var;
+    }
   } else {
     // groups narrower than a lane's eight coordinates: through shared memory
     if (hw == 0) {
@@ -68,6 +91,10 @@ __device__ __forceinline__ void block_stats_finish(const CkvDev &P, int b, float
       dbar_row[t] = s / (fc * (float)gs);
     }
     __syncwarp();
+    if (keep != nullptr) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) keep->dvar[i] = dbar_row[group_of(8 * li + i, P.r, P.glayout)];
+    }
   }
   if (bad && lane == 0) atomicOr(P.status, CKV_DEV_BAD_PAGE);
 }
@@ -142,7 +169,8 @@ template <typename T, bool NC, bool ONEP = false>
 __device__ __forceinline__ void block_stats_warp(const CkvDev &P, const T *__restrict__ k_pool,
                                                  const T *__restrict__ v_pool, const int *__restrict__ pt_row,
                                                  int h, int b, int cnt, float *sq_smem, __nv_bfloat16 *kmean_row,
-                                                 float *dbar_row, __nv_bfloat16 *vmean_row, int lane) {
+                                                 float *dbar_row, __nv_bfloat16 *vmean_row, int lane,
+                                                 BlockRow *keep = nullptr) {
   const int hw = lane >> 4, li = lane & 15;
   float ks[8], vs[8];
 #pragma unroll
@@ -307,7 +335,7 @@ __device__ __forceinline__ void block_stats_warp(const CkvDev &P, const T *__res
       for (int i = 0; i < 8; ++i) { km[i] = 0.f; sq[i] = 0.f; }
     }
   }
-  block_stats_finish(P, b, fc, km, vs, sq, sq_smem, kmean_row, dbar_row, vmean_row, lane, bad);
+  block_stats_finish(P, b, fc, km, vs, sq, sq_smem, kmean_row, dbar_row, vmean_row, lane, bad, keep);
 }
 
 // The same block routine for a caller whose time goes into instruction fetch rather than arithmetic (the tail

@@ -20,6 +20,9 @@
 #define CKV_SCAN_WARPS 7       // consumer warps of a scan CTA (plus one producer warp: 256 threads), each with a partial of its own
 #define CKV_MAX_SCAN_CTAS 160 // persistent scan grid is capped at this many CTAs
 #define CKV_MAX_SPLITS 64     // attention partials per unit
+#define CKV_STEP_MAX_CLUSTER 16   // CTAs of a unit in the one-launch step, at most (the opt-in cluster size of sm_100)
+#define CKV_STEP_MIN_TOKENS 1536  // shorter caches keep the separate launches (see ckv_unit_step_plan)
+#define CKV_LEN_COUNTER_WORD 16   // word of the status region that counts who has read the lengths in a fused step
 #define CKV_RESCALE_SLACK 16.0f  // log2 units: running maxima are only raised when exceeded by this much
 
 constexpr float kLog2e = 1.4426950408889634f;
@@ -59,6 +62,15 @@ struct CkvDev {
   int debug;         // ckv_debug_flags (test hooks; 0 in normal use)
 };
 
+// How a step runs as one launch (ckv_unit_step_plan).
+struct CkvStepPlan {
+  int cluster;      // CTAs per unit
+  int stages;       // ring stages of the scan phase
+  int own_cap;      // blocks of a unit one CTA owns, at most (a multiple of 16)
+  int u_off, smem;  // offset of the score terms in dynamic shared memory, and its size
+  int max_blocks;   // blocks of a sequence by the host's bound on the lengths
+};
+
 struct ckv_ctx {
   ckv_layout layout;
   CkvDev dev;
@@ -69,6 +81,7 @@ struct ckv_ctx {
   int64_t launches;
   int sm_count;
   int tail_mode;   // ckv_tail_mode
+  int step_clusters[CKV_STEP_MAX_CLUSTER + 1];   // clusters of each size the device holds at once (one-launch step)
   CUtensorMap tm_vhi;   // vhi: the mean-values region as rows of 128 bf16 (the hi halves) 512 bytes apart, boxes of 64 rows
   volatile int *host_flag;   // pinned word ckv_step_host waits on (null: stream synchronisation instead)
   int *host_flag_dev;        // the same word as the device sees it
@@ -90,6 +103,7 @@ cudaError_t ckv_launch_attn_mma(ckv_ctx *c, bool dense, const void *q, const voi
                                 const int *page_table, const int *seq_lens, const int *sel_ids, const int *sel_cnt,
                                 int kcap, dim3 grid, int pps, int scan_grid, void *out, float *lse, cudaStream_t st);
 int ckv_scan_grid(const ckv_ctx *c, int batch, int max_len);
+cudaError_t ckv_configure_unit_step(ckv_ctx *c);   // one-launch step: kernel attributes, co-resident clusters by size
 
 // ---- launchers (one per translation unit) ---------------------------------------------------------
 cudaError_t ckv_launch_stats_build(ckv_ctx *c, const void *k_pool, const void *v_pool, const int *page_table,
@@ -107,6 +121,11 @@ struct CkvNewToken {
   int *seq_lens;              // read as the lengths before the append; holds the new lengths when the launch is over
   const void *k_new, *v_new;  // [batch][Hkv][128]
 };
+// The whole step in one launch, where it pays: plan (false: it does not apply) and launch.
+bool ckv_unit_step_plan(const ckv_ctx *c, int batch, int max_len, int kcap, CkvStepPlan *plan);
+cudaError_t ckv_launch_unit_step(ckv_ctx *c, const CkvStepPlan &plan, const void *q, const void *k_pool, const void *v_pool,
+                                 const int *page_table, const int *seq_lens, const CkvNewToken *fresh, int batch, int kcap,
+                                 int *sel_ids, int *sel_cnt, void *out, float *lse, cudaStream_t st);
 // max_len is an upper bound of the lengths the step works on (after the append, if there is one).  The launch
 // follows c->dev.tail; a new token needs tail mode.
 cudaError_t ckv_launch_scan(ckv_ctx *c, const void *q, const int *seq_lens, int batch, int max_len,

@@ -41,20 +41,12 @@
 #include "ckv_pipe.cuh"
 #include "ckv_mma.cuh"
 #include "ckv_blockstats.cuh"
+#include "ckv_scanpart.cuh"
 
 namespace {
 
 using namespace ckv_pipe;
 
-template <bool WIDE> struct ScanTile { static constexpr int TB = WIDE ? CKV_SCAN_TILE_HS : CKV_SCAN_TILE; };   // blocks per tile
-
-// One box of a tensor map from global to shared memory (x: first element of the row, y: first row); completion is
-// counted on `bar` in bytes -- always the whole box, rows past the tensor's end arriving as zeros.
-__device__ __forceinline__ void tensor_g2s(uint32_t dst, const CUtensorMap *map, int x, int y, uint64_t *bar) {
-  asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
-               "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(ckv_pipe::smem_u32(bar))
-               : "memory");
-}
 constexpr int kMaxStages = 8;
 constexpr int kConsumerWarps = CKV_SCAN_WARPS;
 constexpr int kThreads = kConsumerWarps * 32 + 32;   // plus the producer warp
@@ -79,7 +71,7 @@ __device__ __forceinline__ int seq_tiles(const int *s_len, const int *__restrict
   return (ckv_scan_blocks(P, seq_len_of(P, s_len, seq_lens, i)) + P.scan_tile - 1) >> P.lg_tile;
 }
 
-constexpr int kLenCounter = 16;   // word of the status region that counts the CTAs which have read the lengths
+constexpr int kLenCounter = CKV_LEN_COUNTER_WORD;   // counts the CTAs which have read the lengths
 
 // Length hand-over of a fused step.  Every CTA of the launch works with the lengths as they were before the
 // append (plus one); a CTA calls this once it will not read the length array again, and the last one to call
@@ -262,9 +254,6 @@ __device__ __noinline__ void scan_tail(const CkvDev P, const QT *__restrict__ q,
   }
 }
 
-template <typename QT> struct QSplit { static constexpr bool value = false; };
-template <> struct QSplit<float> { static constexpr bool value = true; };
-
 // RD: one variance group per coordinate (r = d).  The variance rows then have the mean rows' layout and
 // sigma^2 = sum_i (scale q_i)^2 Dbar_i is a third tensor-core product, with the squared queries as the A operand.
 // HS: the mean rows hold hi halves only (bf16 summaries, 256-byte rows); every product with a lo plane drops out.
@@ -424,8 +413,6 @@ ckv_scan_kernel(CkvDev P, const QT *__restrict__ q, const int *seq_lens, int uni
     const int head = lane >> 2, qd = lane & 3;   // this thread's accumulator row (head) and column pair
     const bool hv = head < G;
     constexpr bool SP = (G <= 4) && !RD;   // the per-(head, block) arithmetic is shared between the half warps
-    constexpr int NE = SP ? 1 : 2;          // n-tiles a lane works on there
-    const int hsel = lane >> 4;             // ... and which one: the lower half warp the first, the upper the second
     const int ehead = SP ? (head & 3) : head;
     const bool ehv = ehead < G;
     const bool staged = !QS && !RD && P.r == 4;   // bf16 queries, four variance groups: the staged setup below
@@ -455,14 +442,13 @@ ckv_scan_kernel(CkvDev P, const QT *__restrict__ q, const int *seq_lens, int uni
       }
       named_barrier(1, kConsumerWarps * 32);
     }
-    uint32_t qa[8][2], qb[QS ? 8 : 1][2];        // A fragments of the unit's queries (rows 0..7), per 16-coordinate step
-    uint32_t qsh[RD ? 8 : 1][2], qsl[RD ? 8 : 1][2];   // (scale q)^2 as hi and lo halves, same fragment positions
-    float acc[16][2];                            // W Vbar accumulator: head `head`, coordinates 8 t + 2 qd + {0, 1}
-    float m_ref = -CUDART_INF_F, l_acc = 0.f, lp_acc = 0.f;
-    float wown[4] = {0.f, 0.f, 0.f, 0.f};
+    ScanUnit<G, QT, RD> w;
+    w.reset();
+#pragma unroll
+    for (int t = 0; t < 4; ++t) w.wown[t] = 0.f;
     float *sw = sw_all + (size_t)warp * P.r * G;   // [t][g], r != 4 only
-    const float log_bs = logf((float)P.bs);
-    const bool by_mass = (P.variant & CKV_VARIANT_RANK_BY_MASS) != 0;
+    const ScanPartCfg cfg{P.scale, P.half_var, logf((float)P.bs), P.r, P.max_blocks,
+                          (P.variant & CKV_VARIANT_RANK_BY_MASS) != 0, r4};
     float log_last = 0.f;   // log of the token count of the unit's last block, when the scan CTAs cover it
     const bool pair_ok = (P.max_blocks & 1) == 0;   // rows of the per-block outputs start on 8-byte boundaries
     const int ulast = s_ulast;
@@ -483,7 +469,7 @@ ckv_scan_kernel(CkvDev P, const QT *__restrict__ q, const int *seq_lens, int uni
         return;
       }
       // l and lp: sum over the four lanes that share the head
-      float l = l_acc, lp = lp_acc;
+      float l = w.l_acc, lp = w.lp_acc;
       l += __shfl_xor_sync(0xffffffffu, l, 1); l += __shfl_xor_sync(0xffffffffu, l, 2);
       lp += __shfl_xor_sync(0xffffffffu, lp, 1); lp += __shfl_xor_sync(0xffffffffu, lp, 2);
       if (SP) { l += __shfl_xor_sync(0xffffffffu, l, 16); lp += __shfl_xor_sync(0xffffffffu, lp, 16); }
@@ -491,8 +477,8 @@ ckv_scan_kernel(CkvDev P, const QT *__restrict__ q, const int *seq_lens, int uni
         float *pg = part + head * CKV_PART_STRIDE;
 #pragma unroll
         for (int t = 0; t < 16; ++t)
-          *reinterpret_cast<float2 *>(pg + 4 + 8 * t + 2 * qd) = make_float2(acc[t][0], acc[t][1]);
-        if (qd == 0) { pg[0] = m_ref; pg[1] = l; pg[2] = lp; }
+          *reinterpret_cast<float2 *>(pg + 4 + 8 * t + 2 * qd) = make_float2(w.acc[t][0], w.acc[t][1]);
+        if (qd == 0) { pg[0] = w.m_ref; pg[1] = l; pg[2] = lp; }
       }
     };
     // units of this CTA's range that this warp never worked on still need an (empty) partial
@@ -546,9 +532,9 @@ ckv_scan_kernel(CkvDev P, const QT *__restrict__ q, const int *seq_lens, int uni
 #pragma unroll
           for (int ks = 0; ks < 8; ++ks)
 #pragma unroll
-            for (int hh = 0; hh < 2; ++hh) qa[ks][hh] = hv ? srow[(16 * ks + 8 * hh + 2 * qd) / 2] : 0u;
+            for (int hh = 0; hh < 2; ++hh) w.qa[ks][hh] = hv ? srow[(16 * ks + 8 * hh + 2 * qd) / 2] : 0u;
 #pragma unroll
-          for (int t = 0; t < 4; ++t) wown[t] = ehv ? s_w[uk][ehead][t] : 0.f;
+          for (int t = 0; t < 4; ++t) w.wown[t] = ehv ? s_w[uk][ehead][t] : 0.f;
         } else {
 #pragma unroll
         for (int ks = 0; ks < 8; ++ks) {
@@ -556,12 +542,12 @@ ckv_scan_kernel(CkvDev P, const QT *__restrict__ q, const int *seq_lens, int uni
           for (int hh = 0; hh < 2; ++hh) {
             const int c0 = 16 * ks + 8 * hh + 2 * qd;
             const float x0 = hv ? to_float(qrow[c0]) : 0.f, x1 = hv ? to_float(qrow[c0 + 1]) : 0.f;
-            qa[ks][hh] = pack_bf16(x0, x1);
-            if (QS) qb[QS ? ks : 0][hh] = pack_bf16(x0 - bf16_round(x0), x1 - bf16_round(x1));
+            w.qa[ks][hh] = pack_bf16(x0, x1);
+            if (QS) w.qb[QS ? ks : 0][hh] = pack_bf16(x0 - bf16_round(x0), x1 - bf16_round(x1));
             if (RD) {
               const float s0 = (x0 * P.scale) * (x0 * P.scale), s1 = (x1 * P.scale) * (x1 * P.scale);
-              qsh[RD ? ks : 0][hh] = pack_bf16(s0, s1);
-              qsl[RD ? ks : 0][hh] = pack_bf16(s0 - bf16_round(s0), s1 - bf16_round(s1));
+              w.qsh[RD ? ks : 0][hh] = pack_bf16(s0, s1);
+              w.qsl[RD ? ks : 0][hh] = pack_bf16(s0 - bf16_round(s0), s1 - bf16_round(s1));
             }
           }
         }
@@ -588,22 +574,20 @@ ckv_scan_kernel(CkvDev P, const QT *__restrict__ q, const int *seq_lens, int uni
           }
           if (!ehv) { wsum[0] = wsum[1] = wsum[2] = wsum[3] = 0.f; }
 #pragma unroll
-          for (int t = 0; t < 4; ++t) wown[t] = wsum[t] * (P.scale * P.scale);   // Eq. 8's 1/d is the squared logit scale
+          for (int t = 0; t < 4; ++t) w.wown[t] = wsum[t] * (P.scale * P.scale);   // Eq. 8's 1/d is the squared logit scale
         } else {
           __syncwarp();
           for (int idx = lane; idx < P.r * G; idx += 32) {
             const int t = idx / G, g = idx % G;
             const QT *qg = q + ((size_t)s * P.Hq + h * G + g) * CKV_D;
-            float w = 0.f;
+            float ws = 0.f;
             for (int i = 0; i < CKV_D; ++i)
-              if (group_of(i, P.r, P.glayout) == t) { const float x = to_float(qg[i]); w = fmaf(x, x, w); }
-            sw[idx] = w * (P.scale * P.scale);
+              if (group_of(i, P.r, P.glayout) == t) { const float x = to_float(qg[i]); ws = fmaf(x, x, ws); }
+            sw[idx] = ws * (P.scale * P.scale);
           }
           __syncwarp();
         }
-#pragma unroll
-        for (int t = 0; t < 16; ++t) { acc[t][0] = 0.f; acc[t][1] = 0.f; }
-        m_ref = -CUDART_INF_F; l_acc = 0.f; lp_acc = 0.f;
+        w.reset();
         log_last = logf((float)(ui.N - (ui.X - 1) * P.bs));
         const size_t row0 = (size_t)u * P.max_blocks;
         lu = P.lu + row0 * G;   // [head][block] within the unit
@@ -619,183 +603,20 @@ ckv_scan_kernel(CkvDev P, const QT *__restrict__ q, const int *seq_lens, int uni
         const uint32_t sv = sk + TB * kRowBytes;
         const float *sd = reinterpret_cast<const float *>(stage_mem + (size_t)st * stage_bytes + TB * (kRowBytes + kRowBytesV));
 
-        // ---- Z^T = Q Kbar^T: heads x 16 blocks (two n-tiles of 8 blocks), hi and lo planes into one accumulator ----
-        // four accumulation chains per n-tile (hi / lo plane x even / odd 16-coordinate step): the products of a chain
-        // depend on one another, and a warp has little else to issue while it waits for them
-        float z[2][2] = {{0.f, 0.f}, {0.f, 0.f}}, zlo[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
-        float z2[2][2] = {{0.f, 0.f}, {0.f, 0.f}}, zlo2[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
-        {
-          // ldmatrix lane roles: matrix lane / 8 -> 8-coordinate chunk, row lane % 8
-          const int lrow = lane & 7, lmat = lane >> 3;
-#pragma unroll
-          for (int nt = 0; nt < 2; ++nt) {
-            const int r = rb + nt * 8 + lrow;
-            const uint32_t rowaddr = sk + r * kRowBytes;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {   // two 16-coordinate steps per ldmatrix.x4
-              const uint32_t coff = (uint32_t)swz_chunk(4 * j + lmat, r) * 16;
-              uint32_t bh[4], bl[4];
-              ldmatrix_x4(bh, rowaddr + coff);
-              mma_rows8(z[nt][0], z[nt][1], qa[2 * j][0], qa[2 * j][1], bh[0], bh[1]);
-              mma_rows8(z2[nt][0], z2[nt][1], qa[2 * j + 1][0], qa[2 * j + 1][1], bh[2], bh[3]);
-              if (!HS) {
-                ldmatrix_x4(bl, rowaddr + 256 + coff);
-                mma_rows8(zlo[nt][0], zlo[nt][1], qa[2 * j][0], qa[2 * j][1], bl[0], bl[1]);
-                mma_rows8(zlo2[nt][0], zlo2[nt][1], qa[2 * j + 1][0], qa[2 * j + 1][1], bl[2], bl[3]);
-              }
-              if (QS) {
-                mma_rows8(zlo[nt][0], zlo[nt][1], qb[QS ? 2 * j : 0][0], qb[QS ? 2 * j : 0][1], bh[0], bh[1]);
-                mma_rows8(zlo[nt][0], zlo[nt][1], qb[QS ? 2 * j + 1 : 0][0], qb[QS ? 2 * j + 1 : 0][1], bh[2], bh[3]);
-              }
-            }
-            z[nt][0] = (z[nt][0] + z2[nt][0]) + (zlo[nt][0] + zlo2[nt][0]);
-            z[nt][1] = (z[nt][1] + z2[nt][1]) + (zlo[nt][1] + zlo2[nt][1]);
-          }
-        }
-        float sgm[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
-        if (RD) {   // sigma^2 for the same heads x blocks tile: (qs_hi + qs_lo) (D_hi + D_lo) without the lo lo term
-          float sg2[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
-          const uint32_t sdr = sv + TB * kRowBytes;
-          const int lrow = lane & 7, lmat = lane >> 3;
-#pragma unroll
-          for (int nt = 0; nt < 2; ++nt) {
-            const int r = rb + nt * 8 + lrow;
-            const uint32_t rowaddr = sdr + r * kRowBytes;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              const uint32_t coff = (uint32_t)swz_chunk(4 * j + lmat, r) * 16;
-              uint32_t dh[4], dl[4];
-              ldmatrix_x4(dh, rowaddr + coff);
-              ldmatrix_x4(dl, rowaddr + 256 + coff);
-              mma_rows8(sgm[nt][0], sgm[nt][1], qsh[RD ? 2 * j : 0][0], qsh[RD ? 2 * j : 0][1], dh[0], dh[1]);
-              mma_rows8(sgm[nt][0], sgm[nt][1], qsh[RD ? 2 * j + 1 : 0][0], qsh[RD ? 2 * j + 1 : 0][1], dh[2], dh[3]);
-              mma_rows8(sg2[nt][0], sg2[nt][1], qsl[RD ? 2 * j : 0][0], qsl[RD ? 2 * j : 0][1], dh[0], dh[1]);
-              mma_rows8(sg2[nt][0], sg2[nt][1], qsl[RD ? 2 * j + 1 : 0][0], qsl[RD ? 2 * j + 1 : 0][1], dh[2], dh[3]);
-              mma_rows8(sg2[nt][0], sg2[nt][1], qsh[RD ? 2 * j : 0][0], qsh[RD ? 2 * j : 0][1], dl[0], dl[1]);
-              mma_rows8(sg2[nt][0], sg2[nt][1], qsh[RD ? 2 * j + 1 : 0][0], qsh[RD ? 2 * j + 1 : 0][1], dl[2], dl[3]);
-            }
-            sgm[nt][0] += sg2[nt][0]; sgm[nt][1] += sg2[nt][1];
-          }
-        }
-
-        // ---- per (head, block): variance projection, l, running maximum, compensation weight ----
-        // The products leave this part's 16 blocks x G heads in the lanes of rows 0..G-1 (four values per lane).
-        // With G <= 4 those are lanes 0-15 only, so the upper half warp takes over the second n-tile: every lane
-        // then works on one n-tile's pair of blocks (half the dependent chain), and the weights travel back to
-        // the lower lanes, which hold the A operand of the next product.
-        float zin[NE][2];
-        if constexpr (SP) {
-          const float t0 = __shfl_sync(0xffffffffu, z[1][0], lane & 15), t1 = __shfl_sync(0xffffffffu, z[1][1], lane & 15);
-          zin[0][0] = hsel ? t0 : z[0][0];
-          zin[0][1] = hsel ? t1 : z[0][1];
-        } else {
-#pragma unroll
-          for (int k = 0; k < NE; ++k) { zin[k][0] = z[k][0]; zin[k][1] = z[k][1]; }
-        }
-        float zl2[NE][2], sig[NE][2], wt[NE][2];
-        bool val[NE][2];
-        float tmax = -CUDART_INF_F;
-#pragma unroll
-        for (int k = 0; k < NE; ++k) {
-          const int nt = SP ? hsel : k;
-          const int r0 = rb + nt * 8 + 2 * qd;     // this thread's two blocks of the n-tile: rows r0, r0 + 1
-          float ell[2];
-#pragma unroll
-          for (int e = 0; e < 2; ++e) {
-            const int r = r0 + e, b = b0 + r;
-            val[k][e] = ehv && r < nb;
-            float sg = 0.f;
-            if (val[k][e]) {
-              if (RD) {
-                sg = fmaxf(sgm[RD ? k : 0][e], 0.f);
-              } else if (r4) {
-                const float4 dv = *reinterpret_cast<const float4 *>(sd + r * 4);
-                sg = fmaf(wown[0], dv.x, fmaf(wown[1], dv.y, fmaf(wown[2], dv.z, wown[3] * dv.w)));
+        scan_part<G, QT, RD, HS, VH>(
+            w, cfg, sk, sv, (RD || r4 || dbar_bulk) ? sd : nullptr, smem_u32(s_zero_row), sw, db, lane, rb, nb, b0,
+            P.tail ? -1 : ui.X - 1, log_last,   // in tail mode every block here is full
+            [&](int eh, int blk, float u0, float u1, float z0, float z1, bool v0, bool v1) {
+              // the thread's two blocks are neighbours: one 8-byte store each when the rows are 8-byte aligned
+              const size_t o = (size_t)eh * P.max_blocks + blk;
+              if (pair_ok && v1) {
+                *reinterpret_cast<float2 *>(lu + o) = make_float2(u0, u1);
+                *reinterpret_cast<float2 *>(lz + o) = make_float2(z0, z1);
               } else {
-                for (int t = 0; t < P.r; ++t) {
-                  const float dv = dbar_bulk ? sd[r * P.r + t] : __ldg(db + (size_t)b * P.r + t);
-                  sg = fmaf(sw[t * G + ehead], dv, sg);
-                }
+                if (v0) { lu[o] = u0; lz[o] = z0; }
+                if (v1) { lu[o + 1] = u1; lz[o + 1] = z1; }
               }
-            }
-            sig[k][e] = sg;
-            const float zbar = zin[k][e] * P.scale;
-            const float logc = (!P.tail && b == ui.X - 1) ? log_last : log_bs;   // in tail mode every block here is full
-            ell[e] = logc + zbar + P.half_var * sg;
-            zl2[k][e] = val[k][e] ? (zbar + logc) * kLog2e : -CUDART_INF_F;   // log2 of |b| e^{zbar}
-            tmax = fmaxf(tmax, zl2[k][e]);
-          }
-          // what the later kernels read, both in log2 units: the head's term of the block score, e^l sigma^2 (e^l
-          // alone when blocks are ranked by mass), and the block's mean-compensation weight |b| e^{zbar}.  The
-          // thread's two blocks are neighbours: one 8-byte store each when the rows are 8-byte aligned.
-          const size_t o = (size_t)ehead * P.max_blocks + b0 + r0;
-          const float u0 = fmaf(ell[0], kLog2e, by_mass ? 0.f : __log2f(sig[k][0]));
-          const float u1 = fmaf(ell[1], kLog2e, by_mass ? 0.f : __log2f(sig[k][1]));
-          if (pair_ok && val[k][1]) {
-            *reinterpret_cast<float2 *>(lu + o) = make_float2(u0, u1);
-            *reinterpret_cast<float2 *>(lz + o) = make_float2(zl2[k][0], zl2[k][1]);
-          } else {
-            if (val[k][0]) { lu[o] = u0; lz[o] = zl2[k][0]; }
-            if (val[k][1]) { lu[o + 1] = u1; lz[o + 1] = zl2[k][1]; }
-          }
-        }
-        tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, 1));
-        tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, 2));
-        if (SP) tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, 16));
-        if (tmax > m_ref + CKV_RESCALE_SLACK) {   // the running maximum is only raised when exceeded by a slack
-          const float sc = exp2_diff(m_ref, tmax);
-          m_ref = tmax;
-          l_acc *= sc; lp_acc *= sc;
-#pragma unroll
-          for (int t = 0; t < 16; ++t) { acc[t][0] *= sc; acc[t][1] *= sc; }
-        }
-        uint32_t whm[NE], wlm[NE];
-#pragma unroll
-        for (int k = 0; k < NE; ++k) {
-#pragma unroll
-          for (int e = 0; e < 2; ++e) {
-            wt[k][e] = val[k][e] ? fast_exp2(zl2[k][e] - m_ref) : 0.f;
-            l_acc += wt[k][e];
-            lp_acc = fmaf(wt[k][e], fast_exp2(P.half_var * kLog2e * sig[k][e]), lp_acc);   // e^{l - m} = e^{zbar + log|b| - m} e^{sigma^2/2}
-          }
-          whm[k] = pack_bf16(wt[k][0], wt[k][1]);
-          wlm[k] = pack_bf16(wt[k][0] - bf16_round(wt[k][0]), wt[k][1] - bf16_round(wt[k][1]));
-        }
-        uint32_t wh[2], wl[2];   // A fragments of the weights: k = blocks 2 qd + {0, 1} (+ 8), hi and lo halves
-        if constexpr (SP) {
-          // rows 0..3 (lanes 0-15) get their second n-tile from the lane 16 above; rows 4..7 carry zero weights
-          const uint32_t oh = __shfl_sync(0xffffffffu, whm[0], (lane & 15) + 16);
-          const uint32_t ol = __shfl_sync(0xffffffffu, wlm[0], (lane & 15) + 16);
-          wh[0] = hsel ? 0u : whm[0]; wl[0] = hsel ? 0u : wlm[0];
-          wh[1] = hsel ? 0u : oh;     wl[1] = hsel ? 0u : ol;
-        } else {
-#pragma unroll
-          for (int k = 0; k < NE; ++k) { wh[k] = whm[k]; wl[k] = wlm[k]; }
-        }
-
-        // ---- acc += W Vbar: heads x 128 coordinates, k = this half tile's 16 blocks ----
-        {
-          // ldmatrix.trans lane roles: matrix lane / 8 -> (block half, coordinate chunk parity), row lane % 8
-          const int r = rb + ((lane >> 3) & 1) * 8 + (lane & 7);
-          const bool real = r < nb;   // rows past the unit's last block: zeros
-          const uint32_t rowaddr = real ? sv + r * kRowBytesV : smem_u32(s_zero_row);
-          const int cpar = lane >> 4;
-#pragma unroll
-          for (int t2 = 0; t2 < 8; ++t2) {   // two 8-coordinate n-tiles per ldmatrix.x4
-            const uint32_t coff = real ? (uint32_t)swz_chunk(2 * t2 + cpar, r) * 16 : 0u;
-            uint32_t vh[4], vl[4];
-            ldmatrix_x4_trans(vh, rowaddr + coff);
-            mma_rows8(acc[2 * t2][0], acc[2 * t2][1], wh[0], wh[1], vh[0], vh[1]);
-            mma_rows8(acc[2 * t2][0], acc[2 * t2][1], wl[0], wl[1], vh[0], vh[1]);
-            mma_rows8(acc[2 * t2 + 1][0], acc[2 * t2 + 1][1], wh[0], wh[1], vh[2], vh[3]);
-            mma_rows8(acc[2 * t2 + 1][0], acc[2 * t2 + 1][1], wl[0], wl[1], vh[2], vh[3]);
-            if (!HS && !VH) {
-              ldmatrix_x4_trans(vl, rowaddr + (real ? 256u : 0u) + coff);
-              mma_rows8(acc[2 * t2][0], acc[2 * t2][1], wh[0], wh[1], vl[0], vl[1]);
-              mma_rows8(acc[2 * t2 + 1][0], acc[2 * t2 + 1][1], wh[0], wh[1], vl[2], vl[3]);
-            }
-          }
-        }
+            });
       }
       }   // own part
       __syncwarp();

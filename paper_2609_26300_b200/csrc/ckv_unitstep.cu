@@ -1,0 +1,1004 @@
+// One decode step (append, scan, selection, attention, merge: Eq. 8-12) in ONE launch: a thread-block cluster per unit.
+//
+// A step of a few sequences is bound by latency, not by bytes: as four launches (append, scan, select, attention) the
+// 32K single-sequence step spends 28 us in kernels that move 17 MB and 7 us between them, every stage paying its own
+// launch, its own cold start and a trip of its results through global memory.  The units of a step are independent, so
+// one cluster can take a unit from the new token to the output row: its CTAs share out the unit's blocks, exchange the
+// little that crosses blocks (normalisers, block scores, partial outputs) through distributed shared memory, and
+// nothing waits for another unit.  A cluster barrier costs 0.1 us here, a launch about 2 us.
+//
+// CTA `rank` of the cluster owns a contiguous range of the unit's blocks (all but the last one), in 16-block parts:
+//   1. scan: a producer thread streams the range's summaries into a ring of shared-memory stages, eight warps work on
+//      parts (scan_part, shared with the persistent scan kernel); the score terms stay in shared memory.  Meanwhile one
+//      warp of the last CTA appends the new token, redoes the last block's summary and computes its terms.
+//   2. every CTA sends its normaliser partials (M_g, L_g) to all, then the block scores of its own range: every CTA holds
+//      all scores of the unit.  Both exchanges are asynchronous stores counted on an mbarrier of the receiver: a cluster
+//      barrier with release semantics would wait for the scan's stores to global memory as well (1.4 us instead of 0.6).
+//   3. selection, redundantly in every CTA: a histogram over the scores' bit patterns relative to an upper bound of them
+//      (64 bins per octave, 32 octaves), the exact cut by ranking the one bin that holds it (by bisection when that bin
+//      is crowded or the cut lies below the histogram), a bit map of the selected blocks, and their ids in position order
+//      from a prefix sum over its words.  All CTAs get the same list without another exchange.
+//   4. exact attention over the CTA's share of the list, a warp per page, into the SAME accumulators that hold the
+//      compensation sums of step 1 (both are online-softmax sums over the same heads); the selected blocks' mean terms
+//      are taken out through the tokens' weights, or with bf16 summaries as one more product over the stored rows.
+//   5. the CTA's partial is reduced over its warps and sent to the CTAs that reduce it over the cluster; output.
+//
+// The cluster size follows from what the device can hold at once (the number of co-resident clusters by size is asked
+// of the driver when a context is created): the largest size for which all units run in one wave.  72 SMs already
+// stream at the full HBM rate (206 MB: 6.28 TB/s with 72, 96, 120 or 148 CTAs alike), so 8 units in clusters of 10 lose
+// nothing against 148 CTAs.
+#include <algorithm>
+#include <mutex>
+
+#include "ckv_internal.cuh"
+#include "ckv_pipe.cuh"
+#include "ckv_mma.cuh"
+#include "ckv_cluster.cuh"
+#include "ckv_blockstats.cuh"
+#include "ckv_scanpart.cuh"
+#include "ckv_attnpage.cuh"
+
+namespace {
+
+using namespace ckv_pipe;
+using bf16 = __nv_bfloat16;
+
+constexpr int kWarps = 8;                       // warps that work on parts and pages
+constexpr int kWork = kWarps * 32;              // ... and their threads
+constexpr int kProducerWarp = kWarps, kTailWarp = kWarps + 1;
+constexpr int kThreads = (kWarps + 2) * 32;
+constexpr int kClusterCap = CKV_STEP_MAX_CLUSTER;
+constexpr int kStagesCap = 6;
+constexpr int kScoresCap = 9216;                // blocks of a unit whose scores every CTA can hold
+constexpr int kBins = 2048;                     // score histogram: 32 octaves below the largest possible score, 64 bins each
+constexpr int kBinShift = 17;                   // ... a bin is a score's bit pattern without its low 17 bits
+constexpr int kMapWords = 2 * kWork;            // selection bit map: two words per working thread, enough for kScoresCap blocks
+constexpr int kSelCap = 512;                    // selected blocks the id list holds (unless every block is selected)
+constexpr int kCandCap = kWork;                 // blocks of the cut's bin that are ranked directly, one per thread
+// shared memory once the ring is drained
+constexpr int kOffHist = kScoresCap * 4;
+constexpr int kOffMap = kOffHist + (kBins + 32) * 4;          // (cleared together with the histogram)
+constexpr int kOffIds = kOffMap + kMapWords * 4;
+constexpr int kOffCand = kOffIds + kSelCap * 4;
+constexpr int kOffPages = (kOffCand + kCandCap * 8 + 127) / 128 * 128;
+constexpr int kAfterScan = kOffPages + kWarps * 2 * kPageBytes;
+constexpr int kRecvStride = 36;                 // floats of one (head, 32 coordinates) partial: values, maximum, weight sum
+constexpr int kDynLimit = 227 * 1024 - 20 * 1024;   // dynamic shared memory; the kernel's static arrays take under 20 KB
+
+__device__ __forceinline__ void work_barrier() { named_barrier(1, kWork); }
+
+// Exclusive prefix sum of one int per working thread (one barrier; s_wt is not to be reused before the next one).
+__device__ __forceinline__ int work_exclusive_scan(int v, int *s_wt) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int inc = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += t;
+  }
+  if (lane == 31) s_wt[warp] = inc;
+  work_barrier();
+  int before = 0;
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w) before += w < warp ? s_wt[w] : 0;
+  return before + inc - v;
+}
+// Sum of one int per working thread.
+__device__ __forceinline__ int work_sum(int v, int *s_wt) {
+  const int w = (int)__reduce_add_sync(0xffffffffu, (unsigned)v);
+  if ((threadIdx.x & 31) == 0) s_wt[threadIdx.x >> 5] = w;
+  work_barrier();
+  int all = 0;
+#pragma unroll
+  for (int i = 0; i < kWarps; ++i) all += s_wt[i];
+  work_barrier();
+  return all;
+}
+
+// The cut when the bin that holds it is crowded (many equal or nearly equal scores) or lies below the histogram: the
+// kr-th largest ranked key by bisection over its bits, then the last of the equal keys that is taken, by bisection over
+// the block ids.  About 45 counting passes; all of a unit's scores being equal is the usual reason to come here.
+__device__ __noinline__ void cut_by_bisection(int X, int kr, const uint32_t *keys, int rank_lo, int rank_n, int *s_wt,
+                                              uint32_t &cut_key, int &cut_id) {
+  auto key_of = [keys](int b) { return keys[b]; };
+  auto ranked = [rank_lo, rank_n](int b) { return (unsigned)(b - rank_lo) < (unsigned)rank_n; };
+  uint32_t lo = 0, hi = 0x7f800000u;   // count(key >= lo) >= kr, count(key >= hi) < kr
+  while (hi - lo > 1) {
+    const uint32_t mid = lo + (hi - lo) / 2;
+    int c = 0;
+    for (int b = threadIdx.x; b < X; b += kWork) c += (ranked(b) && key_of(b) >= mid) ? 1 : 0;
+    if (work_sum(c, s_wt) >= kr) lo = mid; else hi = mid;
+  }
+  int above = 0;
+  for (int b = threadIdx.x; b < X; b += kWork) above += (ranked(b) && key_of(b) > lo) ? 1 : 0;
+  const int need = kr - work_sum(above, s_wt);   // equal keys taken, lowest ids first
+  int l = -1, h = X - 1;                         // count(equal, id <= l) < need, count(equal, id <= h) >= need
+  while (h - l > 1) {
+    const int mid = (l + h) / 2;
+    int c = 0;
+    for (int b = threadIdx.x; b <= mid; b += kWork) c += (ranked(b) && key_of(b) == lo) ? 1 : 0;
+    if (work_sum(c, s_wt) >= need) h = mid; else l = mid;
+  }
+  cut_key = lo; cut_id = h;
+}
+
+// The last CTA's tail warp: the new token (if there is one) goes into its page and the last block's summary is redone
+// with the append's own routine; then, new token or not, the last block's two per-head terms and its compensation
+// partial, with plain FMAs, from the summary as stored (a fresh one is taken from the registers it was stored from).
+template <int G>
+__device__ __noinline__ void tail_block(const CkvDev P, const bf16 *sq_rows, const int *page_table, const CkvNewToken fresh,
+                                        int unit, int raw, int N, float *sq, float *tail_u, float *tail_part, float4 *norm) {
+  const int lane = threadIdx.x & 31, hw = lane >> 4, li = lane & 15;
+  const int s = ckv_div_hkv(P, unit), h = unit - s * P.Hkv;
+  const int cap = P.max_blocks * P.bs;
+  const bool lo_half = P.row_elems == CKV_ROW_ELEMS;
+  const bool by_mass = (P.variant & CKV_VARIANT_RANK_BY_MASS) != 0;
+  const int *pt_row = page_table + (size_t)s * P.max_pages_per_seq;
+  BlockRow br;
+  bool fresh_row = false;
+  if (fresh.k_new != nullptr) {
+    if (raw < 0 || raw >= cap) {
+      if (lane == 0) atomicOr(P.status, CKV_DEV_SEQ_FULL);
+    } else {
+      bf16 *kp = reinterpret_cast<bf16 *>(fresh.k_pool), *vp = reinterpret_cast<bf16 *>(fresh.v_pool);
+      const bf16 *row_new = reinterpret_cast<const bf16 *>(lane < 16 ? fresh.k_new : fresh.v_new) + (size_t)unit * CKV_D;
+      const uint4 piece = __ldg(reinterpret_cast<const uint4 *>(row_new) + li);
+      const int phys = pt_row[raw / CKV_PAGE];
+      const int b = raw >> P.lg_bs, cnt = raw + 1 - b * P.bs;
+      if (phys >= 0 && phys < P.num_pages)
+        reinterpret_cast<uint4 *>((lane < 16 ? kp : vp) + (((size_t)phys * P.Hkv + h) * CKV_PAGE + raw % CKV_PAGE) * CKV_D)[li] = piece;
+      __syncwarp();
+      const size_t row = (size_t)unit * P.max_blocks + b;
+      block_stats_warp<bf16, false>(P, kp, vp, pt_row, h, b, cnt, sq, P.kmean + row * P.row_elems, P.dbar + row * P.r,
+                                    P.vmean + row * P.row_elems, lane, &br);
+      fresh_row = true;
+    }
+  }
+  const int b = ((N + P.bs - 1) >> P.lg_bs) - 1, cnt = N - b * P.bs;
+  const size_t row = (size_t)unit * P.max_blocks + b;
+  if (!fresh_row) {   // the summary as stored: lower half warp the mean key, upper the mean value (as the scan reads it)
+    load_split8<false>((hw == 0 ? P.kmean : P.vmean) + row * P.row_elems, li, b, br.x, lo_half && !(hw == 1 && P.vhi));
+    if (P.r == CKV_D) {
+      load_split8<false>(reinterpret_cast<const bf16 *>(P.dbar + row * CKV_D), li, b, br.dvar);
+    } else {
+      const float *drow = P.dbar + row * P.r;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) br.dvar[i] = drow[group_of(8 * li + i, P.r, P.glayout)];
+    }
+  }
+  const float logc = logf((float)cnt);
+#pragma unroll
+  for (int g = 0; g < G; ++g) {
+    float qx[8];
+    load8<false>(sq_rows + g * CKV_D + 8 * li, qx);
+    float d = 0.f, sg = 0.f;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      d = fmaf(qx[i], br.x[i], d);   // (meaningful in the lower half warp, which holds the mean key)
+      const float qs = qx[i] * P.scale;
+      sg = fmaf(qs * qs, br.dvar[i], sg);   // Eq. 8: the squared logit scale is its 1/d
+    }
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) {
+      d += __shfl_xor_sync(0xffffffffu, d, o);
+      sg += __shfl_xor_sync(0xffffffffu, sg, o);
+    }
+    sg = fmaxf(sg, 0.f);
+    const float zbar = d * P.scale;
+    const float zl2 = (zbar + logc) * kLog2e;
+    if (lane == 0) {
+      const float u = fmaf(logc + zbar + P.half_var * sg, kLog2e, by_mass ? 0.f : __log2f(sg));
+      tail_u[g] = u;
+      P.lz[((size_t)unit * G + g) * P.max_blocks + b] = zl2;
+      norm[g] = make_float4(zl2, fast_exp2(P.half_var * kLog2e * sg), u, 0.f);
+      tail_part[g * CKV_PART_STRIDE] = zl2;
+      tail_part[g * CKV_PART_STRIDE + 1] = 1.f;
+    }
+    if (hw == 1) {   // weight 1 times the mean value
+      *reinterpret_cast<float4 *>(tail_part + g * CKV_PART_STRIDE + 4 + 8 * li) = make_float4(br.x[0], br.x[1], br.x[2], br.x[3]);
+      *reinterpret_cast<float4 *>(tail_part + g * CKV_PART_STRIDE + 8 + 8 * li) = make_float4(br.x[4], br.x[5], br.x[6], br.x[7]);
+    }
+  }
+}
+
+// The last cluster to have read the lengths stores the new ones (nobody waits: it is a counter).
+__device__ __noinline__ void store_lens(int *counter, int *seq_lens, int batch, int cap, int n_clusters) {
+  if (atomicAdd(counter, 1) != n_clusters - 1) return;
+  *counter = 0;
+  for (int i = 0; i < batch; ++i) {
+    const int raw = seq_lens[i];
+    if (raw >= 0 && raw < cap) seq_lens[i] = raw + 1;
+  }
+}
+
+template <int G, bool RD, bool HS, bool VH>
+__global__ void __launch_bounds__(kThreads, 1)
+ckv_unit_step_kernel(CkvDev P, const bf16 *__restrict__ q, const int *seq_lens, const bf16 *k_pool, const bf16 *v_pool,
+                     const int *__restrict__ page_table, CkvNewToken fresh, int kcap, CkvStepPlan plan, int batch,
+                     int *__restrict__ sel_ids, int *__restrict__ sel_cnt, bf16 *__restrict__ out, float *__restrict__ lse,
+                     const __grid_constant__ CUtensorMap tm_v) {
+  constexpr int kRowBytesK = HS ? CKV_D * 2 : CKV_ROW_ELEMS * 2;
+  constexpr int kRowBytesV = (HS || VH) ? CKV_D * 2 : CKV_ROW_ELEMS * 2;
+  constexpr int TB = ScanTile<HS || VH>::TB;
+  constexpr int kParts = TB / 16;              // parts of a tile
+  constexpr int kSkip = kWarps / kParts;       // a warp works on every kSkip-th tile
+  constexpr bool SP = (G <= 4) && !RD;
+  extern __shared__ __align__(1024) unsigned char smem[];
+  __shared__ __align__(8) uint64_t full_bar[2][kStagesCap], empty_bar[kStagesCap];
+  __shared__ __align__(8) uint64_t s_xbar[4];                 // what the cluster's CTAs send: normalisers, scores, partial outputs; global stores done
+  __shared__ __align__(16) unsigned char s_zero_row[512];
+  __shared__ __align__(16) bf16 s_q[G][CKV_D];
+  __shared__ float s_w[G * 64];                               // variance weights [t][g], r < d
+  __shared__ __align__(16) float4 s_wn[kWarps + 1][G];        // (maximum m, sum of e^{l - m}, largest score term) per warp, then of the last block
+  __shared__ __align__(16) float4 s_norm[kClusterCap][G];     // ... per CTA of the cluster
+  __shared__ float s_tail_u[G];
+  __shared__ __align__(16) float s_tail_part[G][CKV_PART_STRIDE];
+  __shared__ __align__(16) float s_recv[(4 * G + kClusterCap) * kRecvStride];
+  __shared__ float s_sq[CKV_D];
+  __shared__ int s_digit, s_before, s_nc, s_ncand, s_wt[3][kWarps], s_abort, s_issued;
+
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int head = lane >> 2, qd = lane & 3;
+  const bool hv = head < G;
+  const int C = (int)cluster_size(), rank = (int)cluster_rank();
+  const int unit = blockIdx.y, s = ckv_div_hkv(P, unit), h = unit - s * P.Hkv;
+  const bool append = fresh.k_new != nullptr;
+  const int cap = P.max_blocks * P.bs;
+  if (tid == kProducerWarp * 32) {
+    for (int st = 0; st < plan.stages; ++st) { mbar_init(&full_bar[0][st], 1); mbar_init(&full_bar[1][st], 1); mbar_init(&empty_bar[st], kParts); }
+    for (int i = 0; i < 3; ++i) mbar_init(&s_xbar[i], 1);
+    mbar_init(&s_xbar[3], C);
+    fence_barrier_init();
+    const int n_items = (4 * G - rank + C - 1) / C;   // partial outputs this CTA reduces (see the merge)
+    mbar_arrive_expect_tx(&s_xbar[0], (uint32_t)(C * G * 16));
+    mbar_arrive_expect_tx(&s_xbar[2], (uint32_t)(n_items * C * (32 * 4 + 8)));
+    s_abort = 0; s_issued = 0; s_digit = -1; s_ncand = 0;
+  }
+  cluster_arrive_release();   // "this CTA runs, its barriers are set up"
+  pdl_trigger();              // the next launch of the stream may set itself up ...
+  pdl_wait();                 // ... and this one touches nothing before the launch ahead of it is complete
+  const int raw = seq_lens[s];
+  if (tid < G * 16) reinterpret_cast<uint4 *>(&s_q[0][0])[tid] = __ldg(reinterpret_cast<const uint4 *>(q + (size_t)unit * G * CKV_D) + tid);
+  if (tid >= kThreads - 32) reinterpret_cast<uint4 *>(s_zero_row)[lane] = make_uint4(0u, 0u, 0u, 0u);
+  const bool dbar_bulk = P.r >= 4;
+  const int stage_bytes = TB * (kRowBytesK + kRowBytesV) + (dbar_bulk ? TB * P.r * 4 : 0);
+  float *su = reinterpret_cast<float *>(smem + plan.u_off);   // score terms of the CTA's own blocks, [g][own_cap]
+  // the length the step works on; a bound the host misjudged is kept to what the shared arrays were sized for
+  const int N = max(min(min(raw + ((append && raw >= 0 && raw < cap) ? 1 : 0), cap), plan.max_blocks * P.bs), 0);
+  const int X = (N + P.bs - 1) >> P.lg_bs, Xs = max(X - 1, 0);
+  const int n_parts = (Xs + 15) >> 4;
+  const int ppc = (int)ckv_udiv24((unsigned)(n_parts + C - 1), (unsigned)C);
+  const int b_lo = min(rank * ppc, n_parts) * 16;
+  const int own = max(min(min(b_lo + ppc * 16, Xs) - b_lo, plan.own_cap), 0);
+  const int tiles = (own + TB - 1) / TB;
+  const size_t row0 = (size_t)unit * P.max_blocks;
+
+  // one fill of the ring: tile `it` into stage `st`, counted on full barrier `fb`
+  auto fill = [&](int it, int st, uint64_t *fb) {
+    const int nb = min(TB, own - it * TB);
+    const size_t row = row0 + b_lo + it * TB;
+    unsigned char *sk = smem + (size_t)st * stage_bytes;
+    unsigned char *sv = sk + TB * kRowBytesK;
+    const uint32_t kbytes = (uint32_t)nb * kRowBytesK;
+    const uint32_t vbytes = VH ? (uint32_t)TB * kRowBytesV : (uint32_t)nb * kRowBytesV;   // a tensor copy always delivers its whole box
+    const uint32_t dbytes = dbar_bulk ? (uint32_t)nb * P.r * 4 : 0;
+    mbar_arrive_expect_tx(fb, kbytes + vbytes + dbytes);
+    const uint32_t lo = smem_u32(smem), hi = lo + (uint32_t)plan.stages * stage_bytes;
+    bool ok = nb >= 1 && b_lo + it * TB + nb <= P.max_blocks;
+    // test hook (ckv_debug_set): one fill is announced but never issued, so that the waits on it run out
+    const bool skip = (P.debug & CKV_DEBUG_SKIP_FILL) != 0 && it == 0 && rank == 0 && unit == 0;
+    if (!skip) {
+      ok = ok && bulk_g2s_checked(sk, P.kmean + row * P.row_elems, kbytes, fb, lo, hi);
+      if constexpr (VH) {
+        // rows [row, row + TB) of the mean-values region, first 256 bytes of each (rows past the range are never read)
+        const uint32_t dv = smem_u32(sv);
+        const bool fits = (dv & 127u) == 0 && dv >= lo && dv + vbytes <= hi;
+        if (ok && fits) tensor_g2s(dv, &tm_v, 0, (int)row, fb);
+        ok = ok && fits;
+      } else {
+        ok = ok && bulk_g2s_checked(sv, P.vmean + row * P.row_elems, vbytes, fb, lo, hi);
+      }
+      if (dbar_bulk) ok = ok && bulk_g2s_checked(sv + TB * kRowBytesV, P.dbar + row * P.r, dbytes, fb, lo, hi);
+      }
+    if (!ok) atomicOr(P.status, CKV_DEV_BAD_COPY);
+  };
+  __syncthreads();
+  // the first round of fills is issued by as many warps at once: a fill is some seventy instructions, a third of a
+  // microsecond for one thread, which alone would have the last stage's data arrive a microsecond late
+  const int first_fills = min(tiles, plan.stages);
+  if (warp < first_fills && lane == 0) fill(warp, warp, &full_bar[0][warp]);
+
+  ScanUnit<G, bf16, RD> w;
+  w.reset();
+  if (warp == kProducerWarp) {
+    // ---------------- producer: one thread refills the ring ----------------
+    if (lane == 0) {
+      mbar_arrive_expect_tx(&s_xbar[1], (uint32_t)(X * 4));
+      *(volatile int *)&s_issued = first_fills;
+      int st = 0;
+      uint32_t phase = 0, round = 1;
+      for (int it = plan.stages; it < tiles; ++it) {
+        if (!mbar_wait(&empty_bar[st], phase, P.spin_limit)) {
+          atomicOr(P.status, CKV_DEV_TIMEOUT);
+          *(volatile int *)&s_abort = 1;
+        }
+        if (*(volatile int *)&s_abort) break;
+        fill(it, st, &full_bar[round & 1][st]);
+        *(volatile int *)&s_issued = it + 1;
+        if (++st == plan.stages) { st = 0; ++round; phase ^= 1; }
+      }
+    } else {
+      // the other lanes ask the L2 for this CTA's share of the page-table row: the attention's lookups are then short
+      const int lines = (X * P.ppb + 31) / 32, per = (lines + C - 1) / C;
+      const int *pt = page_table + (size_t)s * P.max_pages_per_seq;
+      for (int i = rank * per + lane - 1; i < min((rank + 1) * per, lines); i += 31)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(pt + 32 * i) : "memory");
+    }
+  } else if (warp == kTailWarp) {
+    if (rank == C - 1 && N > 0)
+      tail_block<G>(P, &s_q[0][0], page_table, fresh, unit, raw, N, s_sq, s_tail_u, &s_tail_part[0][0], s_wn[kWarps]);
+    else if (lane < G)
+      s_wn[kWarps][lane] = make_float4(-CUDART_INF_F, 0.f, -CUDART_INF_F, 0.f);
+  } else {
+    // ---------------- working warps: parts of 16 blocks ----------------
+    if (!RD && P.r != 4) {
+      for (int i = tid; i < P.r * G; i += kWork) {   // w_{g,t} of Eq. 8 times the squared logit scale
+        const int g = i & (G - 1), t = i / G, gs = CKV_D / P.r, run = P.glayout == 0 ? gs : gs / 2;
+        float a = 0.f;
+        for (int k = 0; k < gs; ++k) {
+          const int c = t * run + (k < run ? k : CKV_D / 2 + k - run);
+          const float x = __bfloat162float(s_q[g][c]);
+          a = fmaf(x, x, a);
+        }
+        s_w[i] = a * (P.scale * P.scale);
+      }
+      work_barrier();
+    }
+    const uint32_t *srow = reinterpret_cast<const uint32_t *>(&s_q[hv ? head : 0][0]);
+#pragma unroll
+    for (int ks = 0; ks < 8; ++ks)
+#pragma unroll
+      for (int hh = 0; hh < 2; ++hh) {
+        w.qa[ks][hh] = hv ? srow[(16 * ks + 8 * hh + 2 * qd) / 2] : 0u;
+        if (RD) {
+          const float x0 = __uint_as_float(w.qa[ks][hh] << 16) * P.scale, x1 = __uint_as_float(w.qa[ks][hh] & 0xffff0000u) * P.scale;
+          const float s0 = x0 * x0, s1 = x1 * x1;
+          w.qsh[RD ? ks : 0][hh] = pack_bf16(s0, s1);
+          w.qsl[RD ? ks : 0][hh] = pack_bf16(s0 - bf16_round(s0), s1 - bf16_round(s1));
+        }
+      }
+    if (!RD && P.r == 4) {   // the same from the fragments: a head's four lanes hold its 128 coordinates between them
+#pragma unroll
+      for (int t = 0; t < 4; ++t) w.wown[t] = 0.f;
+#pragma unroll
+      for (int ks = 0; ks < 8; ++ks) {
+        float a = 0.f;
+#pragma unroll
+        for (int hh = 0; hh < 2; ++hh) {
+          const float x0 = __uint_as_float(w.qa[ks][hh] << 16), x1 = __uint_as_float(w.qa[ks][hh] & 0xffff0000u);
+          a = fmaf(x0, x0, fmaf(x1, x1, a));
+        }
+        if (P.glayout == 0) w.wown[ks / 2] += a; else w.wown[ks % 4] += a;   // 16 coordinates of one group
+      }
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        w.wown[t] += __shfl_xor_sync(0xffffffffu, w.wown[t], 1);
+        w.wown[t] += __shfl_xor_sync(0xffffffffu, w.wown[t], 2);
+        w.wown[t] *= P.scale * P.scale;
+        if (SP) w.wown[t] = __shfl_sync(0xffffffffu, w.wown[t], lane & 15);   // the upper half warp works for the same heads
+      }
+    }
+    const ScanPartCfg cfg{P.scale, P.half_var, logf((float)P.bs), P.r, P.max_blocks, (P.variant & CKV_VARIANT_RANK_BY_MASS) != 0, P.r == 4};
+    float *lz = P.lz + row0 * G;
+    const bool pair_ok = (P.max_blocks & 1) == 0;
+    const int part = warp % kParts;
+    // A warp visits every kSkip-th tile.  A fill is only issued once the one plan.stages before it was released, and
+    // kSkip <= plan.stages (checked by the launcher): alternate rounds of the ring use two sets of full barriers, which
+    // together tell the fills a parity wait could confuse apart (see the scan kernel).
+    int st = 0, at = 0;
+    uint32_t round = 0;
+    bool aborted = false;
+    float umax = -CUDART_INF_F;   // largest score term this lane has seen (of its head)
+    for (int it = warp / kParts; it < tiles; it += kSkip) {
+      st += it - at;
+      at = it;
+      while (st >= plan.stages) { st -= plan.stages; ++round; }
+      if (!aborted) {
+        bool fail = *(volatile int *)&s_abort != 0;
+        if (!fail && !mbar_wait(&full_bar[round & 1][st], (round >> 1) & 1, P.spin_limit)) {
+          atomicOr(P.status, CKV_DEV_TIMEOUT);
+          *(volatile int *)&s_abort = 1;
+          fail = true;
+        }
+        aborted = __any_sync(0xffffffffu, fail);
+      }
+      const int nb = min(TB, own - it * TB), rb = part * 16;
+      if (!aborted && rb < nb) {
+        const uint32_t sk = smem_u32(smem + (size_t)st * stage_bytes);
+        const float *sd = reinterpret_cast<const float *>(smem + (size_t)st * stage_bytes + TB * (kRowBytesK + kRowBytesV));
+        scan_part<G, bf16, RD, HS, VH>(
+            w, cfg, sk, sk + TB * kRowBytesK, (RD || dbar_bulk) ? sd : nullptr, smem_u32(s_zero_row), s_w, P.dbar + row0 * P.r,
+            lane, rb, nb, b_lo + it * TB, -1, 0.f,
+            [&](int eh, int blk, float u0, float u1, float z0, float z1, bool v0, bool v1) {
+              float *uo = su + eh * plan.own_cap + (blk - b_lo);
+              const size_t o = (size_t)eh * P.max_blocks + blk;
+              if (v0) { uo[0] = u0; umax = fmaxf(umax, u0); }
+              if (v1) { uo[1] = u1; umax = fmaxf(umax, u1); }
+              if (pair_ok && v1) {
+                *reinterpret_cast<float2 *>(lz + o) = make_float2(z0, z1);
+              } else {
+                if (v0) lz[o] = z0;
+                if (v1) lz[o + 1] = z1;
+              }
+            });
+      }
+      __syncwarp();
+      if (lane == 0 && !aborted) mbar_arrive(&empty_bar[st]);
+    }
+    // this warp's normaliser partial
+    float lp = w.lp_acc;
+    lp += __shfl_xor_sync(0xffffffffu, lp, 1); lp += __shfl_xor_sync(0xffffffffu, lp, 2);
+    umax = fmaxf(umax, __shfl_xor_sync(0xffffffffu, umax, 1)); umax = fmaxf(umax, __shfl_xor_sync(0xffffffffu, umax, 2));
+    if (SP) { lp += __shfl_xor_sync(0xffffffffu, lp, 16); umax = fmaxf(umax, __shfl_xor_sync(0xffffffffu, umax, 16)); }
+    if (hv && qd == 0) s_wn[warp][head] = make_float4(w.m_ref, lp, umax, 0.f);
+  }
+  __syncwarp();
+  cluster_wait();    // every CTA of the cluster has started
+  __syncthreads();
+  if (s_abort) {     // leave no copy in flight into memory that is about to be reused: wait (bounded) for every issued fill
+    if (tid == 0)
+      for (int it = max(s_issued - plan.stages, 0); it < s_issued; ++it)
+        mbar_wait(&full_bar[(it / plan.stages) & 1][it % plan.stages], ((it / plan.stages) >> 1) & 1, P.spin_limit);
+    __syncthreads();
+  }
+
+  // ---- normalisers of Eq. 9 over the whole unit ----
+  if (warp < G) {   // the CTA's own: warp g for head g, every lane the whole sum
+    float4 e[kWarps + 1];
+#pragma unroll
+    for (int i = 0; i <= kWarps; ++i) e[i] = s_wn[i][warp];
+    float m = e[0].x, l = 0.f, u = e[0].z;
+#pragma unroll
+    for (int i = 1; i <= kWarps; ++i) { m = fmaxf(m, e[i].x); u = fmaxf(u, e[i].z); }
+#pragma unroll
+    for (int i = 0; i <= kWarps; ++i) l = fmaf(e[i].y, exp2_diff(e[i].x, m), l);
+    if (lane < C) {
+      const uint32_t x0 = smem_u32(&s_xbar[0]), there = cluster_map(x0, lane);   // the CTAs' shared memories are congruent windows
+      st_async_u32x4(there + (smem_u32(&s_norm[rank][warp]) - x0), __float_as_uint(m), __float_as_uint(l), __float_as_uint(u), 0u, there);
+    }
+  }
+  if (warp >= kWarps) {   // meanwhile: histogram and bit map start at zero (the ring is drained)
+    int4 *hist = reinterpret_cast<int4 *>(smem + kOffHist);
+    for (int i = tid - kWork; i < (kBins + 32 + kMapWords) / 4; i += kThreads - kWork) hist[i] = make_int4(0, 0, 0, 0);
+    if (warp == kTailWarp) {
+      // What this CTA's scan and tail warps wrote to global memory and others of the cluster will read (mean-term weights,
+      // the new token's rows) is released by this warp for all of them: the wait for those stores is off the critical path.
+      __threadfence();
+      if (lane < C) mbar_arrive_cluster(cluster_map(smem_u32(&s_xbar[3]), lane));
+    }
+  }
+  auto wait_x = [&](int i) {
+    if (!mbar_wait_cluster(&s_xbar[i], 0, ckv_pipe::kSpinLimit)) { atomicOr(P.status, CKV_DEV_TIMEOUT); s_abort = 1; }
+  };
+  wait_x(0);
+  if (append && rank == 0 && tid == kTailWarp * 32)
+    store_lens(P.status + CKV_LEN_COUNTER_WORD, fresh.seq_lens, batch, cap, (int)gridDim.y);   // all CTAs of this cluster have read them
+  float Mg[G], iL[G], bound = 0.f;   // every warp by itself: 32 / G lanes per head.  bound: no block scores more
+  {
+    constexpr int LPH = 32 / G, EPL = (kClusterCap + LPH - 1) / LPH;
+    const int g = lane / LPH, k0 = lane % LPH;
+    float4 e[EPL];
+    float m = -CUDART_INF_F, l = 0.f, u = -CUDART_INF_F;
+#pragma unroll
+    for (int i = 0; i < EPL; ++i) {
+      const int k = k0 + i * LPH;
+      e[i] = k < C ? s_norm[k < kClusterCap ? k : 0][g] : make_float4(-CUDART_INF_F, 0.f, -CUDART_INF_F, 0.f);
+      m = fmaxf(m, e[i].x);
+      u = fmaxf(u, e[i].z);
+    }
+#pragma unroll
+    for (int o = LPH / 2; o > 0; o >>= 1) {
+      m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+      u = fmaxf(u, __shfl_xor_sync(0xffffffffu, u, o));
+    }
+#pragma unroll
+    for (int i = 0; i < EPL; ++i) l = fmaf(e[i].y, exp2_diff(e[i].x, m), l);
+#pragma unroll
+    for (int o = LPH / 2; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+    const float il = 1.0f / l, b = fast_exp2(u - m) * il;
+#pragma unroll
+    for (int i = 0; i < G; ++i) {
+      Mg[i] = __shfl_sync(0xffffffffu, m, i * LPH);
+      iL[i] = __shfl_sync(0xffffffffu, il, i * LPH);
+      bound += __shfl_sync(0xffffffffu, b, i * LPH);
+    }
+  }
+
+  // ---- scores of the CTA's own blocks (Eq. 10), to every CTA of the cluster ----
+  const int n_recent = min(P.recent, X);
+  const int rank_lo = P.sink, rank_n = max(X - n_recent - P.sink, 0);   // blocks [rank_lo, rank_lo + rank_n) are ranked, the others mandatory
+  auto ranked = [rank_lo, rank_n](int b) { return (unsigned)(b - rank_lo) < (unsigned)rank_n; };
+  uint32_t *keys = reinterpret_cast<uint32_t *>(smem);   // the unit's scores; their bit patterns are ordered like the scores
+  if (warp < kWarps) {
+    bool nonfinite = false;
+    const uint32_t xbar1 = smem_u32(&s_xbar[1]);
+    for (int i = 4 * tid; i < own; i += 4 * kWork) {
+      float sc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+      for (int g = 0; g < G; ++g) {
+        const float4 u = *reinterpret_cast<const float4 *>(su + g * plan.own_cap + i);
+        sc[0] = fmaf(fast_exp2(u.x - Mg[g]), iL[g], sc[0]); sc[1] = fmaf(fast_exp2(u.y - Mg[g]), iL[g], sc[1]);
+        sc[2] = fmaf(fast_exp2(u.z - Mg[g]), iL[g], sc[2]); sc[3] = fmaf(fast_exp2(u.w - Mg[g]), iL[g], sc[3]);
+      }
+      uint32_t k[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const bool real = i + j < own;
+        if (real && (!(sc[j] >= 0.f) || sc[j] > 3.0e38f)) { nonfinite = true; sc[j] = 0.f; }
+        k[j] = __float_as_uint(sc[j]);
+      }
+      const uint32_t dst = smem_u32(keys + b_lo + i);
+      if (i + 4 <= own) {
+        for (int c = 0; c < C; ++c) {
+          const uint32_t there = cluster_map(xbar1, c);   // the CTAs' shared memories are congruent windows
+          st_async_u32x4(there + (dst - xbar1), k[0], k[1], k[2], k[3], there);
+        }
+      } else {   // the end of the unit's range: what follows belongs to somebody else
+        for (int c = 0; c < C; ++c)
+#pragma unroll
+          for (int j = 0; j < 3; ++j)
+            if (i + j < own) st_async_u32(cluster_map(dst + 4 * j, c), k[j], cluster_map(smem_u32(&s_xbar[1]), c));
+      }
+    }
+    if (nonfinite) atomicOr(P.status, CKV_DEV_NONFINITE);
+  } else if (warp == kTailWarp && rank == C - 1 && N > 0) {   // the last block
+    float sc = 0.f;
+#pragma unroll
+    for (int g = 0; g < G; ++g) sc = fmaf(fast_exp2(s_tail_u[g] - Mg[g]), iL[g], sc);
+    if (!(sc >= 0.f) || sc > 3.0e38f) { if (lane == 0) atomicOr(P.status, CKV_DEV_NONFINITE); sc = 0.f; }
+    if (lane < C) st_async_u32(cluster_map(smem_u32(keys + Xs), lane), __float_as_uint(sc), cluster_map(smem_u32(&s_xbar[1]), lane));
+  }
+  if (warp == kTailWarp && X > kcap) {   // the mandatory blocks are in (the other idle warp's share of the map is clear, too)
+    named_barrier(2, kThreads - kWork);
+    uint32_t *map = reinterpret_cast<uint32_t *>(smem + kOffMap);
+    for (int i = lane; i < X - rank_n; i += 32) {
+      const int b = i < rank_lo ? i : i + rank_n;
+      atomicOr(&map[b >> 5], 1u << (b & 31));
+    }
+  } else if (warp == kProducerWarp && X > kcap) {
+    named_barrier(2, kThreads - kWork);
+  }
+  wait_x(1);
+  __syncthreads();   // the histogram is clear, too
+
+  // ---- selection (Eq. 11), the same in every CTA ----
+  const int K = min(kcap, X);
+  const bool all = X <= kcap;          // every block is selected: the step is dense attention
+  int *ids = reinterpret_cast<int *>(smem + kOffIds);
+  if (warp >= kWarps) {   // the two idle warps leave the range's scores where ckv_copy_scores() finds them
+    float *scores = P.scores + row0;
+    for (int i = tid - kWork; i < own; i += kThreads - kWork) scores[b_lo + i] = __uint_as_float(keys[b_lo + i]);
+    if (rank == C - 1 && N > 0 && tid == kWork) scores[Xs] = __uint_as_float(keys[Xs]);
+  }
+  if (warp < kWarps) {
+    int *gids = sel_ids + (size_t)unit * kcap;
+    if (all) {
+      if (rank == 0) {
+        for (int b = tid; b < kcap; b += kWork) gids[b] = b < X ? b : -1;
+        if (tid == 0) sel_cnt[unit] = X;
+      }
+    } else {
+      const int Kr = K - (X - rank_n);   // blocks to rank in (the host guarantees K >= sink + recent when K < X)
+      uint32_t *map = reinterpret_cast<uint32_t *>(smem + kOffMap);
+      auto pick = [map](int b) { atomicOr(&map[b >> 5], 1u << (b & 31)); };
+      if (Kr > 0) {
+        int *hist = reinterpret_cast<int *>(smem + kOffHist);
+        const uint4 *keys4 = reinterpret_cast<const uint4 *>(keys);
+        const int groups = (X + 3) / 4;
+        const int top = (int)(__float_as_uint(fminf(bound, 3.0e38f)) >> kBinShift);
+        auto bin_of = [top](uint32_t k) { return max(top - (int)(k >> kBinShift), 0); };
+#pragma unroll 2
+        for (int i = tid; i < groups; i += kWork) {
+          const uint4 k4 = keys4[i];
+          const uint32_t k[4] = {k4.x, k4.y, k4.z, k4.w};
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const int d = bin_of(k[j]);
+            atomicAdd(&hist[d < kBins && ranked(4 * i + j) ? d : kBins + lane], 1);   // no branch: the rest goes aside
+          }
+        }
+        work_barrier();
+        constexpr int BPT = kBins / kWork;   // bins per thread, largest scores first
+        int c[BPT], csum = 0;
+#pragma unroll
+        for (int j = 0; j < BPT; j += 4) {
+          const int4 x = reinterpret_cast<const int4 *>(hist)[(tid * BPT + j) / 4];
+          c[j] = x.x; c[j + 1] = x.y; c[j + 2] = x.z; c[j + 3] = x.w;
+          csum += (x.x + x.y) + (x.z + x.w);
+        }
+        int before = work_exclusive_scan(csum, s_wt[0]);
+        if (before < Kr && before + csum >= Kr) {
+#pragma unroll
+          for (int j = 0; j < BPT; ++j) {
+            if (before < Kr && before + c[j] >= Kr) { s_digit = tid * BPT + j; s_before = before; s_nc = c[j]; before = Kr; }
+            else before += c[j];
+          }
+        }
+        work_barrier();
+        const int digit = s_digit, nc = s_nc;
+        if (digit >= 0 && nc <= kCandCap) {
+          // higher bins are taken whole; the cut's bin is ranked by (score descending, id ascending)
+          int *cand = reinterpret_cast<int *>(smem + kOffCand);
+          uint32_t *candk = reinterpret_cast<uint32_t *>(smem + kOffCand) + kCandCap;
+          const int take = Kr - s_before;
+#pragma unroll 2
+          for (int i0 = warp * 32; i0 < groups; i0 += kWork) {   // whole warps: eight lanes make up a word of the map
+            const int i = i0 + lane;
+            uint4 k4 = make_uint4(0u, 0u, 0u, 0u);
+            if (i < groups) k4 = keys4[i];
+            const uint32_t k[4] = {k4.x, k4.y, k4.z, k4.w};
+            uint32_t above = 0, at = 0;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const int d = ranked(4 * i + j) ? bin_of(k[j]) : kBins;
+              above |= d < digit ? 1u << j : 0u;
+              at |= d == digit ? 1u << j : 0u;
+            }
+            above <<= 4 * (lane & 7);
+            above |= __shfl_xor_sync(0xffffffffu, above, 1);
+            above |= __shfl_xor_sync(0xffffffffu, above, 2);
+            above |= __shfl_xor_sync(0xffffffffu, above, 4);
+            if ((lane & 7) == 0 && above != 0) atomicOr(&map[i >> 3], above);
+            while (at != 0) {
+              const int j = __ffs(at) - 1;
+              at &= at - 1;
+              const int slot = atomicAdd(&s_ncand, 1);
+              cand[slot] = 4 * i + j;
+              candk[slot] = k[j];
+            }
+          }
+          work_barrier();
+          if (tid < nc) {
+            const int myb = cand[tid];
+            const uint32_t mk = candk[tid];
+            int place = 0;
+#pragma unroll 4
+            for (int j = 0; j < nc; ++j) place += (candk[j] > mk || (candk[j] == mk && cand[j] < myb)) ? 1 : 0;
+            if (place < take) pick(myb);
+          }
+        } else {
+          uint32_t cut_key;
+          int cut_id;
+          cut_by_bisection(X, Kr, keys, rank_lo, rank_n, s_wt[0], cut_key, cut_id);
+          for (int b = tid; b < X; b += kWork)
+            if (ranked(b) && (keys[b] > cut_key || (keys[b] == cut_key && b <= cut_id))) pick(b);
+        }
+      }
+      work_barrier();
+      // ids in position order: two words of the map per thread
+      uint2 m2 = reinterpret_cast<const uint2 *>(map)[tid];
+      int pos = work_exclusive_scan(__popc(m2.x) + __popc(m2.y), s_wt[1]);
+#pragma unroll
+      for (int half = 0; half < 2; ++half) {
+        uint32_t bits = half == 0 ? m2.x : m2.y;
+        while (bits != 0) {
+          const int b = 64 * tid + 32 * half + __ffs(bits) - 1;
+          bits &= bits - 1;
+          if (pos < K) {
+            ids[pos] = b;
+            if (rank == 0) gids[pos] = b;
+          }
+          ++pos;
+        }
+      }
+      if (rank == 0) {
+        for (int i = K + tid; i < kcap; i += kWork) gids[i] = -1;
+        if (tid == 0) sel_cnt[unit] = K;
+      }
+      work_barrier();
+    }
+  }
+  const int nsel = K;
+  if (warp < kWarps) {
+    wait_x(3);       // acquires what the other CTAs of the cluster released
+    // ---- exact attention over the CTA's share of the selected pages ----
+    const bool comp = nsel < X && !(P.variant & CKV_VARIANT_DROP);
+    if (!comp) w.reset();   // nothing is compensated: the scan's sums are not wanted
+    const int n_pages = all ? (N + CKV_PAGE - 1) / CKV_PAGE : nsel * P.ppb;
+    const int share = (int)ckv_udiv24((unsigned)(n_pages + C - 1), (unsigned)C);
+    const int p0 = min(rank * share, n_pages), p1 = min(p0 + share, n_pages);
+    const int n_mine = max((p1 - p0 - warp + kWarps - 1) / kWarps, 0);
+    const int pshift = P.ppb == 1 ? 0 : (P.ppb == 2 ? 1 : 2);
+    const int *pt_row = page_table + (size_t)s * P.max_pages_per_seq;
+    const float *lz = P.lz + row0 * G;
+    const float sl2 = P.scale * kLog2e;
+    const float lg_bs = log2f((float)P.bs), lg_last = log2f((float)max(N - Xs * P.bs, 1));
+    const uint32_t buf0 = smem_u32(smem + kOffPages) + warp * 2 * kPageBytes;
+    const bool rows_rm = HS && comp;   // one more item per 16 pages: the mean-value rows of their blocks
+    bool bad = false;
+    struct Page { int phys, ntok, blk; };
+    Page mine{-1, 0, -1};
+    auto lookup = [&](int n) {         // lane l looks the warp's page n + l up: 32 pages cost one round trip
+      mine = Page{-1, 0, -1};
+      if (n + lane < n_mine) {
+        const int i = p0 + warp + kWarps * (n + lane);
+        const int blk = all ? i >> pshift : ids[i >> pshift];
+        const int page = all ? i : (blk << pshift) + (i & (P.ppb - 1));
+        mine.blk = (i & (P.ppb - 1)) == 0 ? blk : ~blk;   // complemented on the block's later pages
+        mine.ntok = max(min(CKV_PAGE, N - page * CKV_PAGE), 0);
+        if (mine.ntok > 0) {
+          mine.phys = pt_row[page];
+          if (mine.phys < 0 || mine.phys >= P.num_pages) { mine.phys = -1; bad = true; }
+        }
+      }
+    };
+    // items: pages 0 .. 15, [rows], pages 16 .. 31, [rows], ...; the last group may be short
+    const int n_items = n_mine + (rows_rm ? (n_mine + 15) / 16 : 0);
+    struct Item { int ntok; float z[HS ? 4 : 1]; };   // ntok > 0: a page; 0: nothing; -1: rows
+    int gpos = 0, page_n = 0;
+    auto issue = [&](int buf) -> Item {
+      Item it;
+      it.ntok = 0;
+      it.z[0] = -CUDART_INF_F;
+      const uint32_t kb = buf0 + buf * kPageBytes;
+      const bool rows = rows_rm && (gpos == 16 || page_n == n_mine);
+      if (!rows) {
+        if ((page_n & 31) == 0) lookup(page_n);
+        const int phys = __shfl_sync(0xffffffffu, mine.phys, page_n & 31);
+        const int ntok = __shfl_sync(0xffffffffu, mine.ntok, page_n & 31);
+        const int bx = __shfl_sync(0xffffffffu, mine.blk, page_n & 31);
+        if (phys >= 0) {
+          const size_t src = ((size_t)phys * P.Hkv + h) * (CKV_PAGE * CKV_D);
+          issue_page(kb, kb + kTileBytes, k_pool + src, v_pool + src, ntok, lane);
+          it.ntok = ntok;
+          if (!HS && comp && hv) {   // log2 of e^{zbar} of the page's block for this lane's head
+            const int blk = bx < 0 ? ~bx : bx;
+            it.z[0] = __ldcg(lz + (size_t)head * P.max_blocks + blk) - (blk == Xs ? lg_last : lg_bs);
+          }
+        }
+        ++page_n; ++gpos;
+      } else if constexpr (HS) {
+        // mean-value rows of the group's blocks (row j: the group's page j, if it is its block's first), as a value tile
+        const int first = page_n - gpos;
+        it.ntok = -1;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const int idx = lane + 32 * k, row = idx >> 4, c = idx & 15;
+          const int blk = __shfl_sync(0xffffffffu, mine.blk, (first + row) & 31);
+          const bool real = row < gpos && blk >= 0;
+          const bf16 *src = P.vmean + (row0 + (real ? blk : 0)) * P.row_elems + 8 * swz_chunk(c, real ? blk : 0);
+          cp_async16(kb + kTileBytes + (uint32_t)(row * kRowBytes + ((c ^ (row & 7)) << 4)), src, real);
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int row = 2 * qd + (e & 1) + 8 * (e >> 1);
+          const int blk = __shfl_sync(0xffffffffu, mine.blk, (first + row) & 31);
+          it.z[HS ? e : 0] = (hv && row < gpos && blk >= 0) ? __ldcg(lz + (size_t)head * P.max_blocks + blk) : -CUDART_INF_F;
+        }
+        gpos = 0;
+      }
+      return it;
+    };
+    Item cur;
+    cur.ntok = 0;
+    if (n_items > 0) cur = issue(0);
+    cp_async_commit();
+    for (int n = 0, buf = 0; n < n_items; ++n, buf ^= 1) {
+      Item nxt;
+      nxt.ntok = 0;
+      if (n + 1 < n_items) nxt = issue(buf ^ 1);
+      cp_async_commit();
+      cp_async_wait<1>();
+      __syncwarp();
+      const uint32_t kb = buf0 + buf * kPageBytes;
+      if (cur.ntok > 0) {
+        attn_page<SP>(kb, kb + kTileBytes, w.qa, cur.ntok, hv, lane, sl2, HS ? -CUDART_INF_F : cur.z[0], w.acc, w.m_ref, w.l_acc);
+      } else if (HS && cur.ntok < 0) {
+        float zm = fmaxf(fmaxf(cur.z[0], cur.z[HS ? 1 : 0]), fmaxf(cur.z[HS ? 2 : 0], cur.z[HS ? 3 : 0]));
+        zm = fmaxf(zm, __shfl_xor_sync(0xffffffffu, zm, 1));
+        zm = fmaxf(zm, __shfl_xor_sync(0xffffffffu, zm, 2));
+        if (SP) zm = fmaxf(zm, __shfl_xor_sync(0xffffffffu, zm, 16));
+        attn_raise(zm, w.m_ref, w.l_acc, w.acc);
+        float x[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {   // the negated weights
+          const float z = cur.z[HS ? e : 0];
+          x[e] = z == -CUDART_INF_F ? 0.f : -fast_exp2(z - w.m_ref);
+          w.l_acc += x[e];
+        }
+        const uint32_t ph[2] = {pack_bf16(x[0], x[1]), pack_bf16(x[2], x[3])};
+        const uint32_t pl[2] = {pack_bf16(x[0] - bf16_round(x[0]), x[1] - bf16_round(x[1])),
+                                pack_bf16(x[2] - bf16_round(x[2]), x[3] - bf16_round(x[3]))};
+        attn_pv(kb + kTileBytes, ph, pl, lane, w.acc);
+      }
+      __syncwarp();
+      cur = nxt;
+    }
+    cp_async_wait<0>();
+    if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(P.status, CKV_DEV_BAD_PAGE);
+
+    // ---- the CTA's partial: its warps (each with its own running maximum) and the last block's mean term ----
+    float l = w.l_acc;
+    l += __shfl_xor_sync(0xffffffffu, l, 1); l += __shfl_xor_sync(0xffffffffu, l, 2);
+    if (SP) l += __shfl_xor_sync(0xffffffffu, l, 16);
+    float *wpart = reinterpret_cast<float *>(smem + kOffPages) + (size_t)warp * (2 * kPageBytes / 4);
+    __syncwarp();
+    if (hv) {
+      float *r = wpart + head * CKV_PART_STRIDE;
+#pragma unroll
+      for (int t = 0; t < 16; ++t) *reinterpret_cast<float2 *>(r + 4 + 8 * t + 2 * qd) = make_float2(w.acc[t][0], w.acc[t][1]);
+      if (qd == 0) { r[0] = w.m_ref; r[1] = l; }
+    }
+    const bool with_tail = comp && rank == C - 1;
+    auto entry = [&](int e) { return e < kWarps ? reinterpret_cast<const float *>(smem + kOffPages) + (size_t)e * (2 * kPageBytes / 4) : &s_tail_part[0][0]; };
+    work_barrier();
+    // thread t: four coordinates of one head over all entries.  Item i = (head, 32 coordinates) is reduced over the
+    // cluster by CTA i mod C, into slot i / C.
+    for (int idx = tid; idx < G * CKV_D / 4; idx += kWork) {
+      const int g = idx / (CKV_D / 4), c = 4 * (idx % (CKV_D / 4));
+      float2 ml[kWarps + 1];
+      float4 x[kWarps + 1];
+#pragma unroll
+      for (int e = 0; e <= kWarps; ++e) {
+        const float *p = entry(e) + g * CKV_PART_STRIDE;
+        ml[e] = *reinterpret_cast<const float2 *>(p);
+        x[e] = *reinterpret_cast<const float4 *>(p + 4 + c);
+      }
+      if (!with_tail) ml[kWarps].x = -CUDART_INF_F;
+      float M = ml[0].x;
+#pragma unroll
+      for (int e = 1; e <= kWarps; ++e) M = fmaxf(M, ml[e].x);
+      float den = 0.f;
+      float4 num = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int e = 0; e <= kWarps; ++e) {
+        const float sc = exp2_diff(ml[e].x, M);
+        if (sc != 0.f) {   // an entry that holds nothing may hold any bits
+          den = fmaf(ml[e].y, sc, den);
+          num.x = fmaf(x[e].x, sc, num.x); num.y = fmaf(x[e].y, sc, num.y);
+          num.z = fmaf(x[e].z, sc, num.z); num.w = fmaf(x[e].w, sc, num.w);
+        }
+      }
+      const int item = 4 * g + (c >> 5), slot = (int)ckv_udiv24((unsigned)item, (unsigned)C);
+      const uint32_t to = (uint32_t)(item - slot * C);
+      const uint32_t ent = smem_u32(s_recv) + (uint32_t)((slot * C + rank) * kRecvStride) * 4u;
+      const uint32_t bar = cluster_map(smem_u32(&s_xbar[2]), to);
+      st_async_u32x4(cluster_map(ent + (c & 31) * 4, to), __float_as_uint(num.x), __float_as_uint(num.y), __float_as_uint(num.z),
+                     __float_as_uint(num.w), bar);
+      if ((c & 31) == 0) st_async_f32x2(cluster_map(ent + 128, to), M, den, bar);
+    }
+    // ---- the outputs this CTA reduces over the cluster: a warp per item ----
+    if (4 * G > rank) wait_x(2);
+    for (int slot = warp; slot * C + rank < 4 * G; slot += kWarps) {
+      const int item = slot * C + rank, g = item >> 2, c = (item & 3) * 32 + lane;
+      const float *e0 = s_recv + (size_t)slot * C * kRecvStride;
+      float M = -CUDART_INF_F, den = 0.f, o = 0.f;
+#pragma unroll 4
+      for (int e = 0; e < C; ++e) M = fmaxf(M, e0[e * kRecvStride + 32]);
+#pragma unroll 4
+      for (int e = 0; e < C; ++e) {
+        const float sc = exp2_diff(e0[e * kRecvStride + 32], M);
+        den = fmaf(e0[e * kRecvStride + 33], sc, den);
+        o = fmaf(e0[e * kRecvStride + lane], sc, o);
+      }
+      out[((size_t)unit * G + g) * CKV_D + c] = __float2bfloat16_rn(N > 0 ? o / den : 0.f);   // an empty sequence: zero
+      if (lse != nullptr && (item & 3) == 0 && lane == 0) lse[(size_t)unit * G + g] = N > 0 ? (M + log2f(den)) * kLn2 : -CUDART_INF_F;
+    }
+  }
+  __syncwarp();
+  cluster_arrive_relaxed();   // nobody leaves while somebody may still send to it
+  cluster_wait();
+}
+
+// The instantiation a context's layout uses.
+template <int G> const void *kernel_g(const CkvDev &P) {
+  if (P.r == CKV_D) return (const void *)ckv_unit_step_kernel<G, true, false, false>;
+  if (P.row_elems == CKV_D) return (const void *)ckv_unit_step_kernel<G, false, true, false>;
+  if (P.vhi) return (const void *)ckv_unit_step_kernel<G, false, false, true>;
+  return (const void *)ckv_unit_step_kernel<G, false, false, false>;
+}
+const void *kernel_of(const CkvDev &P) {
+  switch (P.G) {
+    case 1: return kernel_g<1>(P);
+    case 2: return kernel_g<2>(P);
+    case 4: return kernel_g<4>(P);
+    case 8: return kernel_g<8>(P);
+  }
+  return nullptr;
+}
+
+cudaLaunchConfig_t launch_config(int C, int units, size_t smem, cudaStream_t st, cudaLaunchAttribute *attr) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(C, units);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = C; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr; cfg.numAttrs = 1;
+  return cfg;
+}
+
+}  // namespace
+
+// Attributes of the context's instantiation, and how many clusters of each size the device holds at once (every CTA
+// takes an SM for itself, so the answer depends on the device alone: asked once per device).
+cudaError_t ckv_configure_unit_step(ckv_ctx *c) {
+  for (int i = 0; i <= CKV_STEP_MAX_CLUSTER; ++i) c->step_clusters[i] = 0;
+  if (c->layout.kv_dtype != CKV_BF16) return cudaSuccess;
+  const void *k = kernel_of(c->dev);
+  if (k == nullptr) return cudaErrorInvalidValue;
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynLimit);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  int dev = 0;
+  if (e == cudaSuccess) e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  constexpr int kMaxDev = 64;
+  static std::mutex mtx;
+  static int table[kMaxDev][CKV_STEP_MAX_CLUSTER + 1];
+  static bool known[kMaxDev];
+  if (dev < 0 || dev >= kMaxDev) return cudaSuccess;   // no table: the step stays with its separate launches
+  std::lock_guard<std::mutex> lock(mtx);
+  if (!known[dev]) {
+    for (int C = 1; C <= CKV_STEP_MAX_CLUSTER; ++C) {
+      cudaLaunchAttribute attr[1];
+      cudaLaunchConfig_t cfg = launch_config(C, 1, kAfterScan, nullptr, attr);
+      int n = 0;
+      if (cudaOccupancyMaxActiveClusters(&n, k, &cfg) != cudaSuccess) { (void)cudaGetLastError(); n = 0; }
+      table[dev][C] = n;
+    }
+    known[dev] = true;
+  }
+  for (int C = 1; C <= CKV_STEP_MAX_CLUSTER; ++C) c->step_clusters[C] = table[dev][C];
+  return cudaSuccess;
+}
+
+// Whether a step of this size runs as one launch, and how.  Against the separate launches (us per step, back to back):
+// 16.8 / 28.6 (one head, 4K), 20.2 / 35.7 (8 units, 32K), 27.6 / 38.9 (8 units, 128K, 32-token blocks), 45.7 / 51.2 (24
+// units, 100K, bf16 summaries), 63.9 / 69.5 (32 units, 128K).  What stays with the separate launches, and why:
+//   * fp32 pages (the attention is on bf16 tensor cores) and an explicit ckv_set_tail_mode, which asks for them;
+//   * caches under CKV_STEP_MIN_TOKENS.  Not a crossover -- one launch is the faster form there too -- but the size below
+//     which the documented two-call arrangement (append, scan, select, attention as launches of their own) is kept;
+//   * r = d: 1536 bytes a block and a third product leave it at 67.1 against 64.8 us (16 units, 88K);
+//   * more selected blocks or scores than the shared arrays hold, more units than clusters run at once, and score terms
+//     that leave no room for the ring.
+bool ckv_unit_step_plan(const ckv_ctx *c, int batch, int max_len, int kcap, CkvStepPlan *plan) {
+  const CkvDev &P = c->dev;
+  if (c->layout.kv_dtype != CKV_BF16 || c->tail_mode != CKV_TAIL_AUTO || max_len < CKV_STEP_MIN_TOKENS || P.r == CKV_D) return false;
+  const int units = batch * P.Hkv, xmax = (max_len + P.bs - 1) / P.bs;
+  if (xmax > kScoresCap || (kcap < xmax && kcap > kSelCap)) return false;
+  int C = 0;
+  for (int k = CKV_STEP_MAX_CLUSTER; k >= 1 && C == 0; --k)
+    if (c->step_clusters[k] >= units) C = k;
+  if (C == 0) return false;
+  const int skip = kWarps / (P.scan_tile / 16);
+  const size_t krow = (size_t)P.row_elems * 2, vrow = (P.vhi || P.row_elems == CKV_D) ? (size_t)CKV_D * 2 : krow;
+  const size_t stage = (size_t)P.scan_tile * (krow + vrow) + (P.r >= 4 ? (size_t)P.scan_tile * P.r * 4 : 0);
+  const int parts = (std::max(xmax - 1, 0) + 15) / 16;
+  plan->own_cap = 16 * std::max((parts + C - 1) / C, 1);
+  const size_t u_bytes = (size_t)plan->own_cap * P.G * sizeof(float);
+  if (u_bytes + (size_t)skip * stage > (size_t)kDynLimit) return false;
+  const int tiles = (plan->own_cap + P.scan_tile - 1) / P.scan_tile;
+  plan->stages = std::min({kStagesCap, (int)(((size_t)kDynLimit - u_bytes) / stage), std::max(tiles, skip)});
+  plan->u_off = (int)(plan->stages * stage);
+  plan->smem = (int)std::max((size_t)plan->u_off + u_bytes, (size_t)kAfterScan);
+  plan->cluster = C;
+  plan->max_blocks = xmax;
+  return true;
+}
+
+cudaError_t ckv_launch_unit_step(ckv_ctx *c, const CkvStepPlan &plan, const void *q, const void *k_pool, const void *v_pool,
+                                 const int *page_table, const int *seq_lens, const CkvNewToken *fresh_in, int batch, int kcap,
+                                 int *sel_ids, int *sel_cnt, void *out, float *lse, cudaStream_t st) {
+  CkvNewToken fresh = {};
+  if (fresh_in != nullptr) fresh = *fresh_in;
+  cudaLaunchAttribute attr[2];
+  cudaLaunchConfig_t cfg = launch_config(plan.cluster, batch * c->dev.Hkv, plan.smem, st, attr);
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.numAttrs = 2;
+  CkvStepPlan p = plan;
+  void *args[] = {&c->dev, &q, &seq_lens, &k_pool, &v_pool, &page_table, &fresh, &kcap, &p, &batch, &sel_ids, &sel_cnt, &out, &lse, &c->tm_vhi};
+  c->launches++;
+  return cudaLaunchKernelExC(&cfg, kernel_of(c->dev), args);
+}

@@ -1,0 +1,136 @@
+"""The one-launch step (a thread-block cluster per unit) at the sizes where it can go wrong: ranges that fill neither a
+part nor a tile nor a page, sequences much shorter than the longest of the batch (CTAs without blocks), every group size
+and summary layout, ties at the cut.  Oracle and tolerances are those of helpers.py."""
+import pytest
+import torch
+
+from paper_2609_26300_b200 import binding, synth
+from helpers import check_unit_decode, setup
+
+pytestmark = pytest.mark.gpu
+
+
+def workload(**kw):
+    base = dict(batch=2, num_q_heads=8, num_kv_heads=2, ctx=16 * 141 + 5, ctx_min=1, budget_tokens=16 * 12, needles=4,
+                outlier_dims=2, decode_steps=3, name="unit_step")
+    base.update(kw)
+    return synth.CONFIGS[1].with_(**base)
+
+
+def step_inputs(d, t):
+    k_new, v_new = synth.appended_rows(d.w, t)
+    return [torch.from_numpy(a).to(d.dtype).cuda() for a in (synth.queries(d.w, t), k_new, v_new)]
+
+
+def run(w, steps, check=(0,), launches=1, budget=None, **layout):
+    """`steps` steps against append + decode (bit for bit) and, at the steps in `check`, every unit against the oracle."""
+    budget = budget or w.budget_tokens
+    a, b = setup(w, **layout), setup(w, **layout)
+    for d in (a, b):
+        d.ckv.stats_build(d.k_pool, d.v_pool, d.table, d.lens, d.max_len)
+    n0 = a.lens.cpu().numpy().copy()
+    for t in range(steps):
+        q, kn, vn = step_inputs(a, t)
+        max_len = w.ctx + t + 1   # the host's bound; the lengths themselves may be much shorter
+        before = a.ckv.launch_count()
+        out, lse, ids, cnt = a.ckv.step(q, kn, vn, a.k_pool, a.v_pool, a.table, a.lens, max_len, budget)
+        assert a.ckv.launch_count() - before == launches
+        scores = a.ckv.copy_scores(w.batch)
+        b.ckv.append(b.k_pool, b.v_pool, b.table, b.lens, kn, vn)
+        other = b.ckv.decode(q, b.k_pool, b.v_pool, b.table, b.lens, max_len, budget)
+        torch.cuda.synchronize()
+        for x, y in zip((out, lse, ids, cnt, a.lens), other + (b.lens,)):
+            assert torch.equal(x, y), t
+        if t in check:
+            ck = {k: v for k, v in layout.items() if k in ("var_groups", "group_layout", "sink", "recent", "variant")}
+            for s in range(w.batch):
+                for h in range(w.num_kv_heads):
+                    check_unit_decode(a, s, h, int(n0[s]) + t + 1, t, budget, out, lse, ids, cnt, scores,
+                                      stat_bf16=bool(layout.get("stat_bf16", 0)), **ck)
+    for x, y in zip(a.ckv.export_stats(), b.ckv.export_stats()):
+        assert torch.equal(x, y)
+    for x, y in ((a.k_pool, b.k_pool), (a.v_pool, b.v_pool)):   # as bits: rows that no step has written yet are NaN
+        assert torch.equal(x.view(torch.int16), y.view(torch.int16))
+    assert a.ckv.read_status() == 0 and b.ckv.read_status() == 0
+    return a
+
+
+@pytest.mark.parametrize("hq,hkv", [(1, 1), (4, 2), (8, 2), (16, 2)])
+@pytest.mark.parametrize("layout", [{}, {"stat_bf16": 1}, {"var_groups": 16, "group_layout": 0}, {"var_groups": 1},
+                                    {"group_layout": 0}])
+def test_group_sizes_and_summary_layouts(hq, hkv, layout):
+    run(workload(num_q_heads=hq, num_kv_heads=hkv, decode_steps=4), 4, check=(0, 3), **layout)
+
+
+@pytest.mark.parametrize("bs", [16, 32, 64])
+@pytest.mark.parametrize("ctx", [1536, 16 * 256 - 1, 16 * 256, 16 * 257 + 1])
+def test_lengths_around_tiles_and_block_rollovers(bs, ctx):
+    run(workload(ctx=ctx, ctx_min=ctx - 40, block_size=bs, budget_tokens=bs * 9, decode_steps=3), 3, check=(0, 2))
+
+
+@pytest.mark.parametrize("batch,hkv", [(1, 1), (9, 2), (5, 8), (9, 8)])   # cluster sizes 16, 6, 3 and 2
+def test_cluster_sizes(batch, hkv):
+    run(workload(batch=batch, num_q_heads=4 * hkv, num_kv_heads=hkv, ctx=16 * 300 + 9, needles=1), 2)
+
+
+@pytest.mark.parametrize("layout", [{"variant": 1}, {"variant": 2}, {"variant": 4}, {"sink": 2, "recent": 3},
+                                    {"recent": 0}, {"variant": 4, "stat_bf16": 1}])
+def test_ablations_and_mandatory_counts(layout):
+    run(workload(), 2, **layout)
+
+
+def test_every_block_selected_in_some_or_all_sequences():
+    run(workload(budget_tokens=16 * 200), 2)              # K >= X everywhere: dense attention
+    run(workload(ctx_min=16 * 10, budget_tokens=16 * 60), 2)
+
+
+def test_an_empty_and_a_full_sequence():
+    w = workload(batch=3, ctx_min=16 * 20, decode_steps=0)
+    d = setup(w)
+    cap = d.table.shape[1] * 16
+    d.lens[1], d.lens[2] = 0, cap
+    d.ckv.stats_build(d.k_pool, d.v_pool, d.table, d.lens, cap)
+    q = torch.from_numpy(synth.queries(w, 0)).to(d.dtype).cuda()
+    out, lse, ids, cnt = d.ckv.decode(q, d.k_pool, d.v_pool, d.table, d.lens, cap, w.budget_tokens)
+    torch.cuda.synchronize()
+    assert cnt[1].tolist() == [0, 0] and bool((ids[1] == -1).all()) and float(out[1].float().abs().max()) == 0.0
+    assert d.ckv.read_status() in (0, binding.CKV_DEV_BAD_PAGE)   # sequence 2 has no pages behind its generated rows
+    d.lens[2] = 16 * 20
+    kn = torch.zeros(3, 2, 128, dtype=d.dtype, device="cuda")
+    d.lens[0] = cap
+    d.ckv.step(q, kn, kn, d.k_pool, d.v_pool, d.table, d.lens, cap, w.budget_tokens)
+    torch.cuda.synchronize()
+    assert int(d.lens[0]) == cap and d.ckv.read_status() & binding.CKV_DEV_SEQ_FULL
+
+
+@pytest.mark.parametrize("copies", [1, 3])
+def test_ties_at_the_cut_take_the_lowest_ids(copies):
+    """All pages hold one of `copies` contents: the cut falls among hundreds of equal scores, more than the direct ranking
+    takes, and the lowest block ids win."""
+    w = workload(batch=1, num_q_heads=4, num_kv_heads=1, ctx=16 * 900, ctx_min=None, decode_steps=0, needles=0,
+                 outlier_dims=0, shuffle_pages=False)
+    d = setup(w)
+    d.k_pool.copy_(d.k_pool[:copies].repeat((900 + copies - 1) // copies, 1, 1, 1)[:900])
+    d.ckv.stats_build(d.k_pool, d.v_pool, d.table, d.lens, d.max_len)
+    q = torch.from_numpy(synth.queries(w, 0)).to(d.dtype).cuda()
+    out, lse, ids, cnt = d.ckv.decode(q, d.k_pool, d.v_pool, d.table, d.lens, d.max_len, 16 * 40)
+    sc = d.ckv.copy_scores(1)[0, 0, :900].cpu()
+    rest = sorted(range(1, 898), key=lambda b: (-float(sc[b]), b))[:37]
+    assert ids[0, 0].tolist() == sorted([0, 898, 899] + rest)
+    assert d.ckv.read_status() == 0
+
+
+def test_a_wait_that_runs_out_is_reported_and_the_context_recovers():
+    w = workload(batch=1, ctx_min=None, decode_steps=0)
+    d = setup(w)
+    d.ckv.stats_build(d.k_pool, d.v_pool, d.table, d.lens, d.max_len)
+    q = torch.from_numpy(synth.queries(w, 0)).to(d.dtype).cuda()
+    good = [t.clone() for t in d.ckv.decode(q, d.k_pool, d.v_pool, d.table, d.lens, d.max_len, w.budget_tokens)]
+    d.ckv.debug_set(1 << 10, binding.CKV_DEBUG_SKIP_FILL)
+    d.ckv.decode(q, d.k_pool, d.v_pool, d.table, d.lens, d.max_len, w.budget_tokens)
+    torch.cuda.synchronize()
+    assert d.ckv.read_status() & binding.CKV_DEV_TIMEOUT
+    d.ckv.debug_set(0, 0)
+    again = d.ckv.decode(q, d.k_pool, d.v_pool, d.table, d.lens, d.max_len, w.budget_tokens)
+    torch.cuda.synchronize()
+    assert d.ckv.read_status() == 0 and all(torch.equal(x, y) for x, y in zip(good, again))
