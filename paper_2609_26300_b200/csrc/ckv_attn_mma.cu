@@ -8,14 +8,14 @@
 // page (16 tokens: a 4 KB K tile and a 4 KB V tile, each contiguous in the paged pool) into one of its two
 // shared-memory buffers with 16-byte cp.async pieces whose destinations are XOR-swizzled by the token row, so
 // that the matrix loads below are conflict-free; rows past the sequence end are zero-filled; the next page is
-// in flight while the current one is multiplied.  Then, with the G heads as the M dimension (rows 0..7 of 16)
-// of mma.sync.m16n8k16:
-//   S^T = Q K^T      heads x 16 tokens, Q fragments held in registers for the whole kernel
-//   P   = 2^(S^T - m) per warp, running maximum raised only when exceeded by a slack; split into bf16 hi + lo
-//   O  += P V        heads x 128 coordinates; the accumulator layout of S^T is the A-operand layout of P V
+// in flight while the current one is multiplied.  Then, with mma.sync.m16n8k16 and the heads as its N dimension
+// (ckv_mma.cuh):
+//   S    = K Q^T     16 tokens x heads, Q fragments held in registers for the whole kernel
+//   P    = 2^(S - m) per warp, running maximum raised only when exceeded by a slack; split into bf16 hi + lo
+//   O^T += V^T P     128 coordinates x heads
 // For every selected block the scan kernel has already added the block's mean term |b| e^{zbar} vbar_b to
 // the all-block compensation sum; here the same terms are subtracted, three blocks at a time, with one more
-// P V-shaped product whose non-zero rows are the blocks' mean values (read as their stored hi + lo halves):
+// P V-shaped product whose non-zero rows are the blocks' stored mean values:
 //   merge = exact(S) + mean(all) - mean(S) = exact(S) + mean(not S).
 //
 // Merge.  The scan's partials of the unit (one per scan CTA and consumer warp) exist before this kernel
@@ -68,8 +68,7 @@ ckv_attn_mma_kernel(CkvDev P, const __nv_bfloat16 *__restrict__ q, const __nv_bf
   if (CL) cluster_arrive_relaxed();   // first phase of the cluster barrier: "this CTA runs, its shared memory exists"
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int head = lane >> 2, qd = lane & 3;
-  const bool hv = head < G;
+  using T = HeadTile<G>;   // which heads a lane works on
   const int unit = blockIdx.y, s = ckv_div_hkv(P, unit), h = unit - s * P.Hkv;
   const int pshift = P.ppb == 1 ? 0 : (P.ppb == 2 ? 1 : 2);
   const int p0 = blockIdx.x * pages_per_split;
@@ -162,10 +161,8 @@ ckv_attn_mma_kernel(CkvDev P, const __nv_bfloat16 *__restrict__ q, const __nv_bf
   if (lane < 16) reinterpret_cast<uint4 *>(waux + kZeroRow)[lane] = make_uint4(0u, 0u, 0u, 0u);
 
   const float sl2 = P.scale * kLog2e;
-  float acc[16][2];
-#pragma unroll
-  for (int t = 0; t < 16; ++t) { acc[t][0] = 0.f; acc[t][1] = 0.f; }
-  float m_ref = -CUDART_INF_F, l_acc = 0.f;
+  HeadAcc<G> w;
+  w.reset();
   const int *pt_row = page_table + (size_t)s * P.max_pages_per_seq;
   const int n_mine = max((p1 - p0 - warp + W - 1) / W, 0);   // this warp's pages: list index p0 + warp + W n
   const float *lz = P.lz + (size_t)unit * P.max_blocks * G;
@@ -267,52 +264,38 @@ ckv_attn_mma_kernel(CkvDev P, const __nv_bfloat16 *__restrict__ q, const __nv_bf
 #pragma unroll
   for (int j = 0; j < kMeanFlush; ++j) { bb[j] = 0; bsl[j] = 0; }
   auto remove_means = [&]() {
-    float zl[2] = {-CUDART_INF_F, -CUDART_INF_F};
-    if (hv && qd < 2) {
+    // row j < nb of the tile is the mean-value row of batch entry j, every other row the row of zeros; this lane's
+    // weights: its heads of batch entry `row`
+    float z[T::NR][2], x[T::NR][2];
 #pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        const int j = 2 * qd + e;
-        if (j < nb) {
-          const int slot = j == 0 ? bsl[0] : (j == 1 ? bsl[1] : bsl[2]);
-          zl[e] = *reinterpret_cast<const float *>(waux + kLsOff + (slot * G + head) * 4);
-        }
+    for (int k = 0; k < T::NR; ++k) {
+      const int j = T::row(lane, k);
+      const int slot = j == 0 ? bsl[0] : (j == 1 ? bsl[1] : bsl[2]);
+#pragma unroll
+      for (int e = 0; e < 2; ++e)
+        z[k][e] = j < nb && T::head(lane, e) < G ? *reinterpret_cast<const float *>(waux + kLsOff + (slot * G + T::head(lane, e)) * 4) : -CUDART_INF_F;
+    }
+    attn_raise<G>(z, w);
+#pragma unroll
+    for (int k = 0; k < T::NR; ++k)
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {   // the negated weights
+        x[k][e] = z[k][e] == -CUDART_INF_F ? 0.f : -fast_exp2(z[k][e] - w.m[e]);
+        w.l[e] += x[k][e];
       }
-    }
-    float zmax = fmaxf(zl[0], zl[1]);
-    zmax = fmaxf(zmax, __shfl_xor_sync(0xffffffffu, zmax, 1));
-    zmax = fmaxf(zmax, __shfl_xor_sync(0xffffffffu, zmax, 2));
-    if (zmax > m_ref + CKV_RESCALE_SLACK) {
-      const float sc = exp2_diff(m_ref, zmax);
-      m_ref = zmax;
-      l_acc *= sc;
-#pragma unroll
-      for (int t = 0; t < 16; ++t) { acc[t][0] *= sc; acc[t][1] *= sc; }
-    }
-    const float w0 = zl[0] == -CUDART_INF_F ? 0.f : fast_exp2(zl[0] - m_ref);
-    const float w1 = zl[1] == -CUDART_INF_F ? 0.f : fast_exp2(zl[1] - m_ref);
-    l_acc -= w0 + w1;
-    // A operand: columns 0..nb-1 (the real rows of the B operand) hold the negated weights
-    const uint32_t wh = pack_bf16(-w0, -w1);
-    const uint32_t wl = pack_bf16(-(w0 - bf16_round(w0)), -(w1 - bf16_round(w1)));
-    // B operand: row j < nb is the mean-value row of batch entry j, every other row the row of zeros
-    const int r = ((lane >> 3) & 1) * 8 + (lane & 7);
+    uint32_t wb[T::NR][2];
+    T::weights(x, lane, wb);
+    const int r = (lane >> 4) * 8 + (lane & 7), cpar = (lane >> 3) & 1;
     const bool real = r < nb;
     const int rblk = r == 0 ? bb[0] : (r == 1 ? bb[1] : bb[2]);
     const int rslot = r == 0 ? bsl[0] : (r == 1 ? bsl[1] : bsl[2]);
     const uint32_t rowaddr = aux_u32 + 512 * (real ? rslot : 0);
-    const int cpar = lane >> 4;
 #pragma unroll
-    for (int t2 = 0; t2 < 8; ++t2) {
-      const uint32_t coff = (uint32_t)(swz_chunk(2 * t2 + cpar, rblk) << 4);
-      uint32_t vh[4], vl[4];
-      ldmatrix_x4_trans(vh, real ? rowaddr + coff : aux_u32 + kZeroRow);
-      ldmatrix_x4_trans(vl, real && mean_lo ? rowaddr + 256 + coff : aux_u32 + kZeroRow);   // no lo halves: zeros
-      mma_rows8(acc[2 * t2][0], acc[2 * t2][1], wh, 0u, vh[0], vh[1]);
-      mma_rows8(acc[2 * t2][0], acc[2 * t2][1], wl, 0u, vh[0], vh[1]);
-      mma_rows8(acc[2 * t2][0], acc[2 * t2][1], wh, 0u, vl[0], vl[1]);
-      mma_rows8(acc[2 * t2 + 1][0], acc[2 * t2 + 1][1], wh, 0u, vh[2], vh[3]);
-      mma_rows8(acc[2 * t2 + 1][0], acc[2 * t2 + 1][1], wl, 0u, vh[2], vh[3]);
-      mma_rows8(acc[2 * t2 + 1][0], acc[2 * t2 + 1][1], wh, 0u, vl[2], vl[3]);
+    for (int t = 0; t < 8; ++t) {
+      uint32_t v[4];
+      ldmatrix_x4_trans(v, real ? rowaddr + (uint32_t)(swz_chunk(2 * t + cpar, rblk) << 4) : aux_u32 + kZeroRow);
+      mma_16816(w.acc[t], v, wb[0][0], wb[0][1]);
+      if constexpr (!T::PAIR) mma_16816(w.acc[t], v, wb[T::NR - 1][0], wb[T::NR - 1][1]);
     }
     nb = 0;
   };
@@ -334,18 +317,15 @@ ckv_attn_mma_kernel(CkvDev P, const __nv_bfloat16 *__restrict__ q, const __nv_bf
   }
   // Everything the first page copy does not need is requested behind it: the queries (first used by the first
   // product) and the place of the unit's scan partials (first used with the last page).
-  // Q fragments: A operand rows 0..7 = heads, scaled logits come out of the products in log2 units
+  // Q fragments: B operand columns = heads (columns without a head of their own hold some head's row: finite values
+  // whose weights are zero, and a load that nothing has to look at before the first product)
   uint32_t qa[8][2];
   {
-    const __nv_bfloat16 *qrow = q + ((size_t)s * P.Hq + h * G + (hv ? head : 0)) * CKV_D;
+    const __nv_bfloat16 *qrow = q + ((size_t)s * P.Hq + h * G + (T::col_head(lane) & (G - 1))) * CKV_D + 2 * (lane & 3);
 #pragma unroll
     for (int ks = 0; ks < 8; ++ks)
 #pragma unroll
-      for (int hh = 0; hh < 2; ++hh) {
-        // rows G..7 repeat head 0: finite values whose products are never used (their weights are zero), and a
-        // load that nothing has to look at before the first product
-        qa[ks][hh] = __ldg(reinterpret_cast<const uint32_t *>(qrow + 16 * ks + 8 * hh + 2 * qd));
-      }
+      for (int hh = 0; hh < 2; ++hh) qa[ks][hh] = __ldg(reinterpret_cast<const uint32_t *>(qrow + 16 * ks + 8 * hh));
   }
   if (comp) {
     int efirst = 0, n_comp = 0;   // where the unit's scan partials sit
@@ -372,11 +352,15 @@ ckv_attn_mma_kernel(CkvDev P, const __nv_bfloat16 *__restrict__ q, const __nv_bf
     if (cur.phys >= 0) {
       const uint32_t kb = wtiles_u32 + buf * kPageBytes;
       const uint32_t vb = kb + kTileBytes;
-      // log2 of e^{zbar} of the page's block for this lane's head (token-weight removal)
-      float lzt = -CUDART_INF_F;
-      if (tok_rm && hv)
-        lzt = *reinterpret_cast<const float *>(waux + kLsOff + (buf * G + head) * 4) - (cur.blk == X - 1 ? lg_last : lg_bs);
-      attn_page<false>(kb, vb, qa, cur.ntok, hv, lane, sl2, lzt, acc, m_ref, l_acc);
+      // log2 of e^{zbar} of the page's block for this lane's heads (token-weight removal)
+      float lzt[2] = {-CUDART_INF_F, -CUDART_INF_F};
+      if (tok_rm) {
+        const float lb = cur.blk == X - 1 ? lg_last : lg_bs;
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+          if (T::head(lane, e) < G) lzt[e] = *reinterpret_cast<const float *>(waux + kLsOff + (buf * G + T::head(lane, e)) * 4) - lb;
+      }
+      attn_page<G>(kb, vb, qa, cur.ntok, lane, sl2, lzt, w);
       if (row_rm && cur.first) {   // its mean-value row sits in aux slot cur_slot
 #pragma unroll
         for (int j = 0; j < kMeanFlush; ++j)
@@ -408,13 +392,14 @@ ckv_attn_mma_kernel(CkvDev P, const __nv_bfloat16 *__restrict__ q, const __nv_bf
   float(*s_scale)[G] = reinterpret_cast<float(*)[G]>(smem + (size_t)W * 2 * kPageBytes);
   int *s_ent = reinterpret_cast<int *>(smem + (size_t)W * 2 * kPageBytes + kMaxEntries * G * 4);
   __syncthreads();   // every warp is done with its aux rows
-  l_acc += __shfl_xor_sync(0xffffffffu, l_acc, 1);
-  l_acc += __shfl_xor_sync(0xffffffffu, l_acc, 2);
-  if (hv) {
-    float *r = sf + region(warp, red_buf(warp)) + head * CKV_PART_STRIDE;
+  {
+    float *r = sf + region(warp, red_buf(warp));
+    w.fold(lane, [&](int g, int c, float v) { r[g * CKV_PART_STRIDE + 4 + c] = v; });
 #pragma unroll
-    for (int t = 0; t < 16; ++t) *reinterpret_cast<float2 *>(r + 4 + 8 * t + 2 * qd) = make_float2(acc[t][0], acc[t][1]);
-    if (qd == 0) { r[0] = m_ref; r[1] = l_acc; }
+    for (int e = 0; e < 2; ++e) {
+      const float l = T::sum_rows(w.l[e]);
+      if (T::owns(lane, e)) { r[T::head(lane, e) * CKV_PART_STRIDE] = w.m[e]; r[T::head(lane, e) * CKV_PART_STRIDE + 1] = l; }
+    }
   }
   if (tid < W + kSlots) {
     int off;

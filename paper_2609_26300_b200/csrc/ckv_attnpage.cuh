@@ -20,7 +20,6 @@ __device__ __forceinline__ void cp_async4(uint32_t dst, const void *src) {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-
 // Start the copies of one page (k, v: its first row): 256 16-byte pieces per tile, 8 per lane; piece c of row r lands at
 // chunk c ^ (r & 7) of the row, so that the matrix loads below are conflict-free; rows at or past ntok are zero-filled.
 __device__ __forceinline__ void issue_page(uint32_t kb, uint32_t vb, const __nv_bfloat16 *k, const __nv_bfloat16 *v, int ntok, int lane) {
@@ -35,86 +34,85 @@ __device__ __forceinline__ void issue_page(uint32_t kb, uint32_t vb, const __nv_
   }
 }
 
-// O += P V for one tile of 16 value rows at vb (swizzled by row): A fragments of the weights as bf16 hi and lo halves.
-__device__ __forceinline__ void attn_pv(uint32_t vb, const uint32_t (&ph)[2], const uint32_t (&pl)[2], int lane, float (&acc)[16][2]) {
-  const int r = ((lane >> 3) & 1) * 8 + (lane & 7);
+// O += rows^T W for the tile of 16 value rows at vb (swizzled by row): the lane's weights x (HeadTile).
+template <int G>
+__device__ __forceinline__ void attn_pv(uint32_t vb, const float (&x)[HeadTile<G>::NR][2], int lane, HeadAcc<G> &w) {
+  uint32_t b[HeadTile<G>::NR][2];
+  HeadTile<G>::weights(x, lane, b);
+  // ldmatrix.trans lane roles: matrix lane / 8 -> (coordinate chunk parity, row half), row lane % 8
+  const int r = (lane >> 4) * 8 + (lane & 7), cpar = (lane >> 3) & 1;
   const uint32_t rowaddr = vb + r * kRowBytes;
-  const int cpar = lane >> 4;
 #pragma unroll
-  for (int t2 = 0; t2 < 8; ++t2) {   // two 8-coordinate n-tiles per ldmatrix.x4
-    uint32_t v[4];
-    ldmatrix_x4_trans(v, rowaddr + (uint32_t)(((2 * t2 + cpar) ^ (r & 7)) << 4));
-    mma_rows8(acc[2 * t2][0], acc[2 * t2][1], ph[0], ph[1], v[0], v[1]);
-    mma_rows8(acc[2 * t2][0], acc[2 * t2][1], pl[0], pl[1], v[0], v[1]);
-    mma_rows8(acc[2 * t2 + 1][0], acc[2 * t2 + 1][1], ph[0], ph[1], v[2], v[3]);
-    mma_rows8(acc[2 * t2 + 1][0], acc[2 * t2 + 1][1], pl[0], pl[1], v[2], v[3]);
+  for (int t = 0; t < 8; ++t) {   // 16 coordinates
+    uint32_t a[4];
+    ldmatrix_x4_trans(a, rowaddr + (uint32_t)(((2 * t + cpar) ^ (r & 7)) << 4));
+    mma_16816(w.acc[t], a, b[0][0], b[0][1]);
+    if constexpr (!HeadTile<G>::PAIR) mma_16816(w.acc[t], a, b[1][0], b[1][1]);
   }
 }
 
-// The running maximum is raised to tmax when that exceeds it by the slack, and what was accumulated is rescaled.
-__device__ __forceinline__ void attn_raise(float tmax, float &m_ref, float &l_acc, float (&acc)[16][2]) {
-  if (tmax > m_ref + CKV_RESCALE_SLACK) {
-    const float sc = exp2_diff(m_ref, tmax);
-    m_ref = tmax;
-    l_acc *= sc;
+// The running maxima are raised to those of z (the lane's values) where these exceed them by the slack.  One vote in the
+// usual case that nothing does.
+template <int G, int N>
+__device__ __forceinline__ void attn_raise(const float (&z)[N][2], HeadAcc<G> &w) {
+  float mx[2] = {z[0][0], z[0][1]};
 #pragma unroll
-    for (int t = 0; t < 16; ++t) { acc[t][0] *= sc; acc[t][1] *= sc; }
+  for (int k = 1; k < N; ++k) { mx[0] = fmaxf(mx[0], z[k][0]); mx[1] = fmaxf(mx[1], z[k][1]); }
+  if (!__any_sync(0xffffffffu, mx[0] > w.m[0] + CKV_RESCALE_SLACK || mx[1] > w.m[1] + CKV_RESCALE_SLACK)) return;
+#pragma unroll
+  for (int e = 0; e < 2; ++e) {
+    const float t = HeadTile<G>::max_rows(mx[e]);
+    if (t > w.m[e] + CKV_RESCALE_SLACK) {
+      w.rescale(e, exp2_diff(w.m[e], t));
+      w.m[e] = t;
+    }
   }
 }
 
-// One page: S^T = Q K^T, P = 2^(S^T - m) - 2^(lzt - m) (lzt: log2 of what is taken off every token's weight, -inf for
-// nothing), O += P V.  sl2: logit scale in log2 units.  hv: this lane's head exists.  SHARED: the lanes 16 above hold
-// partial sums of the same heads (G <= 4) and follow their running maximum.
-template <bool SHARED>
-__device__ __forceinline__ void attn_page(uint32_t kb, uint32_t vb, const uint32_t (&qa)[8][2], int ntok, bool hv, int lane,
-                                          float sl2, float lzt, float (&acc)[16][2], float &m_ref, float &l_acc) {
-  const int qd = lane & 3;
-  // ---- S^T = Q K^T: heads x 16 tokens (two n-tiles of 8 tokens) ----
-  float sv[2][2] = {{0.f, 0.f}, {0.f, 0.f}}, sv2[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
+// One page: logits L = K q^T, weights 2^(L - m) - 2^(lzt - m) (lzt: log2 of what is taken off every token's weight, per
+// head of the lane, -inf for nothing), O += V^T W.  qa: the queries' B fragments; sl2: logit scale in log2 units.
+template <int G>
+__device__ __forceinline__ void attn_page(uint32_t kb, uint32_t vb, const uint32_t (&qa)[8][2], int ntok, int lane, float sl2,
+                                          const float (&lzt)[2], HeadAcc<G> &w) {
+  using T = HeadTile<G>;
+  float z[4] = {0.f, 0.f, 0.f, 0.f}, z2[4] = {0.f, 0.f, 0.f, 0.f};   // two chains: the products of one depend on one another
   {
-    const int lrow = lane & 7, lmat = lane >> 3;
+    // ldmatrix lane roles: matrix lane / 8 -> (row half, coordinate chunk parity), row lane % 8
+    const int r = ((lane >> 3) & 1) * 8 + (lane & 7), cpar = lane >> 4;
+    const uint32_t rowaddr = kb + r * kRowBytes;
 #pragma unroll
-    for (int nt = 0; nt < 2; ++nt) {
-      const int r = nt * 8 + lrow;
-      const uint32_t rowaddr = kb + r * kRowBytes;
+    for (int ks = 0; ks < 8; ks += 2) {
+      uint32_t a[4], a2[4];
+      ldmatrix_x4(a, rowaddr + (uint32_t)(((2 * ks + cpar) ^ (r & 7)) << 4));
+      ldmatrix_x4(a2, rowaddr + (uint32_t)(((2 * ks + 2 + cpar) ^ (r & 7)) << 4));
+      mma_16816(z, a, qa[ks][0], qa[ks][1]);
+      mma_16816(z2, a2, qa[ks + 1][0], qa[ks + 1][1]);
+    }
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {   // two 16-coordinate steps per ldmatrix.x4
-        uint32_t b[4];
-        ldmatrix_x4(b, rowaddr + (uint32_t)(((4 * j + lmat) ^ (r & 7)) << 4));
-        mma_rows8(sv[nt][0], sv[nt][1], qa[2 * j][0], qa[2 * j][1], b[0], b[1]);
-        mma_rows8(sv2[nt][0], sv2[nt][1], qa[2 * j + 1][0], qa[2 * j + 1][1], b[2], b[3]);
-      }
-      sv[nt][0] += sv2[nt][0]; sv[nt][1] += sv2[nt][1];
+    for (int i = 0; i < 4; ++i) z[i] += z2[i];
+  }
+  float s[T::NR + 1][2], x[T::NR][2];
+  {
+    float v[T::NR][2];
+    T::pick(z, lane, v);
+#pragma unroll
+    for (int k = 0; k < T::NR; ++k)
+#pragma unroll
+      for (int e = 0; e < 2; ++e)
+        s[k][e] = T::row(lane, k) < ntok && T::head(lane, e) < G ? v[k][e] * sl2 : -CUDART_INF_F;
+    s[T::NR][0] = lzt[0]; s[T::NR][1] = lzt[1];
+  }
+  attn_raise<G>(s, w);
+#pragma unroll
+  for (int e = 0; e < 2; ++e) {
+    const float off = lzt[e] == -CUDART_INF_F ? 0.f : fast_exp2(lzt[e] - w.m[e]);
+#pragma unroll
+    for (int k = 0; k < T::NR; ++k) {
+      x[k][e] = s[k][e] == -CUDART_INF_F ? 0.f : fast_exp2(s[k][e] - w.m[e]) - off;
+      w.l[e] += x[k][e];
     }
   }
-  // ---- softmax weights for this thread's head and its four tokens ----
-  float tmax = lzt;
-#pragma unroll
-  for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      const bool ok = hv && nt * 8 + 2 * qd + e < ntok;
-      sv[nt][e] = ok ? sv[nt][e] * sl2 : -CUDART_INF_F;
-      tmax = fmaxf(tmax, sv[nt][e]);
-    }
-  tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, 1));
-  tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, 2));
-  if (SHARED) tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, 16));
-  attn_raise(tmax, m_ref, l_acc, acc);
-  const float wtok = lzt == -CUDART_INF_F ? 0.f : fast_exp2(lzt - m_ref);
-  uint32_t ph[2], pl[2];
-#pragma unroll
-  for (int nt = 0; nt < 2; ++nt) {
-    float p[2];
-#pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      p[e] = sv[nt][e] == -CUDART_INF_F ? 0.f : fast_exp2(sv[nt][e] - m_ref) - wtok;
-      l_acc += p[e];
-    }
-    ph[nt] = pack_bf16(p[0], p[1]);
-    pl[nt] = pack_bf16(p[0] - bf16_round(p[0]), p[1] - bf16_round(p[1]));
-  }
-  attn_pv(vb, ph, pl, lane, acc);
+  attn_pv<G>(vb, x, lane, w);
 }
 
 #endif  // CKV_ATTNPAGE_CUH_

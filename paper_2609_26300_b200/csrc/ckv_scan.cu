@@ -11,11 +11,10 @@
 // blocks that end up selected are taken out again by the attention kernel.  That way kbar, Dbar and
 // vbar are each read from HBM exactly once per decode step.
 //
-// The two contractions are the GQA-grouped Q Kbar^T and W Vbar tiles, on mma.sync.m16n8k16 (bf16 in,
-// fp32 accumulate): heads are the M dimension (G <= 8 rows of 16 used), 8 blocks the N dimension of
-// Q Kbar^T, whose accumulator layout is the A-operand layout of W Vbar.  The summaries are stored as
-// split bf16 pairs (hi + lo), so x * y is hi * y + lo * y with no conversion instructions; the weights
-// w = |b| e^{zbar - m} are split the same way (three products per tile: hi hi, lo hi, hi lo).
+// The two contractions are the GQA-grouped Kbar Q^T and Vbar^T W tiles, on mma.sync.m16n8k16 (bf16 in, fp32
+// accumulate): 16 blocks (then 16 coordinates) are the M dimension, the heads the N dimension (ckv_mma.cuh).  The
+// summaries are stored as split bf16 pairs (hi + lo), so x * y is hi * y + lo * y with no conversion instructions; the
+// weights w = |b| e^{zbar - m} are split the same way.
 //
 // Schedule: the launch has two kinds of CTAs.  The first few ("tail" CTAs, one warp per unit) take the LAST block
 // of every sequence -- the only block a decode step can change -- and, in a fused step, first append the step's new
@@ -410,11 +409,7 @@ ckv_scan_kernel(CkvDev P, const QT *__restrict__ q, const int *seq_lens, int uni
     }
   } else {
     // ---------------- consumer warps: half tile j = warp, warp + 8, ... of the CTA's range ----------------
-    const int head = lane >> 2, qd = lane & 3;   // this thread's accumulator row (head) and column pair
-    const bool hv = head < G;
-    constexpr bool SP = (G <= 4) && !RD;   // the per-(head, block) arithmetic is shared between the half warps
-    const int ehead = SP ? (head & 3) : head;
-    const bool ehv = ehead < G;
+    using T = HeadTile<G>;   // which heads a lane works on
     const bool staged = !QS && !RD && P.r == 4;   // bf16 queries, four variance groups: the staged setup below
     if (staged) {
       constexpr int kPieces = G * CKV_D * 2 / 16;   // 16-byte pieces of a unit's G query rows
@@ -444,13 +439,10 @@ ckv_scan_kernel(CkvDev P, const QT *__restrict__ q, const int *seq_lens, int uni
     }
     ScanUnit<G, QT, RD> w;
     w.reset();
-#pragma unroll
-    for (int t = 0; t < 4; ++t) w.wown[t] = 0.f;
     float *sw = sw_all + (size_t)warp * P.r * G;   // [t][g], r != 4 only
     const ScanPartCfg cfg{P.scale, P.half_var, logf((float)P.bs), P.r, P.max_blocks,
                           (P.variant & CKV_VARIANT_RANK_BY_MASS) != 0, r4};
     float log_last = 0.f;   // log of the token count of the unit's last block, when the scan CTAs cover it
-    const bool pair_ok = (P.max_blocks & 1) == 0;   // rows of the per-block outputs start on 8-byte boundaries
     const int ulast = s_ulast;
     int u = s_u0, tl = s_tl0, cur = -1, next_empty = s_u0;
     UnitInfo ui = unit_info(P, s_len, seq_lens, u);
@@ -468,17 +460,14 @@ ckv_scan_kernel(CkvDev P, const QT *__restrict__ q, const int *seq_lens, int uni
         }
         return;
       }
-      // l and lp: sum over the four lanes that share the head
-      float l = w.l_acc, lp = w.lp_acc;
-      l += __shfl_xor_sync(0xffffffffu, l, 1); l += __shfl_xor_sync(0xffffffffu, l, 2);
-      lp += __shfl_xor_sync(0xffffffffu, lp, 1); lp += __shfl_xor_sync(0xffffffffu, lp, 2);
-      if (SP) { l += __shfl_xor_sync(0xffffffffu, l, 16); lp += __shfl_xor_sync(0xffffffffu, lp, 16); }
-      if (hv) {
-        float *pg = part + head * CKV_PART_STRIDE;
+      w.fold(lane, [&](int g, int c, float v) { part[g * CKV_PART_STRIDE + 4 + c] = v; });
 #pragma unroll
-        for (int t = 0; t < 16; ++t)
-          *reinterpret_cast<float2 *>(pg + 4 + 8 * t + 2 * qd) = make_float2(w.acc[t][0], w.acc[t][1]);
-        if (qd == 0) { pg[0] = w.m_ref; pg[1] = l; pg[2] = lp; }
+      for (int e = 0; e < 2; ++e) {
+        const float l = T::sum_rows(w.l[e]), lp = T::sum_rows(w.lp[e]);
+        if (T::owns(lane, e)) {
+          float *pg = part + T::head(lane, e) * CKV_PART_STRIDE;
+          pg[0] = w.m[e]; pg[1] = l; pg[2] = lp;
+        }
       }
     };
     // units of this CTA's range that this warp never worked on still need an (empty) partial
@@ -524,57 +513,50 @@ ckv_scan_kernel(CkvDev P, const QT *__restrict__ q, const int *seq_lens, int uni
         fill_empty_upto(u);
         // per-unit setup: query fragments, variance weights, fresh accumulators
         const int s = ckv_div_hkv(P, u), h = u - s * P.Hkv;
-        const QT *qrow = q + ((size_t)s * P.Hq + h * G + (hv ? head : 0)) * CKV_D;
+        const QT *qrow = q + ((size_t)s * P.Hq + h * G) * CKV_D;
         const int uk = u - s_u0;
         const bool from_smem = staged && uk < kStagedUnits;
         if (from_smem) {
-          const uint32_t *srow = reinterpret_cast<const uint32_t *>(&s_q[uk][hv ? head : 0][0]);
+          w.set_queries(lane, P.scale, [&](int g, int c) {
+            const uint32_t x = *reinterpret_cast<const uint32_t *>(&s_q[uk][g][c]);
+            return make_float2(__uint_as_float(x << 16), __uint_as_float(x & 0xffff0000u));
+          });
 #pragma unroll
-          for (int ks = 0; ks < 8; ++ks)
+          for (int e = 0; e < 2; ++e)
 #pragma unroll
-            for (int hh = 0; hh < 2; ++hh) w.qa[ks][hh] = hv ? srow[(16 * ks + 8 * hh + 2 * qd) / 2] : 0u;
-#pragma unroll
-          for (int t = 0; t < 4; ++t) w.wown[t] = ehv ? s_w[uk][ehead][t] : 0.f;
+            for (int t = 0; t < 4; ++t) w.wown[e][t] = T::head(lane, e) < G ? s_w[uk][T::head(lane, e) & (G - 1)][t] : 0.f;
         } else {
-#pragma unroll
-        for (int ks = 0; ks < 8; ++ks) {
-#pragma unroll
-          for (int hh = 0; hh < 2; ++hh) {
-            const int c0 = 16 * ks + 8 * hh + 2 * qd;
-            const float x0 = hv ? to_float(qrow[c0]) : 0.f, x1 = hv ? to_float(qrow[c0 + 1]) : 0.f;
-            w.qa[ks][hh] = pack_bf16(x0, x1);
-            if (QS) w.qb[QS ? ks : 0][hh] = pack_bf16(x0 - bf16_round(x0), x1 - bf16_round(x1));
-            if (RD) {
-              const float s0 = (x0 * P.scale) * (x0 * P.scale), s1 = (x1 * P.scale) * (x1 * P.scale);
-              w.qsh[RD ? ks : 0][hh] = pack_bf16(s0, s1);
-              w.qsl[RD ? ks : 0][hh] = pack_bf16(s0 - bf16_round(s0), s1 - bf16_round(s1));
-            }
-          }
-        }
+          w.set_queries(lane, P.scale, [&](int g, int c) {
+            return make_float2(to_float(qrow[(size_t)g * CKV_D + c]), to_float(qrow[(size_t)g * CKV_D + c + 1]));
+          });
         }
         if (from_smem) {
           // set up above
         } else if (RD) {
           // nothing to tabulate: the weights are the squared queries held above
         } else if (r4) {
-          // w_{g,t} for this thread's head: every lane of the quad sums all 128 coordinates (once per unit)
-          float wsum[4] = {0.f, 0.f, 0.f, 0.f};
-          const QT *qrow_e = q + ((size_t)s * P.Hq + h * G + (ehv ? ehead : 0)) * CKV_D;
+          // w_{g,t} for this lane's heads: every lane that works on a head sums all 128 coordinates (once per unit)
+#pragma unroll 1
+          for (int e = 0; e < 2; ++e) {
+            float wsum[4] = {0.f, 0.f, 0.f, 0.f};
+            const QT *qrow_e = qrow + (size_t)(T::head(lane, e) & (G - 1)) * CKV_D;
 #pragma unroll
-          for (int c = 0; c < 16; ++c) {
-            float x[8];
-            load8<true>(qrow_e + 8 * c, x);
-            float s8 = 0.f;
+            for (int c = 0; c < 16; ++c) {
+              float x[8];
+              load8<true>(qrow_e + 8 * c, x);
+              float s8 = 0.f;
 #pragma unroll
-            for (int i = 0; i < 8; ++i) s8 = fmaf(x[i], x[i], s8);
-            // an aligned run of 8 coordinates lies in one group for r = 4 (groups are runs of 32 or 16)
-            const int t = P.glayout == 0 ? (8 * c) / 32 : ((8 * c) % 64) / 16;
-            wsum[0] += t == 0 ? s8 : 0.f; wsum[1] += t == 1 ? s8 : 0.f;
-            wsum[2] += t == 2 ? s8 : 0.f; wsum[3] += t == 3 ? s8 : 0.f;
+              for (int i = 0; i < 8; ++i) s8 = fmaf(x[i], x[i], s8);
+              // an aligned run of 8 coordinates lies in one group for r = 4 (groups are runs of 32 or 16)
+              const int t = P.glayout == 0 ? (8 * c) / 32 : ((8 * c) % 64) / 16;
+              wsum[0] += t == 0 ? s8 : 0.f; wsum[1] += t == 1 ? s8 : 0.f;
+              wsum[2] += t == 2 ? s8 : 0.f; wsum[3] += t == 3 ? s8 : 0.f;
+            }
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {   // Eq. 8's 1/d is the squared logit scale
+              if (e == 0) w.wown[0][t] = wsum[t] * (P.scale * P.scale); else w.wown[1][t] = wsum[t] * (P.scale * P.scale);
+            }
           }
-          if (!ehv) { wsum[0] = wsum[1] = wsum[2] = wsum[3] = 0.f; }
-#pragma unroll
-          for (int t = 0; t < 4; ++t) w.wown[t] = wsum[t] * (P.scale * P.scale);   // Eq. 8's 1/d is the squared logit scale
         } else {
           __syncwarp();
           for (int idx = lane; idx < P.r * G; idx += 32) {
@@ -606,16 +588,10 @@ ckv_scan_kernel(CkvDev P, const QT *__restrict__ q, const int *seq_lens, int uni
         scan_part<G, QT, RD, HS, VH>(
             w, cfg, sk, sv, (RD || r4 || dbar_bulk) ? sd : nullptr, smem_u32(s_zero_row), sw, db, lane, rb, nb, b0,
             P.tail ? -1 : ui.X - 1, log_last,   // in tail mode every block here is full
-            [&](int eh, int blk, float u0, float u1, float z0, float z1, bool v0, bool v1) {
-              // the thread's two blocks are neighbours: one 8-byte store each when the rows are 8-byte aligned
-              const size_t o = (size_t)eh * P.max_blocks + blk;
-              if (pair_ok && v1) {
-                *reinterpret_cast<float2 *>(lu + o) = make_float2(u0, u1);
-                *reinterpret_cast<float2 *>(lz + o) = make_float2(z0, z1);
-              } else {
-                if (v0) { lu[o] = u0; lz[o] = z0; }
-                if (v1) { lu[o + 1] = u1; lz[o + 1] = z1; }
-              }
+            [&](int g, int blk, float x, float y) {
+              const size_t o = (size_t)g * P.max_blocks + blk;
+              lu[o] = x;
+              lz[o] = y;
             });
       }
       }   // own part

@@ -4,6 +4,7 @@
 #ifndef CKV_SCANPART_CUH_
 #define CKV_SCANPART_CUH_
 #include "ckv_internal.cuh"
+#include "ckv_attnpage.cuh"
 #include "ckv_mma.cuh"
 #include "ckv_pipe.cuh"
 
@@ -20,20 +21,48 @@ __device__ __forceinline__ void tensor_g2s(uint32_t dst, const CUtensorMap *map,
 template <typename QT> struct QSplit { static constexpr bool value = false; };
 template <> struct QSplit<float> { static constexpr bool value = true; };
 
-// What a warp holds of the unit it works on.  Rows (heads) of the fragments: head = lane / 4 < G, zero otherwise.
+// What a warp holds of the unit it works on.
 template <int G, typename QT, bool RD>
-struct ScanUnit {
-  static constexpr bool QS = QSplit<QT>::value;      // fp32 queries are split into hi + lo like the summaries
-  uint32_t qa[8][2], qb[QS ? 8 : 1][2];              // A fragments of the unit's queries (rows 0..7), per 16-coordinate step
-  uint32_t qsh[RD ? 8 : 1][2], qsl[RD ? 8 : 1][2];   // (scale q)^2 as hi and lo halves, same fragment positions
-  float acc[16][2];                                  // W Vbar accumulator: head `head`, coordinates 8 t + 2 qd + {0, 1}
-  float wown[4];                                     // variance weights of this lane's head (r = 4)
-  float m_ref, l_acc, lp_acc;                        // running maximum, sum of weights, sum of e^{l - m}
+struct ScanUnit : HeadAcc<G> {
+  using T = HeadTile<G>;
+  static constexpr bool QS = QSplit<QT>::value;        // fp32 queries are split into hi + lo like the summaries
+  static constexpr bool QB = QS && !T::PAIR;           // ... as a second operand where columns 4..7 cannot take the lo halves
+  static constexpr bool RB = RD && !T::PAIR;
+  uint32_t qa[8][2], qb[QB ? 8 : 1][2];                // B fragments of the unit's queries, per 16-coordinate step
+  uint32_t qs[RD ? 8 : 1][2], qs2[RB ? 8 : 1][2];      // (scale q)^2, same fragment positions: columns hi | lo, or two operands
+  float wown[2][4];                                    // variance weights of this lane's heads (r = 4)
+  float lp[2];                                         // sum of e^{l - m}
 
   __device__ __forceinline__ void reset() {
+    HeadAcc<G>::reset();
+    lp[0] = lp[1] = 0.f;
+  }
+  // Query fragments; row(head, c): coordinates c, c + 1 of a head as floats.
+  template <class F>
+  __device__ __forceinline__ void set_queries(int lane, float scale, F row) {
+    const int h = T::col_head(lane), qd = lane & 3;
+    const bool hv = h < G, low = T::PAIR && lane >= 16;
 #pragma unroll
-    for (int t = 0; t < 16; ++t) { acc[t][0] = 0.f; acc[t][1] = 0.f; }
-    m_ref = -CUDART_INF_F; l_acc = 0.f; lp_acc = 0.f;
+    for (int ks = 0; ks < 8; ++ks)
+#pragma unroll
+      for (int hh = 0; hh < 2; ++hh) {
+        const float2 x = hv ? row(h, 16 * ks + 8 * hh + 2 * qd) : make_float2(0.f, 0.f);
+        const uint32_t xh = pack_bf16(x.x, x.y);
+        if constexpr (QS) {
+          const uint32_t xl = pack_bf16(x.x - __uint_as_float(xh << 16), x.y - __uint_as_float(xh & 0xffff0000u));
+          qa[ks][hh] = low ? xl : xh;
+          if constexpr (QB) qb[QB ? ks : 0][hh] = xl;
+        } else {
+          qa[ks][hh] = xh;
+        }
+        if constexpr (RD) {
+          const float s0 = (x.x * scale) * (x.x * scale), s1 = (x.y * scale) * (x.y * scale);
+          const uint32_t sh = pack_bf16(s0, s1);
+          const uint32_t sl = pack_bf16(s0 - __uint_as_float(sh << 16), s1 - __uint_as_float(sh & 0xffff0000u));
+          qs[RD ? ks : 0][hh] = low ? sl : sh;
+          if constexpr (RB) qs2[RB ? ks : 0][hh] = sl;
+        }
+      }
   }
 };
 
@@ -50,191 +79,132 @@ struct ScanPartCfg {
 // and those columns are discarded).  b_partial: the block that may hold fewer than block_size tokens (-1: none), with
 // log_partial the log of its token count.  sw: variance weights [t][g] for r not 4 or d; dbar_row0: the unit's variance
 // rows in global memory when the tile does not carry them (sd null).
-// store(head, block, u0, u1, z0, z1, v0, v1): log2 of the score terms and of the mean-term weights of blocks `block` and
-// `block` + 1 for one head; v0 / v1: whether they exist.
+// store(head, block, u, z): log2 of a block's score term and of its mean-term weight, for one head.
 // RD: one variance group per coordinate (r = d): sigma^2 = sum_i (scale q_i)^2 Dbar_i is a third tensor-core product.
 // HS: the mean rows hold hi halves only.  VH: only the mean VALUES' hi halves were brought in.
 template <int G, typename QT, bool RD, bool HS, bool VH, class Store>
 __device__ __forceinline__ void scan_part(ScanUnit<G, QT, RD> &w, const ScanPartCfg &cfg, uint32_t sk, uint32_t sv,
                                           const float *sd, uint32_t zero_row, const float *sw, const float *dbar_row0,
                                           int lane, int rb, int nb, int b0, int b_partial, float log_partial, Store store) {
-  constexpr bool QS = QSplit<QT>::value;
   constexpr int kRowBytes = HS ? CKV_D * 2 : CKV_ROW_ELEMS * 2;            // bytes of one mean-key row in a stage
   constexpr int kRowBytesV = (HS || VH) ? CKV_D * 2 : CKV_ROW_ELEMS * 2;   // ... of one mean-value row
   constexpr int TB = ScanTile<HS || VH>::TB;
-  constexpr bool SP = (G <= 4) && !RD;   // the per-(head, block) arithmetic is shared between the half warps
-  constexpr int NE = SP ? 1 : 2;         // n-tiles a lane works on there
-  const int head = lane >> 2, qd = lane & 3;   // this thread's accumulator row (head) and column pair
-  const int hsel = lane >> 4;                  // ... and which n-tile: the lower half warp the first, the upper the second
-  const int ehead = SP ? (head & 3) : head;
-  const bool ehv = ehead < G;
+  using T = HeadTile<G>;
 
-  // ---- Z^T = Q Kbar^T: heads x 16 blocks (two n-tiles of 8 blocks), hi and lo planes into one accumulator ----
-  // four accumulation chains per n-tile (hi / lo plane x even / odd 16-coordinate step): the products of a chain
-  // depend on one another, and a warp has little else to issue while it waits for them
-  float z[2][2] = {{0.f, 0.f}, {0.f, 0.f}}, zlo[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
-  float z2[2][2] = {{0.f, 0.f}, {0.f, 0.f}}, zlo2[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
+  // ---- Z = Kbar Q^T: 16 blocks x heads, hi and lo planes of the mean keys into one sum ----
+  // four accumulation chains (hi / lo plane x even / odd 16-coordinate step): the products of a chain depend on one
+  // another, and a warp has little else to issue while it waits for them
+  float z[4] = {0.f, 0.f, 0.f, 0.f}, z2[4] = {0.f, 0.f, 0.f, 0.f}, zl[4] = {0.f, 0.f, 0.f, 0.f}, zl2_[4] = {0.f, 0.f, 0.f, 0.f};
+  // ldmatrix lane roles: matrix lane / 8 -> (row half, coordinate chunk parity), row lane % 8
+  const int kr = rb + ((lane >> 3) & 1) * 8 + (lane & 7), kpar = lane >> 4;
   {
-    // ldmatrix lane roles: matrix lane / 8 -> 8-coordinate chunk, row lane % 8
-    const int lrow = lane & 7, lmat = lane >> 3;
+    const uint32_t rowaddr = sk + kr * kRowBytes;
 #pragma unroll
-    for (int nt = 0; nt < 2; ++nt) {
-      const int r = rb + nt * 8 + lrow;
-      const uint32_t rowaddr = sk + r * kRowBytes;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {   // two 16-coordinate steps per ldmatrix.x4
-        const uint32_t coff = (uint32_t)swz_chunk(4 * j + lmat, r) * 16;
-        uint32_t bh[4], bl[4];
-        ldmatrix_x4(bh, rowaddr + coff);
-        mma_rows8(z[nt][0], z[nt][1], w.qa[2 * j][0], w.qa[2 * j][1], bh[0], bh[1]);
-        mma_rows8(z2[nt][0], z2[nt][1], w.qa[2 * j + 1][0], w.qa[2 * j + 1][1], bh[2], bh[3]);
-        if (!HS) {
-          ldmatrix_x4(bl, rowaddr + 256 + coff);
-          mma_rows8(zlo[nt][0], zlo[nt][1], w.qa[2 * j][0], w.qa[2 * j][1], bl[0], bl[1]);
-          mma_rows8(zlo2[nt][0], zlo2[nt][1], w.qa[2 * j + 1][0], w.qa[2 * j + 1][1], bl[2], bl[3]);
-        }
-        if (QS) {
-          mma_rows8(zlo[nt][0], zlo[nt][1], w.qb[QS ? 2 * j : 0][0], w.qb[QS ? 2 * j : 0][1], bh[0], bh[1]);
-          mma_rows8(zlo[nt][0], zlo[nt][1], w.qb[QS ? 2 * j + 1 : 0][0], w.qb[QS ? 2 * j + 1 : 0][1], bh[2], bh[3]);
-        }
+    for (int ks = 0; ks < 8; ++ks) {
+      const uint32_t coff = (uint32_t)swz_chunk(2 * ks + kpar, kr) * 16;
+      uint32_t ah[4], al[4];
+      ldmatrix_x4(ah, rowaddr + coff);
+      mma_16816((ks & 1) ? z2 : z, ah, w.qa[ks][0], w.qa[ks][1]);
+      if (!HS) {
+        ldmatrix_x4(al, rowaddr + 256 + coff);
+        mma_16816((ks & 1) ? zl2_ : zl, al, w.qa[ks][0], w.qa[ks][1]);
       }
-      z[nt][0] = (z[nt][0] + z2[nt][0]) + (zlo[nt][0] + zlo2[nt][0]);
-      z[nt][1] = (z[nt][1] + z2[nt][1]) + (zlo[nt][1] + zlo2[nt][1]);
+      if constexpr (ScanUnit<G, QT, RD>::QB) mma_16816((ks & 1) ? zl2_ : zl, ah, w.qb[ks][0], w.qb[ks][1]);
     }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) z[i] = (z[i] + z2[i]) + (zl[i] + zl2_[i]);
+    if constexpr (QSplit<QT>::value && T::PAIR) T::add_copies(z);   // columns 4..7: the queries' lo halves
   }
-  float sgm[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
-  if (RD) {   // sigma^2 for the same heads x blocks tile: (qs_hi + qs_lo) (D_hi + D_lo) without the lo lo term
-    float sg2[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
-    const uint32_t sdr = sv + TB * kRowBytes;
-    const int lrow = lane & 7, lmat = lane >> 3;
+  float sgm[T::NR][2];
+  if constexpr (RD) {   // sigma^2 for the same tile: (qs_hi + qs_lo) (D_hi + D_lo)
+    float g[4] = {0.f, 0.f, 0.f, 0.f}, g2[4] = {0.f, 0.f, 0.f, 0.f};
+    const uint32_t rowaddr = sv + TB * kRowBytes + kr * kRowBytes;
 #pragma unroll
-    for (int nt = 0; nt < 2; ++nt) {
-      const int r = rb + nt * 8 + lrow;
-      const uint32_t rowaddr = sdr + r * kRowBytes;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const uint32_t coff = (uint32_t)swz_chunk(4 * j + lmat, r) * 16;
-        uint32_t dh[4], dl[4];
-        ldmatrix_x4(dh, rowaddr + coff);
-        ldmatrix_x4(dl, rowaddr + 256 + coff);
-        mma_rows8(sgm[nt][0], sgm[nt][1], w.qsh[RD ? 2 * j : 0][0], w.qsh[RD ? 2 * j : 0][1], dh[0], dh[1]);
-        mma_rows8(sgm[nt][0], sgm[nt][1], w.qsh[RD ? 2 * j + 1 : 0][0], w.qsh[RD ? 2 * j + 1 : 0][1], dh[2], dh[3]);
-        mma_rows8(sg2[nt][0], sg2[nt][1], w.qsl[RD ? 2 * j : 0][0], w.qsl[RD ? 2 * j : 0][1], dh[0], dh[1]);
-        mma_rows8(sg2[nt][0], sg2[nt][1], w.qsl[RD ? 2 * j + 1 : 0][0], w.qsl[RD ? 2 * j + 1 : 0][1], dh[2], dh[3]);
-        mma_rows8(sg2[nt][0], sg2[nt][1], w.qsh[RD ? 2 * j : 0][0], w.qsh[RD ? 2 * j : 0][1], dl[0], dl[1]);
-        mma_rows8(sg2[nt][0], sg2[nt][1], w.qsh[RD ? 2 * j + 1 : 0][0], w.qsh[RD ? 2 * j + 1 : 0][1], dl[2], dl[3]);
-      }
-      sgm[nt][0] += sg2[nt][0]; sgm[nt][1] += sg2[nt][1];
+    for (int ks = 0; ks < 8; ++ks) {
+      const uint32_t coff = (uint32_t)swz_chunk(2 * ks + kpar, kr) * 16;
+      uint32_t dh[4], dl[4];
+      ldmatrix_x4(dh, rowaddr + coff);
+      ldmatrix_x4(dl, rowaddr + 256 + coff);
+      mma_16816(g, dh, w.qs[RD ? ks : 0][0], w.qs[RD ? ks : 0][1]);
+      mma_16816(g2, dl, w.qs[RD ? ks : 0][0], w.qs[RD ? ks : 0][1]);
+      if constexpr (!T::PAIR) mma_16816(g2, dh, w.qs2[ks][0], w.qs2[ks][1]);
     }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) g[i] += g2[i];
+    if constexpr (T::PAIR) T::add_copies(g);
+    T::pick(g, lane, sgm);
   }
 
-  // ---- per (head, block): variance projection, l, running maximum, compensation weight ----
-  // The products leave this part's 16 blocks x G heads in the lanes of rows 0..G-1 (four values per lane).
-  // With G <= 4 those are lanes 0-15 only, so the upper half warp takes over the second n-tile: every lane
-  // then works on one n-tile's pair of blocks (half the dependent chain), and the weights travel back to
-  // the lower lanes, which hold the A operand of the next product.
-  float zin[NE][2];
-  if constexpr (SP) {
-    const float t0 = __shfl_sync(0xffffffffu, z[1][0], lane & 15), t1 = __shfl_sync(0xffffffffu, z[1][1], lane & 15);
-    zin[0][0] = hsel ? t0 : z[0][0];
-    zin[0][1] = hsel ? t1 : z[0][1];
-  } else {
+  // ---- per (block, head): variance projection, l, running maximum, compensation weight ----
+  float zin[T::NR][2], zw[T::NR][2], sig[T::NR][2], wt[T::NR][2];
+  T::pick(z, lane, zin);
 #pragma unroll
-    for (int k = 0; k < NE; ++k) { zin[k][0] = z[k][0]; zin[k][1] = z[k][1]; }
-  }
-  float zl2[NE][2], sig[NE][2], wt[NE][2];
-  bool val[NE][2];
-  float tmax = -CUDART_INF_F;
-#pragma unroll
-  for (int k = 0; k < NE; ++k) {
-    const int nt = SP ? hsel : k;
-    const int r0 = rb + nt * 8 + 2 * qd;     // this thread's two blocks of the n-tile: rows r0, r0 + 1
-    float ell[2];
+  for (int k = 0; k < T::NR; ++k) {
+    const int r = rb + T::row(lane, k), b = b0 + r;
+    const bool real = r < nb;
+    const float logc = b == b_partial ? log_partial : cfg.log_bs;
+    float4 dv = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (!RD && cfg.r4 && real) dv = *reinterpret_cast<const float4 *>(sd + r * 4);
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
-      const int r = r0 + e, b = b0 + r;
-      val[k][e] = ehv && r < nb;
+      const int head = T::head(lane, e);
+      const bool val = real && head < G;
       float sg = 0.f;
-      if (val[k][e]) {
-        if (RD) {
-          sg = fmaxf(sgm[RD ? k : 0][e], 0.f);
+      if (val) {
+        if constexpr (RD) {
+          sg = fmaxf(sgm[k][e], 0.f);
         } else if (cfg.r4) {
-          const float4 dv = *reinterpret_cast<const float4 *>(sd + r * 4);
-          sg = fmaf(w.wown[0], dv.x, fmaf(w.wown[1], dv.y, fmaf(w.wown[2], dv.z, w.wown[3] * dv.w)));
+          sg = fmaf(w.wown[e][0], dv.x, fmaf(w.wown[e][1], dv.y, fmaf(w.wown[e][2], dv.z, w.wown[e][3] * dv.w)));
         } else {
           for (int t = 0; t < cfg.r; ++t) {
-            const float dv = sd != nullptr ? sd[r * cfg.r + t] : __ldg(dbar_row0 + (size_t)b * cfg.r + t);
-            sg = fmaf(sw[t * G + ehead], dv, sg);
+            const float d = sd != nullptr ? sd[r * cfg.r + t] : __ldg(dbar_row0 + (size_t)b * cfg.r + t);
+            sg = fmaf(sw[t * G + head], d, sg);
           }
         }
       }
       sig[k][e] = sg;
       const float zbar = zin[k][e] * cfg.scale;
-      const float logc = b == b_partial ? log_partial : cfg.log_bs;
-      ell[e] = logc + zbar + cfg.half_var * sg;
-      zl2[k][e] = val[k][e] ? (zbar + logc) * kLog2e : -CUDART_INF_F;   // log2 of |b| e^{zbar}
-      tmax = fmaxf(tmax, zl2[k][e]);
+      const float ell = logc + zbar + cfg.half_var * sg;
+      zw[k][e] = val ? (zbar + logc) * kLog2e : -CUDART_INF_F;   // log2 of |b| e^{zbar}
+      // what the later stages read, both in log2 units: the head's term of the block score, e^l sigma^2 (e^l alone
+      // when blocks are ranked by mass), and the block's mean-compensation weight |b| e^{zbar}
+      if (val) store(head, b, fmaf(ell, kLog2e, cfg.by_mass ? 0.f : __log2f(sg)), zw[k][e]);
     }
-    // what the later stages read, both in log2 units: the head's term of the block score, e^l sigma^2 (e^l
-    // alone when blocks are ranked by mass), and the block's mean-compensation weight |b| e^{zbar}
-    const float u0 = fmaf(ell[0], kLog2e, cfg.by_mass ? 0.f : __log2f(sig[k][0]));
-    const float u1 = fmaf(ell[1], kLog2e, cfg.by_mass ? 0.f : __log2f(sig[k][1]));
-    store(ehead, b0 + r0, u0, u1, zl2[k][0], zl2[k][1], val[k][0], val[k][1]);
   }
-  tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, 1));
-  tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, 2));
-  if (SP) tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, 16));
-  if (tmax > w.m_ref + CKV_RESCALE_SLACK) {   // the running maximum is only raised when exceeded by a slack
-    const float sc = exp2_diff(w.m_ref, tmax);
-    w.m_ref = tmax;
-    w.l_acc *= sc; w.lp_acc *= sc;
-#pragma unroll
-    for (int t = 0; t < 16; ++t) { w.acc[t][0] *= sc; w.acc[t][1] *= sc; }
+  {   // the running maximum is only raised when exceeded by a slack
+    const float m0 = w.m[0], m1 = w.m[1];
+    attn_raise<G>(zw, w);
+    if (w.m[0] != m0) w.lp[0] *= exp2_diff(m0, w.m[0]);
+    if (w.m[1] != m1) w.lp[1] *= exp2_diff(m1, w.m[1]);
   }
-  uint32_t whm[NE], wlm[NE];
 #pragma unroll
-  for (int k = 0; k < NE; ++k) {
+  for (int k = 0; k < T::NR; ++k)
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
-      wt[k][e] = val[k][e] ? fast_exp2(zl2[k][e] - w.m_ref) : 0.f;
-      w.l_acc += wt[k][e];
-      w.lp_acc = fmaf(wt[k][e], fast_exp2(cfg.half_var * kLog2e * sig[k][e]), w.lp_acc);   // e^{l - m} = e^{zbar + log|b| - m} e^{sigma^2/2}
+      wt[k][e] = zw[k][e] == -CUDART_INF_F ? 0.f : fast_exp2(zw[k][e] - w.m[e]);
+      w.l[e] += wt[k][e];
+      w.lp[e] = fmaf(wt[k][e], fast_exp2(cfg.half_var * kLog2e * sig[k][e]), w.lp[e]);   // e^{l - m} = e^{zbar + log|b| - m} e^{sigma^2/2}
     }
-    whm[k] = pack_bf16(wt[k][0], wt[k][1]);
-    wlm[k] = pack_bf16(wt[k][0] - bf16_round(wt[k][0]), wt[k][1] - bf16_round(wt[k][1]));
-  }
-  uint32_t wh[2], wl[2];   // A fragments of the weights: k = blocks 2 qd + {0, 1} (+ 8), hi and lo halves
-  if constexpr (SP) {
-    // rows 0..3 (lanes 0-15) get their second n-tile from the lane 16 above; rows 4..7 carry zero weights
-    const uint32_t oh = __shfl_sync(0xffffffffu, whm[0], (lane & 15) + 16);
-    const uint32_t ol = __shfl_sync(0xffffffffu, wlm[0], (lane & 15) + 16);
-    wh[0] = hsel ? 0u : whm[0]; wl[0] = hsel ? 0u : wlm[0];
-    wh[1] = hsel ? 0u : oh;     wl[1] = hsel ? 0u : ol;
-  } else {
-#pragma unroll
-    for (int k = 0; k < NE; ++k) { wh[k] = whm[k]; wl[k] = wlm[k]; }
-  }
 
-  // ---- acc += W Vbar: heads x 128 coordinates, k = this part's 16 blocks ----
+  // ---- acc += Vbar^T W: 128 coordinates x heads, k = this part's 16 blocks ----
   {
-    // ldmatrix.trans lane roles: matrix lane / 8 -> (block half, coordinate chunk parity), row lane % 8
-    const int r = rb + ((lane >> 3) & 1) * 8 + (lane & 7);
+    uint32_t b[T::NR][2];
+    T::weights(wt, lane, b);
+    // ldmatrix.trans lane roles: matrix lane / 8 -> (coordinate chunk parity, row half), row lane % 8
+    const int r = rb + (lane >> 4) * 8 + (lane & 7), cpar = (lane >> 3) & 1;
     const bool real = r < nb;   // rows past the last block: zeros
     const uint32_t rowaddr = real ? sv + r * kRowBytesV : zero_row;
-    const int cpar = lane >> 4;
 #pragma unroll
-    for (int t2 = 0; t2 < 8; ++t2) {   // two 8-coordinate n-tiles per ldmatrix.x4
-      const uint32_t coff = real ? (uint32_t)swz_chunk(2 * t2 + cpar, r) * 16 : 0u;
-      uint32_t vh[4], vl[4];
+    for (int t = 0; t < 8; ++t) {
+      const uint32_t coff = real ? (uint32_t)swz_chunk(2 * t + cpar, r) * 16 : 0u;
+      uint32_t vh[4];
       ldmatrix_x4_trans(vh, rowaddr + coff);
-      mma_rows8(w.acc[2 * t2][0], w.acc[2 * t2][1], wh[0], wh[1], vh[0], vh[1]);
-      mma_rows8(w.acc[2 * t2][0], w.acc[2 * t2][1], wl[0], wl[1], vh[0], vh[1]);
-      mma_rows8(w.acc[2 * t2 + 1][0], w.acc[2 * t2 + 1][1], wh[0], wh[1], vh[2], vh[3]);
-      mma_rows8(w.acc[2 * t2 + 1][0], w.acc[2 * t2 + 1][1], wl[0], wl[1], vh[2], vh[3]);
-      if (!HS && !VH) {
+      mma_16816(w.acc[t], vh, b[0][0], b[0][1]);
+      if constexpr (!T::PAIR) mma_16816(w.acc[t], vh, b[T::NR - 1][0], b[T::NR - 1][1]);
+      if constexpr (!HS && !VH) {
+        uint32_t vl[4];
         ldmatrix_x4_trans(vl, rowaddr + (real ? 256u : 0u) + coff);
-        mma_rows8(w.acc[2 * t2][0], w.acc[2 * t2][1], wh[0], wh[1], vl[0], vl[1]);
-        mma_rows8(w.acc[2 * t2 + 1][0], w.acc[2 * t2 + 1][1], wh[0], wh[1], vl[2], vl[3]);
+        mma_16816(w.acc[t], vl, b[0][0], b[0][1]);
       }
     }
   }

@@ -222,7 +222,6 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *__restrict__ q, const int *seq_lens, 
   constexpr int TB = ScanTile<HS || VH>::TB;
   constexpr int kParts = TB / 16;              // parts of a tile
   constexpr int kSkip = kWarps / kParts;       // a warp works on every kSkip-th tile
-  constexpr bool SP = (G <= 4) && !RD;
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ __align__(8) uint64_t full_bar[2][kStagesCap], empty_bar[kStagesCap];
   __shared__ __align__(8) uint64_t s_xbar[4];                 // what the cluster's CTAs send: normalisers, scores, partial outputs; global stores done
@@ -238,8 +237,7 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *__restrict__ q, const int *seq_lens, 
   __shared__ int s_digit, s_before, s_nc, s_ncand, s_wt[3][kWarps], s_abort, s_issued;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int head = lane >> 2, qd = lane & 3;
-  const bool hv = head < G;
+  using T = HeadTile<G>;       // which heads a lane works on
   const int C = (int)cluster_size(), rank = (int)cluster_rank();
   const int unit = blockIdx.y, s = ckv_div_hkv(P, unit), h = unit - s * P.Hkv;
   const bool append = fresh.k_new != nullptr;
@@ -262,7 +260,8 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *__restrict__ q, const int *seq_lens, 
   if (tid >= kThreads - 32) reinterpret_cast<uint4 *>(s_zero_row)[lane] = make_uint4(0u, 0u, 0u, 0u);
   const bool dbar_bulk = P.r >= 4;
   const int stage_bytes = TB * (kRowBytesK + kRowBytesV) + (dbar_bulk ? TB * P.r * 4 : 0);
-  float *su = reinterpret_cast<float *>(smem + plan.u_off);   // score terms of the CTA's own blocks, [g][own_cap]
+  float *su = reinterpret_cast<float *>(smem + plan.u_off);   // score terms of the CTA's own blocks, [g][u_stride]
+  const int u_stride = plan.own_cap + 8;   // a tile's eight rows x four heads then fall into 32 different banks
   // the length the step works on; a bound the host misjudged is kept to what the shared arrays were sized for
   const int N = max(min(min(raw + ((append && raw >= 0 && raw < cap) ? 1 : 0), cap), plan.max_blocks * P.bs), 0);
   const int X = (N + P.bs - 1) >> P.lg_bs, Xs = max(X - 1, 0);
@@ -354,43 +353,33 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *__restrict__ q, const int *seq_lens, 
       }
       work_barrier();
     }
-    const uint32_t *srow = reinterpret_cast<const uint32_t *>(&s_q[hv ? head : 0][0]);
-#pragma unroll
-    for (int ks = 0; ks < 8; ++ks)
-#pragma unroll
-      for (int hh = 0; hh < 2; ++hh) {
-        w.qa[ks][hh] = hv ? srow[(16 * ks + 8 * hh + 2 * qd) / 2] : 0u;
-        if (RD) {
-          const float x0 = __uint_as_float(w.qa[ks][hh] << 16) * P.scale, x1 = __uint_as_float(w.qa[ks][hh] & 0xffff0000u) * P.scale;
-          const float s0 = x0 * x0, s1 = x1 * x1;
-          w.qsh[RD ? ks : 0][hh] = pack_bf16(s0, s1);
-          w.qsl[RD ? ks : 0][hh] = pack_bf16(s0 - bf16_round(s0), s1 - bf16_round(s1));
-        }
-      }
-    if (!RD && P.r == 4) {   // the same from the fragments: a head's four lanes hold its 128 coordinates between them
-#pragma unroll
-      for (int t = 0; t < 4; ++t) w.wown[t] = 0.f;
+    w.set_queries(lane, P.scale, [&](int g, int c) {
+      const uint32_t x = *reinterpret_cast<const uint32_t *>(&s_q[g][c]);
+      return make_float2(__uint_as_float(x << 16), __uint_as_float(x & 0xffff0000u));
+    });
+    if (!RD && P.r == 4) {   // the same from the fragments: a column's four lanes hold its head's 128 coordinates between them
+      float a[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
       for (int ks = 0; ks < 8; ++ks) {
-        float a = 0.f;
+        float sq = 0.f;
 #pragma unroll
         for (int hh = 0; hh < 2; ++hh) {
           const float x0 = __uint_as_float(w.qa[ks][hh] << 16), x1 = __uint_as_float(w.qa[ks][hh] & 0xffff0000u);
-          a = fmaf(x0, x0, fmaf(x1, x1, a));
+          sq = fmaf(x0, x0, fmaf(x1, x1, sq));
         }
-        if (P.glayout == 0) w.wown[ks / 2] += a; else w.wown[ks % 4] += a;   // 16 coordinates of one group
+        if (P.glayout == 0) a[ks / 2] += sq; else a[ks % 4] += sq;   // 16 coordinates of one group
       }
 #pragma unroll
       for (int t = 0; t < 4; ++t) {
-        w.wown[t] += __shfl_xor_sync(0xffffffffu, w.wown[t], 1);
-        w.wown[t] += __shfl_xor_sync(0xffffffffu, w.wown[t], 2);
-        w.wown[t] *= P.scale * P.scale;
-        if (SP) w.wown[t] = __shfl_sync(0xffffffffu, w.wown[t], lane & 15);   // the upper half warp works for the same heads
+        a[t] += __shfl_xor_sync(0xffffffffu, a[t], 1);
+        a[t] += __shfl_xor_sync(0xffffffffu, a[t], 2);
+        a[t] *= P.scale * P.scale;
+#pragma unroll
+        for (int e = 0; e < 2; ++e) w.wown[e][t] = __shfl_sync(0xffffffffu, a[t], 4 * T::head(lane, e));   // column = head
       }
     }
     const ScanPartCfg cfg{P.scale, P.half_var, logf((float)P.bs), P.r, P.max_blocks, (P.variant & CKV_VARIANT_RANK_BY_MASS) != 0, P.r == 4};
     float *lz = P.lz + row0 * G;
-    const bool pair_ok = (P.max_blocks & 1) == 0;
     const int part = warp % kParts;
     // A warp visits every kSkip-th tile.  A fill is only issued once the one plan.stages before it was released, and
     // kSkip <= plan.stages (checked by the launcher): alternate rounds of the ring use two sets of full barriers, which
@@ -398,7 +387,7 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *__restrict__ q, const int *seq_lens, 
     int st = 0, at = 0;
     uint32_t round = 0;
     bool aborted = false;
-    float umax = -CUDART_INF_F;   // largest score term this lane has seen (of its head)
+    float umax[2] = {-CUDART_INF_F, -CUDART_INF_F};   // largest score terms this lane has seen, of its heads
     for (int it = warp / kParts; it < tiles; it += kSkip) {
       st += it - at;
       at = it;
@@ -419,28 +408,21 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *__restrict__ q, const int *seq_lens, 
         scan_part<G, bf16, RD, HS, VH>(
             w, cfg, sk, sk + TB * kRowBytesK, (RD || dbar_bulk) ? sd : nullptr, smem_u32(s_zero_row), s_w, P.dbar + row0 * P.r,
             lane, rb, nb, b_lo + it * TB, -1, 0.f,
-            [&](int eh, int blk, float u0, float u1, float z0, float z1, bool v0, bool v1) {
-              float *uo = su + eh * plan.own_cap + (blk - b_lo);
-              const size_t o = (size_t)eh * P.max_blocks + blk;
-              if (v0) { uo[0] = u0; umax = fmaxf(umax, u0); }
-              if (v1) { uo[1] = u1; umax = fmaxf(umax, u1); }
-              if (pair_ok && v1) {
-                *reinterpret_cast<float2 *>(lz + o) = make_float2(z0, z1);
-              } else {
-                if (v0) lz[o] = z0;
-                if (v1) lz[o + 1] = z1;
-              }
+            [&](int g, int blk, float x, float y) {
+              su[g * u_stride + (blk - b_lo)] = x;
+              lz[(size_t)g * P.max_blocks + blk] = y;
+              if (g & 1) umax[1] = fmaxf(umax[1], x); else umax[0] = fmaxf(umax[0], x);
             });
       }
       __syncwarp();
       if (lane == 0 && !aborted) mbar_arrive(&empty_bar[st]);
     }
     // this warp's normaliser partial
-    float lp = w.lp_acc;
-    lp += __shfl_xor_sync(0xffffffffu, lp, 1); lp += __shfl_xor_sync(0xffffffffu, lp, 2);
-    umax = fmaxf(umax, __shfl_xor_sync(0xffffffffu, umax, 1)); umax = fmaxf(umax, __shfl_xor_sync(0xffffffffu, umax, 2));
-    if (SP) { lp += __shfl_xor_sync(0xffffffffu, lp, 16); umax = fmaxf(umax, __shfl_xor_sync(0xffffffffu, umax, 16)); }
-    if (hv && qd == 0) s_wn[warp][head] = make_float4(w.m_ref, lp, umax, 0.f);
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const float lp = T::sum_rows(w.lp[e]), um = T::max_rows(umax[e]);
+      if (T::owns(lane, e)) s_wn[warp][T::head(lane, e)] = make_float4(w.m[e], lp, um, 0.f);
+    }
   }
   __syncwarp();
   cluster_wait();    // every CTA of the cluster has started
@@ -526,7 +508,7 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *__restrict__ q, const int *seq_lens, 
       float sc[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
       for (int g = 0; g < G; ++g) {
-        const float4 u = *reinterpret_cast<const float4 *>(su + g * plan.own_cap + i);
+        const float4 u = *reinterpret_cast<const float4 *>(su + g * u_stride + i);
         sc[0] = fmaf(fast_exp2(u.x - Mg[g]), iL[g], sc[0]); sc[1] = fmaf(fast_exp2(u.y - Mg[g]), iL[g], sc[1]);
         sc[2] = fmaf(fast_exp2(u.z - Mg[g]), iL[g], sc[2]); sc[3] = fmaf(fast_exp2(u.w - Mg[g]), iL[g], sc[3]);
       }
@@ -734,12 +716,12 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *__restrict__ q, const int *seq_lens, 
     };
     // items: pages 0 .. 15, [rows], pages 16 .. 31, [rows], ...; the last group may be short
     const int n_items = n_mine + (rows_rm ? (n_mine + 15) / 16 : 0);
-    struct Item { int ntok; float z[HS ? 4 : 1]; };   // ntok > 0: a page; 0: nothing; -1: rows
+    struct Item { int ntok; float z[HS ? T::NR : 1][2]; };   // ntok > 0: a page; 0: nothing; -1: rows
     int gpos = 0, page_n = 0;
     auto issue = [&](int buf) -> Item {
       Item it;
       it.ntok = 0;
-      it.z[0] = -CUDART_INF_F;
+      it.z[0][0] = it.z[0][1] = -CUDART_INF_F;
       const uint32_t kb = buf0 + buf * kPageBytes;
       const bool rows = rows_rm && (gpos == 16 || page_n == n_mine);
       if (!rows) {
@@ -751,9 +733,12 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *__restrict__ q, const int *seq_lens, 
           const size_t src = ((size_t)phys * P.Hkv + h) * (CKV_PAGE * CKV_D);
           issue_page(kb, kb + kTileBytes, k_pool + src, v_pool + src, ntok, lane);
           it.ntok = ntok;
-          if (!HS && comp && hv) {   // log2 of e^{zbar} of the page's block for this lane's head
+          if (!HS && comp) {   // log2 of e^{zbar} of the page's block for this lane's heads
             const int blk = bx < 0 ? ~bx : bx;
-            it.z[0] = __ldcg(lz + (size_t)head * P.max_blocks + blk) - (blk == Xs ? lg_last : lg_bs);
+            const float lb = blk == Xs ? lg_last : lg_bs;
+#pragma unroll
+            for (int e = 0; e < 2; ++e)
+              if (T::head(lane, e) < G) it.z[0][e] = __ldcg(lz + (size_t)T::head(lane, e) * P.max_blocks + blk) - lb;
           }
         }
         ++page_n; ++gpos;
@@ -770,10 +755,12 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *__restrict__ q, const int *seq_lens, 
           cp_async16(kb + kTileBytes + (uint32_t)(row * kRowBytes + ((c ^ (row & 7)) << 4)), src, real);
         }
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const int row = 2 * qd + (e & 1) + 8 * (e >> 1);
+        for (int k = 0; k < T::NR; ++k) {
+          const int row = T::row(lane, k);
           const int blk = __shfl_sync(0xffffffffu, mine.blk, (first + row) & 31);
-          it.z[HS ? e : 0] = (hv && row < gpos && blk >= 0) ? __ldcg(lz + (size_t)head * P.max_blocks + blk) : -CUDART_INF_F;
+#pragma unroll
+          for (int e = 0; e < 2; ++e)
+            it.z[HS ? k : 0][e] = (T::head(lane, e) < G && row < gpos && blk >= 0) ? __ldcg(lz + (size_t)T::head(lane, e) * P.max_blocks + blk) : -CUDART_INF_F;
         }
         gpos = 0;
       }
@@ -792,24 +779,21 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *__restrict__ q, const int *seq_lens, 
       __syncwarp();
       const uint32_t kb = buf0 + buf * kPageBytes;
       if (cur.ntok > 0) {
-        attn_page<SP>(kb, kb + kTileBytes, w.qa, cur.ntok, hv, lane, sl2, HS ? -CUDART_INF_F : cur.z[0], w.acc, w.m_ref, w.l_acc);
-      } else if (HS && cur.ntok < 0) {
-        float zm = fmaxf(fmaxf(cur.z[0], cur.z[HS ? 1 : 0]), fmaxf(cur.z[HS ? 2 : 0], cur.z[HS ? 3 : 0]));
-        zm = fmaxf(zm, __shfl_xor_sync(0xffffffffu, zm, 1));
-        zm = fmaxf(zm, __shfl_xor_sync(0xffffffffu, zm, 2));
-        if (SP) zm = fmaxf(zm, __shfl_xor_sync(0xffffffffu, zm, 16));
-        attn_raise(zm, w.m_ref, w.l_acc, w.acc);
-        float x[4];
+        const float lzt[2] = {HS ? -CUDART_INF_F : cur.z[0][0], HS ? -CUDART_INF_F : cur.z[0][1]};
+        attn_page<G>(kb, kb + kTileBytes, w.qa, cur.ntok, lane, sl2, lzt, w);
+      } else if constexpr (HS) {
+        if (cur.ntok < 0) {
+          attn_raise<G>(cur.z, w);
+          float x[T::NR][2];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {   // the negated weights
-          const float z = cur.z[HS ? e : 0];
-          x[e] = z == -CUDART_INF_F ? 0.f : -fast_exp2(z - w.m_ref);
-          w.l_acc += x[e];
+          for (int k = 0; k < T::NR; ++k)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {   // the negated weights
+              x[k][e] = cur.z[k][e] == -CUDART_INF_F ? 0.f : -fast_exp2(cur.z[k][e] - w.m[e]);
+              w.l[e] += x[k][e];
+            }
+          attn_pv<G>(kb + kTileBytes, x, lane, w);
         }
-        const uint32_t ph[2] = {pack_bf16(x[0], x[1]), pack_bf16(x[2], x[3])};
-        const uint32_t pl[2] = {pack_bf16(x[0] - bf16_round(x[0]), x[1] - bf16_round(x[1])),
-                                pack_bf16(x[2] - bf16_round(x[2]), x[3] - bf16_round(x[3]))};
-        attn_pv(kb + kTileBytes, ph, pl, lane, w.acc);
       }
       __syncwarp();
       cur = nxt;
@@ -818,16 +802,13 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *__restrict__ q, const int *seq_lens, 
     if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(P.status, CKV_DEV_BAD_PAGE);
 
     // ---- the CTA's partial: its warps (each with its own running maximum) and the last block's mean term ----
-    float l = w.l_acc;
-    l += __shfl_xor_sync(0xffffffffu, l, 1); l += __shfl_xor_sync(0xffffffffu, l, 2);
-    if (SP) l += __shfl_xor_sync(0xffffffffu, l, 16);
     float *wpart = reinterpret_cast<float *>(smem + kOffPages) + (size_t)warp * (2 * kPageBytes / 4);
     __syncwarp();
-    if (hv) {
-      float *r = wpart + head * CKV_PART_STRIDE;
+    w.fold(lane, [&](int g, int c, float v) { wpart[g * CKV_PART_STRIDE + 4 + c] = v; });
 #pragma unroll
-      for (int t = 0; t < 16; ++t) *reinterpret_cast<float2 *>(r + 4 + 8 * t + 2 * qd) = make_float2(w.acc[t][0], w.acc[t][1]);
-      if (qd == 0) { r[0] = w.m_ref; r[1] = l; }
+    for (int e = 0; e < 2; ++e) {
+      const float l = T::sum_rows(w.l[e]);
+      if (T::owns(lane, e)) { wpart[T::head(lane, e) * CKV_PART_STRIDE] = w.m[e]; wpart[T::head(lane, e) * CKV_PART_STRIDE + 1] = l; }
     }
     const bool with_tail = comp && rank == C - 1;
     auto entry = [&](int e) { return e < kWarps ? reinterpret_cast<const float *>(smem + kOffPages) + (size_t)e * (2 * kPageBytes / 4) : &s_tail_part[0][0]; };
@@ -954,8 +935,8 @@ cudaError_t ckv_configure_unit_step(ckv_ctx *c) {
 }
 
 // Whether a step of this size runs as one launch, and how.  Against the separate launches (us per step, back to back):
-// 16.8 / 28.6 (one head, 4K), 20.2 / 35.7 (8 units, 32K), 27.6 / 38.9 (8 units, 128K, 32-token blocks), 45.7 / 51.2 (24
-// units, 100K, bf16 summaries), 63.9 / 69.5 (32 units, 128K).  What stays with the separate launches, and why:
+// 15.3 / 27.4 (one head, 4K), 17.4 / 35.8 (8 units, 32K), 22.4 / 38.6 (8 units, 128K, 32-token blocks), 32.2 / 51.2 (24
+// units, 100K, bf16 summaries), 56.1 / 69.2 (32 units, 128K).  What stays with the separate launches, and why:
 //   * fp32 pages (the attention is on bf16 tensor cores) and an explicit ckv_set_tail_mode, which asks for them;
 //   * caches under CKV_STEP_MIN_TOKENS.  Not a crossover -- one launch is the faster form there too -- but the size below
 //     which the documented two-call arrangement (append, scan, select, attention as launches of their own) is kept;
@@ -976,7 +957,7 @@ bool ckv_unit_step_plan(const ckv_ctx *c, int batch, int max_len, int kcap, CkvS
   const size_t stage = (size_t)P.scan_tile * (krow + vrow) + (P.r >= 4 ? (size_t)P.scan_tile * P.r * 4 : 0);
   const int parts = (std::max(xmax - 1, 0) + 15) / 16;
   plan->own_cap = 16 * std::max((parts + C - 1) / C, 1);
-  const size_t u_bytes = (size_t)plan->own_cap * P.G * sizeof(float);
+  const size_t u_bytes = (size_t)(plan->own_cap + 8) * P.G * sizeof(float);
   if (u_bytes + (size_t)skip * stage > (size_t)kDynLimit) return false;
   const int tiles = (plan->own_cap + P.scan_tile - 1) / P.scan_tile;
   plan->stages = std::min({kStagesCap, (int)(((size_t)kDynLimit - u_bytes) / stage), std::max(tiles, skip)});
