@@ -49,6 +49,7 @@ constexpr int kProducerWarp = kWarps, kTailWarp = kWarps + 1;
 constexpr int kThreads = (kWarps + 2) * 32;
 constexpr int kClusterCap = CKV_STEP_MAX_CLUSTER;
 constexpr int kStagesCap = 6;
+constexpr int kMinRing = 3;                     // stages the score terms have to leave room for, or they go through global memory
 constexpr int kScoresCap = 9216;                // blocks of a unit whose scores every CTA can hold
 constexpr int kBins = 2048;                     // score histogram: 32 octaves below the largest possible score, 64 bins each
 constexpr int kBinShift = 17;                   // ... a bin is a score's bit pattern without its low 17 bits
@@ -379,7 +380,7 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *__restrict__ q, const int *seq_lens, 
       }
     }
     const ScanPartCfg cfg{P.scale, P.half_var, logf((float)P.bs), P.r, P.max_blocks, (P.variant & CKV_VARIANT_RANK_BY_MASS) != 0, P.r == 4};
-    float *lz = P.lz + row0 * G;
+    float *lz = P.lz + row0 * G, *lu = P.lu + row0 * G;
     const int part = warp % kParts;
     // A warp visits every kSkip-th tile.  A fill is only issued once the one plan.stages before it was released, and
     // kSkip <= plan.stages (checked by the launcher): alternate rounds of the ring use two sets of full barriers, which
@@ -409,7 +410,7 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *__restrict__ q, const int *seq_lens, 
             w, cfg, sk, sk + TB * kRowBytesK, (RD || dbar_bulk) ? sd : nullptr, smem_u32(s_zero_row), s_w, P.dbar + row0 * P.r,
             lane, rb, nb, b_lo + it * TB, -1, 0.f,
             [&](int g, int blk, float x, float y) {
-              su[g * u_stride + (blk - b_lo)] = x;
+              if (plan.u_global) lu[(size_t)g * P.max_blocks + blk] = x; else su[g * u_stride + (blk - b_lo)] = x;
               lz[(size_t)g * P.max_blocks + blk] = y;
               if (g & 1) umax[1] = fmaxf(umax[1], x); else umax[0] = fmaxf(umax[0], x);
             });
@@ -504,13 +505,27 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *__restrict__ q, const int *seq_lens, 
   if (warp < kWarps) {
     bool nonfinite = false;
     const uint32_t xbar1 = smem_u32(&s_xbar[1]);
+    // the score terms of the CTA's blocks, in shared memory or in the workspace (where a head's row may start anywhere)
+    const float *ub = plan.u_global ? P.lu + row0 * G + b_lo : su;
+    const size_t us = plan.u_global ? (size_t)P.max_blocks : (size_t)u_stride;
+    const bool wide = (us & 3) == 0;
     for (int i = 4 * tid; i < own; i += 4 * kWork) {
       float sc[4] = {0.f, 0.f, 0.f, 0.f};
+      float4 u[G];   // all heads' loads before the first use: they may be trips to the L2
+      if (wide) {
+#pragma unroll
+        for (int g = 0; g < G; ++g) u[g] = *reinterpret_cast<const float4 *>(ub + g * us + i);
+      } else {
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+          const float *up = ub + g * us + i;
+          u[g] = make_float4(up[0], i + 1 < own ? up[1] : 0.f, i + 2 < own ? up[2] : 0.f, i + 3 < own ? up[3] : 0.f);
+        }
+      }
 #pragma unroll
       for (int g = 0; g < G; ++g) {
-        const float4 u = *reinterpret_cast<const float4 *>(su + g * u_stride + i);
-        sc[0] = fmaf(fast_exp2(u.x - Mg[g]), iL[g], sc[0]); sc[1] = fmaf(fast_exp2(u.y - Mg[g]), iL[g], sc[1]);
-        sc[2] = fmaf(fast_exp2(u.z - Mg[g]), iL[g], sc[2]); sc[3] = fmaf(fast_exp2(u.w - Mg[g]), iL[g], sc[3]);
+        sc[0] = fmaf(fast_exp2(u[g].x - Mg[g]), iL[g], sc[0]); sc[1] = fmaf(fast_exp2(u[g].y - Mg[g]), iL[g], sc[1]);
+        sc[2] = fmaf(fast_exp2(u[g].z - Mg[g]), iL[g], sc[2]); sc[3] = fmaf(fast_exp2(u[g].w - Mg[g]), iL[g], sc[3]);
       }
       uint32_t k[4];
 #pragma unroll
@@ -936,16 +951,17 @@ cudaError_t ckv_configure_unit_step(ckv_ctx *c) {
 
 // Whether a step of this size runs as one launch, and how.  Against the separate launches (us per step, back to back):
 // 15.3 / 27.4 (one head, 4K), 17.4 / 35.8 (8 units, 32K), 22.4 / 38.6 (8 units, 128K, 32-token blocks), 32.2 / 51.2 (24
-// units, 100K, bf16 summaries), 56.1 / 69.2 (32 units, 128K).  What stays with the separate launches, and why:
+// units, 100K, bf16 summaries), 41.9 / 60.3 (16 units, 88K, r = d), 56.1 / 69.2 (32 units, 128K), 60 / 70 (64 units, 64K),
+// 61 / 81 (72 units, 58K), 95 / 147 (80 units, r = 16), 73 / 80 (88 units of 14K, r = d), 71 / 81 (128 units, 32K), 82 / 89
+// (128 ragged units, G = 8: one CTA per unit, score terms through global memory).  What stays with the separate launches:
 //   * fp32 pages (the attention is on bf16 tensor cores) and an explicit ckv_set_tail_mode, which asks for them;
 //   * caches under CKV_STEP_MIN_TOKENS.  Not a crossover -- one launch is the faster form there too -- but the size below
 //     which the documented two-call arrangement (append, scan, select, attention as launches of their own) is kept;
-//   * r = d: 1536 bytes a block and a third product leave it at 67.1 against 64.8 us (16 units, 88K);
-//   * more selected blocks or scores than the shared arrays hold, more units than clusters run at once, and score terms
-//     that leave no room for the ring.
+//   * more units than CTAs run at once: a last wave that is nearly empty costs a whole wave (192 units: 92 / 90);
+//   * more selected blocks or scores than the shared arrays hold.
 bool ckv_unit_step_plan(const ckv_ctx *c, int batch, int max_len, int kcap, CkvStepPlan *plan) {
   const CkvDev &P = c->dev;
-  if (c->layout.kv_dtype != CKV_BF16 || c->tail_mode != CKV_TAIL_AUTO || max_len < CKV_STEP_MIN_TOKENS || P.r == CKV_D) return false;
+  if (c->layout.kv_dtype != CKV_BF16 || c->tail_mode != CKV_TAIL_AUTO || max_len < CKV_STEP_MIN_TOKENS) return false;
   const int units = batch * P.Hkv, xmax = (max_len + P.bs - 1) / P.bs;
   if (xmax > kScoresCap || (kcap < xmax && kcap > kSelCap)) return false;
   int C = 0;
@@ -957,10 +973,13 @@ bool ckv_unit_step_plan(const ckv_ctx *c, int batch, int max_len, int kcap, CkvS
   const size_t stage = (size_t)P.scan_tile * (krow + vrow) + (P.r >= 4 ? (size_t)P.scan_tile * P.r * 4 : 0);
   const int parts = (std::max(xmax - 1, 0) + 15) / 16;
   plan->own_cap = 16 * std::max((parts + C - 1) / C, 1);
-  const size_t u_bytes = (size_t)(plan->own_cap + 8) * P.G * sizeof(float);
-  if (u_bytes + (size_t)skip * stage > (size_t)kDynLimit) return false;
+  size_t u_bytes = (size_t)(plan->own_cap + 8) * P.G * sizeof(float);
+  const int min_ring = std::max(kMinRing, skip);   // a warp visits every skip-th tile: the ring must hold that many (see the kernel)
+  plan->u_global = u_bytes + (size_t)min_ring * stage > (size_t)kDynLimit;
+  if (plan->u_global) u_bytes = 0;
   const int tiles = (plan->own_cap + P.scan_tile - 1) / P.scan_tile;
   plan->stages = std::min({kStagesCap, (int)(((size_t)kDynLimit - u_bytes) / stage), std::max(tiles, skip)});
+  if (plan->stages < skip) return false;
   plan->u_off = (int)(plan->stages * stage);
   plan->smem = (int)std::max((size_t)plan->u_off + u_bytes, (size_t)kAfterScan);
   plan->cluster = C;
