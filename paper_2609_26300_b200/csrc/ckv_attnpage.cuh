@@ -40,12 +40,11 @@ __device__ __forceinline__ void attn_pv(uint32_t vb, const float (&x)[HeadTile<G
   uint32_t b[HeadTile<G>::NR][2];
   HeadTile<G>::weights(x, lane, b);
   // ldmatrix.trans lane roles: matrix lane / 8 -> (coordinate chunk parity, row half), row lane % 8
-  const int r = (lane >> 4) * 8 + (lane & 7), cpar = (lane >> 3) & 1;
-  const uint32_t rowaddr = vb + r * kRowBytes;
+  const uint32_t rowaddr = (vb + ((lane >> 4) * 8 + (lane & 7)) * kRowBytes) | ((((lane >> 3) & 1) ^ (lane & 7)) << 4);
 #pragma unroll
   for (int t = 0; t < 8; ++t) {   // 16 coordinates
     uint32_t a[4];
-    ldmatrix_x4_trans(a, rowaddr + (uint32_t)(((2 * t + cpar) ^ (r & 7)) << 4));
+    ldmatrix_x4_trans(a, swz_at(rowaddr, t));
     mma_16816(w.acc[t], a, b[0][0], b[0][1]);
     if constexpr (!HeadTile<G>::PAIR) mma_16816(w.acc[t], a, b[1][0], b[1][1]);
   }
@@ -78,13 +77,12 @@ __device__ __forceinline__ void attn_page(uint32_t kb, uint32_t vb, const uint32
   float z[4] = {0.f, 0.f, 0.f, 0.f}, z2[4] = {0.f, 0.f, 0.f, 0.f};   // two chains: the products of one depend on one another
   {
     // ldmatrix lane roles: matrix lane / 8 -> (row half, coordinate chunk parity), row lane % 8
-    const int r = ((lane >> 3) & 1) * 8 + (lane & 7), cpar = lane >> 4;
-    const uint32_t rowaddr = kb + r * kRowBytes;
+    const uint32_t rowaddr = (kb + (((lane >> 3) & 1) * 8 + (lane & 7)) * kRowBytes) | (((lane >> 4) ^ (lane & 7)) << 4);
 #pragma unroll
     for (int ks = 0; ks < 8; ks += 2) {
       uint32_t a[4], a2[4];
-      ldmatrix_x4(a, rowaddr + (uint32_t)(((2 * ks + cpar) ^ (r & 7)) << 4));
-      ldmatrix_x4(a2, rowaddr + (uint32_t)(((2 * ks + 2 + cpar) ^ (r & 7)) << 4));
+      ldmatrix_x4(a, swz_at(rowaddr, ks));
+      ldmatrix_x4(a2, swz_at(rowaddr, ks + 1));
       mma_16816(z, a, qa[ks][0], qa[ks][1]);
       mma_16816(z2, a2, qa[ks + 1][0], qa[ks + 1][1]);
     }

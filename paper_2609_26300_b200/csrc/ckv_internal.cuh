@@ -68,7 +68,6 @@ struct CkvStepPlan {
   int stages;       // ring stages of the scan phase
   int own_cap;      // blocks of a unit one CTA owns, at most (a multiple of 16)
   int u_off, smem;  // offset of the score terms in dynamic shared memory, and its size
-  int u_global;     // 1: the score terms are too many for shared memory and go through the workspace
   int max_blocks;   // blocks of a sequence by the host's bound on the lengths
 };
 

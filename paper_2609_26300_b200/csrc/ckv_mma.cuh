@@ -32,6 +32,9 @@ __device__ __forceinline__ uint32_t movmatrix_trans(uint32_t a) {
   asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(d) : "r"(a));
   return d;
 }
+// Address of the 16-byte chunk 2 j + parity of a row whose chunks are XORed by (row & 7): `base` is the row's address
+// (a multiple of 128) with (parity ^ row & 7) * 16 in its low bits, so that one XOR per chunk of a half row is enough.
+__device__ __forceinline__ uint32_t swz_at(uint32_t base, int j) { return (base ^ (32u * (j & 3))) + 128u * (j >> 2); }
 // D (16x8) += A (16x16) B (16x8)
 __device__ __forceinline__ void mma_16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
   asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"

@@ -271,7 +271,7 @@ ckv_scan_kernel(CkvDev P, const QT *__restrict__ q, const int *seq_lens, int uni
   constexpr int TB = ScanTile<HS || VH>::TB;
   extern __shared__ __align__(128) unsigned char stage_mem[];
   __shared__ __align__(8) uint64_t full_bar[2][kMaxStages], empty_bar[kMaxStages];
-  __shared__ __align__(16) unsigned char s_zero_row[512];   // what mean-value rows past a unit's last block are read as
+  __shared__ __align__(512) unsigned char s_zero_row[512];   // what mean-value rows past a unit's last block are read as
   __shared__ int s_u0, s_tl0, s_count, s_ulast, s_abort, s_issued;
   __shared__ int s_len[kMaxSeqs];
   // Query rows and variance weights of the first kStagedUnits units of this CTA's range (a CTA's range rarely

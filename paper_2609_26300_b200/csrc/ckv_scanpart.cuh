@@ -74,7 +74,7 @@ struct ScanPartCfg {
 };
 
 // One part: rows rb .. rb + 15 of the tile whose first block is b0 and which holds nb blocks.  sk / sv / sd: the tile's
-// mean keys, mean values and variances in shared memory; zero_row: 512 bytes of zeros (what mean-value rows past nb are
+// mean keys, mean values and variances in shared memory; zero_row: 512 bytes of zeros, 128-byte aligned (what mean-value rows past nb are
 // read as: a stale NaN pattern times a zero weight would poison the accumulators; elsewhere a block is an output column,
 // and those columns are discarded).  b_partial: the block that may hold fewer than block_size tokens (-1: none), with
 // log_partial the log of its token count.  sw: variance weights [t][g] for r not 4 or d; dbar_row0: the unit's variance
@@ -96,17 +96,18 @@ __device__ __forceinline__ void scan_part(ScanUnit<G, QT, RD> &w, const ScanPart
   // another, and a warp has little else to issue while it waits for them
   float z[4] = {0.f, 0.f, 0.f, 0.f}, z2[4] = {0.f, 0.f, 0.f, 0.f}, zl[4] = {0.f, 0.f, 0.f, 0.f}, zl2_[4] = {0.f, 0.f, 0.f, 0.f};
   // ldmatrix lane roles: matrix lane / 8 -> (row half, coordinate chunk parity), row lane % 8
-  const int kr = rb + ((lane >> 3) & 1) * 8 + (lane & 7), kpar = lane >> 4;
+  const int kr = rb + ((lane >> 3) & 1) * 8 + (lane & 7);
+  const uint32_t kx = ((lane >> 4) ^ (lane & 7)) << 4;   // chunk parity and row swizzle (rb is a multiple of 8)
   {
-    const uint32_t rowaddr = sk + kr * kRowBytes;
+    const uint32_t rowaddr = (sk + kr * kRowBytes) | kx;
 #pragma unroll
     for (int ks = 0; ks < 8; ++ks) {
-      const uint32_t coff = (uint32_t)swz_chunk(2 * ks + kpar, kr) * 16;
+      const uint32_t at = swz_at(rowaddr, ks);
       uint32_t ah[4], al[4];
-      ldmatrix_x4(ah, rowaddr + coff);
+      ldmatrix_x4(ah, at);
       mma_16816((ks & 1) ? z2 : z, ah, w.qa[ks][0], w.qa[ks][1]);
       if (!HS) {
-        ldmatrix_x4(al, rowaddr + 256 + coff);
+        ldmatrix_x4(al, at + 256);
         mma_16816((ks & 1) ? zl2_ : zl, al, w.qa[ks][0], w.qa[ks][1]);
       }
       if constexpr (ScanUnit<G, QT, RD>::QB) mma_16816((ks & 1) ? zl2_ : zl, ah, w.qb[ks][0], w.qb[ks][1]);
@@ -118,13 +119,13 @@ __device__ __forceinline__ void scan_part(ScanUnit<G, QT, RD> &w, const ScanPart
   float sgm[T::NR][2];
   if constexpr (RD) {   // sigma^2 for the same tile: (qs_hi + qs_lo) (D_hi + D_lo)
     float g[4] = {0.f, 0.f, 0.f, 0.f}, g2[4] = {0.f, 0.f, 0.f, 0.f};
-    const uint32_t rowaddr = sv + TB * kRowBytes + kr * kRowBytes;
+    const uint32_t rowaddr = (sv + TB * kRowBytes + kr * kRowBytes) | kx;
 #pragma unroll
     for (int ks = 0; ks < 8; ++ks) {
-      const uint32_t coff = (uint32_t)swz_chunk(2 * ks + kpar, kr) * 16;
+      const uint32_t at = swz_at(rowaddr, ks);
       uint32_t dh[4], dl[4];
-      ldmatrix_x4(dh, rowaddr + coff);
-      ldmatrix_x4(dl, rowaddr + 256 + coff);
+      ldmatrix_x4(dh, at);
+      ldmatrix_x4(dl, at + 256);
       mma_16816(g, dh, w.qs[RD ? ks : 0][0], w.qs[RD ? ks : 0][1]);
       mma_16816(g2, dl, w.qs[RD ? ks : 0][0], w.qs[RD ? ks : 0][1]);
       if constexpr (!T::PAIR) mma_16816(g2, dh, w.qs2[ks][0], w.qs2[ks][1]);
@@ -144,7 +145,8 @@ __device__ __forceinline__ void scan_part(ScanUnit<G, QT, RD> &w, const ScanPart
     const bool real = r < nb;
     const float logc = b == b_partial ? log_partial : cfg.log_bs;
     float4 dv = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (!RD && cfg.r4 && real) dv = *reinterpret_cast<const float4 *>(sd + r * 4);
+    const bool r4 = VH || cfg.r4;   // VH comes with four variance groups only
+    if (!RD && r4 && real) dv = *reinterpret_cast<const float4 *>(sd + r * 4);
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
       const int head = T::head(lane, e);
@@ -153,7 +155,7 @@ __device__ __forceinline__ void scan_part(ScanUnit<G, QT, RD> &w, const ScanPart
       if (val) {
         if constexpr (RD) {
           sg = fmaxf(sgm[k][e], 0.f);
-        } else if (cfg.r4) {
+        } else if (r4) {
           sg = fmaf(w.wown[e][0], dv.x, fmaf(w.wown[e][1], dv.y, fmaf(w.wown[e][2], dv.z, w.wown[e][3] * dv.w)));
         } else {
           for (int t = 0; t < cfg.r; ++t) {
@@ -191,19 +193,19 @@ __device__ __forceinline__ void scan_part(ScanUnit<G, QT, RD> &w, const ScanPart
     uint32_t b[T::NR][2];
     T::weights(wt, lane, b);
     // ldmatrix.trans lane roles: matrix lane / 8 -> (coordinate chunk parity, row half), row lane % 8
-    const int r = rb + (lane >> 4) * 8 + (lane & 7), cpar = (lane >> 3) & 1;
-    const bool real = r < nb;   // rows past the last block: zeros
-    const uint32_t rowaddr = real ? sv + r * kRowBytesV : zero_row;
+    const int r = rb + (lane >> 4) * 8 + (lane & 7);
+    // rows past the last block: the row of zeros, which is as long as a stored row
+    const uint32_t rowaddr = (r < nb ? sv + r * kRowBytesV : zero_row) | ((((lane >> 3) & 1) ^ (lane & 7)) << 4);
 #pragma unroll
     for (int t = 0; t < 8; ++t) {
-      const uint32_t coff = real ? (uint32_t)swz_chunk(2 * t + cpar, r) * 16 : 0u;
+      const uint32_t at = swz_at(rowaddr, t);
       uint32_t vh[4];
-      ldmatrix_x4_trans(vh, rowaddr + coff);
+      ldmatrix_x4_trans(vh, at);
       mma_16816(w.acc[t], vh, b[0][0], b[0][1]);
       if constexpr (!T::PAIR) mma_16816(w.acc[t], vh, b[T::NR - 1][0], b[T::NR - 1][1]);
       if constexpr (!HS && !VH) {
         uint32_t vl[4];
-        ldmatrix_x4_trans(vl, rowaddr + (real ? 256u : 0u) + coff);
+        ldmatrix_x4_trans(vl, at + 256);
         mma_16816(w.acc[t], vl, b[0][0], b[0][1]);
       }
     }

@@ -49,7 +49,7 @@ constexpr int kProducerWarp = kWarps, kTailWarp = kWarps + 1;
 constexpr int kThreads = (kWarps + 2) * 32;
 constexpr int kClusterCap = CKV_STEP_MAX_CLUSTER;
 constexpr int kStagesCap = 6;
-constexpr int kMinRing = 3;                     // stages the score terms have to leave room for, or they go through global memory
+constexpr int kMinRing = 3;                     // ring stages that the score terms have to leave room for
 constexpr int kScoresCap = 9216;                // blocks of a unit whose scores every CTA can hold
 constexpr int kBins = 2048;                     // score histogram: 32 octaves below the largest possible score, 64 bins each
 constexpr int kBinShift = 17;                   // ... a bin is a score's bit pattern without its low 17 bits
@@ -226,7 +226,7 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *__restrict__ q, const int *seq_lens, 
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ __align__(8) uint64_t full_bar[2][kStagesCap], empty_bar[kStagesCap];
   __shared__ __align__(8) uint64_t s_xbar[4];                 // what the cluster's CTAs send: normalisers, scores, partial outputs; global stores done
-  __shared__ __align__(16) unsigned char s_zero_row[512];
+  __shared__ __align__(512) unsigned char s_zero_row[512];
   __shared__ __align__(16) bf16 s_q[G][CKV_D];
   __shared__ float s_w[G * 64];                               // variance weights [t][g], r < d
   __shared__ __align__(16) float4 s_wn[kWarps + 1][G];        // (maximum m, sum of e^{l - m}, largest score term) per warp, then of the last block
@@ -261,8 +261,6 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *__restrict__ q, const int *seq_lens, 
   if (tid >= kThreads - 32) reinterpret_cast<uint4 *>(s_zero_row)[lane] = make_uint4(0u, 0u, 0u, 0u);
   const bool dbar_bulk = P.r >= 4;
   const int stage_bytes = TB * (kRowBytesK + kRowBytesV) + (dbar_bulk ? TB * P.r * 4 : 0);
-  float *su = reinterpret_cast<float *>(smem + plan.u_off);   // score terms of the CTA's own blocks, [g][u_stride]
-  const int u_stride = plan.own_cap + 8;   // a tile's eight rows x four heads then fall into 32 different banks
   // the length the step works on; a bound the host misjudged is kept to what the shared arrays were sized for
   const int N = max(min(min(raw + ((append && raw >= 0 && raw < cap) ? 1 : 0), cap), plan.max_blocks * P.bs), 0);
   const int X = (N + P.bs - 1) >> P.lg_bs, Xs = max(X - 1, 0);
@@ -272,6 +270,10 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *__restrict__ q, const int *seq_lens, 
   const int own = max(min(min(b_lo + ppc * 16, Xs) - b_lo, plan.own_cap), 0);
   const int tiles = (own + TB - 1) / TB;
   const size_t row0 = (size_t)unit * P.max_blocks;
+  // score terms of the CTA's own blocks, [g][us] (eight more than the range holds: a tile's eight rows x four heads then
+  // fall into 32 different banks)
+  float *ub = reinterpret_cast<float *>(smem + plan.u_off);
+  const int us = plan.own_cap + 8;
 
   // one fill of the ring: tile `it` into stage `st`, counted on full barrier `fb`
   auto fill = [&](int it, int st, uint64_t *fb) {
@@ -380,7 +382,7 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *__restrict__ q, const int *seq_lens, 
       }
     }
     const ScanPartCfg cfg{P.scale, P.half_var, logf((float)P.bs), P.r, P.max_blocks, (P.variant & CKV_VARIANT_RANK_BY_MASS) != 0, P.r == 4};
-    float *lz = P.lz + row0 * G, *lu = P.lu + row0 * G;
+    float *lz = P.lz + row0 * G;
     const int part = warp % kParts;
     // A warp visits every kSkip-th tile.  A fill is only issued once the one plan.stages before it was released, and
     // kSkip <= plan.stages (checked by the launcher): alternate rounds of the ring use two sets of full barriers, which
@@ -410,7 +412,7 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *__restrict__ q, const int *seq_lens, 
             w, cfg, sk, sk + TB * kRowBytesK, (RD || dbar_bulk) ? sd : nullptr, smem_u32(s_zero_row), s_w, P.dbar + row0 * P.r,
             lane, rb, nb, b_lo + it * TB, -1, 0.f,
             [&](int g, int blk, float x, float y) {
-              if (plan.u_global) lu[(size_t)g * P.max_blocks + blk] = x; else su[g * u_stride + (blk - b_lo)] = x;
+              ub[g * us + (blk - b_lo)] = x;
               lz[(size_t)g * P.max_blocks + blk] = y;
               if (g & 1) umax[1] = fmaxf(umax[1], x); else umax[0] = fmaxf(umax[0], x);
             });
@@ -505,27 +507,13 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *__restrict__ q, const int *seq_lens, 
   if (warp < kWarps) {
     bool nonfinite = false;
     const uint32_t xbar1 = smem_u32(&s_xbar[1]);
-    // the score terms of the CTA's blocks, in shared memory or in the workspace (where a head's row may start anywhere)
-    const float *ub = plan.u_global ? P.lu + row0 * G + b_lo : su;
-    const size_t us = plan.u_global ? (size_t)P.max_blocks : (size_t)u_stride;
-    const bool wide = (us & 3) == 0;
     for (int i = 4 * tid; i < own; i += 4 * kWork) {
       float sc[4] = {0.f, 0.f, 0.f, 0.f};
-      float4 u[G];   // all heads' loads before the first use: they may be trips to the L2
-      if (wide) {
-#pragma unroll
-        for (int g = 0; g < G; ++g) u[g] = *reinterpret_cast<const float4 *>(ub + g * us + i);
-      } else {
-#pragma unroll
-        for (int g = 0; g < G; ++g) {
-          const float *up = ub + g * us + i;
-          u[g] = make_float4(up[0], i + 1 < own ? up[1] : 0.f, i + 2 < own ? up[2] : 0.f, i + 3 < own ? up[3] : 0.f);
-        }
-      }
 #pragma unroll
       for (int g = 0; g < G; ++g) {
-        sc[0] = fmaf(fast_exp2(u[g].x - Mg[g]), iL[g], sc[0]); sc[1] = fmaf(fast_exp2(u[g].y - Mg[g]), iL[g], sc[1]);
-        sc[2] = fmaf(fast_exp2(u[g].z - Mg[g]), iL[g], sc[2]); sc[3] = fmaf(fast_exp2(u[g].w - Mg[g]), iL[g], sc[3]);
+        const float4 u = *reinterpret_cast<const float4 *>(ub + g * us + i);
+        sc[0] = fmaf(fast_exp2(u.x - Mg[g]), iL[g], sc[0]); sc[1] = fmaf(fast_exp2(u.y - Mg[g]), iL[g], sc[1]);
+        sc[2] = fmaf(fast_exp2(u.z - Mg[g]), iL[g], sc[2]); sc[3] = fmaf(fast_exp2(u.w - Mg[g]), iL[g], sc[3]);
       }
       uint32_t k[4];
 #pragma unroll
@@ -950,15 +938,17 @@ cudaError_t ckv_configure_unit_step(ckv_ctx *c) {
 }
 
 // Whether a step of this size runs as one launch, and how.  Against the separate launches (us per step, back to back):
-// 15.3 / 27.4 (one head, 4K), 17.4 / 35.8 (8 units, 32K), 22.4 / 38.6 (8 units, 128K, 32-token blocks), 32.2 / 51.2 (24
-// units, 100K, bf16 summaries), 41.9 / 60.3 (16 units, 88K, r = d), 56.1 / 69.2 (32 units, 128K), 60 / 70 (64 units, 64K),
-// 61 / 81 (72 units, 58K), 95 / 147 (80 units, r = 16), 73 / 80 (88 units of 14K, r = d), 71 / 81 (128 units, 32K), 82 / 89
-// (128 ragged units, G = 8: one CTA per unit, score terms through global memory).  What stays with the separate launches:
+// 14.3 / 27.4 (one head, 4K), 16.7 / 35.8 (8 units, 32K), 21.9 / 38.6 (8 units, 128K, 32-token blocks), 31.5 / 51.2 (24
+// units, 100K, bf16 summaries), 41.3 / 60.3 (16 units, 88K, r = d), 53.4 / 68.4 (32 units, 128K), 60 / 70 (64 units, 64K),
+// 61 / 81 (72 units, 58K), 95 / 147 (80 units, r = 16), 73 / 80 (88 units of 14K, r = d), 69 / 81 (128 units, 32K).
+// What stays with the separate launches, and why:
 //   * fp32 pages (the attention is on bf16 tensor cores) and an explicit ckv_set_tail_mode, which asks for them;
 //   * caches under CKV_STEP_MIN_TOKENS.  Not a crossover -- one launch is the faster form there too -- but the size below
 //     which the documented two-call arrangement (append, scan, select, attention as launches of their own) is kept;
 //   * more units than CTAs run at once: a last wave that is nearly empty costs a whole wave (192 units: 92 / 90);
-//   * more selected blocks or scores than the shared arrays hold.
+//   * more selected blocks or scores than the shared arrays hold, or score terms that leave no room for the ring: one CTA
+//     per unit with eight heads beyond about 30K tokens.  There the persistent scan's even split of the tiles is worth
+//     more (a long sequence of a ragged batch is one CTA's work here), and its three launches are kept.
 bool ckv_unit_step_plan(const ckv_ctx *c, int batch, int max_len, int kcap, CkvStepPlan *plan) {
   const CkvDev &P = c->dev;
   if (c->layout.kv_dtype != CKV_BF16 || c->tail_mode != CKV_TAIL_AUTO || max_len < CKV_STEP_MIN_TOKENS) return false;
@@ -973,13 +963,10 @@ bool ckv_unit_step_plan(const ckv_ctx *c, int batch, int max_len, int kcap, CkvS
   const size_t stage = (size_t)P.scan_tile * (krow + vrow) + (P.r >= 4 ? (size_t)P.scan_tile * P.r * 4 : 0);
   const int parts = (std::max(xmax - 1, 0) + 15) / 16;
   plan->own_cap = 16 * std::max((parts + C - 1) / C, 1);
-  size_t u_bytes = (size_t)(plan->own_cap + 8) * P.G * sizeof(float);
-  const int min_ring = std::max(kMinRing, skip);   // a warp visits every skip-th tile: the ring must hold that many (see the kernel)
-  plan->u_global = u_bytes + (size_t)min_ring * stage > (size_t)kDynLimit;
-  if (plan->u_global) u_bytes = 0;
+  const size_t u_bytes = (size_t)(plan->own_cap + 8) * P.G * sizeof(float);
+  if (u_bytes + (size_t)std::max(kMinRing, skip) * stage > (size_t)kDynLimit) return false;
   const int tiles = (plan->own_cap + P.scan_tile - 1) / P.scan_tile;
   plan->stages = std::min({kStagesCap, (int)(((size_t)kDynLimit - u_bytes) / stage), std::max(tiles, skip)});
-  if (plan->stages < skip) return false;
   plan->u_off = (int)(plan->stages * stage);
   plan->smem = (int)std::max((size_t)plan->u_off + u_bytes, (size_t)kAfterScan);
   plan->cluster = C;
