@@ -27,9 +27,8 @@ struct ScanUnit : HeadAcc<G> {
   using T = HeadTile<G>;
   static constexpr bool QS = QSplit<QT>::value;        // fp32 queries are split into hi + lo like the summaries
   static constexpr bool QB = QS && !T::PAIR;           // ... as a second operand where columns 4..7 cannot take the lo halves
-  static constexpr bool RB = RD && !T::PAIR;
   uint32_t qa[8][2], qb[QB ? 8 : 1][2];                // B fragments of the unit's queries, per 16-coordinate step
-  uint32_t qs[RD ? 8 : 1][2], qs2[RB ? 8 : 1][2];      // (scale q)^2, same fragment positions: columns hi | lo, or two operands
+  uint32_t qs[RD ? 8 : 1][2], qs2[RD ? 8 : 1][2];      // (scale q)^2 as hi and lo halves, same fragment positions
   float wown[2][4];                                    // variance weights of this lane's heads (r = 4)
   float lp[2];                                         // sum of e^{l - m}
 
@@ -59,8 +58,8 @@ struct ScanUnit : HeadAcc<G> {
           const float s0 = (x.x * scale) * (x.x * scale), s1 = (x.y * scale) * (x.y * scale);
           const uint32_t sh = pack_bf16(s0, s1);
           const uint32_t sl = pack_bf16(s0 - __uint_as_float(sh << 16), s1 - __uint_as_float(sh & 0xffff0000u));
-          qs[RD ? ks : 0][hh] = low ? sl : sh;
-          if constexpr (RB) qs2[RB ? ks : 0][hh] = sl;
+          qs[RD ? ks : 0][hh] = sh;
+          qs2[RD ? ks : 0][hh] = sl;
         }
       }
   }
@@ -117,22 +116,26 @@ __device__ __forceinline__ void scan_part(ScanUnit<G, QT, RD> &w, const ScanPart
     if constexpr (QSplit<QT>::value && T::PAIR) T::add_copies(z);   // columns 4..7: the queries' lo halves
   }
   float sgm[T::NR][2];
-  if constexpr (RD) {   // sigma^2 for the same tile: (qs_hi + qs_lo) (D_hi + D_lo)
+  if constexpr (RD) {   // sigma^2 for the same tile: (qs_hi + qs_lo) (D_hi + D_lo) without the lo lo term
     float g[4] = {0.f, 0.f, 0.f, 0.f}, g2[4] = {0.f, 0.f, 0.f, 0.f};
     const uint32_t rowaddr = (sv + TB * kRowBytes + kr * kRowBytes) | kx;
 #pragma unroll
-    for (int ks = 0; ks < 8; ++ks) {
-      const uint32_t at = swz_at(rowaddr, ks);
-      uint32_t dh[4], dl[4];
-      ldmatrix_x4(dh, at);
-      ldmatrix_x4(dl, at + 256);
-      mma_16816(g, dh, w.qs[RD ? ks : 0][0], w.qs[RD ? ks : 0][1]);
-      mma_16816(g2, dl, w.qs[RD ? ks : 0][0], w.qs[RD ? ks : 0][1]);
-      if constexpr (!T::PAIR) mma_16816(g2, dh, w.qs2[ks][0], w.qs2[ks][1]);
+    for (int ks = 0; ks < 8; ks += 2) {   // the order of the chains is part of the result: scores that differ in the last bit
+      uint32_t dh[2][4], dl[2][4];        // can swap blocks at the cut
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const uint32_t at = swz_at(rowaddr, ks + j);
+        ldmatrix_x4(dh[j], at);
+        ldmatrix_x4(dl[j], at + 256);
+        mma_16816(g, dh[j], w.qs[RD ? ks + j : 0][0], w.qs[RD ? ks + j : 0][1]);
+      }
+#pragma unroll
+      for (int j = 0; j < 2; ++j) mma_16816(g2, dh[j], w.qs2[RD ? ks + j : 0][0], w.qs2[RD ? ks + j : 0][1]);
+#pragma unroll
+      for (int j = 0; j < 2; ++j) mma_16816(g2, dl[j], w.qs[RD ? ks + j : 0][0], w.qs[RD ? ks + j : 0][1]);
     }
 #pragma unroll
     for (int i = 0; i < 4; ++i) g[i] += g2[i];
-    if constexpr (T::PAIR) T::add_copies(g);
     T::pick(g, lane, sgm);
   }
 

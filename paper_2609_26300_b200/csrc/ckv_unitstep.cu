@@ -126,8 +126,11 @@ __device__ __noinline__ void cut_by_bisection(int X, int kr, const uint32_t *key
 // The last CTA's tail warp: the new token (if there is one) goes into its page and the last block's summary is redone
 // with the append's own routine; then, new token or not, the last block's two per-head terms and its compensation
 // partial, with plain FMAs, from the summary as stored (a fresh one is taken from the registers it was stored from).
+// The cluster waits for this warp, whose time is one chain of dependent loads and cold code (4.3 us beside 2.7 us of scan
+// at 32K): so every load that depends on nothing is requested first, the new row is put among the page's other rows in
+// registers instead of being read back, and the sums of all heads share one tree of shuffles.
 template <int G>
-__device__ __noinline__ void tail_block(const CkvDev P, const bf16 *sq_rows, const int *page_table, const CkvNewToken fresh,
+__device__ __noinline__ void tail_block(const CkvDev P, const bf16 *q_rows, const int *page_table, const CkvNewToken fresh,
                                         int unit, int raw, int N, float *sq, float *tail_u, float *tail_part, float4 *norm) {
   const int lane = threadIdx.x & 31, hw = lane >> 4, li = lane & 15;
   const int s = ckv_div_hkv(P, unit), h = unit - s * P.Hkv;
@@ -135,70 +138,87 @@ __device__ __noinline__ void tail_block(const CkvDev P, const bf16 *sq_rows, con
   const bool lo_half = P.row_elems == CKV_ROW_ELEMS;
   const bool by_mass = (P.variant & CKV_VARIANT_RANK_BY_MASS) != 0;
   const int *pt_row = page_table + (size_t)s * P.max_pages_per_seq;
-  BlockRow br;
-  bool fresh_row = false;
-  if (fresh.k_new != nullptr) {
-    if (raw < 0 || raw >= cap) {
-      if (lane == 0) atomicOr(P.status, CKV_DEV_SEQ_FULL);
-    } else {
-      bf16 *kp = reinterpret_cast<bf16 *>(fresh.k_pool), *vp = reinterpret_cast<bf16 *>(fresh.v_pool);
-      const bf16 *row_new = reinterpret_cast<const bf16 *>(lane < 16 ? fresh.k_new : fresh.v_new) + (size_t)unit * CKV_D;
-      const uint4 piece = __ldg(reinterpret_cast<const uint4 *>(row_new) + li);
-      const int phys = pt_row[raw / CKV_PAGE];
-      const int b = raw >> P.lg_bs, cnt = raw + 1 - b * P.bs;
-      if (phys >= 0 && phys < P.num_pages)
-        reinterpret_cast<uint4 *>((lane < 16 ? kp : vp) + (((size_t)phys * P.Hkv + h) * CKV_PAGE + raw % CKV_PAGE) * CKV_D)[li] = piece;
-      __syncwarp();
-      const size_t row = (size_t)unit * P.max_blocks + b;
-      block_stats_warp<bf16, false>(P, kp, vp, pt_row, h, b, cnt, sq, P.kmean + row * P.row_elems, P.dbar + row * P.r,
-                                    P.vmean + row * P.row_elems, lane, &br);
-      fresh_row = true;
-    }
+  const bool append = fresh.k_new != nullptr && raw >= 0 && raw < cap;
+  int phys = -1;
+  uint4 kn, vn;   // this lane's eight coordinates of the new rows
+  kn = vn = make_uint4(0u, 0u, 0u, 0u);
+  if (append) {
+    phys = pt_row[raw / CKV_PAGE];
+    kn = __ldg(reinterpret_cast<const uint4 *>(reinterpret_cast<const bf16 *>(fresh.k_new) + (size_t)unit * CKV_D) + li);
+    vn = __ldg(reinterpret_cast<const uint4 *>(reinterpret_cast<const bf16 *>(fresh.v_new) + (size_t)unit * CKV_D) + li);
   }
+  uint4 qr[G];    // ... and of the queries
+#pragma unroll
+  for (int g = 0; g < G; ++g) qr[g] = __ldg(reinterpret_cast<const uint4 *>(q_rows + (size_t)g * CKV_D) + li);
   const int b = ((N + P.bs - 1) >> P.lg_bs) - 1, cnt = N - b * P.bs;
   const size_t row = (size_t)unit * P.max_blocks + b;
-  if (!fresh_row) {   // the summary as stored: lower half warp the mean key, upper the mean value (as the scan reads it)
-    load_split8<false>((hw == 0 ? P.kmean : P.vmean) + row * P.row_elems, li, b, br.x, lo_half && !(hw == 1 && P.vhi));
-    if (P.r == CKV_D) {
-      load_split8<false>(reinterpret_cast<const bf16 *>(P.dbar + row * CKV_D), li, b, br.dvar);
-    } else {
-      const float *drow = P.dbar + row * P.r;
+  __nv_bfloat16 *kmean_row = P.kmean + row * P.row_elems, *vmean_row = P.vmean + row * P.row_elems;
+  float *dbar_row = P.dbar + row * P.r;
+  BlockRow br;
+  if (append) {
+    bf16 *kp = reinterpret_cast<bf16 *>(fresh.k_pool), *vp = reinterpret_cast<bf16 *>(fresh.v_pool);
+    const bool ok = phys >= 0 && phys < P.num_pages;
+    const size_t base = ok ? ((size_t)phys * P.Hkv + h) * CKV_PAGE * CKV_D + 8 * li : 0;
+    const size_t at = base + (size_t)(raw % CKV_PAGE) * CKV_D;
+    if (cnt <= CKV_PAGE) {   // the token's page is all there is of its block
+      uint4 kraw[8], vraw[8];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) br.dvar[i] = drow[group_of(8 * li + i, P.r, P.glayout)];
+      for (int j = 0; j < 8; ++j) {
+        const int t = hw + 2 * j;
+        kraw[j] = kn; vraw[j] = vn;
+        if (ok && t < cnt - 1) {
+          kraw[j] = *reinterpret_cast<const uint4 *>(kp + base + (size_t)t * CKV_D);
+          vraw[j] = *reinterpret_cast<const uint4 *>(vp + base + (size_t)t * CKV_D);
+        }
+      }
+      if (ok) *reinterpret_cast<uint4 *>((hw == 0 ? kp : vp) + at) = hw == 0 ? kn : vn;
+      float km[8], vs[8], ssq[8];
+      block_stats_rows16(kraw, vraw, ok, cnt, lane, km, vs, ssq);
+      block_stats_finish(P, b, (float)cnt, km, vs, ssq, sq, kmean_row, dbar_row, vmean_row, lane, !ok, &br);
+    } else {
+      if (ok) *reinterpret_cast<uint4 *>((hw == 0 ? kp : vp) + at) = hw == 0 ? kn : vn;
+      __syncwarp();
+      block_stats_warp<bf16, false>(P, kp, vp, pt_row, h, b, cnt, sq, kmean_row, dbar_row, vmean_row, lane, &br);
+    }
+  } else {   // the summary as stored: lower half warp the mean key, upper the mean value (as the scan reads it)
+    if (fresh.k_new != nullptr && lane == 0) atomicOr(P.status, CKV_DEV_SEQ_FULL);
+    load_split8<false>(hw == 0 ? kmean_row : vmean_row, li, b, br.x, lo_half && !(hw == 1 && P.vhi));
+    if (P.r == CKV_D) {
+      load_split8<false>(reinterpret_cast<const bf16 *>(dbar_row), li, b, br.dvar);
+    } else {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) br.dvar[i] = dbar_row[group_of(8 * li + i, P.r, P.glayout)];
     }
   }
-  const float logc = logf((float)cnt);
+  // sums over the 16 lanes of a half warp, d_0 .. d_{G-1}, sigma^2_0 .. sigma^2_{G-1} (the d of the lower half count: it holds the mean key)
+  float v[2 * G];
 #pragma unroll
   for (int g = 0; g < G; ++g) {
     float qx[8];
-    load8<false>(sq_rows + g * CKV_D + 8 * li, qx);
-    float d = 0.f, sg = 0.f;
+    bf16x8_to_float(qr[g], qx);
+    v[g] = v[G + g] = 0.f;
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      d = fmaf(qx[i], br.x[i], d);   // (meaningful in the lower half warp, which holds the mean key)
+      v[g] = fmaf(qx[i], br.x[i], v[g]);
       const float qs = qx[i] * P.scale;
-      sg = fmaf(qs * qs, br.dvar[i], sg);   // Eq. 8: the squared logit scale is its 1/d
-    }
-#pragma unroll
-    for (int o = 8; o > 0; o >>= 1) {
-      d += __shfl_xor_sync(0xffffffffu, d, o);
-      sg += __shfl_xor_sync(0xffffffffu, sg, o);
-    }
-    sg = fmaxf(sg, 0.f);
-    const float zbar = d * P.scale;
-    const float zl2 = (zbar + logc) * kLog2e;
-    if (lane == 0) {
-      const float u = fmaf(logc + zbar + P.half_var * sg, kLog2e, by_mass ? 0.f : __log2f(sg));
-      tail_u[g] = u;
-      P.lz[((size_t)unit * G + g) * P.max_blocks + b] = zl2;
-      norm[g] = make_float4(zl2, fast_exp2(P.half_var * kLog2e * sg), u, 0.f);
-      tail_part[g * CKV_PART_STRIDE] = zl2;
-      tail_part[g * CKV_PART_STRIDE + 1] = 1.f;
+      v[G + g] = fmaf(qs * qs, br.dvar[i], v[G + g]);   // Eq. 8: the squared logit scale is its 1/d
     }
     if (hw == 1) {   // weight 1 times the mean value
       *reinterpret_cast<float4 *>(tail_part + g * CKV_PART_STRIDE + 4 + 8 * li) = make_float4(br.x[0], br.x[1], br.x[2], br.x[3]);
       *reinterpret_cast<float4 *>(tail_part + g * CKV_PART_STRIDE + 8 + 8 * li) = make_float4(br.x[4], br.x[5], br.x[6], br.x[7]);
     }
+  }
+  reduce16<2 * G, 1>(v, li);   // half-warp lane i now holds sum i / (8 / G)
+  const float d = __shfl_sync(0xffffffffu, v[0], (lane * (8 / G)) & 15);
+  const float sg = fmaxf(__shfl_sync(0xffffffffu, v[0], ((G + lane) * (8 / G)) & 15), 0.f);
+  if (lane < G) {
+    const float zbar = d * P.scale, logc = logf((float)cnt), zl2 = (zbar + logc) * kLog2e;
+    const float u = fmaf(logc + zbar + P.half_var * sg, kLog2e, by_mass ? 0.f : __log2f(sg));
+    tail_u[lane] = u;
+    P.lz[((size_t)unit * G + lane) * P.max_blocks + b] = zl2;
+    norm[lane] = make_float4(zl2, fast_exp2(P.half_var * kLog2e * sg), u, 0.f);
+    tail_part[lane * CKV_PART_STRIDE] = zl2;
+    tail_part[lane * CKV_PART_STRIDE + 1] = 1.f;
   }
 }
 
@@ -304,7 +324,9 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *__restrict__ q, const int *seq_lens, 
       }
     if (!ok) atomicOr(P.status, CKV_DEV_BAD_COPY);
   };
-  __syncthreads();
+  // The tail warp does not wait here: it needs nothing that the others set up, and the cluster will wait for it.
+  if (warp == kTailWarp) named_arrive(3, kThreads);
+  else named_barrier(3, kThreads);
   // the first round of fills is issued by as many warps at once: a fill is some seventy instructions, a third of a
   // microsecond for one thread, which alone would have the last stage's data arrive a microsecond late
   const int first_fills = min(tiles, plan.stages);
@@ -338,15 +360,18 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *__restrict__ q, const int *seq_lens, 
     }
   } else if (warp == kTailWarp) {
     if (rank == C - 1 && N > 0)
-      tail_block<G>(P, &s_q[0][0], page_table, fresh, unit, raw, N, s_sq, s_tail_u, &s_tail_part[0][0], s_wn[kWarps]);
+      tail_block<G>(P, q + (size_t)unit * G * CKV_D, page_table, fresh, unit, raw, N, s_sq, s_tail_u, &s_tail_part[0][0], s_wn[kWarps]);
     else if (lane < G)
       s_wn[kWarps][lane] = make_float4(-CUDART_INF_F, 0.f, -CUDART_INF_F, 0.f);
   } else {
     // ---------------- working warps: parts of 16 blocks ----------------
-    if (!RD && P.r != 4) {
-      for (int i = tid; i < P.r * G; i += kWork) {   // w_{g,t} of Eq. 8 times the squared logit scale
+    if (!RD) {
+      // w_{g,t} of Eq. 8 times the squared logit scale, summed in coordinate order as every kernel does it: scores that
+      // differ in the last bit can swap blocks at the cut.  (The first tile's data is still on its way.)
+      for (int i = tid; i < P.r * G; i += kWork) {
         const int g = i & (G - 1), t = i / G, gs = CKV_D / P.r, run = P.glayout == 0 ? gs : gs / 2;
         float a = 0.f;
+#pragma unroll 8
         for (int k = 0; k < gs; ++k) {
           const int c = t * run + (k < run ? k : CKV_D / 2 + k - run);
           const float x = __bfloat162float(s_q[g][c]);
@@ -360,26 +385,11 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *__restrict__ q, const int *seq_lens, 
       const uint32_t x = *reinterpret_cast<const uint32_t *>(&s_q[g][c]);
       return make_float2(__uint_as_float(x << 16), __uint_as_float(x & 0xffff0000u));
     });
-    if (!RD && P.r == 4) {   // the same from the fragments: a column's four lanes hold its head's 128 coordinates between them
-      float a[4] = {0.f, 0.f, 0.f, 0.f};
+    if (!RD && P.r == 4) {
 #pragma unroll
-      for (int ks = 0; ks < 8; ++ks) {
-        float sq = 0.f;
+      for (int e = 0; e < 2; ++e)
 #pragma unroll
-        for (int hh = 0; hh < 2; ++hh) {
-          const float x0 = __uint_as_float(w.qa[ks][hh] << 16), x1 = __uint_as_float(w.qa[ks][hh] & 0xffff0000u);
-          sq = fmaf(x0, x0, fmaf(x1, x1, sq));
-        }
-        if (P.glayout == 0) a[ks / 2] += sq; else a[ks % 4] += sq;   // 16 coordinates of one group
-      }
-#pragma unroll
-      for (int t = 0; t < 4; ++t) {
-        a[t] += __shfl_xor_sync(0xffffffffu, a[t], 1);
-        a[t] += __shfl_xor_sync(0xffffffffu, a[t], 2);
-        a[t] *= P.scale * P.scale;
-#pragma unroll
-        for (int e = 0; e < 2; ++e) w.wown[e][t] = __shfl_sync(0xffffffffu, a[t], 4 * T::head(lane, e));   // column = head
-      }
+        for (int t = 0; t < 4; ++t) w.wown[e][t] = T::head(lane, e) < G ? s_w[t * G + T::head(lane, e)] : 0.f;
     }
     const ScanPartCfg cfg{P.scale, P.half_var, logf((float)P.bs), P.r, P.max_blocks, (P.variant & CKV_VARIANT_RANK_BY_MASS) != 0, P.r == 4};
     float *lz = P.lz + row0 * G;
