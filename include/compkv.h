@@ -254,7 +254,8 @@ int ckv_copy_scores(ckv_ctx *ctx, float *dst, int batch, ckv_stream stream);
  * (all work the call put on the stream has then finished).  Host buffers should be pinned: buffers the
  * device can address (pinned, registered or managed memory, 16-byte aligned) are moved by two small
  * kernels of the library and the call waits on a pinned word its last kernel stores; pageable buffers
- * take six copies and a stream synchronisation (about 20 us more per call).  A caller that comes back with the
+ * take six copies and a stream synchronisation (about 20 us more per call).  Where the step is one launch (see ckv_step),
+ * that launch reads the pinned inputs and writes the pinned results itself.  Otherwise a caller that comes back with the
  * same buffers, arrays and sizes on a stream of its own (not the default stream, not a capturing one) has its
  * second such call captured as a CUDA graph and the later ones replayed (the length bound is rounded up to a
  * multiple of 1024 inside, so the graph lasts that many steps); the graph is the context's and goes with it.

@@ -133,8 +133,17 @@ def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
     return t.data_ptr()
 
 
-def _stream() -> int:
+def _public_stream() -> int:
     return torch.cuda.current_stream().cuda_stream
+
+
+def _raw_stream() -> int:
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+
+
+# The current stream's handle.  Building a torch.cuda.Stream object for it costs 3.3 us a call (a whole step of one short
+# sequence takes 13 us on the GPU), reading the handle 0.2 us.
+_stream = _raw_stream if hasattr(torch._C, "_cuda_getCurrentRawStream") and hasattr(torch._C, "_cuda_getDevice") else _public_stream
 
 
 def dense_decode_static(layout: ckv_layout, q, k_pool, v_pool, page_table, seq_lens, max_seq_len: int, out=None,

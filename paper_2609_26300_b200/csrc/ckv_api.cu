@@ -261,8 +261,8 @@ bool device_view(const void *host, void **dev) {
   *dev = a.devicePointer;
   return true;
 }
+constexpr size_t kHostReadBytes = 160 * 1024;   // see ckv_step_host
 bool aligned16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
-constexpr int kHostEpochWord = 20;   // word of the status region that counts the ckv_step_host calls completed on the device
 
 // three source ranges to three destination ranges, 16 bytes per thread and iteration (sizes are multiples of 16)
 __global__ void __launch_bounds__(1024) ckv_move3_kernel(const uint4 *__restrict__ a, uint4 *__restrict__ da, int na,
@@ -326,7 +326,7 @@ int decode_impl(ckv_ctx *c, const void *q, const void *k_pool, const void *v_poo
     return CKV_ERR_BUDGET_TOO_SMALL;
   CkvStepPlan plan;
   if (ev == nullptr && ckv_unit_step_plan(c, batch, max_seq_len_host, kcap, &plan)) {
-    CKV_CUDA(ckv_launch_unit_step(c, plan, q, k_pool, v_pool, page_table, seq_lens, fresh, batch, kcap, sel_ids, sel_cnt, out, lse, s));
+    CKV_CUDA(ckv_launch_unit_step(c, plan, q, k_pool, v_pool, page_table, seq_lens, fresh, batch, kcap, sel_ids, sel_cnt, out, lse, CkvHostDone{}, s));
     return CKV_OK;
   }
   int scan_grid = 0, n_splits = 0;
@@ -487,7 +487,7 @@ int ckv_step_host(ckv_ctx *c, const void *q_host, const void *k_new_host, const 
                       device_view(out_host, &ho) && device_view(sel_ids_host, &hi) && device_view(sel_cnt_host, &hc) &&
                       aligned16(hq) && aligned16(hk) && aligned16(hv) && aligned16(ho) && aligned16(hi);
   const bool flagged = direct && c->host_flag != nullptr;
-  int *done_count = c->dev.status + kHostEpochWord;
+  int *done_count = c->dev.status + CKV_HOST_EPOCH_WORD;
   // the three parts of the call as launches on `on`: inputs in, the step, results out (+ completion word)
   auto enqueue = [&](cudaStream_t on, int max_len) -> int {
     if (direct) {
@@ -520,6 +520,25 @@ int ckv_step_host(ckv_ctx *c, const void *q_host, const void *k_new_host, const 
     c->host_epoch = *c->host_flag;
     return CKV_OK;
   };
+
+  // A step that is one launch reads its inputs from the pinned buffers and writes its results there itself, completion
+  // word included: nothing is staged and there is one kernel to launch (a graph of copy-in, step and copy-out took 64 us
+  // a call at 128K where this takes 56 us).  Every CTA of a unit reads the unit's queries, so this is for steps whose CTAs
+  // read no more than kHostReadBytes over the bus; larger ones bring the inputs in with one kernel first.
+  CkvStepPlan plan;
+  if (flagged && ckv_unit_step_plan(c, batch, max_seq_len_host, kcap, &plan)) {
+    if (!k_pool || !v_pool || !page_table || !seq_lens) return CKV_ERR_INVALID_ARG;
+    if (kcap < L.sink_blocks + L.recent_blocks && (long long)kcap * L.block_size < max_seq_len_host) return CKV_ERR_BUDGET_TOO_SMALL;
+    const void *sq = hq, *sk = hk, *sv = hv;
+    if (q_bytes * plan.cluster > kHostReadBytes) {
+      CKV_CUDA(ckv_launch_host_in(c, hq, hk, hv, dq, dk, dv, q_bytes, kv_bytes, s));
+      sq = dq; sk = dk; sv = dv;
+    }
+    const CkvNewToken fresh = {k_pool, v_pool, page_table, seq_lens, sk, sv};
+    CKV_CUDA(ckv_launch_unit_step(c, plan, sq, k_pool, v_pool, page_table, seq_lens, &fresh, batch, kcap, (int *)hi, (int *)hc, ho, nullptr,
+                                  CkvHostDone{c->host_flag_dev, done_count, c->dev.status + CKV_CTA_COUNTER_WORD}, s));
+    return wait_done();
+  }
 
   // A caller that comes back with the same buffers and sizes (a decode loop) gets its second call captured as a
   // CUDA graph and every later one replayed: one driver call instead of five launches.  The length bound is part

@@ -23,6 +23,8 @@
 #define CKV_STEP_MAX_CLUSTER 16   // CTAs of a unit in the one-launch step, at most (the opt-in cluster size of sm_100)
 #define CKV_STEP_MIN_TOKENS 1536  // shorter caches keep the separate launches (see ckv_unit_step_plan)
 #define CKV_LEN_COUNTER_WORD 16   // word of the status region that counts who has read the lengths in a fused step
+#define CKV_HOST_EPOCH_WORD 20    // ... that counts the ckv_step_host calls completed on the device
+#define CKV_CTA_COUNTER_WORD 24   // ... that counts the CTAs of a one-launch step whose results are in host memory
 #define CKV_RESCALE_SLACK 16.0f  // log2 units: running maxima are only raised when exceeded by this much
 
 constexpr float kLog2e = 1.4426950408889634f;
@@ -61,6 +63,10 @@ struct CkvDev {
   uint32_t spin_limit;  // polls a bounded wait makes before it gives up (ckv_debug_set; default ckv_pipe::kSpinLimit)
   int debug;         // ckv_debug_flags (test hooks; 0 in normal use)
 };
+
+// The completion word a host-buffer call waits on: the kernel's last CTA adds one to *count and stores it to *flag (pinned),
+// after every result has reached host memory.  flag null: nobody waits.
+struct CkvHostDone { int *flag, *count, *ctas; };
 
 // How a step runs as one launch (ckv_unit_step_plan).
 struct CkvStepPlan {
@@ -125,7 +131,7 @@ struct CkvNewToken {
 bool ckv_unit_step_plan(const ckv_ctx *c, int batch, int max_len, int kcap, CkvStepPlan *plan);
 cudaError_t ckv_launch_unit_step(ckv_ctx *c, const CkvStepPlan &plan, const void *q, const void *k_pool, const void *v_pool,
                                  const int *page_table, const int *seq_lens, const CkvNewToken *fresh, int batch, int kcap,
-                                 int *sel_ids, int *sel_cnt, void *out, float *lse, cudaStream_t st);
+                                 int *sel_ids, int *sel_cnt, void *out, float *lse, const CkvHostDone &done, cudaStream_t st);
 // max_len is an upper bound of the lengths the step works on (after the append, if there is one).  The launch
 // follows c->dev.tail; a new token needs tail mode.
 cudaError_t ckv_launch_scan(ckv_ctx *c, const void *q, const int *seq_lens, int batch, int max_len,

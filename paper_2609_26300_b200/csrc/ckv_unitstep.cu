@@ -237,7 +237,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 ckv_unit_step_kernel(CkvDev P, const bf16 *__restrict__ q, const int *seq_lens, const bf16 *k_pool, const bf16 *v_pool,
                      const int *__restrict__ page_table, CkvNewToken fresh, int kcap, CkvStepPlan plan, int batch,
                      int *__restrict__ sel_ids, int *__restrict__ sel_cnt, bf16 *__restrict__ out, float *__restrict__ lse,
-                     const __grid_constant__ CUtensorMap tm_v) {
+                     CkvHostDone done, const __grid_constant__ CUtensorMap tm_v) {
   constexpr int kRowBytesK = HS ? CKV_D * 2 : CKV_ROW_ELEMS * 2;
   constexpr int kRowBytesV = (HS || VH) ? CKV_D * 2 : CKV_ROW_ELEMS * 2;
   constexpr int TB = ScanTile<HS || VH>::TB;
@@ -879,6 +879,18 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *__restrict__ q, const int *seq_lens, 
       if (lse != nullptr && (item & 3) == 0 && lane == 0) lse[(size_t)unit * G + g] = N > 0 ? (M + log2f(den)) * kLn2 : -CUDART_INF_F;
     }
   }
+  if (done.flag != nullptr) {   // the results are in the caller's host buffers: the last CTA to say so stores the word
+    __syncthreads();
+    if (tid == 0) {
+      __threadfence_system();
+      if (atomicAdd(done.ctas, 1) == (int)(gridDim.x * gridDim.y) - 1) {
+        *done.ctas = 0;
+        const int e = *done.count + 1;   // counted on the device, call after call
+        *done.count = e;
+        *(volatile int *)done.flag = e;
+      }
+    }
+  }
   __syncwarp();
   cluster_arrive_relaxed();   // nobody leaves while somebody may still send to it
   cluster_wait();
@@ -986,7 +998,8 @@ bool ckv_unit_step_plan(const ckv_ctx *c, int batch, int max_len, int kcap, CkvS
 
 cudaError_t ckv_launch_unit_step(ckv_ctx *c, const CkvStepPlan &plan, const void *q, const void *k_pool, const void *v_pool,
                                  const int *page_table, const int *seq_lens, const CkvNewToken *fresh_in, int batch, int kcap,
-                                 int *sel_ids, int *sel_cnt, void *out, float *lse, cudaStream_t st) {
+                                 int *sel_ids, int *sel_cnt, void *out, float *lse, const CkvHostDone &done_in, cudaStream_t st) {
+  CkvHostDone done = done_in;
   CkvNewToken fresh = {};
   if (fresh_in != nullptr) fresh = *fresh_in;
   cudaLaunchAttribute attr[2];
@@ -995,7 +1008,7 @@ cudaError_t ckv_launch_unit_step(ckv_ctx *c, const CkvStepPlan &plan, const void
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.numAttrs = 2;
   CkvStepPlan p = plan;
-  void *args[] = {&c->dev, &q, &seq_lens, &k_pool, &v_pool, &page_table, &fresh, &kcap, &p, &batch, &sel_ids, &sel_cnt, &out, &lse, &c->tm_vhi};
+  void *args[] = {&c->dev, &q, &seq_lens, &k_pool, &v_pool, &page_table, &fresh, &kcap, &p, &batch, &sel_ids, &sel_cnt, &out, &lse, &done, &c->tm_vhi};
   c->launches++;
   return cudaLaunchKernelExC(&cfg, kernel_of(c->dev), args);
 }

@@ -134,3 +134,27 @@ def test_a_wait_that_runs_out_is_reported_and_the_context_recovers():
     again = d.ckv.decode(q, d.k_pool, d.v_pool, d.table, d.lens, d.max_len, w.budget_tokens)
     torch.cuda.synchronize()
     assert d.ckv.read_status() == 0 and all(torch.equal(x, y) for x, y in zip(good, again))
+
+
+@pytest.mark.parametrize("batch,hq,hkv", [(1, 8, 2), (9, 64, 8)])   # inputs read over the bus; brought in by a kernel first
+def test_host_buffers_in_one_launch(batch, hq, hkv):
+    w = workload(batch=batch, num_q_heads=hq, num_kv_heads=hkv, ctx=16 * 200 + 3, needles=0, decode_steps=4)
+    a, b = setup(w), setup(w)
+    for d in (a, b):
+        d.ckv.stats_build(d.k_pool, d.v_pool, d.table, d.lens, d.max_len)
+    kcap = w.budget_tokens // 16
+    pin = dict(pin_memory=True)
+    ho = torch.zeros(batch, hq, 128, dtype=torch.bfloat16, **pin)
+    hi, hc = torch.zeros(batch, hkv, kcap, dtype=torch.int32, **pin), torch.zeros(batch, hkv, dtype=torch.int32, **pin)
+    for t in range(4):
+        q, kn, vn = step_inputs(a, t)
+        before = a.ckv.launch_count()
+        a.ckv.step_host(q.cpu().pin_memory(), kn.cpu().pin_memory(), vn.cpu().pin_memory(), a.k_pool, a.v_pool, a.table,
+                        a.lens, w.ctx + t + 1, w.budget_tokens, ho, hi, hc)
+        got = [x.clone() for x in (ho, hi, hc)]   # complete when the call returns
+        assert a.ckv.launch_count() - before == (1 if batch == 1 else 2)
+        out, lse, ids, cnt = b.ckv.step(q, kn, vn, b.k_pool, b.v_pool, b.table, b.lens, w.ctx + t + 1, w.budget_tokens)
+        torch.cuda.synchronize()
+        for x, y in zip(got, (out, ids, cnt)):
+            assert torch.equal(x, y.cpu()), t
+    assert torch.equal(a.lens, b.lens) and a.ckv.read_status() == 0
