@@ -35,6 +35,7 @@
 #include "ckv_mma.cuh"
 #include "ckv_cluster.cuh"
 #include "ckv_attnpage.cuh"
+#include "ckv_pipe.cuh"
 
 namespace {
 
@@ -65,6 +66,8 @@ ckv_attn_mma_kernel(CkvDev P, const __nv_bfloat16 *__restrict__ q, const __nv_bf
   // Cluster merge: where the other splits of the unit deposit their partials of the heads this CTA reduces.
   // Entry (j * cluster size + source rank) belongs to head (this rank + j * cluster size).
   __shared__ __align__(16) float s_recv[CL ? (G + kMaxCluster) * CKV_PART_STRIDE : 4];
+  if (DENSE) ckv_pipe::pdl_trigger();   // (see ckv_launch_pdl on the sparse form)
+  ckv_pipe::pdl_wait();
   if (CL) cluster_arrive_relaxed();   // first phase of the cluster barrier: "this CTA runs, its shared memory exists"
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -559,35 +562,15 @@ cudaError_t launch_g(ckv_ctx *c, bool dense, const void *q, const void *k_pool, 
                      dim3 grid, int pps, int scan_grid, void *out, float *lse, cudaStream_t st) {
   const int units = (int)grid.y;
   const __nv_bfloat16 *qp = (const __nv_bfloat16 *)q, *kp = (const __nv_bfloat16 *)k_pool, *vp = (const __nv_bfloat16 *)v_pool;
-  if (dense) {
-    ckv_attn_mma_kernel<G, true, kDenseWarps, false, false><<<grid, kDenseWarps * 32, dyn_smem<kDenseWarps>(), st>>>(
-        c->dev, qp, kp, vp, page_table, seq_lens, sel_ids, sel_cnt, kcap, pps, scan_grid, units, (__nv_bfloat16 *)out, lse);
-    return cudaGetLastError();
-  }
+  if (dense)
+    return ckv_launch_pdl(ckv_attn_mma_kernel<G, true, kDenseWarps, false, false>, grid, dim3(kDenseWarps * 32), dyn_smem<kDenseWarps>(), st, 0,
+                          c->dev, qp, kp, vp, page_table, seq_lens, sel_ids, sel_cnt, kcap, pps, scan_grid, units, (__nv_bfloat16 *)out, lse);
   const bool rm = c->dev.row_elems == CKV_D;   // bf16 summaries: removal with the stored mean-value rows
-  if (cluster_fits<G>((int)grid.x, st)) {   // the unit's splits as one cluster: partials never leave the SMs
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(kSparseWarps * 32);
-    cfg.dynamicSmemBytes = dyn_smem<kSparseWarps>();
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = grid.x; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
-    if (rm)
-      return cudaLaunchKernelEx(&cfg, ckv_attn_mma_kernel<G, false, kSparseWarps, true, true>, c->dev, qp, kp, vp, page_table,
-                                seq_lens, sel_ids, sel_cnt, kcap, pps, scan_grid, units, (__nv_bfloat16 *)out, lse);
-    return cudaLaunchKernelEx(&cfg, ckv_attn_mma_kernel<G, false, kSparseWarps, true, false>, c->dev, qp, kp, vp, page_table,
-                              seq_lens, sel_ids, sel_cnt, kcap, pps, scan_grid, units, (__nv_bfloat16 *)out, lse);
-  }
-  if (rm)
-    ckv_attn_mma_kernel<G, false, kSparseWarps, false, true><<<grid, kSparseWarps * 32, dyn_smem<kSparseWarps>(), st>>>(
-        c->dev, qp, kp, vp, page_table, seq_lens, sel_ids, sel_cnt, kcap, pps, scan_grid, units, (__nv_bfloat16 *)out, lse);
-  else
-    ckv_attn_mma_kernel<G, false, kSparseWarps, false, false><<<grid, kSparseWarps * 32, dyn_smem<kSparseWarps>(), st>>>(
-        c->dev, qp, kp, vp, page_table, seq_lens, sel_ids, sel_cnt, kcap, pps, scan_grid, units, (__nv_bfloat16 *)out, lse);
-  return cudaGetLastError();
+  const bool cl = cluster_fits<G>((int)grid.x, st);   // the unit's splits as one cluster: partials never leave the SMs
+  auto kernel = cl ? (rm ? ckv_attn_mma_kernel<G, false, kSparseWarps, true, true> : ckv_attn_mma_kernel<G, false, kSparseWarps, true, false>)
+                   : (rm ? ckv_attn_mma_kernel<G, false, kSparseWarps, false, true> : ckv_attn_mma_kernel<G, false, kSparseWarps, false, false>);
+  return ckv_launch_pdl(kernel, grid, dim3(kSparseWarps * 32), dyn_smem<kSparseWarps>(), st, cl ? (int)grid.x : 0,
+                        c->dev, qp, kp, vp, page_table, seq_lens, sel_ids, sel_cnt, kcap, pps, scan_grid, units, (__nv_bfloat16 *)out, lse);
 }
 
 template <int G>

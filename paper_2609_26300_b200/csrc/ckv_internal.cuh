@@ -100,6 +100,25 @@ struct ckv_ctx {
   bool hg_key_valid, hg_disabled;
 };
 
+// A launch that may start while the launch before it in the stream is still running (programmatic dependent launch): the
+// kernel calls pdl_wait() before it touches global memory.  Gaps of 2 to 3 us between kernels all but vanish (prefill chunks
+// 129 -> 124 us, the three-launch step of 128 units 87.4 -> 80.7).  pdl_trigger() lets the next kernel's CTAs in before this
+// one's are done: good where the next one is alike (builds, chunks, dense passes, one-launch steps), bad among the scan,
+// selection and attention kernels, whose CTAs then sit on SMs that the running kernel still needs (80.7 -> 92.3): those do
+// not call it.  cluster_x: CTAs of a cluster (0: no clusters).
+template <class... Params, class... Args>
+inline cudaError_t ckv_launch_pdl(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, int cluster_x, Args... args) {
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = cluster_x; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
+  cfg.attrs = attr; cfg.numAttrs = cluster_x > 0 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, kernel, Params(args)...);
+}
+
 int ckv_record_cuda_error(cudaError_t e);   // remembers e for ckv_last_cuda_error() on this thread; returns CKV_ERR_CUDA
 cudaError_t ckv_configure_kernels();   // selection kernel attributes
 cudaError_t ckv_configure_scan(ckv_ctx *c);   // scan kernel attributes (and, with vhi, the tensor map of the mean values)

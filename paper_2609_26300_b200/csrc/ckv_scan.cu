@@ -295,6 +295,7 @@ ckv_scan_kernel(CkvDev P, const QT *__restrict__ q, const int *seq_lens, int uni
   const int cap = P.max_blocks * P.bs;
   // length the step works on: one more than stored when a token is being appended (a full sequence keeps its length)
   auto eff_len = [&](int raw) { return max(min(raw + ((append && raw >= 0 && raw < cap) ? 1 : 0), cap), 0); };
+  pdl_wait();
   const int len_mine = tid < batch ? seq_lens[tid] : 0;
   if ((int)blockIdx.x < n_tail) {
     // ---------------- tail CTAs: the new token and the last block of every unit ----------------
@@ -638,20 +639,19 @@ cudaError_t launch_gt(ckv_ctx *c, const void *q, const int *seq_lens, int units,
   const ScanCfg cfg = scan_cfg(c->dev, G);
   if (cfg.stages == 0) return cudaErrorInvalidConfiguration;
   if (c->dev.r == CKV_D)
-    ckv_scan_kernel<G, QT, true, false, false><<<grid, kThreads, cfg.smem, st>>>(c->dev, (const QT *)q, seq_lens, units, cfg.stages, fresh, n_tail, c->tm_vhi);
+    return ckv_launch_pdl(ckv_scan_kernel<G, QT, true, false, false>, dim3(grid), dim3(kThreads), cfg.smem, st, 0, c->dev, (const QT *)q, seq_lens, units, cfg.stages, fresh, n_tail, c->tm_vhi);
   else if (c->dev.row_elems == CKV_D) {
     if constexpr (!QSplit<QT>::value)   // bf16 summaries come with bf16 pages and queries only
-      ckv_scan_kernel<G, QT, false, true, false><<<grid, kThreads, cfg.smem, st>>>(c->dev, (const QT *)q, seq_lens, units, cfg.stages, fresh, n_tail, c->tm_vhi);
+      return ckv_launch_pdl(ckv_scan_kernel<G, QT, false, true, false>, dim3(grid), dim3(kThreads), cfg.smem, st, 0, c->dev, (const QT *)q, seq_lens, units, cfg.stages, fresh, n_tail, c->tm_vhi);
     else
       return cudaErrorInvalidValue;
   } else if (c->dev.vhi) {
     if constexpr (!QSplit<QT>::value)
-      ckv_scan_kernel<G, QT, false, false, true><<<grid, kThreads, cfg.smem, st>>>(c->dev, (const QT *)q, seq_lens, units, cfg.stages, fresh, n_tail, c->tm_vhi);
+      return ckv_launch_pdl(ckv_scan_kernel<G, QT, false, false, true>, dim3(grid), dim3(kThreads), cfg.smem, st, 0, c->dev, (const QT *)q, seq_lens, units, cfg.stages, fresh, n_tail, c->tm_vhi);
     else
       return cudaErrorInvalidValue;
   } else
-    ckv_scan_kernel<G, QT, false, false, false><<<grid, kThreads, cfg.smem, st>>>(c->dev, (const QT *)q, seq_lens, units, cfg.stages, fresh, n_tail, c->tm_vhi);
-  return cudaGetLastError();
+    return ckv_launch_pdl(ckv_scan_kernel<G, QT, false, false, false>, dim3(grid), dim3(kThreads), cfg.smem, st, 0, c->dev, (const QT *)q, seq_lens, units, cfg.stages, fresh, n_tail, c->tm_vhi);
 }
 
 template <int G>

@@ -14,6 +14,7 @@
 // in the bin that holds the threshold (falling back to 12 + 8 more bits on heavy ties); ids come out in position
 // order from a prefix sum over selection flags.
 #include "ckv_internal.cuh"
+#include "ckv_pipe.cuh"
 
 namespace {
 
@@ -63,6 +64,9 @@ __global__ void __launch_bounds__(kThreads) ckv_select_kernel(CkvDev P, const in
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int unit = blockIdx.x, s = ckv_div_hkv(P, unit);
+  if (tid == 0) s_ncand = 0;
+  for (int i = tid; i < kBins; i += kThreads) s_hist[i] = 0;   // the first radix pass fills it while scoring
+  ckv_pipe::pdl_wait();
   const int N = max(min(seq_lens[s], P.max_blocks * P.bs), 0);
   const int X = (N + P.bs - 1) >> P.lg_bs;
   int *ids = sel_ids + (size_t)unit * kcap;
@@ -77,8 +81,6 @@ __global__ void __launch_bounds__(kThreads) ckv_select_kernel(CkvDev P, const in
   // ---- normalisers of Eq. 9: M_g, L_g from the scan partials of this unit (entries (c + unit) * W + w, c in
   // [cfirst, cfirst + ccount)).  Warp g works them out for head g; its loads are issued before the much larger
   // batch of score-term loads below, which would otherwise sit in front of them in the memory pipeline. ----
-  if (tid == 0) s_ncand = 0;
-  for (int i = tid; i < kBins; i += kThreads) s_hist[i] = 0;   // the first radix pass fills it while scoring
   float pm[4], pl[4];
   const float *cp = nullptr;
   int n_part = 0;
@@ -311,8 +313,7 @@ template <int G>
 cudaError_t launch_g(ckv_ctx *c, const int *seq_lens, int units, int kcap, int scan_grid, int *sel_ids, int *sel_cnt,
                      cudaStream_t st) {
   const size_t smem = (size_t)kSmemKeys * sizeof(uint32_t);
-  ckv_select_kernel<G><<<units, kThreads, smem, st>>>(c->dev, seq_lens, kcap, scan_grid, units, sel_ids, sel_cnt);
-  return cudaGetLastError();
+  return ckv_launch_pdl(ckv_select_kernel<G>, dim3(units), dim3(kThreads), smem, st, 0, c->dev, seq_lens, kcap, scan_grid, units, sel_ids, sel_cnt);
 }
 
 template <int G>

@@ -8,13 +8,31 @@
 // operations in the same order, so their results are bit-identical.
 #include "ckv_internal.cuh"
 #include "ckv_blockstats.cuh"
+#include "ckv_pipe.cuh"
 
 namespace {
 
-constexpr int kBuildRounds = 8;   // blocks per warp of the build kernel
-constexpr int kPrefillRounds = 4; // blocks per warp of the prefill kernel's register-resident variant
+constexpr int kBuildRounds = 8;   // blocks per warp of the build kernel, at most
+constexpr int kPrefillRounds = 4; // blocks per warp of the prefill kernel's register-resident variants, at most
 
-// A warp takes kBuildRounds blocks, eight blocks apart.  Two CTAs per SM: the block routine holds a page's 16 key and
+// Blocks per warp of a launch over `units` units of `blocks` blocks each (CTAs of eight warps, two CTAs per SM).  All CTAs
+// take about the same time, so a launch takes waves * rounds of it, and what is lost is the last wave: 2K-token chunks of
+// one sequence with four rounds 133 us, with one 69; 8K chunks of two sequences 125 us with four (one wave, in lockstep),
+// 136 with three (1.2 waves), 116 with two; 9K caches of 32-token blocks 46 us with eight rounds, 39 with two.  Among equals
+// the most rounds (fewest CTAs to start) that still leave two waves to overlap, else the fewest.
+int rounds_for(int blocks, int units, int sms, int most) {
+  int best = 1;
+  long long best_cost = 0;
+  bool best_two = false;
+  for (int r = 1; r <= most; ++r) {
+    const long long ctas = (long long)((blocks + 8 * r - 1) / (8 * r)) * units, waves = (ctas + 2 * sms - 1) / (2 * sms);
+    const long long cost = waves * r;
+    if (r == 1 || cost < best_cost || (cost == best_cost && waves >= 2 && best_two)) { best = r; best_cost = cost; best_two = waves >= 2; }
+  }
+  return best;
+}
+
+// A warp takes `rounds` blocks, eight blocks apart (rounds_for).  Two CTAs per SM: the block routine holds a page's 16 key and
 // 16 value rows in registers, which does not fit three CTAs' register share without spills, and the kernel was bound
 // by instruction issue, not by DRAM, while it spilled.  The 16 warps of an SM keep enough rows in flight by
 // themselves: asking the L2 for a warp's next block ahead of time (which paid while the block routine was long) now
@@ -24,16 +42,18 @@ template <typename T, bool ONEP>
 __global__ void __launch_bounds__(256, 2) ckv_stats_build_kernel(CkvDev P, const T *__restrict__ k_pool,
                                                               const T *__restrict__ v_pool,
                                                               const int *__restrict__ page_table,
-                                                              const int *__restrict__ seq_lens) {
+                                                              const int *__restrict__ seq_lens, int rounds) {
   __shared__ float sq_smem[8][CKV_D];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int unit = blockIdx.y, s = unit / P.Hkv, h = unit % P.Hkv;
+  ckv_pipe::pdl_trigger();
+  ckv_pipe::pdl_wait();
   const int N = min(seq_lens[s], P.max_blocks * P.bs);
   const int X = (N + P.bs - 1) / P.bs;
   const int *pt_row = page_table + (size_t)s * P.max_pages_per_seq;
 #pragma unroll 1
-  for (int i = 0; i < kBuildRounds; ++i) {
-    const int b = (blockIdx.x * kBuildRounds + i) * 8 + warp;
+  for (int i = 0; i < rounds; ++i) {
+    const int b = (blockIdx.x * rounds + i) * 8 + warp;
     if (b >= X) return;
     const int cnt = min(P.bs, N - b * P.bs);
     const size_t row = (size_t)unit * P.max_blocks + b;
@@ -50,6 +70,8 @@ __global__ void __launch_bounds__(256) ckv_append_kernel(CkvDev P, T *k_pool, T 
   __shared__ float sq_smem[8][CKV_D];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
   const int s = blockIdx.x;
+  ckv_pipe::pdl_trigger();
+  ckv_pipe::pdl_wait();
   const int N = seq_lens[s];
   // the new row of this warp's first head does not depend on N: it is requested together with it, so that the
   // chain length -> page -> row has no fourth link (16-byte pieces: lanes 0-15 hold K, lanes 16-31 hold V)
@@ -102,20 +124,23 @@ template <typename T, int REG>
 __global__ void __launch_bounds__(256, REG ? 2 : 1) ckv_prefill_kernel(CkvDev P, T *k_pool, T *v_pool,
                                                           const int *__restrict__ page_table, int *seq_lens,
                                                           const T *__restrict__ k_src, const T *__restrict__ v_src,
-                                                          const int *__restrict__ new_lens, int src_stride, int batch) {
+                                                          const int *__restrict__ new_lens, int src_stride, int batch,
+                                                          int rounds) {
   __shared__ float sq_smem[8][CKV_D];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int unit = blockIdx.y, s = unit / P.Hkv, h = unit % P.Hkv;
   const int cap = P.max_blocks * P.bs;
+  ckv_pipe::pdl_trigger();
+  ckv_pipe::pdl_wait();
   const int N = seq_lens[s], M = new_lens[s];
   const int m_eff = N < 0 ? 0 : max(min(min(M, src_stride), cap - N), 0);   // tokens that fit
   if (M > m_eff && blockIdx.x == 0 && threadIdx.x == 0) atomicOr(P.status, CKV_DEV_SEQ_FULL);
-  // the register-resident variant gives a warp kPrefillRounds blocks, eight blocks apart (L2 requests for the next
+  // the register-resident variants give a warp `rounds` blocks, eight blocks apart (L2 requests for the next
   // block's rows ahead of time made it slower once the block routine had been trimmed: 763 against 728 us)
-  constexpr int kRounds = REG ? kPrefillRounds : 1;
+  const int n_rounds = REG ? rounds : 1;
 #pragma unroll 1
-  for (int rnd = 0; rnd < kRounds; ++rnd) {
-  const int b = (N >= 0 ? N / P.bs : 0) + (blockIdx.x * kRounds + rnd) * 8 + warp;
+  for (int rnd = 0; rnd < n_rounds; ++rnd) {
+  const int b = (N >= 0 ? N / P.bs : 0) + (blockIdx.x * n_rounds + rnd) * 8 + warp;
   if (m_eff > 0 && b <= (N + m_eff - 1) / P.bs) {
     const int *pt_row = page_table + (size_t)s * P.max_pages_per_seq;
     const int p_lo = max(b * P.bs, N), p_hi = min((b + 1) * P.bs, N + m_eff);
@@ -296,18 +321,18 @@ cudaError_t ckv_launch_stats_build(ckv_ctx *c, const void *k_pool, const void *v
   const CkvDev &P = c->dev;
   const int xmax = (max_len + P.bs - 1) / P.bs;
   if (xmax <= 0 || batch <= 0) return cudaSuccess;
-  dim3 grid((xmax + 8 * kBuildRounds - 1) / (8 * kBuildRounds), batch * P.Hkv);
+  const int sms = c->sm_count > 0 ? c->sm_count : 148;
+  const int rounds = rounds_for(xmax, batch * P.Hkv, sms, kBuildRounds);
+  dim3 grid((xmax + 8 * rounds - 1) / (8 * rounds), batch * P.Hkv);
+  cudaError_t e;
   if (c->layout.kv_dtype == CKV_BF16 && P.ppb == 1)
-    ckv_stats_build_kernel<__nv_bfloat16, true><<<grid, 256, 0, st>>>(P, (const __nv_bfloat16 *)k_pool,
-                                                                      (const __nv_bfloat16 *)v_pool, page_table, seq_lens);
+    e = ckv_launch_pdl(ckv_stats_build_kernel<__nv_bfloat16, true>, dim3(grid), dim3(256), 0, st, 0, P, (const __nv_bfloat16 *)k_pool, (const __nv_bfloat16 *)v_pool, page_table, seq_lens, rounds);
   else if (c->layout.kv_dtype == CKV_BF16)
-    ckv_stats_build_kernel<__nv_bfloat16, false><<<grid, 256, 0, st>>>(P, (const __nv_bfloat16 *)k_pool,
-                                                                       (const __nv_bfloat16 *)v_pool, page_table, seq_lens);
+    e = ckv_launch_pdl(ckv_stats_build_kernel<__nv_bfloat16, false>, dim3(grid), dim3(256), 0, st, 0, P, (const __nv_bfloat16 *)k_pool, (const __nv_bfloat16 *)v_pool, page_table, seq_lens, rounds);
   else
-    ckv_stats_build_kernel<float, false><<<grid, 256, 0, st>>>(P, (const float *)k_pool, (const float *)v_pool, page_table,
-                                                               seq_lens);
+    e = ckv_launch_pdl(ckv_stats_build_kernel<float, false>, dim3(grid), dim3(256), 0, st, 0, P, (const float *)k_pool, (const float *)v_pool, page_table, seq_lens, rounds);
   c->launches++;
-  return cudaGetLastError();
+  return e;
 }
 
 cudaError_t ckv_launch_prefill(ckv_ctx *c, void *k_pool, void *v_pool, const int *page_table, int *seq_lens,
@@ -317,20 +342,18 @@ cudaError_t ckv_launch_prefill(ckv_ctx *c, void *k_pool, void *v_pool, const int
   if (batch <= 0 || max_new <= 0) return cudaSuccess;
   const int touched = (max_new + P.bs - 1) / P.bs + 1;   // a chunk that starts inside a block touches one more
   dim3 grid((touched + 7) / 8, batch * P.Hkv);
-  const dim3 grid_one((touched + 8 * kPrefillRounds - 1) / (8 * kPrefillRounds), batch * P.Hkv);
+  const int sms = c->sm_count > 0 ? c->sm_count : 148;
+  const int rounds = rounds_for(touched, batch * P.Hkv, sms, kPrefillRounds);
+  const dim3 grid_one((touched + 8 * rounds - 1) / (8 * rounds), batch * P.Hkv);
+  cudaError_t e;
   if (c->layout.kv_dtype == CKV_BF16 && P.ppb == 1)
-    ckv_prefill_kernel<__nv_bfloat16, 1><<<grid_one, 256, 0, st>>>(P, (__nv_bfloat16 *)k_pool, (__nv_bfloat16 *)v_pool,
-                                                                  page_table, seq_lens, (const __nv_bfloat16 *)k_src,
-                                                                  (const __nv_bfloat16 *)v_src, new_lens, src_stride, batch);
+    e = ckv_launch_pdl(ckv_prefill_kernel<__nv_bfloat16, 1>, dim3(grid_one), dim3(256), 0, st, 0, P, (__nv_bfloat16 *)k_pool, (__nv_bfloat16 *)v_pool, page_table, seq_lens, (const __nv_bfloat16 *)k_src, (const __nv_bfloat16 *)v_src, new_lens, src_stride, batch, rounds);
   else if (c->layout.kv_dtype == CKV_BF16)
-    ckv_prefill_kernel<__nv_bfloat16, 2><<<grid_one, 256, 0, st>>>(P, (__nv_bfloat16 *)k_pool, (__nv_bfloat16 *)v_pool,
-                                                                   page_table, seq_lens, (const __nv_bfloat16 *)k_src,
-                                                                   (const __nv_bfloat16 *)v_src, new_lens, src_stride, batch);
+    e = ckv_launch_pdl(ckv_prefill_kernel<__nv_bfloat16, 2>, dim3(grid_one), dim3(256), 0, st, 0, P, (__nv_bfloat16 *)k_pool, (__nv_bfloat16 *)v_pool, page_table, seq_lens, (const __nv_bfloat16 *)k_src, (const __nv_bfloat16 *)v_src, new_lens, src_stride, batch, rounds);
   else
-    ckv_prefill_kernel<float, 0><<<grid, 256, 0, st>>>(P, (float *)k_pool, (float *)v_pool, page_table, seq_lens,
-                                                    (const float *)k_src, (const float *)v_src, new_lens, src_stride, batch);
+    e = ckv_launch_pdl(ckv_prefill_kernel<float, 0>, dim3(grid), dim3(256), 0, st, 0, P, (float *)k_pool, (float *)v_pool, page_table, seq_lens, (const float *)k_src, (const float *)v_src, new_lens, src_stride, batch, rounds);
   c->launches++;
-  return cudaGetLastError();
+  return e;
 }
 
 cudaError_t ckv_launch_append(ckv_ctx *c, void *k_pool, void *v_pool, const int *page_table, int *seq_lens,
@@ -338,13 +361,11 @@ cudaError_t ckv_launch_append(ckv_ctx *c, void *k_pool, void *v_pool, const int 
   const CkvDev &P = c->dev;
   if (batch <= 0) return cudaSuccess;
   const int threads = 32 * min(P.Hkv, 8);
+  cudaError_t e;
   if (c->layout.kv_dtype == CKV_BF16)
-    ckv_append_kernel<__nv_bfloat16><<<batch, threads, 0, st>>>(P, (__nv_bfloat16 *)k_pool, (__nv_bfloat16 *)v_pool,
-                                                                page_table, seq_lens, (const __nv_bfloat16 *)k_new,
-                                                                (const __nv_bfloat16 *)v_new);
+    e = ckv_launch_pdl(ckv_append_kernel<__nv_bfloat16>, dim3(batch), dim3(threads), 0, st, 0, P, (__nv_bfloat16 *)k_pool, (__nv_bfloat16 *)v_pool, page_table, seq_lens, (const __nv_bfloat16 *)k_new, (const __nv_bfloat16 *)v_new);
   else
-    ckv_append_kernel<float><<<batch, threads, 0, st>>>(P, (float *)k_pool, (float *)v_pool, page_table, seq_lens,
-                                                        (const float *)k_new, (const float *)v_new);
+    e = ckv_launch_pdl(ckv_append_kernel<float>, dim3(batch), dim3(threads), 0, st, 0, P, (float *)k_pool, (float *)v_pool, page_table, seq_lens, (const float *)k_new, (const float *)v_new);
   c->launches++;
-  return cudaGetLastError();
+  return e;
 }

@@ -96,3 +96,31 @@ def test_prefill_then_decode_steps_and_capacity():
     torch.cuda.synchronize()
     assert d.ckv.read_status() & 2
     assert torch.all(cur == torch.minimum(before + room + 7, torch.full_like(cur, cap)))
+
+
+@pytest.mark.parametrize("batch,tokens,bs", [(1, 2048, 16), (2, 8200, 16), (3, 20011, 16), (2, 16390, 32)])   # 1, 2 and more blocks per warp
+def test_prefill_and_build_with_several_blocks_per_warp(batch, tokens, bs):
+    """Launches of one and of several waves: both give the plain means (fp32 sums of 16 to 64 bf16 rows in [-6, 6] err by less
+    than 64 * 6 * 2^-24, the stored pairs by 2^-18 of 6), and the prefill the same bits as the build."""
+    from paper_2609_26300_b200 import binding
+    hkv, pages = 8, -(-tokens // 64) * 4
+    gen = torch.Generator(device="cuda").manual_seed(tokens)
+    k_src, v_src = (torch.randn(batch, tokens, hkv, 128, generator=gen, device="cuda").clamp(-6, 6).bfloat16() for _ in range(2))
+    table = torch.randperm(batch * pages, generator=gen, device="cuda").int().view(batch, pages).contiguous()
+    pools = [torch.zeros(batch * pages, hkv, 16, 128, dtype=torch.bfloat16, device="cuda") for _ in range(2)]
+    ckv = binding.CompKV(32, hkv, batch, pages * 16 // bs, batch * pages, block_size=bs)
+    lens = torch.zeros(batch, dtype=torch.int32, device="cuda")
+    new = torch.full_like(lens, tokens)
+    new[-1] -= 5
+    ckv.prefill(pools[0], pools[1], table, lens, k_src, v_src, new, tokens)
+    got = [t.clone() for t in ckv.export_stats()]
+    ckv.stats_build(pools[0], pools[1], table, lens, tokens)
+    again = ckv.export_stats()
+    torch.cuda.synchronize()
+    assert torch.equal(lens, new) and ckv.read_status() == 0
+    for s in range(batch):
+        full, x = int(lens[s]) // bs, -(-int(lens[s]) // bs)
+        for a, b in zip(got, again):
+            assert torch.equal(a[s, :, :x], b[s, :, :x])
+        want = k_src[s, :full * bs].view(full, bs, hkv, 128).double().mean(1).transpose(0, 1)
+        assert float((got[0][s, :, :full].double() - want).abs().max()) <= 64 * 6 * 2.0 ** -24 + 6 * 2.0 ** -18
