@@ -22,15 +22,17 @@ template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile(
 
 // Start the copies of one page (k, v: its first row): 256 16-byte pieces per tile, 8 per lane; piece c of row r lands at
 // chunk c ^ (r & 7) of the row, so that the matrix loads below are conflict-free; rows at or past ntok are zero-filled.
+// A lane's rows lane / 16 + 2 i differ in their swizzle by an XOR with 2 i.
 __device__ __forceinline__ void issue_page(uint32_t kb, uint32_t vb, const __nv_bfloat16 *k, const __nv_bfloat16 *v, int ntok, int lane) {
+  const int r0 = lane >> 4, c = lane & 15;
+  const uint32_t at = (uint32_t)(r0 * kRowBytes + ((c ^ r0) << 4));
+  const __nv_bfloat16 *ks = k + r0 * CKV_D + 8 * c, *vs = v + r0 * CKV_D + 8 * c;
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
-    const int idx = lane + 32 * i, row = idx >> 4, c = idx & 15;
-    const uint32_t off = (uint32_t)(row * kRowBytes + ((c ^ (row & 7)) << 4));
-    const bool valid = row < ntok;
-    const size_t so = (size_t)(valid ? row : 0) * CKV_D + 8 * c;
-    cp_async16(kb + off, k + so, valid);
-    cp_async16(vb + off, v + so, valid);
+    const uint32_t off = (at ^ (uint32_t)(((2 * i) & 7) << 4)) + (uint32_t)(2 * i * kRowBytes);
+    const bool valid = r0 + 2 * i < ntok;   // (a copy of no bytes fills with zeros; its source is not read)
+    cp_async16(kb + off, ks + 2 * i * CKV_D, valid);
+    cp_async16(vb + off, vs + 2 * i * CKV_D, valid);
   }
 }
 
