@@ -608,7 +608,7 @@ def main():
         "dtype": DTYPE, "data": "synthetic",
         "config": {"workload": describe(w, is_default).replace("fp32 summaries", "bf16 summaries") if args.stat_bf16
                    else describe(w, is_default),
-                   "step": "ckv_step (summary scan with the new token's append in its tail CTAs, select, attention + merge: three launches) replayed as one CUDA graph; CUDA events around each replay",
+                   "step": "ckv_step (append, summary scan, selection, attention and merge of a unit by one thread-block cluster: one launch where the units fit a wave, else three) replayed as one CUDA graph; CUDA events around each replay",
                    "l2": "flushed between steps (256 MiB memset then 256 MiB read, outside the events); per-step inputs exceed L2",
                    "replicas": "every rank runs the whole workload (the path does not shard)",
                    "kv_storage": "bf16", "seed": w.seed},
@@ -633,8 +633,7 @@ def main():
         "stages_us": {"append": float(stage_us[0]), "scan": float(stage_us[1]), "select": float(stage_us[2]),
                       "attention": float(stage_us[3]), "merge": float(stage_us[4]),
                       "note": "the two-call route (ckv_append, then ckv_decode) launched eagerly with events between "
-                              "the kernels; in the timed ckv_step the append runs inside the scan launch, beside "
-                              "the scan CTAs, so its time does not add"},
+                              "the kernels; the timed ckv_step does the same work in one launch at this size"},
         "prefill": prefill,
         "stats_build": {"us": build_us, "gbs": build_bytes / (build_us * 1e-6) / 1e9, "bytes": build_bytes},
         "roofline": {"kernel": "ckv_scan_kernel", "bound": "hbm", "achieved": scan_gbs, "peak": peak,
