@@ -8,11 +8,14 @@
 // The scan kernel leaves, per head and block, u_{g,b} = log2(e^{l_{g,b}} sigma_hat^2_{g,b}) (4 bytes) and the
 // normalisers (M_g, L_g) as per-CTA partials, so S_b = sum_g 2^{u_{g,b} - M_g} / L_g and every term is read
 // once.  The normaliser loads are issued before the (much larger) batch of u loads, which would otherwise sit in
-// front of them in the memory pipeline.  The K-th largest score is found exactly with a most-significant-
-// digit-first radix select on the fp32 bit patterns (scores are >= 0, so unsigned order is numeric order): a
-// 4096-bin histogram of the top 12 bits, built while the scores are computed, then a direct ranking of the blocks
-// in the bin that holds the threshold (falling back to 12 + 8 more bits on heavy ties); ids come out in position
-// order from a prefix sum over selection flags.
+// front of them in the memory pipeline.  The K-th largest score is found exactly on the fp32 bit patterns (scores are
+// >= 0, so unsigned order is numeric order): a histogram built while the scores are computed, then a direct ranking of
+// the blocks in the bin that holds the threshold; ids come out in position order from a prefix sum over selection flags.
+// The histogram has 64 bins an octave over 64 octaves, which leaves the ranking a handful of blocks and the shared-memory
+// atomics few collisions: with the top 12 bits of the key (8 bins an octave) a step of 128 / 192 / 256 / 512 units took
+// 80.8 / 89.4 / 89.3 / 113.9 us, this way 80.3 / 87.5 / 87.5 / 111.8.  The ranking takes a bin of up to 1024 blocks whose
+// keys are in shared memory (24576 a unit); equal scores by the thousand and longer units go through radix passes of
+// 12, 12 and 8 bits.
 #include "ckv_internal.cuh"
 #include "ckv_pipe.cuh"
 
@@ -21,8 +24,11 @@ namespace {
 constexpr int kThreads = 1024;
 constexpr int kSmemKeys = 24576;   // keys cached in shared memory (96 KB); longer units re-read global scores
 constexpr int kBins = 4096;
+constexpr int kFineShift = 17;                  // the first histogram: 64 bins an octave ...
+constexpr int kFineBase = (127 - 54) << 6;      // ... from 2^-54 to 2^10; what lies outside goes into the end bins
 
-// Exclusive prefix sum of one int per thread over the CTA; *total receives the sum.
+// Exclusive prefix sum of one int per thread over the CTA; *total (if given) receives the sum.  A caller's next use of
+// the same warp_tot lies behind a barrier of its own.
 __device__ __forceinline__ int block_exclusive_scan(int v, int *warp_tot, int *total) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int inc = v;
@@ -42,12 +48,10 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int *warp_tot, int *t
       if (lane >= o) winc += t;
     }
     warp_tot[lane] = winc - w;
-    if (lane == 31) *total = winc;
+    if (total != nullptr && lane == 31) *total = winc;
   }
   __syncthreads();
-  const int res = warp_tot[warp] + inc - v;
-  __syncthreads();
-  return res;
+  return warp_tot[warp] + inc - v;
 }
 
 template <int G>
@@ -55,12 +59,11 @@ __global__ void __launch_bounds__(kThreads) ckv_select_kernel(CkvDev P, const in
                                                               int scan_grid, int units, int *__restrict__ sel_ids,
                                                               int *__restrict__ sel_cnt) {
   extern __shared__ uint32_t skeys[];
-  __shared__ int s_hist[kBins];
+  __shared__ __align__(16) int s_hist[kBins];
   __shared__ float s_M[G], s_invL[G];
-  __shared__ int s_wtot[32];
+  __shared__ int s_wtot[3][32];
   __shared__ int s_total, s_digit, s_remaining, s_ncand;
-  __shared__ int s_cand[kThreads];
-  __shared__ uint32_t s_candk[kThreads];   // the candidates' keys, so that the ranking loop reads no key through an id
+  __shared__ uint64_t s_cand[kThreads];   // (key, complement of the id): the larger one is ranked first
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int unit = blockIdx.x, s = ckv_div_hkv(P, unit);
@@ -135,8 +138,12 @@ __global__ void __launch_bounds__(kThreads) ckv_select_kernel(CkvDev P, const in
   if (P.sink + n_tail > X) nF = X;
   const int Kr = K - nF;   // blocks to rank in (the host guarantees K >= sink + recent when K < X)
   if (tid == 0) { s_remaining = Kr; s_total = 0; }   // read after the barrier that follows the scoring loop
-  const bool hist0 = X > kcap && Kr > 0;   // the first radix pass (top 12 bits of every ranked key) is built on the fly
+  const bool hist0 = X > kcap && Kr > 0;   // the first histogram is built on the fly
   const bool cached = X <= kSmemKeys;
+  // keys at hand are ranked in the bin that holds the threshold, by a fine histogram; units too long for that take the
+  // radix passes, of which the first (top 12 bits) is this histogram
+  const int shift0 = cached ? kFineShift : 20, base0 = cached ? kFineBase : 0;
+  auto bin0 = [shift0, base0](uint32_t k) { return min(max((int)(k >> shift0) - base0, 0), kBins - 1); };
   bool nonfinite = false;
   for (int base = 0; base < X; base += NB * kThreads) {
     if (base > 0) load_batch(base);
@@ -150,7 +157,7 @@ __global__ void __launch_bounds__(kThreads) ckv_select_kernel(CkvDev P, const in
         if (!(sc >= 0.f) || sc > 3.0e38f) { nonfinite = true; sc = 0.f; }
         scores[b] = sc;
         if (cached) skeys[b] = __float_as_uint(sc);
-        if (hist0 && !mandatory(b)) atomicAdd(&s_hist[__float_as_uint(sc) >> 20], 1);
+        if (hist0 && !mandatory(b)) atomicAdd(&s_hist[bin0(__float_as_uint(sc))], 1);
       }
     }
   }
@@ -160,103 +167,94 @@ __global__ void __launch_bounds__(kThreads) ckv_select_kernel(CkvDev P, const in
 
   const uint32_t *keys = cached ? skeys : reinterpret_cast<const uint32_t *>(scores);
 
-  // ---- the Kr-th largest ranked score: one 12-bit radix pass, then either a direct ranking of the blocks in the
-  //      digit bin that holds it (the usual case: a few dozen blocks) or the remaining radix passes ----
-  uint32_t prefix = 0, pmask = 0;
-  int eq_total = 0;   // blocks scoring exactly the threshold (radix path)
-  bool ranked = false;   // direct-ranking path taken: chosen blocks carry the sign bit in skeys
-  if (Kr > 0) {
-#pragma unroll 1
-    for (int pass = 0; pass < 3; ++pass) {
-      const int shift = pass == 0 ? 20 : (pass == 1 ? 8 : 0);
-      const int bins = pass == 2 ? 256 : kBins;
-      if (pass > 0) {   // pass 0's histogram was built while the scores were computed
-        for (int i = tid; i < bins; i += kThreads) s_hist[i] = 0;
-        __syncthreads();
-        for (int b = tid; b < X; b += kThreads) {
-          if (mandatory(b)) continue;
-          const uint32_t k = keys[b];
-          if ((k & pmask) == prefix) atomicAdd(&s_hist[(k >> shift) & (bins - 1)], 1);
-        }
-        __syncthreads();
-      }
-      // thread t owns the four bins bins-1-4t ... bins-4-4t (highest digits first)
-      int c[4], c4 = 0;
+  // ---- the Kr-th largest ranked score: the bin that holds it, then either a direct ranking of the blocks in that bin
+  //      (the usual case: a few dozen blocks) or radix passes of 12, 12 and 8 bits ----
+  uint32_t prefix = 0, floor_key = 0;
+  int eq_total = 0;      // blocks scoring exactly the threshold (radix path)
+  bool direct = false;   // direct-ranking path taken: chosen blocks carry the sign bit in skeys
+  // The bin (of `bins`, largest digits first) that holds the s_remaining-th key -> s_digit; its count -> s_total; how many
+  // of it are taken -> s_remaining.
+  auto find_digit = [&](int bins) {
+    int c[4] = {0, 0, 0, 0};   // thread t owns the four bins bins-1-4t ... bins-4-4t
+    if (4 * tid < bins) {
+      const int4 x = *reinterpret_cast<const int4 *>(s_hist + bins - 4 - 4 * tid);
+      c[0] = x.w; c[1] = x.z; c[2] = x.y; c[3] = x.x;
+    }
+    const int c4 = (c[0] + c[1]) + (c[2] + c[3]);
+    const int remaining = s_remaining;
+    int before = block_exclusive_scan(c4, s_wtot[0], nullptr);   // keys with a higher digit than this thread's bins
+    if (before < remaining && before + c4 >= remaining) {
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const int bin = bins - 1 - 4 * tid - j;
-        c[j] = bin >= 0 ? s_hist[bin] : 0;
-        c4 += c[j];
-      }
-      const int remaining = s_remaining;
-      int before = block_exclusive_scan(c4, s_wtot, &s_total);   // keys with a higher digit than this thread's bins
-      if (before < remaining && before + c4 >= remaining) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          if (before < remaining && before + c[j] >= remaining) {
-            s_digit = bins - 1 - 4 * tid - j;
-            s_remaining = remaining - before;
-            s_total = c[j];
-            before = remaining;   // stop
-          } else {
-            before += c[j];
-          }
+        if (before < remaining && before + c[j] >= remaining) {
+          s_digit = bins - 1 - 4 * tid - j;
+          s_remaining = remaining - before;
+          s_total = c[j];
+          before = remaining;   // stop
+        } else {
+          before += c[j];
         }
       }
+    }
+    __syncthreads();
+  };
+  if (Kr > 0) {
+    find_digit(kBins);
+    direct = cached && s_total <= kThreads;
+    if (direct) {   // rank the bin's blocks by (score descending, id ascending) and mark the first `take`
+      const int digit = s_digit, take = s_remaining, nc = s_total;
+      for (int b = tid; b < X; b += kThreads) {
+        const uint32_t k = skeys[b];
+        if (bin0(k) == digit && !mandatory(b)) s_cand[atomicAdd(&s_ncand, 1)] = (uint64_t)k << 32 | (uint32_t)~b;
+      }
       __syncthreads();
-      prefix |= (uint32_t)s_digit << shift;
-      pmask |= (uint32_t)(bins - 1) << shift;
-      eq_total = s_total;
-      const int take = s_remaining;
-      __syncthreads();
-      if (pass == 0 && cached && eq_total <= kThreads) {
-        // rank the bin's blocks by (score descending, id ascending) and mark the first `take`
-        for (int b = tid; b < X; b += kThreads) {
-          if (mandatory(b)) continue;
-          const uint32_t k = keys[b];
-          if ((k & pmask) == prefix) {
-            const int slot = atomicAdd(&s_ncand, 1);
-            s_cand[slot] = b;
-            s_candk[slot] = k;
-          }
-        }
-        __syncthreads();
-        const int nc = s_ncand;
-        bool chosen = false;
-        int myb = -1;
-        if (tid < nc) {
-          myb = s_cand[tid];
-          const uint32_t mk = s_candk[tid];
-          int rank = 0;
+      if (tid < nc) {
+        const uint64_t mine = s_cand[tid];
+        int rank = 0;
 #pragma unroll 8
-          for (int j = 0; j < nc; ++j) {
-            const int ob = s_cand[j];
-            const uint32_t ok = s_candk[j];
-            rank += (ok > mk || (ok == mk && ob < myb)) ? 1 : 0;
-          }
-          chosen = rank < take;
-        }
-        __syncthreads();   // every rank is computed before any key is marked
-        if (chosen) skeys[myb] |= 0x80000000u;
-        __syncthreads();
-        ranked = true;
-        break;
+        for (int j = 0; j < nc; ++j) rank += s_cand[j] > mine ? 1 : 0;
+        if (rank < take) skeys[~(uint32_t)mine] |= 0x80000000u;
       }
+      // a marked key carries the sign bit and a key of a higher bin is at least the first of the next: both are >= this
+      floor_key = digit == kBins - 1 ? 0x80000000u : (uint32_t)(kFineBase + digit + 1) << kFineShift;
+      __syncthreads();
+    } else {
+      __syncthreads();   // everyone has read s_total
+      if (cached && tid == 0) s_remaining = Kr;
+      uint32_t pmask = 0;
+#pragma unroll 1
+      for (int pass = 0; pass < 3; ++pass) {
+        const int shift = pass == 0 ? 20 : (pass == 1 ? 8 : 0);
+        const int bins = pass == 2 ? 256 : kBins;
+        if (cached || pass > 0) {   // the first histogram was this one's if the unit is too long for the fine one
+          for (int i = tid; i < bins; i += kThreads) s_hist[i] = 0;
+          __syncthreads();
+          for (int b = tid; b < X; b += kThreads) {
+            if (mandatory(b)) continue;
+            const uint32_t k = keys[b];
+            if ((k & pmask) == prefix) atomicAdd(&s_hist[(k >> shift) & (bins - 1)], 1);
+          }
+          __syncthreads();
+          find_digit(bins);
+        }
+        prefix |= (uint32_t)s_digit << shift;
+        pmask |= (uint32_t)(bins - 1) << shift;
+      }
+      eq_total = s_total;
     }
   }
   const uint32_t thr = prefix;          // radix path: bit pattern of the Kr-th largest ranked score
   const int need_eq = s_remaining;      // ... and how many blocks scoring exactly thr are taken (lowest ids first)
-  const uint32_t digit0 = prefix >> 20; // ranking path: the 12-bit digit of the bin that was ranked
 
   // ---- ordered emission: thread t owns a contiguous range of blocks (odd length: conflict-free smem reads) ----
   const int per = ((X + kThreads - 1) / kThreads) | 1;
   const int b0 = min(tid * per, X), b1 = min(b0 + per, X);
   int eq_rank = 0;
   const bool all_eq = need_eq >= eq_total;   // every block at the threshold is taken: no rank among ties needed
-  if (Kr > 0 && !ranked && !all_eq) {
+  if (Kr > 0 && !direct && !all_eq) {
     int c_eq = 0;
     for (int b = b0; b < b1; ++b) c_eq += (!mandatory(b) && keys[b] == thr) ? 1 : 0;
-    eq_rank = block_exclusive_scan(c_eq, s_wtot, &s_total);
+    eq_rank = block_exclusive_scan(c_eq, s_wtot[1], nullptr);
   }
   auto walk = [&](auto &&emit) {   // calls emit(b) for every selected block of this thread's range, in order
     int e = eq_rank;
@@ -264,8 +262,8 @@ __global__ void __launch_bounds__(kThreads) ckv_select_kernel(CkvDev P, const in
       bool sel = mandatory(b);
       if (!sel && Kr > 0) {
         const uint32_t k = keys[b];
-        if (ranked) {
-          sel = (k & 0x80000000u) != 0 || (k >> 20) > digit0;
+        if (direct) {
+          sel = k >= floor_key;
         } else if (k > thr) {
           sel = true;
         } else if (k == thr) {
@@ -280,10 +278,7 @@ __global__ void __launch_bounds__(kThreads) ckv_select_kernel(CkvDev P, const in
   int c_sel = 0;
   uint32_t picked = 0;
   const bool masked = per <= 32;
-  if (ranked && cached && masked) {
-    // the usual case in one comparison per key: marked keys carry the sign bit and every key of a higher bin is at
-    // least (digit + 1) << 20, so "selected" is an unsigned >= ; mandatory blocks only matter at the two ends
-    const uint32_t floor_key = (digit0 + 1u) << 20;
+  if (direct && masked) {   // the usual case in one comparison per key: mandatory blocks only matter at the two ends
     const bool ends = b0 < P.sink || b1 > X - n_tail;
     for (int b = b0; b < b1; ++b) {
       const bool sel = skeys[b] >= floor_key || (ends && mandatory(b));
@@ -293,7 +288,7 @@ __global__ void __launch_bounds__(kThreads) ckv_select_kernel(CkvDev P, const in
   } else {
     walk([&](int b) { ++c_sel; if (masked) picked |= 1u << (b - b0); });
   }
-  int pos = block_exclusive_scan(c_sel, s_wtot, &s_total);
+  int pos = block_exclusive_scan(c_sel, s_wtot[2], &s_total);
   const int total = s_total;
   if (masked) {
     while (picked != 0) {
