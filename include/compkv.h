@@ -71,7 +71,9 @@ enum ckv_device_status {
   CKV_DEV_SEQ_FULL = 2,     /* append past max_blocks_per_seq * block_size: the token was dropped */
   CKV_DEV_NONFINITE = 4,    /* a block score was NaN/Inf: it was ranked as 0 */
   CKV_DEV_TIMEOUT = 8,      /* a bounded wait inside a kernel ran out: the step's results are invalid */
-  CKV_DEV_BAD_COPY = 16     /* a kernel refused to issue a bulk copy whose arguments failed its checks */
+  CKV_DEV_BAD_COPY = 16,    /* a kernel refused to issue a bulk copy whose arguments failed its checks */
+  CKV_DEV_BAD_BOUND = 32    /* a sequence is longer than max_seq_len_host said, and the step was sized for no more: its
+                               cache, summaries and length are right, its result covers the blocks within the bound */
 };
 
 /* Bits of ckv_layout.variant: the scorer / merge ablations of Sec. 5.3 and App. A.6.  0 is the method as printed. */

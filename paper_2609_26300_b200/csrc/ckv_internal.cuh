@@ -74,7 +74,7 @@ struct CkvStepPlan {
   int stages;       // ring stages of the scan phase
   int own_cap;      // blocks of a unit one CTA owns, at most (a multiple of 16)
   int u_off, smem;  // offset of the score terms in dynamic shared memory, and its size
-  int max_blocks;   // blocks of a sequence by the host's bound on the lengths
+  int max_blocks;   // blocks of a sequence the step can work on (the capacity, or the host's bound on the lengths)
 };
 
 struct ckv_ctx {

@@ -151,7 +151,11 @@ __device__ __noinline__ void tail_block(const CkvDev P, const bf16 *q_rows, cons
 #pragma unroll
   for (int g = 0; g < G; ++g) qr[g] = __ldg(reinterpret_cast<const uint4 *>(q_rows + (size_t)g * CKV_D) + li);
   const int b = ((N + P.bs - 1) >> P.lg_bs) - 1, cnt = N - b * P.bs;
-  const size_t row = (size_t)unit * P.max_blocks + b;
+  // the block the token lands in: the last one, unless the sequence has outgrown the host's bound -- then its summary is
+  // kept up to date all the same, and the block whose terms are wanted is one that the step does not change
+  const int ab = append ? raw >> P.lg_bs : b, acnt = append ? raw + 1 - ab * P.bs : cnt;
+  const bool past = append && raw + 1 > N;
+  const size_t row = (size_t)unit * P.max_blocks + ab;
   __nv_bfloat16 *kmean_row = P.kmean + row * P.row_elems, *vmean_row = P.vmean + row * P.row_elems;
   float *dbar_row = P.dbar + row * P.r;
   BlockRow br;
@@ -160,34 +164,38 @@ __device__ __noinline__ void tail_block(const CkvDev P, const bf16 *q_rows, cons
     const bool ok = phys >= 0 && phys < P.num_pages;
     const size_t base = ok ? ((size_t)phys * P.Hkv + h) * CKV_PAGE * CKV_D + 8 * li : 0;
     const size_t at = base + (size_t)(raw % CKV_PAGE) * CKV_D;
-    if (cnt <= CKV_PAGE) {   // the token's page is all there is of its block
+    if (acnt <= CKV_PAGE) {   // the token's page is all there is of its block
       uint4 kraw[8], vraw[8];
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
         const int t = hw + 2 * j;
         kraw[j] = kn; vraw[j] = vn;
-        if (ok && t < cnt - 1) {
+        if (ok && t < acnt - 1) {
           kraw[j] = *reinterpret_cast<const uint4 *>(kp + base + (size_t)t * CKV_D);
           vraw[j] = *reinterpret_cast<const uint4 *>(vp + base + (size_t)t * CKV_D);
         }
       }
       if (ok) *reinterpret_cast<uint4 *>((hw == 0 ? kp : vp) + at) = hw == 0 ? kn : vn;
       float km[8], vs[8], ssq[8];
-      block_stats_rows16(kraw, vraw, ok, cnt, lane, km, vs, ssq);
-      block_stats_finish(P, b, (float)cnt, km, vs, ssq, sq, kmean_row, dbar_row, vmean_row, lane, !ok, &br);
+      block_stats_rows16(kraw, vraw, ok, acnt, lane, km, vs, ssq);
+      block_stats_finish(P, ab, (float)acnt, km, vs, ssq, sq, kmean_row, dbar_row, vmean_row, lane, !ok, &br);
     } else {
       if (ok) *reinterpret_cast<uint4 *>((hw == 0 ? kp : vp) + at) = hw == 0 ? kn : vn;
       __syncwarp();
-      block_stats_warp<bf16, false>(P, kp, vp, pt_row, h, b, cnt, sq, kmean_row, dbar_row, vmean_row, lane, &br);
+      block_stats_warp<bf16, false>(P, kp, vp, pt_row, h, ab, acnt, sq, kmean_row, dbar_row, vmean_row, lane, &br);
     }
-  } else {   // the summary as stored: lower half warp the mean key, upper the mean value (as the scan reads it)
-    if (fresh.k_new != nullptr && lane == 0) atomicOr(P.status, CKV_DEV_SEQ_FULL);
-    load_split8<false>(hw == 0 ? kmean_row : vmean_row, li, b, br.x, lo_half && !(hw == 1 && P.vhi));
+  } else if (fresh.k_new != nullptr && lane == 0) {
+    atomicOr(P.status, CKV_DEV_SEQ_FULL);
+  }
+  if (!append || past) {   // the summary as stored: lower half warp the mean key, upper the mean value (as the scan reads it)
+    const size_t r0 = (size_t)unit * P.max_blocks + b;
+    load_split8<false>((hw == 0 ? P.kmean : P.vmean) + r0 * P.row_elems, li, b, br.x, lo_half && !(hw == 1 && P.vhi));
+    const float *drow = P.dbar + r0 * P.r;
     if (P.r == CKV_D) {
-      load_split8<false>(reinterpret_cast<const bf16 *>(dbar_row), li, b, br.dvar);
+      load_split8<false>(reinterpret_cast<const bf16 *>(drow), li, b, br.dvar);
     } else {
 #pragma unroll
-      for (int i = 0; i < 8; ++i) br.dvar[i] = dbar_row[group_of(8 * li + i, P.r, P.glayout)];
+      for (int i = 0; i < 8; ++i) br.dvar[i] = drow[group_of(8 * li + i, P.r, P.glayout)];
     }
   }
   // sums over the 16 lanes of a half warp, d_0 .. d_{G-1}, sigma^2_0 .. sigma^2_{G-1} (the d of the lower half count: it holds the mean key)
@@ -281,8 +289,10 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *__restrict__ q, const int *seq_lens, 
   if (tid >= kThreads - 32) reinterpret_cast<uint4 *>(s_zero_row)[lane] = make_uint4(0u, 0u, 0u, 0u);
   const bool dbar_bulk = P.r >= 4;
   const int stage_bytes = TB * (kRowBytesK + kRowBytesV) + (dbar_bulk ? TB * P.r * 4 : 0);
-  // the length the step works on; a bound the host misjudged is kept to what the shared arrays were sized for
-  const int N = max(min(min(raw + ((append && raw >= 0 && raw < cap) ? 1 : 0), cap), plan.max_blocks * P.bs), 0);
+  // the length the step works on; of a sequence longer than the host's bound, what the shared arrays were sized for
+  const int N_all = max(min(raw + ((append && raw >= 0 && raw < cap) ? 1 : 0), cap), 0);
+  const int N = min(N_all, plan.max_blocks * P.bs);
+  if (N < N_all && rank == 0 && tid == 0) atomicOr(P.status, CKV_DEV_BAD_BOUND);
   const int X = (N + P.bs - 1) >> P.lg_bs, Xs = max(X - 1, 0);
   const int n_parts = (Xs + 15) >> 4;
   const int ppc = (int)ckv_udiv24((unsigned)(n_parts + C - 1), (unsigned)C);
@@ -983,16 +993,23 @@ bool ckv_unit_step_plan(const ckv_ctx *c, int batch, int max_len, int kcap, CkvS
   const int skip = kWarps / (P.scan_tile / 16);
   const size_t krow = (size_t)P.row_elems * 2, vrow = (P.vhi || P.row_elems == CKV_D) ? (size_t)CKV_D * 2 : krow;
   const size_t stage = (size_t)P.scan_tile * (krow + vrow) + (P.r >= 4 ? (size_t)P.scan_tile * P.r * 4 : 0);
-  const int parts = (std::max(xmax - 1, 0) + 15) / 16;
-  plan->own_cap = 16 * std::max((parts + C - 1) / C, 1);
-  const size_t u_bytes = (size_t)(plan->own_cap + 8) * P.G * sizeof(float);
-  if (u_bytes + (size_t)std::max(kMinRing, skip) * stage > (size_t)kDynLimit) return false;
+  auto blocks_per_cta = [C](int x) { const int parts = (std::max(x - 1, 0) + 15) / 16; return 16 * std::max((parts + C - 1) / C, 1); };
+  auto term_bytes = [&P](int own) { return (size_t)(own + 8) * P.G * sizeof(float); };
+  plan->own_cap = blocks_per_cta(xmax);
+  if (term_bytes(plan->own_cap) + (size_t)std::max(kMinRing, skip) * stage > (size_t)kDynLimit) return false;
   const int tiles = (plan->own_cap + P.scan_tile - 1) / P.scan_tile;
-  plan->stages = std::min({kStagesCap, (int)(((size_t)kDynLimit - u_bytes) / stage), std::max(tiles, skip)});
+  plan->stages = std::min({kStagesCap, (int)(((size_t)kDynLimit - term_bytes(plan->own_cap)) / stage), std::max(tiles, skip)});
   plan->u_off = (int)(plan->stages * stage);
-  plan->smem = (int)std::max((size_t)plan->u_off + u_bytes, (size_t)kAfterScan);
-  plan->cluster = C;
   plan->max_blocks = xmax;
+  // Where the arrays can be sized for the cache's capacity beside the same ring, they are: a bound that turns out too small
+  // (a captured step replayed once too often) then costs nothing.
+  const int full = blocks_per_cta(P.max_blocks);
+  if (P.max_blocks <= kScoresCap && (kcap >= P.max_blocks || kcap <= kSelCap) && plan->u_off + term_bytes(full) <= (size_t)kDynLimit) {
+    plan->own_cap = full;
+    plan->max_blocks = P.max_blocks;
+  }
+  plan->smem = (int)std::max(plan->u_off + term_bytes(plan->own_cap), (size_t)kAfterScan);
+  plan->cluster = C;
   return true;
 }
 

@@ -103,6 +103,54 @@ def test_an_empty_and_a_full_sequence():
     assert int(d.lens[0]) == cap and d.ckv.read_status() & binding.CKV_DEV_SEQ_FULL
 
 
+def with_capacity(d, max_blocks):
+    """The same cache behind page-table rows, summaries and a context for `max_blocks` blocks a sequence."""
+    w, pages = d.w, max_blocks * d.w.block_size // 16
+    table = torch.full((w.batch, pages), -1, dtype=torch.int32, device="cuda")
+    table[:, :d.table.shape[1]] = d.table
+    d.table = table
+    d.ckv = binding.CompKV(w.num_q_heads, w.num_kv_heads, w.batch, max_blocks, d.k_pool.shape[0], block_size=w.block_size)
+    return d
+
+
+@pytest.mark.parametrize("bs,over", [(16, 1), (16, 17), (64, 1), (64, 21)])
+@pytest.mark.parametrize("tight", [False, True])
+def test_a_length_bound_that_is_too_small(bs, over, tight):
+    """Lengths `over` tokens past what the host says.  Where the capacity fits the step's shared memory the bound makes no
+    difference; where it does not (eight heads, one CTA a unit, 57 344 tokens and more) the step says so, and pages,
+    summaries and lengths are still those of ckv_append."""
+    bound = 16 * 112
+    batch, hq = (10, 64) if tight else (2, 8)
+    hkv = hq // 8 if tight else 2
+    w = workload(batch=batch, num_q_heads=hq, num_kv_heads=hkv, ctx=bound + over - 1, ctx_min=bound + over - 1, block_size=bs,
+                 budget_tokens=bs * 8, needles=1, decode_steps=2)
+    blocks = 64 * 1024 // bs if tight else 2048 // bs
+    if tight and bs == 64:
+        blocks = 4096   # the shared memory counts blocks: 262 144 tokens
+    a, b = (with_capacity(setup(w), blocks) for _ in range(2))
+    for d in (a, b):
+        d.ckv.stats_build(d.k_pool, d.v_pool, d.table, d.lens, w.ctx)
+    for t, max_len in enumerate((bound, w.ctx + 2)):   # the second step gets a right bound
+        q, kn, vn = step_inputs(a, t)
+        before = a.ckv.launch_count()
+        got = a.ckv.step(q, kn, vn, a.k_pool, a.v_pool, a.table, a.lens, max_len, w.budget_tokens)
+        assert a.ckv.launch_count() - before == 1
+        b.ckv.append(b.k_pool, b.v_pool, b.table, b.lens, kn, vn)
+        want = b.ckv.decode(q, b.k_pool, b.v_pool, b.table, b.lens, w.ctx + 2, w.budget_tokens)
+        torch.cuda.synchronize()
+        assert a.ckv.read_status() == (binding.CKV_DEV_BAD_BOUND if tight and t == 0 else 0) and b.ckv.read_status() == 0
+        assert torch.equal(a.lens, b.lens)
+        for x, y in zip(a.ckv.export_stats(), b.ckv.export_stats()):
+            assert torch.equal(x, y)
+        for x, y in ((a.k_pool, b.k_pool), (a.v_pool, b.v_pool)):
+            assert torch.equal(x.view(torch.int16), y.view(torch.int16))
+        if not (tight and t == 0):
+            for x, y in zip(got, want):
+                assert torch.equal(x, y)
+        else:   # what the bound covers: every id a block of it
+            assert int(got[2].max()) < bound // bs and bool(torch.isfinite(got[0].float()).all())
+
+
 @pytest.mark.parametrize("copies", [1, 3])
 def test_ties_at_the_cut_take_the_lowest_ids(copies):
     """All pages hold one of `copies` contents: the cut falls among hundreds of equal scores, more than the direct ranking
