@@ -138,7 +138,7 @@ __device__ __noinline__ void tail_block(const CkvDev P, const bf16 *q_rows, cons
   const bool lo_half = P.row_elems == CKV_ROW_ELEMS;
   const bool by_mass = (P.variant & CKV_VARIANT_RANK_BY_MASS) != 0;
   const int *pt_row = page_table + (size_t)s * P.max_pages_per_seq;
-  const bool append = fresh.k_new != nullptr && raw >= 0 && raw < cap;
+  const bool append = fresh.k_new != nullptr && raw + 1 == N;   // (past the host's bound: see append_past_bound)
   int phys = -1;
   uint4 kn, vn;   // this lane's eight coordinates of the new rows
   kn = vn = make_uint4(0u, 0u, 0u, 0u);
@@ -151,11 +151,7 @@ __device__ __noinline__ void tail_block(const CkvDev P, const bf16 *q_rows, cons
 #pragma unroll
   for (int g = 0; g < G; ++g) qr[g] = __ldg(reinterpret_cast<const uint4 *>(q_rows + (size_t)g * CKV_D) + li);
   const int b = ((N + P.bs - 1) >> P.lg_bs) - 1, cnt = N - b * P.bs;
-  // the block the token lands in: the last one, unless the sequence has outgrown the host's bound -- then its summary is
-  // kept up to date all the same, and the block whose terms are wanted is one that the step does not change
-  const int ab = append ? raw >> P.lg_bs : b, acnt = append ? raw + 1 - ab * P.bs : cnt;
-  const bool past = append && raw + 1 > N;
-  const size_t row = (size_t)unit * P.max_blocks + ab;
+  const size_t row = (size_t)unit * P.max_blocks + b;
   __nv_bfloat16 *kmean_row = P.kmean + row * P.row_elems, *vmean_row = P.vmean + row * P.row_elems;
   float *dbar_row = P.dbar + row * P.r;
   BlockRow br;
@@ -164,38 +160,34 @@ __device__ __noinline__ void tail_block(const CkvDev P, const bf16 *q_rows, cons
     const bool ok = phys >= 0 && phys < P.num_pages;
     const size_t base = ok ? ((size_t)phys * P.Hkv + h) * CKV_PAGE * CKV_D + 8 * li : 0;
     const size_t at = base + (size_t)(raw % CKV_PAGE) * CKV_D;
-    if (acnt <= CKV_PAGE) {   // the token's page is all there is of its block
+    if (cnt <= CKV_PAGE) {   // the token's page is all there is of its block
       uint4 kraw[8], vraw[8];
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
         const int t = hw + 2 * j;
         kraw[j] = kn; vraw[j] = vn;
-        if (ok && t < acnt - 1) {
+        if (ok && t < cnt - 1) {
           kraw[j] = *reinterpret_cast<const uint4 *>(kp + base + (size_t)t * CKV_D);
           vraw[j] = *reinterpret_cast<const uint4 *>(vp + base + (size_t)t * CKV_D);
         }
       }
       if (ok) *reinterpret_cast<uint4 *>((hw == 0 ? kp : vp) + at) = hw == 0 ? kn : vn;
       float km[8], vs[8], ssq[8];
-      block_stats_rows16(kraw, vraw, ok, acnt, lane, km, vs, ssq);
-      block_stats_finish(P, ab, (float)acnt, km, vs, ssq, sq, kmean_row, dbar_row, vmean_row, lane, !ok, &br);
+      block_stats_rows16(kraw, vraw, ok, cnt, lane, km, vs, ssq);
+      block_stats_finish(P, b, (float)cnt, km, vs, ssq, sq, kmean_row, dbar_row, vmean_row, lane, !ok, &br);
     } else {
       if (ok) *reinterpret_cast<uint4 *>((hw == 0 ? kp : vp) + at) = hw == 0 ? kn : vn;
       __syncwarp();
-      block_stats_warp<bf16, false>(P, kp, vp, pt_row, h, ab, acnt, sq, kmean_row, dbar_row, vmean_row, lane, &br);
+      block_stats_warp<bf16, false>(P, kp, vp, pt_row, h, b, cnt, sq, kmean_row, dbar_row, vmean_row, lane, &br);
     }
-  } else if (fresh.k_new != nullptr && lane == 0) {
-    atomicOr(P.status, CKV_DEV_SEQ_FULL);
-  }
-  if (!append || past) {   // the summary as stored: lower half warp the mean key, upper the mean value (as the scan reads it)
-    const size_t r0 = (size_t)unit * P.max_blocks + b;
-    load_split8<false>((hw == 0 ? P.kmean : P.vmean) + r0 * P.row_elems, li, b, br.x, lo_half && !(hw == 1 && P.vhi));
-    const float *drow = P.dbar + r0 * P.r;
+  } else {   // the summary as stored: lower half warp the mean key, upper the mean value (as the scan reads it)
+    if (fresh.k_new != nullptr && raw >= cap && lane == 0) atomicOr(P.status, CKV_DEV_SEQ_FULL);
+    load_split8<false>(hw == 0 ? kmean_row : vmean_row, li, b, br.x, lo_half && !(hw == 1 && P.vhi));
     if (P.r == CKV_D) {
-      load_split8<false>(reinterpret_cast<const bf16 *>(drow), li, b, br.dvar);
+      load_split8<false>(reinterpret_cast<const bf16 *>(dbar_row), li, b, br.dvar);
     } else {
 #pragma unroll
-      for (int i = 0; i < 8; ++i) br.dvar[i] = drow[group_of(8 * li + i, P.r, P.glayout)];
+      for (int i = 0; i < 8; ++i) br.dvar[i] = dbar_row[group_of(8 * li + i, P.r, P.glayout)];
     }
   }
   // sums over the 16 lanes of a half warp, d_0 .. d_{G-1}, sigma^2_0 .. sigma^2_{G-1} (the d of the lower half count: it holds the mean key)
@@ -228,6 +220,25 @@ __device__ __noinline__ void tail_block(const CkvDev P, const bf16 *q_rows, cons
     tail_part[lane * CKV_PART_STRIDE] = zl2;
     tail_part[lane * CKV_PART_STRIDE + 1] = 1.f;
   }
+}
+
+// The append of a sequence that has outgrown the host's bound: the token lands in a block that the step does not look at,
+// whose summary is kept up to date all the same.
+__device__ __noinline__ void append_past_bound(const CkvDev P, const int *page_table, const CkvNewToken fresh, int unit, int raw, float *sq) {
+  const int lane = threadIdx.x & 31, hw = lane >> 4, li = lane & 15;
+  const int s = ckv_div_hkv(P, unit), h = unit - s * P.Hkv;
+  const int *pt_row = page_table + (size_t)s * P.max_pages_per_seq;
+  bf16 *kp = reinterpret_cast<bf16 *>(fresh.k_pool), *vp = reinterpret_cast<bf16 *>(fresh.v_pool);
+  const int phys = pt_row[raw / CKV_PAGE], b = raw >> P.lg_bs;
+  if (phys >= 0 && phys < P.num_pages) {
+    const bf16 *src = reinterpret_cast<const bf16 *>(hw == 0 ? fresh.k_new : fresh.v_new) + (size_t)unit * CKV_D + 8 * li;
+    bf16 *dst = (hw == 0 ? kp : vp) + (((size_t)phys * P.Hkv + h) * CKV_PAGE + raw % CKV_PAGE) * CKV_D + 8 * li;
+    *reinterpret_cast<uint4 *>(dst) = *reinterpret_cast<const uint4 *>(src);
+  }
+  __syncwarp();
+  const size_t row = (size_t)unit * P.max_blocks + b;
+  block_stats_warp<bf16, false>(P, kp, vp, pt_row, h, b, raw + 1 - b * P.bs, sq, P.kmean + row * P.row_elems, P.dbar + row * P.r,
+                                P.vmean + row * P.row_elems, lane);
 }
 
 // The last cluster to have read the lengths stores the new ones (nobody waits: it is a counter).
@@ -369,6 +380,7 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *__restrict__ q, const int *seq_lens, 
         asm volatile("prefetch.global.L2 [%0];" ::"l"(pt + 32 * i) : "memory");
     }
   } else if (warp == kTailWarp) {
+    if (rank == C - 1 && append && raw >= N && raw < cap) append_past_bound(P, page_table, fresh, unit, raw, s_sq);
     if (rank == C - 1 && N > 0)
       tail_block<G>(P, q + (size_t)unit * G * CKV_D, page_table, fresh, unit, raw, N, s_sq, s_tail_u, &s_tail_part[0][0], s_wn[kWarps]);
     else if (lane < G)
