@@ -316,6 +316,8 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *__restrict__ q, const int *seq_lens, 
   float *ub = reinterpret_cast<float *>(smem + plan.u_off);
   const int us = plan.own_cap + 8;
 
+  // test hook (ckv_debug_set): one fill is announced but never issued, so that the waits on it run out
+  auto withheld = [&](int it) { return (P.debug & CKV_DEBUG_SKIP_FILL) != 0 && it == 0 && rank == 0 && unit == 0; };
   // one fill of the ring: tile `it` into stage `st`, counted on full barrier `fb`
   auto fill = [&](int it, int st, uint64_t *fb) {
     const int nb = min(TB, own - it * TB);
@@ -328,9 +330,7 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *__restrict__ q, const int *seq_lens, 
     mbar_arrive_expect_tx(fb, kbytes + vbytes + dbytes);
     const uint32_t lo = smem_u32(smem), hi = lo + (uint32_t)plan.stages * stage_bytes;
     bool ok = nb >= 1 && b_lo + it * TB + nb <= P.max_blocks;
-    // test hook (ckv_debug_set): one fill is announced but never issued, so that the waits on it run out
-    const bool skip = (P.debug & CKV_DEBUG_SKIP_FILL) != 0 && it == 0 && rank == 0 && unit == 0;
-    if (!skip) {
+    if (!withheld(it)) {
       ok = ok && bulk_g2s_checked(sk, P.kmean + row * P.row_elems, kbytes, fb, lo, hi);
       if constexpr (VH) {
         // rows [row, row + TB) of the mean-values region, first 256 bytes of each (rows past the range are never read)
@@ -342,7 +342,7 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *__restrict__ q, const int *seq_lens, 
         ok = ok && bulk_g2s_checked(sv, P.vmean + row * P.row_elems, vbytes, fb, lo, hi);
       }
       if (dbar_bulk) ok = ok && bulk_g2s_checked(sv + TB * kRowBytesV, P.dbar + row * P.r, dbytes, fb, lo, hi);
-      }
+    }
     if (!ok) atomicOr(P.status, CKV_DEV_BAD_COPY);
   };
   // The tail warp does not wait here: it needs nothing that the others set up, and the cluster will wait for it.
@@ -465,7 +465,7 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *__restrict__ q, const int *seq_lens, 
   if (s_abort) {     // leave no copy in flight into memory that is about to be reused: wait (bounded) for every issued fill
     if (tid == 0)
       for (int it = max(s_issued - plan.stages, 0); it < s_issued; ++it)
-        mbar_wait(&full_bar[(it / plan.stages) & 1][it % plan.stages], ((it / plan.stages) >> 1) & 1, P.spin_limit);
+        if (!withheld(it)) mbar_wait(&full_bar[(it / plan.stages) & 1][it % plan.stages], ((it / plan.stages) >> 1) & 1);
     __syncthreads();
   }
 
@@ -495,11 +495,14 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *__restrict__ q, const int *seq_lens, 
     }
   }
   auto wait_x = [&](int i) {
-    if (!mbar_wait_cluster(&s_xbar[i], 0, ckv_pipe::kSpinLimit)) { atomicOr(P.status, CKV_DEV_TIMEOUT); s_abort = 1; }
+    if (mbar_wait_cluster(&s_xbar[i], 0, P.spin_limit)) return true;
+    atomicOr(P.status, CKV_DEV_TIMEOUT);
+    *(volatile int *)&s_abort = 1;
+    return false;
   };
-  wait_x(0);
-  if (append && rank == 0 && tid == kTailWarp * 32)
-    store_lens(P.status + CKV_LEN_COUNTER_WORD, fresh.seq_lens, batch, cap, (int)gridDim.y);   // all CTAs of this cluster have read them
+  const bool normed = wait_x(0);   // false: a CTA of the cluster may still be scanning, its ring in use and the lengths unread
+  const bool counts = append && rank == 0 && tid == kTailWarp * 32;
+  if (counts && normed) store_lens(P.status + CKV_LEN_COUNTER_WORD, fresh.seq_lens, batch, cap, (int)gridDim.y);   // all CTAs of this cluster have read them
   float Mg[G], iL[G], bound = 0.f;   // every warp by itself: 32 / G lanes per head.  bound: no block scores more
   {
     constexpr int LPH = 32 / G, EPL = (kClusterCap + LPH - 1) / LPH;
@@ -536,7 +539,9 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *__restrict__ q, const int *seq_lens, 
   const int rank_lo = P.sink, rank_n = max(X - n_recent - P.sink, 0);   // blocks [rank_lo, rank_lo + rank_n) are ranked, the others mandatory
   auto ranked = [rank_lo, rank_n](int b) { return (unsigned)(b - rank_lo) < (unsigned)rank_n; };
   uint32_t *keys = reinterpret_cast<uint32_t *>(smem);   // the unit's scores; their bit patterns are ordered like the scores
-  if (warp < kWarps) {
+  if (!normed) {
+    // nothing is sent into a CTA that may not be ready for it: its wait for the scores runs out, too
+  } else if (warp < kWarps) {
     bool nonfinite = false;
     const uint32_t xbar1 = smem_u32(&s_xbar[1]);
     for (int i = 4 * tid; i < own; i += 4 * kWork) {
@@ -586,20 +591,27 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *__restrict__ q, const int *seq_lens, 
     named_barrier(2, kThreads - kWork);
   }
   wait_x(1);
-  __syncthreads();   // the histogram is clear, too
+  // (the histogram is clear, too.)  A CTA one of whose waits ran out has scores that never came: it selects nothing and
+  // contributes an empty partial, so that the others get what they wait for.
+  const bool dead = __syncthreads_or(*(volatile int *)&s_abort) != 0;
 
   // ---- selection (Eq. 11), the same in every CTA ----
   const int K = min(kcap, X);
   const bool all = X <= kcap;          // every block is selected: the step is dense attention
   int *ids = reinterpret_cast<int *>(smem + kOffIds);
-  if (warp >= kWarps) {   // the two idle warps leave the range's scores where ckv_copy_scores() finds them
+  if (warp >= kWarps && !dead) {   // the two idle warps leave the range's scores where ckv_copy_scores() finds them
     float *scores = P.scores + row0;
     for (int i = tid - kWork; i < own; i += kThreads - kWork) scores[b_lo + i] = __uint_as_float(keys[b_lo + i]);
     if (rank == C - 1 && N > 0 && tid == kWork) scores[Xs] = __uint_as_float(keys[Xs]);
   }
   if (warp < kWarps) {
     int *gids = sel_ids + (size_t)unit * kcap;
-    if (all) {
+    if (dead) {
+      if (rank == 0) {
+        for (int i = tid; i < kcap; i += kWork) gids[i] = -1;
+        if (tid == 0) sel_cnt[unit] = 0;
+      }
+    } else if (all) {
       if (rank == 0) {
         for (int b = tid; b < kcap; b += kWork) gids[b] = b < X ? b : -1;
         if (tid == 0) sel_cnt[unit] = X;
@@ -670,8 +682,7 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *__restrict__ q, const int *seq_lens, 
               const int j = __ffs(at) - 1;
               at &= at - 1;
               const int slot = atomicAdd(&s_ncand, 1);
-              cand[slot] = 4 * i + j;
-              candk[slot] = k[j];
+              if (slot < kCandCap) { cand[slot] = 4 * i + j; candk[slot] = k[j]; }
             }
           }
           work_barrier();
@@ -719,9 +730,9 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *__restrict__ q, const int *seq_lens, 
   if (warp < kWarps) {
     wait_x(3);       // acquires what the other CTAs of the cluster released
     // ---- exact attention over the CTA's share of the selected pages ----
-    const bool comp = nsel < X && !(P.variant & CKV_VARIANT_DROP);
+    const bool comp = nsel < X && !dead && !(P.variant & CKV_VARIANT_DROP);
     if (!comp) w.reset();   // nothing is compensated: the scan's sums are not wanted
-    const int n_pages = all ? (N + CKV_PAGE - 1) / CKV_PAGE : nsel * P.ppb;
+    const int n_pages = dead ? 0 : (all ? (N + CKV_PAGE - 1) / CKV_PAGE : nsel * P.ppb);
     const int share = (int)ckv_udiv24((unsigned)(n_pages + C - 1), (unsigned)C);
     const int p0 = min(rank * share, n_pages), p1 = min(p0 + share, n_pages);
     const int n_mine = max((p1 - p0 - warp + kWarps - 1) / kWarps, 0);
@@ -742,7 +753,7 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *__restrict__ q, const int *seq_lens, 
         const int blk = all ? i >> pshift : ids[i >> pshift];
         const int page = all ? i : (blk << pshift) + (i & (P.ppb - 1));
         mine.blk = (i & (P.ppb - 1)) == 0 ? blk : ~blk;   // complemented on the block's later pages
-        mine.ntok = max(min(CKV_PAGE, N - page * CKV_PAGE), 0);
+        mine.ntok = (unsigned)blk < (unsigned)X ? max(min(CKV_PAGE, N - page * CKV_PAGE), 0) : 0;
         if (mine.ntok > 0) {
           mine.phys = pt_row[page];
           if (mine.phys < 0 || mine.phys >= P.num_pages) { mine.phys = -1; bad = true; }
@@ -916,6 +927,7 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *__restrict__ q, const int *seq_lens, 
   __syncwarp();
   cluster_arrive_relaxed();   // nobody leaves while somebody may still send to it
   cluster_wait();
+  if (counts && !normed) store_lens(P.status + CKV_LEN_COUNTER_WORD, fresh.seq_lens, batch, cap, (int)gridDim.y);
 }
 
 // The instantiation a context's layout uses.

@@ -184,6 +184,34 @@ def test_a_wait_that_runs_out_is_reported_and_the_context_recovers():
     assert d.ckv.read_status() == 0 and all(torch.equal(x, y) for x, y in zip(good, again))
 
 
+@pytest.mark.parametrize("polls", [1, 64])
+@pytest.mark.parametrize("batch", [1, 9])
+def test_waits_that_run_out_in_the_exchanges(polls, batch):
+    """With next to no polls the waits for the other CTAs' normalisers, scores and partial outputs run out as well (one
+    CTA's copy never comes): the launch returns, names no block that does not exist, and lengths, pages and summaries are
+    as after any step."""
+    w = workload(batch=batch, num_q_heads=16, num_kv_heads=4, ctx=16 * 300 + 9, ctx_min=None, decode_steps=2, needles=1)
+    a, b = setup(w), setup(w)
+    for d in (a, b):
+        d.ckv.stats_build(d.k_pool, d.v_pool, d.table, d.lens, d.max_len)
+    a.ckv.debug_set(polls, binding.CKV_DEBUG_SKIP_FILL)
+    for t in range(2):
+        q, kn, vn = step_inputs(a, t)
+        got = a.ckv.step(q, kn, vn, a.k_pool, a.v_pool, a.table, a.lens, w.ctx + t + 1, w.budget_tokens)
+        want = b.ckv.step(q, kn, vn, b.k_pool, b.v_pool, b.table, b.lens, w.ctx + t + 1, w.budget_tokens)
+        torch.cuda.synchronize()
+        assert torch.equal(a.lens, b.lens) and b.ckv.read_status() == 0
+        status = a.ckv.read_status()
+        if t == 0:
+            assert status & binding.CKV_DEV_TIMEOUT
+            assert int(got[2].min()) >= -1 and int(got[2].max()) <= w.ctx // 16
+            a.ckv.debug_set(0, 0)
+        else:
+            assert status == 0 and all(torch.equal(x, y) for x, y in zip(got, want))
+    for x, y in zip(a.ckv.export_stats(), b.ckv.export_stats()):
+        assert torch.equal(x, y)
+
+
 @pytest.mark.parametrize("batch,hq,hkv", [(1, 8, 2), (9, 64, 8)])   # inputs read over the bus; brought in by a kernel first
 def test_host_buffers_in_one_launch(batch, hq, hkv):
     w = workload(batch=batch, num_q_heads=hq, num_kv_heads=hkv, ctx=16 * 200 + 3, needles=0, decode_steps=4)
