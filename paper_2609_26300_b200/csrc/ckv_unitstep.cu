@@ -915,8 +915,9 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *__restrict__ q, const int *seq_lens, 
   if (done.flag != nullptr) {   // the results are in the caller's host buffers: the last CTA to say so stores the word
     __syncthreads();
     if (tid == 0) {
-      __threadfence_system();
+      __threadfence();   // the CTA's results before its count ...
       if (atomicAdd(done.ctas, 1) == (int)(gridDim.x * gridDim.y) - 1) {
+        __threadfence_system();   // ... and all that were counted before the word, as the host sees it
         *done.ctas = 0;
         const int e = *done.count + 1;   // counted on the device, call after call
         *done.count = e;
