@@ -55,11 +55,9 @@ constexpr int kMaxCluster = 8;    // splits of a unit that can be one cluster (t
 // through the tokens' weights, and the row machinery is not compiled in.
 template <int G, bool DENSE, int W, bool CL, bool RM>
 __global__ void __launch_bounds__(W * 32, DENSE ? 1 : 2)
-ckv_attn_mma_kernel(CkvDev P, const __nv_bfloat16 *__restrict__ q, const __nv_bfloat16 *__restrict__ k_pool,
-                    const __nv_bfloat16 *__restrict__ v_pool, const int *__restrict__ page_table,
-                    const int *__restrict__ seq_lens, const int *__restrict__ sel_ids,
-                    const int *__restrict__ sel_cnt, int kcap, int pages_per_split, int scan_grid, int units,
-                    __nv_bfloat16 *__restrict__ out, float *__restrict__ lse) {
+ckv_attn_mma_kernel(CkvDev P, const __nv_bfloat16 *q, const __nv_bfloat16 *k_pool, const __nv_bfloat16 *v_pool,
+                    const int *page_table, const int *seq_lens, const int *sel_ids, const int *sel_cnt, int kcap,
+                    int pages_per_split, int scan_grid, int units, __nv_bfloat16 *__restrict__ out, float *__restrict__ lse) {
   extern __shared__ __align__(128) unsigned char smem[];   // [W warps][2 buffers][K tile | V tile], then [W warps][aux]
   __shared__ float s_M[G], s_den[G];
   __shared__ int s_last;
@@ -328,7 +326,7 @@ ckv_attn_mma_kernel(CkvDev P, const __nv_bfloat16 *__restrict__ q, const __nv_bf
 #pragma unroll
     for (int ks = 0; ks < 8; ++ks)
 #pragma unroll
-      for (int hh = 0; hh < 2; ++hh) qa[ks][hh] = __ldg(reinterpret_cast<const uint32_t *>(qrow + 16 * ks + 8 * hh));
+      for (int hh = 0; hh < 2; ++hh) qa[ks][hh] = *reinterpret_cast<const uint32_t *>(qrow + 16 * ks + 8 * hh);
   }
   if (comp) {
     int efirst = 0, n_comp = 0;   // where the unit's scan partials sit

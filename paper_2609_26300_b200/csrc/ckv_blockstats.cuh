@@ -162,12 +162,11 @@ __device__ __forceinline__ void block_stats_rows16(const uint4 (&kraw)[8], const
   }
 }
 
-// NC: the pools are read-only for the whole kernel (loads may use the non-coherent path).
+// ALONE: the caller's warp works on one block only, so that asking the L2 for all of its pages first pays.
 // ONEP: the caller's layout has one-page blocks of bf16 rows, and only that path is compiled (fewer registers).
 // sq_smem: 128 floats of shared memory owned by the calling warp.
-template <typename T, bool NC, bool ONEP = false>
-__device__ __forceinline__ void block_stats_warp(const CkvDev &P, const T *__restrict__ k_pool,
-                                                 const T *__restrict__ v_pool, const int *__restrict__ pt_row,
+template <typename T, bool ALONE, bool ONEP = false>
+__device__ __forceinline__ void block_stats_warp(const CkvDev &P, const T *k_pool, const T *v_pool, const int *pt_row,
                                                  int h, int b, int cnt, float *sq_smem, __nv_bfloat16 *kmean_row,
                                                  float *dbar_row, __nv_bfloat16 *vmean_row, int lane,
                                                  BlockRow *keep = nullptr) {
@@ -196,8 +195,8 @@ __device__ __forceinline__ void block_stats_warp(const CkvDev &P, const T *__res
       if (ok && cnt == CKV_PAGE) {   // a full block (all but the last of a sequence): no per-row tests
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-          kraw[j] = NC ? __ldg(kp + j * kStep) : kp[j * kStep];
-          vraw[j] = NC ? __ldg(vp + j * kStep) : vp[j * kStep];
+          kraw[j] = kp[j * kStep];
+          vraw[j] = vp[j * kStep];
         }
         block_stats_rows16<true>(kraw, vraw, true, CKV_PAGE, lane, km, vs, sq);
       } else {
@@ -205,8 +204,8 @@ __device__ __forceinline__ void block_stats_warp(const CkvDev &P, const T *__res
         for (int j = 0; j < 8; ++j) {
           const bool valid = ok && hw + 2 * j < cnt;
           const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
-          kraw[j] = valid ? (NC ? __ldg(kp + j * kStep) : kp[j * kStep]) : zero;
-          vraw[j] = valid ? (NC ? __ldg(vp + j * kStep) : vp[j * kStep]) : zero;
+          kraw[j] = valid ? kp[j * kStep] : zero;
+          vraw[j] = valid ? vp[j * kStep] : zero;
         }
         block_stats_rows16(kraw, vraw, ok, cnt, lane, km, vs, sq);
       }
@@ -219,7 +218,7 @@ __device__ __forceinline__ void block_stats_warp(const CkvDev &P, const T *__res
       // block only (the append, the chunked prefill) the L2 is asked for all pages first, so that only the first one
       // costs a DRAM round trip.  (The build kernel asks for its next block itself.)
       done = true;
-      if constexpr (!NC) {
+      if constexpr (ALONE) {
         if (lane < npages) {
           const int phys = pt_row[b * P.ppb + lane];
           if (phys >= 0 && phys < P.num_pages) {
@@ -247,8 +246,8 @@ __device__ __forceinline__ void block_stats_warp(const CkvDev &P, const T *__res
         if (ntok == CKV_PAGE) {   // a full page: no per-row tests
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
-            kraw[j] = NC ? __ldg(kp + j * kStep) : kp[j * kStep];
-            vraw[j] = NC ? __ldg(vp + j * kStep) : vp[j * kStep];
+            kraw[j] = kp[j * kStep];
+            vraw[j] = vp[j * kStep];
           }
           block_stats_rows16<true>(kraw, vraw, true, CKV_PAGE, lane, mb, vb, qb);
         } else {
@@ -256,8 +255,8 @@ __device__ __forceinline__ void block_stats_warp(const CkvDev &P, const T *__res
           for (int j = 0; j < 8; ++j) {
             const bool valid = hw + 2 * j < ntok;
             const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
-            kraw[j] = valid ? (NC ? __ldg(kp + j * kStep) : kp[j * kStep]) : zero;
-            vraw[j] = valid ? (NC ? __ldg(vp + j * kStep) : vp[j * kStep]) : zero;
+            kraw[j] = valid ? kp[j * kStep] : zero;
+            vraw[j] = valid ? vp[j * kStep] : zero;
           }
           block_stats_rows16(kraw, vraw, true, ntok, lane, mb, vb, qb);
         }
@@ -272,7 +271,7 @@ __device__ __forceinline__ void block_stats_warp(const CkvDev &P, const T *__res
   }
   if constexpr (sizeof(T) != 2) {
   if (!done) {
-    if constexpr (!NC) {
+    if constexpr (ALONE) {
       // A block of several pages (32- or 64-token blocks) is read page after page, twice: when the caller works on
       // one block only (the append, the chunked prefill) the L2 is asked for all of its pages first, so that only
       // the first page costs a DRAM round trip.  (The build kernel asks for its next block itself.)
@@ -296,8 +295,8 @@ __device__ __forceinline__ void block_stats_warp(const CkvDev &P, const T *__res
         const int t = hw + 2 * j;
         if (t < ntok) {
           float a[8], c[8];
-          load8<NC>(k_pool + base + (size_t)t * CKV_D, a);
-          load8<NC>(v_pool + base + (size_t)t * CKV_D, c);
+          load8<false>(k_pool + base + (size_t)t * CKV_D, a);
+          load8<false>(v_pool + base + (size_t)t * CKV_D, c);
 #pragma unroll
           for (int i = 0; i < 8; ++i) { ks[i] += a[i]; vs[i] += c[i]; }
         }
@@ -320,7 +319,7 @@ __device__ __forceinline__ void block_stats_warp(const CkvDev &P, const T *__res
         const int t = hw + 2 * j;
         if (t < ntok) {
           float a[8];
-          load8<NC>(k_pool + base + (size_t)t * CKV_D, a);
+          load8<false>(k_pool + base + (size_t)t * CKV_D, a);
 #pragma unroll
           for (int i = 0; i < 8; ++i) { const float dv = a[i] - km[i]; sq[i] = fmaf(dv, dv, sq[i]); }
         }

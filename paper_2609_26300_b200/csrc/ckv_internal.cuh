@@ -106,6 +106,9 @@ struct ckv_ctx {
 // one's are done: good where the next one is alike (builds, chunks, dense passes, one-launch steps), bad among the scan,
 // selection and attention kernels, whose CTAs then sit on SMs that the running kernel still needs (80.7 -> 92.3): those do
 // not call it.  cluster_x: CTAs of a cluster (0: no clusters).
+// Whatever such a kernel reads may have been written while it was already running, by the launch ahead of it: its loads
+// promise nothing (no __ldg, no const __restrict__), or the compiler may take them for invariant and move them up past
+// pdl_wait().  The plain loads measure the same.
 template <class... Params, class... Args>
 inline cudaError_t ckv_launch_pdl(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, int cluster_x, Args... args) {
   cudaLaunchAttribute attr[2];
@@ -218,8 +221,8 @@ __device__ __forceinline__ void sub_bf16x8(const uint4 &u, const float (&m)[8], 
   }
 }
 
-// Eight consecutive elements as floats.  NC = read-only (non-coherent) path; use NC = false for
-// data the same kernel has just written.
+// Eight consecutive elements as floats.  NC = read-only (non-coherent) path; use NC = false for data the same kernel has
+// just written, and in every kernel that may start before the launch ahead of it is complete (ckv_launch_pdl).
 template <bool NC>
 __device__ __forceinline__ void load8(const __nv_bfloat16 *p, float (&o)[8]) {
   uint4 u;

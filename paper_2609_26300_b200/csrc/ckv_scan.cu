@@ -55,10 +55,10 @@ struct UnitInfo { int N, X, tiles; };   // X: the blocks the scan CTAs cover (in
 
 // s_len holds the clamped lengths (after this step's append, if any) of the first kMaxSeqs sequences, staged once
 // per CTA; longer batches never come with an append and read the device array
-__device__ __forceinline__ int seq_len_of(const CkvDev &P, const int *s_len, const int *__restrict__ seq_lens, int s) {
+__device__ __forceinline__ int seq_len_of(const CkvDev &P, const int *s_len, const int *seq_lens, int s) {
   return s < kMaxSeqs ? s_len[s] : max(min(seq_lens[s], P.max_blocks * P.bs), 0);
 }
-__device__ __forceinline__ UnitInfo unit_info(const CkvDev &P, const int *s_len, const int *__restrict__ seq_lens, int u) {
+__device__ __forceinline__ UnitInfo unit_info(const CkvDev &P, const int *s_len, const int *seq_lens, int u) {
   UnitInfo ui;
   ui.N = seq_len_of(P, s_len, seq_lens, ckv_div_hkv(P, u));
   ui.X = ckv_scan_blocks(P, ui.N);
@@ -66,7 +66,7 @@ __device__ __forceinline__ UnitInfo unit_info(const CkvDev &P, const int *s_len,
   return ui;
 }
 
-__device__ __forceinline__ int seq_tiles(const int *s_len, const int *__restrict__ seq_lens, const CkvDev &P, int i) {
+__device__ __forceinline__ int seq_tiles(const int *s_len, const int *seq_lens, const CkvDev &P, int i) {
   return (ckv_scan_blocks(P, seq_len_of(P, s_len, seq_lens, i)) + P.scan_tile - 1) >> P.lg_tile;
 }
 
@@ -116,7 +116,7 @@ __device__ __noinline__ void lens_arrive(int *counter, const int *seq_lens, int 
 // kernel's size and the scan CTAs stalled on instruction fetch (the launch went from 55 to 68 us); handed a
 // reference, the compiler moves the parameter block to local memory for every CTA, scan loop included.
 template <int G, typename QT>
-__device__ __noinline__ void scan_tail(const CkvDev P, const QT *__restrict__ q, const int *seq_lens, int *s_len,
+__device__ __noinline__ void scan_tail(const CkvDev P, const QT *q, const int *seq_lens, int *s_len,
                                        int len_mine, int units, int nscan, const CkvNewToken fresh, int n_tail,
                                        float *smem_f, int smem_bytes) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, hw = lane >> 4, li = lane & 15;
@@ -140,7 +140,7 @@ __device__ __noinline__ void scan_tail(const CkvDev P, const QT *__restrict__ q,
   if (append && u_first < units) {
     const uint4 *src = reinterpret_cast<const uint4 *>((lane < 16 ? k_new : v_new) + (size_t)u_first * CKV_D);
 #pragma unroll
-    for (int k = 0; k < PP; ++k) piece[k] = __ldg(src + li + 16 * k);
+    for (int k = 0; k < PP; ++k) piece[k] = src[li + 16 * k];
   }
   auto eff_len = [&](int raw) { return max(min(raw + ((append && raw >= 0 && raw < cap) ? 1 : 0), cap), 0); };
   if (tid < batch) s_len[tid] = eff_len(len_mine);
@@ -176,7 +176,7 @@ __device__ __noinline__ void scan_tail(const CkvDev P, const QT *__restrict__ q,
           if (u != u_first) {
             const uint4 *src = reinterpret_cast<const uint4 *>((lane < 16 ? k_new : v_new) + (size_t)u * CKV_D);
 #pragma unroll
-            for (int k = 0; k < PP; ++k) piece[k] = __ldg(src + li + 16 * k);
+            for (int k = 0; k < PP; ++k) piece[k] = src[li + 16 * k];
           }
           uint4 *dst = reinterpret_cast<uint4 *>((lane < 16 ? k_pool : v_pool) +
                                                  (((size_t)phys * P.Hkv + h) * CKV_PAGE + slot) * CKV_D);
@@ -192,7 +192,7 @@ __device__ __noinline__ void scan_tail(const CkvDev P, const QT *__restrict__ q,
                                       reinterpret_cast<unsigned char *>(smem_f + 8 * CKV_D) + (size_t)warp * kStageBytes, sq,
                                       P.kmean + row * P.row_elems, P.dbar + row * P.r, P.vmean + row * P.row_elems, lane);
         else
-          block_stats_warp<QT, false>(P, k_pool, v_pool, pt_row, h, b, cnt, sq, P.kmean + row * P.row_elems,
+          block_stats_warp<QT, true>(P, k_pool, v_pool, pt_row, h, b, cnt, sq, P.kmean + row * P.row_elems,
                                       P.dbar + row * P.r, P.vmean + row * P.row_elems, lane);
       }
     }
@@ -221,7 +221,7 @@ __device__ __noinline__ void scan_tail(const CkvDev P, const QT *__restrict__ q,
 #pragma unroll 1
     for (int g = 0; g < G; ++g) {
       float qx[8];   // this lane's 8 coordinates of query row u G + g
-      load8<true>(q + ((size_t)u * G + g) * CKV_D + 8 * li, qx);
+      load8<false>(q + ((size_t)u * G + g) * CKV_D + 8 * li, qx);
       float d = 0.f, sg = 0.f;
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
@@ -262,7 +262,7 @@ __device__ __noinline__ void scan_tail(const CkvDev P, const QT *__restrict__ q,
 // bf16 output).
 template <int G, typename QT, bool RD, bool HS, bool VH>
 __global__ void __launch_bounds__(kThreads, 1)
-ckv_scan_kernel(CkvDev P, const QT *__restrict__ q, const int *seq_lens, int units, int stages, CkvNewToken fresh,
+ckv_scan_kernel(CkvDev P, const QT *q, const int *seq_lens, int units, int stages, CkvNewToken fresh,
                 int n_tail, const __grid_constant__ CUtensorMap tm_v) {
   constexpr bool QS = QSplit<QT>::value;   // fp32 queries are split into hi + lo like the summaries
   static_assert(!(VH && (HS || RD)), "VH is a variant of the full-precision layout with four variance groups");
@@ -419,7 +419,7 @@ ckv_scan_kernel(CkvDev P, const QT *__restrict__ q, const int *seq_lens, int uni
         if (uu <= s_ulast && uu < units) {
           const int s2 = ckv_div_hkv(P, uu), h2 = uu - s2 * P.Hkv;
           const uint4 *src = reinterpret_cast<const uint4 *>(q + ((size_t)s2 * P.Hq + h2 * G) * CKV_D);
-          reinterpret_cast<uint4 *>(&s_q[k][0][0])[pc] = __ldg(src + pc);
+          reinterpret_cast<uint4 *>(&s_q[k][0][0])[pc] = src[pc];
         }
       }
       named_barrier(1, kConsumerWarps * 32);
@@ -544,7 +544,7 @@ ckv_scan_kernel(CkvDev P, const QT *__restrict__ q, const int *seq_lens, int uni
 #pragma unroll
             for (int c = 0; c < 16; ++c) {
               float x[8];
-              load8<true>(qrow_e + 8 * c, x);
+              load8<false>(qrow_e + 8 * c, x);
               float s8 = 0.f;
 #pragma unroll
               for (int i = 0; i < 8; ++i) s8 = fmaf(x[i], x[i], s8);

@@ -162,7 +162,7 @@ __device__ __forceinline__ void scan_part(ScanUnit<G, QT, RD> &w, const ScanPart
           sg = fmaf(w.wown[e][0], dv.x, fmaf(w.wown[e][1], dv.y, fmaf(w.wown[e][2], dv.z, w.wown[e][3] * dv.w)));
         } else {
           for (int t = 0; t < cfg.r; ++t) {
-            const float d = sd != nullptr ? sd[r * cfg.r + t] : __ldg(dbar_row0 + (size_t)b * cfg.r + t);
+            const float d = sd != nullptr ? sd[r * cfg.r + t] : dbar_row0[(size_t)b * cfg.r + t];
             sg = fmaf(sw[t * G + head], d, sg);
           }
         }

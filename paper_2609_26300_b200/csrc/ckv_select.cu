@@ -55,7 +55,7 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int *warp_tot, int *t
 }
 
 template <int G>
-__global__ void __launch_bounds__(kThreads) ckv_select_kernel(CkvDev P, const int *__restrict__ seq_lens, int kcap,
+__global__ void __launch_bounds__(kThreads) ckv_select_kernel(CkvDev P, const int *seq_lens, int kcap,
                                                               int scan_grid, int units, int *__restrict__ sel_ids,
                                                               int *__restrict__ sel_cnt) {
   extern __shared__ uint32_t skeys[];

@@ -39,10 +39,8 @@ int rounds_for(int blocks, int units, int sms, int most) {
 // only costs instructions, and with blocks of several pages it cost a third of the time.
 // ONEP: one-page blocks of bf16 rows (the default layout), compiled without the other paths of the block routine.
 template <typename T, bool ONEP>
-__global__ void __launch_bounds__(256, 2) ckv_stats_build_kernel(CkvDev P, const T *__restrict__ k_pool,
-                                                              const T *__restrict__ v_pool,
-                                                              const int *__restrict__ page_table,
-                                                              const int *__restrict__ seq_lens, int rounds) {
+__global__ void __launch_bounds__(256, 2) ckv_stats_build_kernel(CkvDev P, const T *k_pool, const T *v_pool,
+                                                                 const int *page_table, const int *seq_lens, int rounds) {
   __shared__ float sq_smem[8][CKV_D];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int unit = blockIdx.y, s = unit / P.Hkv, h = unit % P.Hkv;
@@ -57,7 +55,7 @@ __global__ void __launch_bounds__(256, 2) ckv_stats_build_kernel(CkvDev P, const
     if (b >= X) return;
     const int cnt = min(P.bs, N - b * P.bs);
     const size_t row = (size_t)unit * P.max_blocks + b;
-    block_stats_warp<T, true, ONEP>(P, k_pool, v_pool, pt_row, h, b, cnt, sq_smem[warp], P.kmean + row * P.row_elems,
+    block_stats_warp<T, false, ONEP>(P, k_pool, v_pool, pt_row, h, b, cnt, sq_smem[warp], P.kmean + row * P.row_elems,
                                     P.dbar + row * P.r, P.vmean + row * P.row_elems, lane);
   }
 }
@@ -65,8 +63,8 @@ __global__ void __launch_bounds__(256, 2) ckv_stats_build_kernel(CkvDev P, const
 // One CTA per sequence, one warp per KV head (looping when there are more heads than warps).
 template <typename T>
 __global__ void __launch_bounds__(256) ckv_append_kernel(CkvDev P, T *k_pool, T *v_pool,
-                                                         const int *__restrict__ page_table, int *seq_lens,
-                                                         const T *__restrict__ k_new, const T *__restrict__ v_new) {
+                                                         const int *page_table, int *seq_lens, const T *k_new,
+                                                         const T *v_new) {
   __shared__ float sq_smem[8][CKV_D];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
   const int s = blockIdx.x;
@@ -81,7 +79,7 @@ __global__ void __launch_bounds__(256) ckv_append_kernel(CkvDev P, T *k_pool, T 
   if (warp < P.Hkv) {
     const uint4 *src = reinterpret_cast<const uint4 *>((lane < 16 ? k_new : v_new) + ((size_t)s * P.Hkv + warp) * CKV_D);
 #pragma unroll
-    for (int k = 0; k < PP; ++k) fresh[k] = __ldg(src + (lane & 15) + 16 * k);
+    for (int k = 0; k < PP; ++k) fresh[k] = src[(lane & 15) + 16 * k];
   }
   __syncthreads();   // every warp has read N before thread 0 may change it
   if (N < 0 || N >= P.max_blocks * P.bs) {
@@ -98,7 +96,7 @@ __global__ void __launch_bounds__(256) ckv_append_kernel(CkvDev P, T *k_pool, T 
       if (h != warp) {   // further heads of this warp (more KV heads than warps)
         const uint4 *src = reinterpret_cast<const uint4 *>((lane < 16 ? k_new : v_new) + ((size_t)s * P.Hkv + h) * CKV_D);
 #pragma unroll
-        for (int k = 0; k < PP; ++k) fresh[k] = __ldg(src + (lane & 15) + 16 * k);
+        for (int k = 0; k < PP; ++k) fresh[k] = src[(lane & 15) + 16 * k];
       }
       uint4 *dst = reinterpret_cast<uint4 *>((lane < 16 ? k_pool : v_pool) +
                                              (((size_t)phys * P.Hkv + h) * CKV_PAGE + slot) * CKV_D);
@@ -107,7 +105,7 @@ __global__ void __launch_bounds__(256) ckv_append_kernel(CkvDev P, T *k_pool, T 
     }
     __syncwarp();
     const size_t row = ((size_t)s * P.Hkv + h) * P.max_blocks + b;
-    block_stats_warp<T, false>(P, k_pool, v_pool, pt_row, h, b, cnt, sq_smem[warp], P.kmean + row * P.row_elems,
+    block_stats_warp<T, true>(P, k_pool, v_pool, pt_row, h, b, cnt, sq_smem[warp], P.kmean + row * P.row_elems,
                                P.dbar + row * P.r, P.vmean + row * P.row_elems, lane);
   }
   __syncthreads();
@@ -122,9 +120,8 @@ __global__ void __launch_bounds__(256) ckv_append_kernel(CkvDev P, T *k_pool, T 
 // rows never leave the registers; 0 = the general form (fp32 pages).
 template <typename T, int REG>
 __global__ void __launch_bounds__(256, REG ? 2 : 1) ckv_prefill_kernel(CkvDev P, T *k_pool, T *v_pool,
-                                                          const int *__restrict__ page_table, int *seq_lens,
-                                                          const T *__restrict__ k_src, const T *__restrict__ v_src,
-                                                          const int *__restrict__ new_lens, int src_stride, int batch,
+                                                          const int *page_table, int *seq_lens, const T *k_src,
+                                                          const T *v_src, const int *new_lens, int src_stride, int batch,
                                                           int rounds) {
   __shared__ float sq_smem[8][CKV_D];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -165,8 +162,8 @@ __global__ void __launch_bounds__(256, REG ? 2 : 1) ckv_prefill_kernel(CkvDev P,
           const size_t sstep = (size_t)2 * P.Hkv * CKV_D;   // two chunk rows on
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
-            kraw[j] = __ldg(reinterpret_cast<const uint4 *>(k_src + so + j * sstep));
-            vraw[j] = __ldg(reinterpret_cast<const uint4 *>(v_src + so + j * sstep));
+            kraw[j] = *reinterpret_cast<const uint4 *>(k_src + so + j * sstep);
+            vraw[j] = *reinterpret_cast<const uint4 *>(v_src + so + j * sstep);
           }
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
@@ -183,8 +180,8 @@ __global__ void __launch_bounds__(256, REG ? 2 : 1) ckv_prefill_kernel(CkvDev P,
             if (t < ntok) {
               if (p >= p_lo) {
                 const size_t so = (((size_t)s * src_stride + (p - N)) * P.Hkv + h) * CKV_D + 8 * li;
-                kraw[j] = __ldg(reinterpret_cast<const uint4 *>(k_src + so));
-                vraw[j] = __ldg(reinterpret_cast<const uint4 *>(v_src + so));
+                kraw[j] = *reinterpret_cast<const uint4 *>(k_src + so);
+                vraw[j] = *reinterpret_cast<const uint4 *>(v_src + so);
               } else {
                 kraw[j] = *reinterpret_cast<const uint4 *>(k_pool + pbase + (size_t)t * CKV_D);
                 vraw[j] = *reinterpret_cast<const uint4 *>(v_pool + pbase + (size_t)t * CKV_D);
@@ -248,7 +245,7 @@ __global__ void __launch_bounds__(256, REG ? 2 : 1) ckv_prefill_kernel(CkvDev P,
         if (p >= p_lo && p < p_hi) {
           const uint4 *src = reinterpret_cast<const uint4 *>(src_base + (((size_t)s * src_stride + (p - N)) * P.Hkv + h) * CKV_D);
 #pragma unroll
-          for (int k = 0; k < PP; ++k) r[t][k] = __ldg(src + (lane & 15) + 16 * k);
+          for (int k = 0; k < PP; ++k) r[t][k] = src[(lane & 15) + 16 * k];
         }
       }
 #pragma unroll
@@ -265,7 +262,7 @@ __global__ void __launch_bounds__(256, REG ? 2 : 1) ckv_prefill_kernel(CkvDev P,
     __syncwarp();
     const int cnt = min(P.bs, N + m_eff - b * P.bs);
     const size_t row = (size_t)unit * P.max_blocks + b;
-    block_stats_warp<T, false>(P, k_pool, v_pool, pt_row, h, b, cnt, sq_smem[warp], P.kmean + row * P.row_elems,
+    block_stats_warp<T, true>(P, k_pool, v_pool, pt_row, h, b, cnt, sq_smem[warp], P.kmean + row * P.row_elems,
                                P.dbar + row * P.r, P.vmean + row * P.row_elems, lane);
     }
   }

@@ -144,12 +144,12 @@ __device__ __noinline__ void tail_block(const CkvDev P, const bf16 *q_rows, cons
   kn = vn = make_uint4(0u, 0u, 0u, 0u);
   if (append) {
     phys = pt_row[raw / CKV_PAGE];
-    kn = __ldg(reinterpret_cast<const uint4 *>(reinterpret_cast<const bf16 *>(fresh.k_new) + (size_t)unit * CKV_D) + li);
-    vn = __ldg(reinterpret_cast<const uint4 *>(reinterpret_cast<const bf16 *>(fresh.v_new) + (size_t)unit * CKV_D) + li);
+    kn = reinterpret_cast<const uint4 *>(reinterpret_cast<const bf16 *>(fresh.k_new) + (size_t)unit * CKV_D)[li];
+    vn = reinterpret_cast<const uint4 *>(reinterpret_cast<const bf16 *>(fresh.v_new) + (size_t)unit * CKV_D)[li];
   }
   uint4 qr[G];    // ... and of the queries
 #pragma unroll
-  for (int g = 0; g < G; ++g) qr[g] = __ldg(reinterpret_cast<const uint4 *>(q_rows + (size_t)g * CKV_D) + li);
+  for (int g = 0; g < G; ++g) qr[g] = reinterpret_cast<const uint4 *>(q_rows + (size_t)g * CKV_D)[li];
   const int b = ((N + P.bs - 1) >> P.lg_bs) - 1, cnt = N - b * P.bs;
   const size_t row = (size_t)unit * P.max_blocks + b;
   __nv_bfloat16 *kmean_row = P.kmean + row * P.row_elems, *vmean_row = P.vmean + row * P.row_elems;
@@ -178,7 +178,7 @@ __device__ __noinline__ void tail_block(const CkvDev P, const bf16 *q_rows, cons
     } else {
       if (ok) *reinterpret_cast<uint4 *>((hw == 0 ? kp : vp) + at) = hw == 0 ? kn : vn;
       __syncwarp();
-      block_stats_warp<bf16, false>(P, kp, vp, pt_row, h, b, cnt, sq, kmean_row, dbar_row, vmean_row, lane, &br);
+      block_stats_warp<bf16, true>(P, kp, vp, pt_row, h, b, cnt, sq, kmean_row, dbar_row, vmean_row, lane, &br);
     }
   } else {   // the summary as stored: lower half warp the mean key, upper the mean value (as the scan reads it)
     if (fresh.k_new != nullptr && raw >= cap && lane == 0) atomicOr(P.status, CKV_DEV_SEQ_FULL);
@@ -237,7 +237,7 @@ __device__ __noinline__ void append_past_bound(const CkvDev P, const int *page_t
   }
   __syncwarp();
   const size_t row = (size_t)unit * P.max_blocks + b;
-  block_stats_warp<bf16, false>(P, kp, vp, pt_row, h, b, raw + 1 - b * P.bs, sq, P.kmean + row * P.row_elems, P.dbar + row * P.r,
+  block_stats_warp<bf16, true>(P, kp, vp, pt_row, h, b, raw + 1 - b * P.bs, sq, P.kmean + row * P.row_elems, P.dbar + row * P.r,
                                 P.vmean + row * P.row_elems, lane);
 }
 
@@ -253,8 +253,8 @@ __device__ __noinline__ void store_lens(int *counter, int *seq_lens, int batch, 
 
 template <int G, bool RD, bool HS, bool VH>
 __global__ void __launch_bounds__(kThreads, 1)
-ckv_unit_step_kernel(CkvDev P, const bf16 *__restrict__ q, const int *seq_lens, const bf16 *k_pool, const bf16 *v_pool,
-                     const int *__restrict__ page_table, CkvNewToken fresh, int kcap, CkvStepPlan plan, int batch,
+ckv_unit_step_kernel(CkvDev P, const bf16 *q, const int *seq_lens, const bf16 *k_pool, const bf16 *v_pool,
+                     const int *page_table, CkvNewToken fresh, int kcap, CkvStepPlan plan, int batch,
                      int *__restrict__ sel_ids, int *__restrict__ sel_cnt, bf16 *__restrict__ out, float *__restrict__ lse,
                      CkvHostDone done, const __grid_constant__ CUtensorMap tm_v) {
   constexpr int kRowBytesK = HS ? CKV_D * 2 : CKV_ROW_ELEMS * 2;
@@ -296,7 +296,7 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *__restrict__ q, const int *seq_lens, 
   pdl_trigger();              // the next launch of the stream may set itself up ...
   pdl_wait();                 // ... and this one touches nothing before the launch ahead of it is complete
   const int raw = seq_lens[s];
-  if (tid < G * 16) reinterpret_cast<uint4 *>(&s_q[0][0])[tid] = __ldg(reinterpret_cast<const uint4 *>(q + (size_t)unit * G * CKV_D) + tid);
+  if (tid < G * 16) reinterpret_cast<uint4 *>(&s_q[0][0])[tid] = reinterpret_cast<const uint4 *>(q + (size_t)unit * G * CKV_D)[tid];
   if (tid >= kThreads - 32) reinterpret_cast<uint4 *>(s_zero_row)[lane] = make_uint4(0u, 0u, 0u, 0u);
   const bool dbar_bulk = P.r >= 4;
   const int stage_bytes = TB * (kRowBytesK + kRowBytesV) + (dbar_bulk ? TB * P.r * 4 : 0);

@@ -18,3 +18,18 @@ def test_completion_word_is_stored_behind_what_the_counter_showed():
     count, store = src.index("atomicAdd(done.ctas"), src.index("(volatile int *)done.flag = ")
     assert "__threadfence" in src[:count].rsplit("__syncthreads()", 1)[1]
     assert "__threadfence_system()" in src[count:store]
+
+
+def test_kernels_that_start_early_do_not_call_their_inputs_constant():
+    """A programmatic dependent launch runs while the launch ahead of it still writes: `__ldg` and `const __restrict__`
+    would let the compiler move loads up past griddepcontrol.wait."""
+    kernels = re.compile(r"ckv_launch_pdl\(\s*\(?(\w+)")
+    early = {"ckv_attn_mma.cu", "ckv_scan.cu", "ckv_select.cu", "ckv_stats.cu", "ckv_unitstep.cu"}
+    found = {f for f in os.listdir(CSRC) if f.endswith(".cu") and (kernels.search(code(f)) or "griddepcontrol" in code(f)
+                                                                    or "cudaLaunchAttributeProgrammatic" in code(f))}
+    assert found == early   # a new one belongs into the list
+    for name in sorted(early | {"ckv_blockstats.cuh", "ckv_scanpart.cuh", "ckv_attnpage.cuh"}):
+        src = code(name)
+        src = re.sub(r"__global__[^;{]*ckv_stats_export_kernel.*?\n}\n", "", src, flags=re.S)   # an ordinary launch
+        for bad in (r"__ldg", r"ld\.global\.nc", r"load8<true>", r"load8<NC>", r"load_split8\(", r"const\s+[\w ]+\*\s*__restrict__"):
+            assert not re.search(bad, src), (name, bad)
