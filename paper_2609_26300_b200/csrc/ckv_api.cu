@@ -311,11 +311,23 @@ cudaError_t ckv_launch_host_out(ckv_ctx *c, const void *dout, const int32_t *did
   return cudaGetLastError();
 }
 
-// The launches of a sparse decode step; ev (may be null) receives 5 events bracketing them.  With `fresh` the
-// scan launch also appends the step's new token (its tail CTAs do, beside the scan CTAs).
+// How a step is arranged: one launch, or separate ones with the last block left to the scan's tail CTAs or not.  The
+// arrangements agree to rounding only, so a call decides once, from the length bound it was given.
+struct Route { bool one, tail; CkvStepPlan plan; };
+Route route_of(const ckv_ctx *c, int batch, int max_len, int kcap) {
+  Route r = {};
+  r.one = ckv_unit_step_plan(c, batch, max_len, kcap, &r.plan);
+  r.tail = !r.one && ckv_scan_wants_tail(c, batch, max_len);
+  return r;
+}
+
+// The launches of a sparse decode step; ev (may be null) receives 5 events bracketing them.  With `fresh` the step's new
+// token is appended by its only launch, or by the scan launch (its tail CTAs do, beside the scan CTAs).  route: null, or
+// what the caller has decided.
 int decode_impl(ckv_ctx *c, const void *q, const void *k_pool, const void *v_pool, const int32_t *page_table,
                 const int32_t *seq_lens, int batch, int max_seq_len_host, int budget_tokens, void *out, float *lse,
-                int32_t *sel_ids, int32_t *sel_cnt, cudaStream_t s, cudaEvent_t *ev, const CkvNewToken *fresh = nullptr) {
+                int32_t *sel_ids, int32_t *sel_cnt, cudaStream_t s, cudaEvent_t *ev, const CkvNewToken *fresh = nullptr,
+                const Route *route = nullptr) {
   const int st = check_step_args(c, batch, max_seq_len_host);
   if (st != CKV_OK) return st;
   if (!q || !k_pool || !v_pool || !page_table || !seq_lens || !out || !sel_ids || !sel_cnt) return CKV_ERR_INVALID_ARG;
@@ -324,13 +336,16 @@ int decode_impl(ckv_ctx *c, const void *q, const void *k_pool, const void *v_poo
   if (budget_tokens <= 0 || kcap <= 0) return CKV_ERR_BUDGET_TOO_SMALL;
   if (kcap < L.sink_blocks + L.recent_blocks && (long long)kcap * L.block_size < max_seq_len_host)
     return CKV_ERR_BUDGET_TOO_SMALL;
-  CkvStepPlan plan;
-  if (ev == nullptr && ckv_unit_step_plan(c, batch, max_seq_len_host, kcap, &plan)) {
-    CKV_CUDA(ckv_launch_unit_step(c, plan, q, k_pool, v_pool, page_table, seq_lens, fresh, batch, kcap, sel_ids, sel_cnt, out, lse, CkvHostDone{}, s));
+  Route rt;
+  if (route != nullptr) rt = *route;
+  else if (ev == nullptr) rt = route_of(c, batch, max_seq_len_host, kcap);
+  else rt = Route{false, ckv_scan_wants_tail(c, batch, max_seq_len_host), {}};   // the profile is of the separate launches
+  if (rt.one) {
+    CKV_CUDA(ckv_launch_unit_step(c, rt.plan, q, k_pool, v_pool, page_table, seq_lens, fresh, batch, kcap, sel_ids, sel_cnt, out, lse, CkvHostDone{}, s));
     return CKV_OK;
   }
   int scan_grid = 0, n_splits = 0;
-  c->dev.tail = (fresh != nullptr || ckv_scan_wants_tail(c, batch, max_seq_len_host)) ? 1 : 0;   // one mode for the step's launches
+  c->dev.tail = rt.tail ? 1 : 0;   // one mode for the step's launches
   if (ev) CKV_CUDA(cudaEventRecord(ev[0], s));
   CKV_CUDA(ckv_launch_scan(c, q, seq_lens, batch, max_seq_len_host, fresh, &scan_grid, s));
   if (ev) CKV_CUDA(cudaEventRecord(ev[1], s));
@@ -345,6 +360,28 @@ int decode_impl(ckv_ctx *c, const void *q, const void *k_pool, const void *v_poo
   return CKV_OK;
 }
 
+// One step; route: null, or what the caller has decided.
+int step_impl(ckv_ctx *c, const void *q, const void *k_new, const void *v_new, void *k_pool, void *v_pool,
+              const int32_t *page_table, int32_t *seq_lens, int batch, int max_seq_len_host, int budget_tokens, void *out,
+              float *lse, int32_t *sel_ids, int32_t *sel_cnt, cudaStream_t s, const Route *route) {
+  // validate the decode half before anything is appended, so that a refused step leaves the cache untouched
+  const int st = check_step_args(c, batch, max_seq_len_host);
+  if (st != CKV_OK) return st;
+  if (!q || !out || !sel_ids || !sel_cnt) return CKV_ERR_INVALID_ARG;
+  const ckv_layout &L = c->layout;
+  const int kcap = budget_tokens / L.block_size;
+  if (budget_tokens <= 0 || kcap <= 0) return CKV_ERR_BUDGET_TOO_SMALL;
+  if (kcap < L.sink_blocks + L.recent_blocks && (long long)kcap * L.block_size < max_seq_len_host)
+    return CKV_ERR_BUDGET_TOO_SMALL;
+  if (!k_pool || !v_pool || !page_table || !seq_lens || !k_new || !v_new) return CKV_ERR_INVALID_ARG;
+  const Route rt = route != nullptr ? *route : route_of(c, batch, max_seq_len_host, kcap);
+  CkvNewToken fresh = {k_pool, v_pool, page_table, seq_lens, k_new, v_new};
+  const bool rides = rt.one || rt.tail;   // the append rides in the step's only launch, or in the scan launch (three per step)
+  if (!rides) CKV_CUDA(ckv_launch_append(c, k_pool, v_pool, page_table, seq_lens, k_new, v_new, batch, s));
+  return decode_impl(c, q, k_pool, v_pool, page_table, seq_lens, batch, max_seq_len_host, budget_tokens, out, lse, sel_ids,
+                     sel_cnt, s, nullptr, rides ? &fresh : nullptr, &rt);
+}
+
 }  // namespace
 
 int ckv_decode(ckv_ctx *c, const void *q, const void *k_pool, const void *v_pool, const int32_t *page_table,
@@ -357,27 +394,8 @@ int ckv_decode(ckv_ctx *c, const void *q, const void *k_pool, const void *v_pool
 int ckv_step(ckv_ctx *c, const void *q, const void *k_new, const void *v_new, void *k_pool, void *v_pool,
              const int32_t *page_table, int32_t *seq_lens, int batch, int max_seq_len_host, int budget_tokens, void *out,
              float *lse, int32_t *sel_ids, int32_t *sel_cnt, ckv_stream stream) {
-  // validate the decode half before anything is appended, so that a refused step leaves the cache untouched
-  const int st = check_step_args(c, batch, max_seq_len_host);
-  if (st != CKV_OK) return st;
-  if (!q || !out || !sel_ids || !sel_cnt) return CKV_ERR_INVALID_ARG;
-  const ckv_layout &L = c->layout;
-  const int kcap = budget_tokens / L.block_size;
-  if (budget_tokens <= 0 || kcap <= 0) return CKV_ERR_BUDGET_TOO_SMALL;
-  if (kcap < L.sink_blocks + L.recent_blocks && (long long)kcap * L.block_size < max_seq_len_host)
-    return CKV_ERR_BUDGET_TOO_SMALL;
-  if (!k_pool || !v_pool || !page_table || !seq_lens || !k_new || !v_new) return CKV_ERR_INVALID_ARG;
-  CkvStepPlan plan;
-  // the append rides in the step's only launch, or in the scan launch (three launches per step)
-  if (ckv_unit_step_plan(c, batch, max_seq_len_host, kcap, &plan) || ckv_scan_wants_tail(c, batch, max_seq_len_host)) {
-    const CkvNewToken fresh = {k_pool, v_pool, page_table, seq_lens, k_new, v_new};
-    return decode_impl(c, q, k_pool, v_pool, page_table, seq_lens, batch, max_seq_len_host, budget_tokens, out, lse,
-                       sel_ids, sel_cnt, (cudaStream_t)stream, nullptr, &fresh);
-  }
-  const int r = ckv_append(c, k_pool, v_pool, page_table, seq_lens, k_new, v_new, batch, stream);
-  if (r != CKV_OK) return r;
-  return ckv_decode(c, q, k_pool, v_pool, page_table, seq_lens, batch, max_seq_len_host, budget_tokens, out, lse, sel_ids,
-                    sel_cnt, stream);
+  return step_impl(c, q, k_new, v_new, k_pool, v_pool, page_table, seq_lens, batch, max_seq_len_host, budget_tokens, out, lse,
+                   sel_ids, sel_cnt, (cudaStream_t)stream, nullptr);
 }
 
 int ckv_decode_profile(ckv_ctx *c, const void *q, const void *k_pool, const void *v_pool, const int32_t *page_table,
@@ -488,6 +506,7 @@ int ckv_step_host(ckv_ctx *c, const void *q_host, const void *k_new_host, const 
                       aligned16(hq) && aligned16(hk) && aligned16(hv) && aligned16(ho) && aligned16(hi);
   const bool flagged = direct && c->host_flag != nullptr;
   int *done_count = c->dev.status + CKV_HOST_EPOCH_WORD;
+  const Route rt = route_of(c, batch, max_seq_len_host, kcap);
   // the three parts of the call as launches on `on`: inputs in, the step, results out (+ completion word)
   auto enqueue = [&](cudaStream_t on, int max_len) -> int {
     if (direct) {
@@ -497,8 +516,8 @@ int ckv_step_host(ckv_ctx *c, const void *q_host, const void *k_new_host, const 
       CKV_CUDA(cudaMemcpyAsync(dk, k_new_host, kv_bytes, cudaMemcpyHostToDevice, on));
       CKV_CUDA(cudaMemcpyAsync(dv, v_new_host, kv_bytes, cudaMemcpyHostToDevice, on));
     }
-    const int r = ckv_step(c, dq, dk, dv, k_pool, v_pool, page_table, seq_lens, batch, max_len, budget_tokens, dout, nullptr,
-                           dids, dcnt, (ckv_stream)on);
+    const int r = step_impl(c, dq, dk, dv, k_pool, v_pool, page_table, seq_lens, batch, max_len, budget_tokens, dout, nullptr,
+                            dids, dcnt, on, &rt);
     if (r != CKV_OK) return r;
     if (direct) {
       CKV_CUDA(ckv_launch_host_out(c, dout, dids, dcnt, ho, hi, hc, q_bytes, ids_bytes, cnt_bytes,
@@ -525,8 +544,8 @@ int ckv_step_host(ckv_ctx *c, const void *q_host, const void *k_new_host, const 
   // word included: nothing is staged and there is one kernel to launch (a graph of copy-in, step and copy-out took 64 us
   // a call at 128K where this takes 56 us).  Every CTA of a unit reads the unit's queries, so this is for steps whose CTAs
   // read no more than kHostReadBytes over the bus; larger ones bring the inputs in with one kernel first.
-  CkvStepPlan plan;
-  if (flagged && ckv_unit_step_plan(c, batch, max_seq_len_host, kcap, &plan)) {
+  if (flagged && rt.one) {
+    const CkvStepPlan &plan = rt.plan;
     if (!k_pool || !v_pool || !page_table || !seq_lens) return CKV_ERR_INVALID_ARG;
     if (kcap < L.sink_blocks + L.recent_blocks && (long long)kcap * L.block_size < max_seq_len_host) return CKV_ERR_BUDGET_TOO_SMALL;
     const void *sq = hq, *sk = hk, *sv = hv;
@@ -542,7 +561,8 @@ int ckv_step_host(ckv_ctx *c, const void *q_host, const void *k_new_host, const 
 
   // A caller that comes back with the same buffers and sizes (a decode loop) gets its second call captured as a
   // CUDA graph and every later one replayed: one driver call instead of five launches.  The length bound is part
-  // of the captured launches, so it is rounded up (it only has to be an upper bound) and the graph lasts 1024 steps.
+  // of the captured launches, so it is rounded up (it only has to be an upper bound) and the graph lasts 1024 steps; the
+  // arrangement is the one of the bound that was given, and part of the key.
   cudaStreamCaptureStatus cap_state = cudaStreamCaptureStatusActive;
   const bool own_stream = s != nullptr && s != cudaStreamLegacy && s != cudaStreamPerThread &&
                           cudaStreamIsCapturing(s, &cap_state) == cudaSuccess && cap_state == cudaStreamCaptureStatusNone;
@@ -550,7 +570,7 @@ int ckv_step_host(ckv_ctx *c, const void *q_host, const void *k_new_host, const 
     const int cap_tokens = L.max_blocks_per_seq * L.block_size;
     const int len_r = std::min((max_seq_len_host + 1023) / 1024 * 1024, cap_tokens);
     const void *key[10] = {q_host, k_new_host, v_new_host, out_host, sel_ids_host, sel_cnt_host, k_pool, v_pool, page_table, seq_lens};
-    const int ints[4] = {batch, len_r, budget_tokens, c->tail_mode};
+    const int ints[5] = {batch, len_r, budget_tokens, c->tail_mode, rt.tail ? 1 : 0};
     const bool same = c->hg_key_valid && memcmp(key, c->hg_key, sizeof(key)) == 0 && memcmp(ints, c->hg_ints, sizeof(ints)) == 0;
     if (same && c->hg_exec == nullptr) {   // second call in a row with this key: capture it
       const int64_t before = c->launches;

@@ -95,7 +95,7 @@ struct ckv_ctx {
   // ckv_step_host replays a captured graph when it is called again with the same buffers and sizes
   void *hg_exec;             // cudaGraphExec_t, or null
   const void *hg_key[10];    // the six host buffers, pools, page table, lengths array
-  int hg_ints[4];            // batch, rounded length bound, budget, tail mode
+  int hg_ints[5];            // batch, rounded length bound, budget, tail mode, arrangement
   int hg_launches;           // kernel launches one replay stands for
   bool hg_key_valid, hg_disabled;
 };

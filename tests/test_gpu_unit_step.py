@@ -234,3 +234,31 @@ def test_host_buffers_in_one_launch(batch, hq, hkv):
         for x, y in zip(got, (out, ids, cnt)):
             assert torch.equal(x, y.cpu()), t
     assert torch.equal(a.lens, b.lens) and a.ckv.read_status() == 0
+
+
+def test_host_buffer_calls_below_the_one_launch_length_are_arranged_alike():
+    """Bounds from 1200 tokens on a cache of 2048: the captured call rounds its bound up past the length from which one
+    launch is taken; every call is arranged by the bound it was given, and equals ckv_step bit for bit."""
+    w = workload(ctx=1200, ctx_min=None, needles=0, decode_steps=4)
+    a, b = (with_capacity(setup(w), 128) for _ in range(2))
+    for d in (a, b):
+        d.ckv.stats_build(d.k_pool, d.v_pool, d.table, d.lens, w.ctx)
+    kcap = w.budget_tokens // 16
+    pinned = [x.pin_memory() for x in (torch.zeros(2, 8, 128, dtype=torch.bfloat16), torch.zeros(2, 2, 128, dtype=torch.bfloat16),
+                                       torch.zeros(2, 2, 128, dtype=torch.bfloat16), torch.zeros(2, 8, 128, dtype=torch.bfloat16),
+                                       torch.zeros(2, 2, kcap, dtype=torch.int32), torch.zeros(2, 2, dtype=torch.int32))]
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    for t in range(4):
+        inputs = step_inputs(a, t)
+        for x, y in zip(pinned, inputs):
+            x.copy_(y)
+        before = a.ckv.launch_count()
+        with torch.cuda.stream(side):
+            a.ckv.step_host(*pinned[:3], a.k_pool, a.v_pool, a.table, a.lens, w.ctx + t + 1, w.budget_tokens, *pinned[3:])
+        assert a.ckv.launch_count() - before == 6, t   # in, append, scan, selection, attention, out
+        out, lse, ids, cnt = b.ckv.step(*inputs, b.k_pool, b.v_pool, b.table, b.lens, w.ctx + t + 1, w.budget_tokens)
+        torch.cuda.synchronize()
+        for x, y in zip(pinned[3:] + [a.lens], (out, ids, cnt, b.lens)):
+            assert torch.equal(x.cpu(), y.cpu()), t
+    assert a.ckv.read_status() == 0
