@@ -385,6 +385,7 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *q, const int *seq_lens, const bf16 *k
       tail_block<G>(P, q + (size_t)unit * G * CKV_D, page_table, fresh, unit, raw, N, s_sq, s_tail_u, &s_tail_part[0][0], s_wn[kWarps]);
     else if (lane < G)
       s_wn[kWarps][lane] = make_float4(-CUDART_INF_F, 0.f, -CUDART_INF_F, 0.f);
+    if (append && raw < 0 && rank == C - 1 && lane == 0) atomicOr(P.status, CKV_DEV_SEQ_FULL);   // no place for the token
   } else {
     // ---------------- working warps: parts of 16 blocks ----------------
     if (!RD) {

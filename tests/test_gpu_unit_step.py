@@ -103,6 +103,20 @@ def test_an_empty_and_a_full_sequence():
     assert int(d.lens[0]) == cap and d.ckv.read_status() & binding.CKV_DEV_SEQ_FULL
 
 
+@pytest.mark.parametrize("tail", [binding.CKV_TAIL_AUTO, binding.CKV_TAIL_OFF, binding.CKV_TAIL_ON])
+def test_a_negative_length_drops_the_token_in_every_arrangement(tail):
+    w = workload(ctx_min=16 * 20, decode_steps=1)
+    d = setup(w)
+    n0 = int(d.lens[0])
+    d.lens[1] = -5
+    d.ckv.set_tail_mode(tail)
+    d.ckv.stats_build(d.k_pool, d.v_pool, d.table, d.lens, d.max_len)
+    out, lse, ids, cnt = d.ckv.step(*step_inputs(d, 0), d.k_pool, d.v_pool, d.table, d.lens, w.ctx + 1, w.budget_tokens)
+    torch.cuda.synchronize()
+    assert d.lens.tolist() == [n0 + 1, -5] and d.ckv.read_status() == binding.CKV_DEV_SEQ_FULL
+    assert cnt[1].tolist() == [0, 0] and bool((out[1] == 0).all()) and bool((lse[1] == -float("inf")).all())
+
+
 def with_capacity(d, max_blocks):
     """The same cache behind page-table rows, summaries and a context for `max_blocks` blocks a sequence."""
     w, pages = d.w, max_blocks * d.w.block_size // 16
