@@ -757,7 +757,11 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *q, const int *seq_lens, const bf16 *k
         mine.ntok = (unsigned)blk < (unsigned)X ? max(min(CKV_PAGE, N - page * CKV_PAGE), 0) : 0;
         if (mine.ntok > 0) {
           mine.phys = pt_row[page];
-          if (mine.phys < 0 || mine.phys >= P.num_pages) { mine.phys = -1; bad = true; }
+          if (mine.phys < 0 || mine.phys >= P.num_pages) {   // skipped: nothing is added, and no mean row taken off
+            mine.phys = -1;
+            mine.blk = mine.blk < 0 ? mine.blk : ~mine.blk;
+            bad = true;
+          }
         }
       }
     };

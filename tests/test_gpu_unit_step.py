@@ -117,6 +117,34 @@ def test_a_negative_length_drops_the_token_in_every_arrangement(tail):
     assert cnt[1].tolist() == [0, 0] and bool((out[1] == 0).all()) and bool((lse[1] == -float("inf")).all())
 
 
+@pytest.mark.parametrize("bs,page", [(16, 0), (32, 0), (32, 1)])
+@pytest.mark.parametrize("layout", [{}, {"stat_bf16": 1}])
+def test_a_bad_page_among_the_selected_is_skipped_as_the_attention_kernel_skips_it(bs, page, layout):
+    """One page of the best-scoring block is struck from the table: the block's mean term stays in the sums or not, but it
+    does so in both arrangements."""
+    w = workload(batch=1, num_q_heads=8, num_kv_heads=2, ctx_min=None, block_size=bs, budget_tokens=bs * 6, decode_steps=0)
+    d = setup(w, **layout)
+    d.ckv.stats_build(d.k_pool, d.v_pool, d.table, d.lens, d.max_len)
+    q = torch.from_numpy(synth.queries(w, 0)).to(d.dtype).cuda()
+    call = (q, d.k_pool, d.v_pool, d.table, d.lens, d.max_len, w.budget_tokens)
+    good = [t.clone() for t in d.ckv.decode(*call)]
+    best = int(d.ckv.copy_scores(1)[0, 0, 1:w.ctx // bs - 2].argmax()) + 1
+    assert best in good[2][0, 0].tolist()
+    d.table[0, best * bs // 16 + page] = -1
+    res = []
+    for tail, launches in ((binding.CKV_TAIL_AUTO, 1), (binding.CKV_TAIL_OFF, 3)):
+        d.ckv.set_tail_mode(tail)
+        before = d.ckv.launch_count()
+        res.append([t.clone() for t in d.ckv.decode(*call)])
+        assert d.ckv.launch_count() - before == launches
+        torch.cuda.synchronize()
+        assert d.ckv.read_status() == binding.CKV_DEV_BAD_PAGE
+    assert torch.equal(res[0][2], res[1][2])
+    # log-sum-exps as close as the two arrangements are on good pages (fp32 sums in another order), rows to bf16 rounding
+    assert float((res[0][1] - res[1][1]).abs().max()) <= 1e-4 and float((res[0][1] - good[1]).abs().max()) > 1e-2
+    assert float((res[0][0].float() - res[1][0].float()).abs().max()) <= 2.0 ** -7 * float(res[1][0].float().abs().max())
+
+
 def with_capacity(d, max_blocks):
     """The same cache behind page-table rows, summaries and a context for `max_blocks` blocks a sequence."""
     w, pages = d.w, max_blocks * d.w.block_size // 16
