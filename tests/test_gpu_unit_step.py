@@ -210,6 +210,46 @@ def test_ties_at_the_cut_take_the_lowest_ids(copies):
     assert d.ckv.read_status() == 0
 
 
+@pytest.mark.parametrize("keys,X", [("spread", 1100), ("spread", 8192), ("spread", 9216), ("alike", 259), ("alike", 260),
+                                    ("alike", 8192), ("alike", 9216), ("two kinds", 5000), ("far apart", 4000)])
+@pytest.mark.parametrize("K", [4, 200, 512])
+def test_selected_ids_are_the_best_of_the_scores(keys, X, K):
+    """Exact: the ids against a stable sort of the scores the launch itself left behind.  Cuts in a bin of exactly and of more
+    than the 256 blocks that are ranked directly, and below the histogram."""
+    g = torch.Generator("cuda").manual_seed(X)
+    k, v = (torch.randn((X, 1, 16, 128), generator=g, device="cuda") for _ in range(2))
+    q = torch.randn((1, 4, 128), generator=g, device="cuda").bfloat16()
+    if keys == "alike":
+        k.copy_(k[:1].clone().expand_as(k))
+    elif keys == "two kinds":
+        k.copy_(k[torch.randint(0, 2, (X,), generator=g, device="cuda")])
+    elif keys == "far apart":   # block means far apart, keys of a block close together: e^l stays near e^(mean logit)
+        k = 0.1 * k + 30.0 * torch.randn((X, 1, 1, 128), generator=g, device="cuda")
+    k, v = k.bfloat16(), v.bfloat16()
+    ckv = binding.CompKV(4, 1, max_batch=1, max_blocks_per_seq=max(X, 1024), num_pages=X, block_size=16, sink_blocks=1,
+                         recent_blocks=2)
+    table = torch.full((1, max(X, 1024)), -1, dtype=torch.int32, device="cuda")
+    table[0, :X] = torch.arange(X, dtype=torch.int32, device="cuda")
+    lens = torch.tensor([16 * X - 3], dtype=torch.int32, device="cuda")
+    ckv.stats_build(k, v, table, lens, 16 * X)
+    before = ckv.launch_count()
+    ids, cnt = ckv.decode(q, k, v, table, lens, 16 * X, 16 * K)[2:4]
+    assert ckv.launch_count() - before == 1
+    S = ckv.copy_scores(1)[0, 0, :X]
+    torch.cuda.synchronize()
+    assert ckv.read_status() == 0
+    if K >= X:
+        assert cnt.tolist() == [[X]] and ids[0, 0].tolist() == list(range(X)) + [-1] * (K - X)
+        return
+    ranked = S[1:X - 2]
+    if keys == "alike":
+        assert bool((ranked == ranked[0]).all())
+    best = 1 + torch.sort(ranked, descending=True, stable=True).indices[:K - 3]
+    if keys == "far apart" and K == 512:   # more than 32 octaves below the largest
+        assert float(ranked[best[-1] - 1]) < 2.0 ** -33 * float(ranked.max())
+    assert cnt.tolist() == [[K]] and ids[0, 0, :K].tolist() == sorted([0, X - 2, X - 1] + best.tolist())
+
+
 def test_a_wait_that_runs_out_is_reported_and_the_context_recovers():
     w = workload(batch=1, ctx_min=None, decode_steps=0)
     d = setup(w)
