@@ -55,6 +55,7 @@ constexpr int kBins = 2048;                     // score histogram: 32 octaves b
 constexpr int kBinShift = 17;                   // ... a bin is a score's bit pattern without its low 17 bits
 constexpr int kMapWords = 2 * kWork;            // selection bit map: two words per working thread, enough for kScoresCap blocks
 constexpr int kSelCap = 512;                    // selected blocks the id list holds (unless every block is selected)
+constexpr int kOwnMost = 2800, kSeqCtas = 24;   // blocks a CTA may own where a sequence gets few CTAs (see ckv_unit_step_plan)
 constexpr int kCandCap = kWork;                 // blocks of the cut's bin that are ranked directly, one per thread
 // shared memory once the ring is drained
 constexpr int kOffHist = kScoresCap * 4;
@@ -1025,6 +1026,13 @@ cudaError_t ckv_configure_unit_step(ckv_ctx *c) {
 //   * caches under CKV_STEP_MIN_TOKENS.  Not a crossover -- one launch is the faster form there too -- but the size below
 //     which the documented two-call arrangement (append, scan, select, attention as launches of their own) is kept;
 //   * more units than CTAs run at once: a last wave that is nearly empty costs a whole wave (192 units: 92 / 90);
+//   * more than kOwnMost blocks a CTA where a sequence gets fewer than kSeqCtas of them.  The host knows the longest
+//     sequence only: alone among short ones, its few CTAs are all that works.  One launch / separate ones, 128 units of the
+//     default layout, all long, then lengths of a quarter and up, then one long and 15 of 1K: 32K 56.3 / 63.8, 49.5 / 55.3,
+//     42.2 / 34.5; 40K 66.3 / 73.0, 58.9 / 64.2, 47.6 / 35.9; 56K 84.1 / 89.8, 72.4 / 72.2, 58.7 / 39.7; one head a group,
+//     130K 147 / 161, 127 / 121, 106 / 49.  At 45K a CTA the last of the usual spread's gain goes, and the uneven batch loses a
+//     quarter.  (24 CTAs a sequence, 128K: 59.2 / 71.1, 54.8 / 63.3, 44.0 / 40.5: no line.  Groups other than 4 and 128: one
+//     launch is ahead either way, 75.0 / 143, 70.9 / 162, 68.3 / 101 at 32K with 16 of them.);
 //   * more selected blocks or scores than the shared arrays hold, or score terms that leave no room for the ring: one CTA
 //     per unit with eight heads beyond about 30K tokens.  There the persistent scan's even split of the tiles is worth
 //     more (a long sequence of a ragged batch is one CTA's work here), and its three launches are kept.
@@ -1043,6 +1051,7 @@ bool ckv_unit_step_plan(const ckv_ctx *c, int batch, int max_len, int kcap, CkvS
   auto blocks_per_cta = [C](int x) { const int parts = (std::max(x - 1, 0) + 15) / 16; return 16 * std::max((parts + C - 1) / C, 1); };
   auto term_bytes = [&P](int own) { return (size_t)(own + 8) * P.G * sizeof(float); };
   plan->own_cap = blocks_per_cta(xmax);
+  if (plan->own_cap > kOwnMost && P.Hkv * C < kSeqCtas && (P.r == 4 || P.r == CKV_D)) return false;
   if (term_bytes(plan->own_cap) + (size_t)std::max(kMinRing, skip) * stage > (size_t)kDynLimit) return false;
   const int tiles = (plan->own_cap + P.scan_tile - 1) / P.scan_tile;
   plan->stages = std::min({kStagesCap, (int)(((size_t)kDynLimit - term_bytes(plan->own_cap)) / stage), std::max(tiles, skip)});

@@ -145,13 +145,14 @@ def test_a_bad_page_among_the_selected_is_skipped_as_the_attention_kernel_skips_
     assert float((res[0][0].float() - res[1][0].float()).abs().max()) <= 2.0 ** -7 * float(res[1][0].float().abs().max())
 
 
-def with_capacity(d, max_blocks):
+def with_capacity(d, max_blocks, **layout):
     """The same cache behind page-table rows, summaries and a context for `max_blocks` blocks a sequence."""
     w, pages = d.w, max_blocks * d.w.block_size // 16
     table = torch.full((w.batch, pages), -1, dtype=torch.int32, device="cuda")
     table[:, :d.table.shape[1]] = d.table
     d.table = table
-    d.ckv = binding.CompKV(w.num_q_heads, w.num_kv_heads, w.batch, max_blocks, d.k_pool.shape[0], block_size=w.block_size)
+    d.ckv = binding.CompKV(w.num_q_heads, w.num_kv_heads, w.batch, max_blocks, d.k_pool.shape[0], block_size=w.block_size,
+                           **layout)
     return d
 
 
@@ -208,6 +209,24 @@ def test_ties_at_the_cut_take_the_lowest_ids(copies):
     rest = sorted(range(1, 898), key=lambda b: (-float(sc[b]), b))[:37]
     assert ids[0, 0].tolist() == sorted([0, 898, 899] + rest)
     assert d.ckv.read_status() == 0
+
+
+@pytest.mark.parametrize("batch,layout,launches", [(10, {}, 3), (5, {}, 1), (10, {"var_groups": 16}, 1)])
+def test_a_long_bound_with_few_ctas_a_sequence_takes_separate_launches(batch, layout, launches):
+    """From 2801 blocks a CTA on (80 units: one CTA each, eight a sequence) the host's bound decides; 40 units get 24 CTAs a
+    sequence, and with 16 groups one launch is always ahead.  Same ids, and rows to bf16 rounding, on either side."""
+    w = workload(batch=batch, num_q_heads=32, num_kv_heads=8, ctx=16 * 100, ctx_min=16 * 20, needles=1, decode_steps=0)
+    d = with_capacity(setup(w), 3000, **layout)
+    d.ckv.stats_build(d.k_pool, d.v_pool, d.table, d.lens, w.ctx)
+    q = torch.from_numpy(synth.queries(w, 0)).to(d.dtype).cuda()
+    res = []
+    for blocks, n in ((2801, 1), (2802, launches)):   # the last block is nobody's
+        before = d.ckv.launch_count()
+        res.append([t.clone() for t in d.ckv.decode(q, d.k_pool, d.v_pool, d.table, d.lens, 16 * blocks, w.budget_tokens)])
+        assert d.ckv.launch_count() - before == n
+    torch.cuda.synchronize()
+    assert d.ckv.read_status() == 0 and torch.equal(res[0][2], res[1][2]) and torch.equal(res[0][3], res[1][3])
+    assert float((res[0][0].float() - res[1][0].float()).abs().max()) <= 2.0 ** -7 * float(res[0][0].float().abs().max())
 
 
 @pytest.mark.parametrize("keys,X", [("spread", 1100), ("spread", 8192), ("spread", 9216), ("alike", 259), ("alike", 260),
