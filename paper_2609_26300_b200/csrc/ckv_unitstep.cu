@@ -56,6 +56,7 @@ constexpr int kBinShift = 17;                   // ... a bin is a score's bit pa
 constexpr int kMapWords = 2 * kWork;            // selection bit map: two words per working thread, enough for kScoresCap blocks
 constexpr int kSelCap = 512;                    // selected blocks the id list holds (unless every block is selected)
 constexpr int kOwnMost = 2800, kSeqCtas = 24;   // blocks a CTA may own where a sequence gets few CTAs (see ckv_unit_step_plan)
+constexpr long long kIdleMost = 80000000;   // bytes: selected keys and values times the share of SMs without a CTA (see ckv_unit_step_plan)
 constexpr int kCandCap = kWork;                 // blocks of the cut's bin that are ranked directly, one per thread
 // shared memory once the ring is drained
 constexpr int kOffHist = kScoresCap * 4;
@@ -1037,6 +1038,12 @@ cudaError_t ckv_configure_unit_step(ckv_ctx *c) {
 //     130K 147 / 161, 127 / 121, 106 / 49.  At 45K a CTA the last of the usual spread's gain goes, and the uneven batch loses a
 //     quarter.  (24 CTAs a sequence, 128K: 59.2 / 71.1, 54.8 / 63.3, 44.0 / 40.5: no line.  Groups other than 4 and 128: one
 //     launch is ahead either way, 75.0 / 143, 70.9 / 162, 68.3 / 101 at 32K with 16 of them.);
+//   * large selections where the clusters leave SMs idle (selected bytes x idle share from kIdleMost on): the attention is most
+//     of such a step, and a launch of its own keeps the whole chip at it.  One launch / separate ones / the product: 80 units
+//     (68 SMs idle) 4K tokens of 32K 73.8 / 68.3 / 77 MB, 8K of 16K 95.8 / 81.7 / 154, 32K of 40K 290 / 216 / 616; 104 units
+//     8K of 16K 103.3 / 99.5 / 130; 128 units 8K of 16K 104.6 / 104.7 / 72, 16K of 40K 189 / 184 / 145.  Not where the
+//     attention's own clusters fill more than nine tenths of their places, two a SM, and no longer pack: 72 units in
+//     clusters of 4 (288 CTAs), 32K of 40K 205 / 256;
 //   * more selected blocks or scores than the shared arrays hold, or score terms that leave no room for the ring: one CTA
 //     per unit with eight heads beyond about 30K tokens.  There the persistent scan's even split of the tiles is worth
 //     more (a long sequence of a ragged batch is one CTA's work here), and its three launches are kept.
@@ -1049,6 +1056,11 @@ bool ckv_unit_step_plan(const ckv_ctx *c, int batch, int max_len, int kcap, CkvS
   for (int k = CKV_STEP_MAX_CLUSTER; k >= 1 && C == 0; --k)
     if (c->step_clusters[k] >= units) C = k;
   if (C == 0) return false;
+  if (kcap < xmax) {
+    const int sms = c->sm_count, splits = std::min(std::max(2 * sms / units, 1), 8);   // as ckv_launch_attn splits it
+    const long long selected = (long long)units * kcap * P.bs * (2 * CKV_D * 2), idle = std::max(sms - C * units, 0);
+    if (selected * idle >= kIdleMost * sms && splits * units * 10 <= 2 * sms * 9) return false;
+  }
   const int skip = kWarps / (P.scan_tile / 16);
   const size_t krow = (size_t)P.row_elems * 2, vrow = (P.vhi || P.row_elems == CKV_D) ? (size_t)CKV_D * 2 : krow;
   const size_t stage = (size_t)P.scan_tile * (krow + vrow) + (P.r >= 4 ? (size_t)P.scan_tile * P.r * 4 : 0);

@@ -238,6 +238,27 @@ def test_a_long_bound_with_few_ctas_a_sequence_takes_separate_launches(batch, la
     assert float((res[0][0].float() - res[1][0].float()).abs().max()) <= 2.0 ** -7 * float(res[0][0].float().abs().max())
 
 
+@pytest.mark.parametrize("batch,hkv,blocks,launches", [(10, 8, 66, 1), (10, 8, 67, 3), (16, 8, 141, 1), (16, 8, 142, 3), (9, 8, 512, 1)])
+def test_large_selections_beside_idle_sms_take_separate_launches(batch, hkv, blocks, launches):
+    """Selected bytes times the share of SMs without a CTA: 64-token blocks, 80 units (68 SMs idle) on either side of the
+    line, 128 units on either side, and 72 units, whose attention clusters do not pack.  The bound is long, the lengths are
+    short (every block is selected): same rows as the separate launches to bf16 rounding."""
+    w = workload(batch=batch, num_q_heads=4 * hkv, num_kv_heads=hkv, ctx=64 * 30 + 9, ctx_min=64 * 20, block_size=64, needles=1,
+                 budget_tokens=64 * 8, decode_steps=0)
+    d = with_capacity(setup(w), 600)
+    d.ckv.stats_build(d.k_pool, d.v_pool, d.table, d.lens, w.ctx)
+    q = torch.from_numpy(synth.queries(w, 0)).to(d.dtype).cuda()
+    res = []
+    for tail, n in ((binding.CKV_TAIL_AUTO, launches), (binding.CKV_TAIL_OFF, 3)):
+        d.ckv.set_tail_mode(tail)
+        before = d.ckv.launch_count()
+        res.append([t.clone() for t in d.ckv.decode(q, d.k_pool, d.v_pool, d.table, d.lens, 64 * 600, 64 * blocks)])
+        assert d.ckv.launch_count() - before == n
+    torch.cuda.synchronize()
+    assert d.ckv.read_status() == 0 and torch.equal(res[0][2], res[1][2]) and torch.equal(res[0][3], res[1][3])
+    assert float((res[0][0].float() - res[1][0].float()).abs().max()) <= 2.0 ** -7 * float(res[0][0].float().abs().max())
+
+
 @pytest.mark.parametrize("keys,X", [("spread", 1100), ("spread", 8192), ("spread", 9216), ("alike", 259), ("alike", 260),
                                     ("alike", 8192), ("alike", 9216), ("two kinds", 5000), ("far apart", 4000)])
 @pytest.mark.parametrize("K", [4, 200, 512])
