@@ -6,6 +6,8 @@
 // first, then deviations from it) over a page of rows held in registers; the pages of a longer
 // block are joined pairwise (ckv_blockstats.cuh).  Build, append and chunked prefill run the same
 // operations in the same order, so their results are bit-identical.
+#include <algorithm>
+
 #include "ckv_internal.cuh"
 #include "ckv_blockstats.cuh"
 #include "ckv_pipe.cuh"
@@ -15,21 +17,23 @@ namespace {
 constexpr int kBuildRounds = 8;   // blocks per warp of the build kernel, at most
 constexpr int kPrefillRounds = 4; // blocks per warp of the prefill kernel's register-resident variants, at most
 
-// Blocks per warp of a launch over `units` units of `blocks` blocks each (CTAs of eight warps, two CTAs per SM).  All CTAs
-// take about the same time, so a launch takes waves * rounds of it, and what is lost is the last wave: 2K-token chunks of
-// one sequence with four rounds 133 us, with one 69; 8K chunks of two sequences 125 us with four (one wave, in lockstep),
-// 136 with three (1.2 waves), 116 with two; 9K caches of 32-token blocks 46 us with eight rounds, 39 with two.  Among equals
-// the most rounds (fewest CTAs to start) that still leave two waves to overlap, else the fewest.
-int rounds_for(int blocks, int units, int sms, int most) {
-  int best = 1;
-  long long best_cost = 0;
-  bool best_two = false;
-  for (int r = 1; r <= most; ++r) {
+// Blocks per warp of a launch over `units` units of `blocks` blocks of `ppb` pages each (CTAs of eight warps, two CTAs per
+// SM).  A launch takes waves * rounds block times, and what is lost is the last wave; on top of that a CTA costs about a
+// third of a page's time to start, working or not, which is most of a ragged batch's time when CTAs are small (stats_build
+// of 16 sequences: 32K each 382 us with one round, 354 with eight; one of 32K and 15 of 1K 90.8 and 49.9).  A single wave
+// runs in lockstep and counts a tenth more (8K chunks of two sequences 125 us in one, 116 in two).  Of several sequences,
+// among what is within five hundredths of the least, the fewest rounds: short ones then leave fewer warps idle (16 x 2K
+// 26.5 us with four rounds and 25.9 with eight; one of 2K and 15 of 1K 11.4 and 18.3).
+int rounds_for(int blocks, int batch, int units, int ppb, int sms, int most) {
+  auto cost = [&](int r) {
     const long long ctas = (long long)((blocks + 8 * r - 1) / (8 * r)) * units, waves = (ctas + 2 * sms - 1) / (2 * sms);
-    const long long cost = waves * r;
-    if (r == 1 || cost < best_cost || (cost == best_cost && waves >= 2 && best_two)) { best = r; best_cost = cost; best_two = waves >= 2; }
-  }
-  return best;
+    return (double)waves * (r + 0.3 / ppb) * (waves == 1 && r > 1 ? 1.1 : 1.0);
+  };
+  double least = cost(1);
+  for (int r = 2; r <= most; ++r) least = std::min(least, cost(r));
+  int r = 1;
+  while (cost(r) > (batch > 1 ? 1.05 : 1.0) * least) ++r;
+  return r;
 }
 
 // A warp takes `rounds` blocks, eight blocks apart (rounds_for).  Two CTAs per SM: the block routine holds a page's 16 key and
@@ -319,7 +323,7 @@ cudaError_t ckv_launch_stats_build(ckv_ctx *c, const void *k_pool, const void *v
   const int xmax = (max_len + P.bs - 1) / P.bs;
   if (xmax <= 0 || batch <= 0) return cudaSuccess;
   const int sms = c->sm_count > 0 ? c->sm_count : 148;
-  const int rounds = rounds_for(xmax, batch * P.Hkv, sms, kBuildRounds);
+  const int rounds = rounds_for(xmax, batch, batch * P.Hkv, P.ppb, sms, kBuildRounds);
   dim3 grid((xmax + 8 * rounds - 1) / (8 * rounds), batch * P.Hkv);
   cudaError_t e;
   if (c->layout.kv_dtype == CKV_BF16 && P.ppb == 1)
@@ -340,7 +344,7 @@ cudaError_t ckv_launch_prefill(ckv_ctx *c, void *k_pool, void *v_pool, const int
   const int touched = (max_new + P.bs - 1) / P.bs + 1;   // a chunk that starts inside a block touches one more
   dim3 grid((touched + 7) / 8, batch * P.Hkv);
   const int sms = c->sm_count > 0 ? c->sm_count : 148;
-  const int rounds = rounds_for(touched, batch * P.Hkv, sms, kPrefillRounds);
+  const int rounds = rounds_for(touched, batch, batch * P.Hkv, P.ppb, sms, kPrefillRounds);
   const dim3 grid_one((touched + 8 * rounds - 1) / (8 * rounds), batch * P.Hkv);
   cudaError_t e;
   if (c->layout.kv_dtype == CKV_BF16 && P.ppb == 1)

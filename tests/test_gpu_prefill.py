@@ -124,3 +124,28 @@ def test_prefill_and_build_with_several_blocks_per_warp(batch, tokens, bs):
             assert torch.equal(a[s, :, :x], b[s, :, :x])
         want = k_src[s, :full * bs].view(full, bs, hkv, 128).double().mean(1).transpose(0, 1)
         assert float((got[0][s, :, :full].double() - want).abs().max()) <= 64 * 6 * 2.0 ** -24 + 6 * 2.0 ** -18
+
+
+@pytest.mark.parametrize("bs", [16, 32, 64])
+@pytest.mark.parametrize("bound", [4096, 16384, 65536])
+def test_build_of_a_long_sequence_among_short_ones(bs, bound):
+    """The blocks a warp takes follow from the host's bound and the batch: every sequence's summaries are those of a build
+    of that sequence alone, whatever the bound."""
+    w = small(batch=9, block_size=bs, ctx=16 * 90 + 11, ctx_min=5)
+    d = setup(w)
+    d.ckv.stats_build(d.k_pool, d.v_pool, d.table, d.lens, d.max_len)
+    ref = [t.clone() for t in d.ckv.export_stats(w.batch)]
+    blocks = bound // bs
+    from paper_2609_26300_b200 import binding
+    table = torch.full((w.batch, bound // 16), -1, dtype=torch.int32, device="cuda")
+    table[:, :d.table.shape[1]] = d.table
+    ckv = binding.CompKV(8, 2, w.batch, blocks, d.k_pool.shape[0], block_size=bs)
+    ckv.stats_build(d.k_pool, d.v_pool, table, d.lens, bound)
+    got = ckv.export_stats(w.batch)
+    one = binding.CompKV(8, 2, 1, blocks, d.k_pool.shape[0], block_size=bs)
+    for s in range(w.batch):
+        n = -(-int(d.lens[s]) // bs)
+        one.stats_build(d.k_pool, d.v_pool, table[s:s + 1].contiguous(), d.lens[s:s + 1].contiguous(), int(d.lens[s]))
+        for x, y, z in zip(ref, got, one.export_stats(1)):
+            assert torch.equal(x[s, :, :n], y[s, :, :n]) and torch.equal(x[s, :, :n], z[0, :, :n])
+    assert d.ckv.read_status() == 0 and ckv.read_status() == 0 and one.read_status() == 0
