@@ -104,8 +104,8 @@ struct ckv_ctx {
 // kernel calls pdl_wait() before it touches global memory.  Gaps of 2 to 3 us between kernels all but vanish (prefill chunks
 // 129 -> 124 us, the three-launch step of 128 units 87.4 -> 80.7).  pdl_trigger() lets the next kernel's CTAs in before this
 // one's are done: good where the next one is alike (builds, chunks, dense passes, one-launch steps), bad among the scan,
-// selection and attention kernels, whose CTAs then sit on SMs that the running kernel still needs (80.7 -> 92.3): those do
-// not call it.  cluster_x: CTAs of a cluster (0: no clusters).
+// selection and attention kernels, whose CTAs then sit on SMs that the running kernel still needs (80.7 -> 92.3), and in
+// the append ahead of a scan (steps of one 500-token sequence 17.5 -> 19.2): those do not call it.  cluster_x: CTAs of a cluster (0: no clusters).
 // Whatever such a kernel reads may have been written while it was already running, by the launch ahead of it: its loads
 // promise nothing (no __ldg, no const __restrict__), or the compiler may take them for invariant and move them up past
 // pdl_wait().  The plain loads measure the same.

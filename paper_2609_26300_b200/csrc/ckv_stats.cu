@@ -72,7 +72,6 @@ __global__ void __launch_bounds__(256) ckv_append_kernel(CkvDev P, T *k_pool, T 
   __shared__ float sq_smem[8][CKV_D];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
   const int s = blockIdx.x;
-  ckv_pipe::pdl_trigger();
   ckv_pipe::pdl_wait();
   const int N = seq_lens[s];
   // the new row of this warp's first head does not depend on N: it is requested together with it, so that the
