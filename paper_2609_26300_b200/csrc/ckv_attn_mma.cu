@@ -39,10 +39,11 @@
 
 namespace {
 
-constexpr int kMeanSlots = 4;                         // mean-value rows (512 B each) a warp can hold
+constexpr int kMeanRow = CKV_D * 2;                    // a stored mean-value row of the bf16 summaries
+constexpr int kMeanSlots = 4;                         // ... of which a warp can hold this many
 constexpr int kMeanFlush = 3;                         // ... of which at most 3 wait for removal while one is in flight
-constexpr int kZeroRow = kMeanSlots * 512;            // offset of the row of zeros inside the aux area
-constexpr int kLsOff = kZeroRow + 256;                // then log2 of the blocks' mean-compensation weights: [slot][G] float
+constexpr int kZeroRow = kMeanSlots * kMeanRow;           // offset of the row of zeros inside the aux area
+constexpr int kLsOff = kZeroRow + kMeanRow;               // then log2 of the blocks' mean-compensation weights: [slot][G] float
 constexpr int kAuxBytes = kLsOff + 256;
 constexpr int kMaxEntries = 32;                       // partials a CTA folds per round: one per lane
 constexpr int kPartBytes = CKV_PART_STRIDE * 4;       // one head's partial
@@ -168,7 +169,6 @@ ckv_attn_mma_kernel(CkvDev P, const __nv_bfloat16 *q, const __nv_bfloat16 *k_poo
   const int n_mine = max((p1 - p0 - warp + W - 1) / W, 0);   // this warp's pages: list index p0 + warp + W n
   const float *lz = P.lz + (size_t)unit * P.max_blocks * G;
   const __nv_bfloat16 *vmean = P.vmean + (size_t)unit * P.max_blocks * P.row_elems;
-  const bool mean_lo = P.row_elems == CKV_ROW_ELEMS;   // the mean-value rows carry lo halves (fp32-precision summaries)
   // How a selected block's mean term |b| e^{zbar} vbar_b (part of the scan's all-block sum) is taken out again.
   // vbar_b is the mean of the block's value rows, so with full-precision summaries it is enough to lower the weight
   // of each of the block's tokens by e^{zbar}: sum_j (p_j - e^{zbar}) v_j = sum_j p_j v_j - |b| e^{zbar} vbar_b up to
@@ -248,9 +248,8 @@ ckv_attn_mma_kernel(CkvDev P, const __nv_bfloat16 *q, const __nv_bfloat16 *k_poo
       const uint32_t kb = wtiles_u32 + buf * kPageBytes;
       const uint32_t vb = kb + kTileBytes;
       issue_page(kb, vb, k_pool + src, v_pool + src, r.ntok, lane);
-      if (row_rm && r.first) {   // verbatim: hi halves then lo halves, swizzled by block index
-        if (mean_lo || lane < 16)
-          cp_async16(aux_u32 + 512 * slot + 16 * lane, vmean + (size_t)r.blk * P.row_elems + 8 * lane, true);
+      if (row_rm && r.first) {   // verbatim: swizzled by block index
+        if (lane < 16) cp_async16(aux_u32 + kMeanRow * slot + 16 * lane, vmean + (size_t)r.blk * CKV_D + 8 * lane, true);
         if (lane < G)          // and log2 of the weight of its mean term, for every head
           cp_async4(aux_u32 + kLsOff + (slot * G + lane) * 4, lz + (size_t)lane * P.max_blocks + r.blk);
       }
@@ -290,7 +289,7 @@ ckv_attn_mma_kernel(CkvDev P, const __nv_bfloat16 *q, const __nv_bfloat16 *k_poo
     const bool real = r < nb;
     const int rblk = r == 0 ? bb[0] : (r == 1 ? bb[1] : bb[2]);
     const int rslot = r == 0 ? bsl[0] : (r == 1 ? bsl[1] : bsl[2]);
-    const uint32_t rowaddr = aux_u32 + 512 * (real ? rslot : 0);
+    const uint32_t rowaddr = aux_u32 + kMeanRow * (real ? rslot : 0);
 #pragma unroll
     for (int t = 0; t < 8; ++t) {
       uint32_t v[4];

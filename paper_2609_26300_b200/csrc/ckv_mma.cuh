@@ -46,7 +46,6 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<const uint32_t *>(&v);
 }
-__device__ __forceinline__ float bf16_round(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
 
 // Which (row, head) pairs of a tile a lane works on: rows row(lane, k), k < NR, heads head(lane, 0) and head(lane, 1)
 // (beyond G: the lane's values are padding).  `copy` lanes hold the same heads as the lane two below, for other rows.
