@@ -174,6 +174,8 @@ int ckv_append(ckv_ctx *ctx, void *k_pool, void *v_pool, const int32_t *page_tab
  *   out:     attention output, kv_dtype (fp32 accumulation, rounded once; App. D.1).
  *   sel_ids: selected block ids per unit in position order; sel_cnt their number.
  * The cache is read through page_table; summaries must be current (build / append).
+ * max_seq_len_host: an upper bound (host) on seq_lens[s].  A sequence that is longer all the same is worked on in full
+ * where the step's shared memory holds the cache's capacity; otherwise CKV_DEV_BAD_BOUND is set.
  * Returns CKV_ERR_BUDGET_TOO_SMALL when K < sink_blocks + recent_blocks and K * block_size <
  * max_seq_len_host (some sequence could not hold its mandatory blocks). */
 int ckv_decode(ckv_ctx *ctx, const void *q, const void *k_pool, const void *v_pool,
@@ -200,8 +202,9 @@ int ckv_prefill(ckv_ctx *ctx, void *k_pool, void *v_pool, const int32_t *page_ta
  * ckv_append(k_new, v_new) followed by ckv_decode(q, ...), bit for bit (Sec. 4.3: the new token enters the cache
  * and the summaries before blocks are selected; seq_lens holds N on entry and N + 1 once the step has run;
  * max_seq_len_host bounds the lengths after the append).  Where a unit's blocks fit a thread-block cluster (bf16 pages,
- * caches of 1536 tokens and more, as many units as clusters run at once) the whole step is ONE launch, and ckv_decode is
- * the same launch without a new token.  Otherwise it is three launches on long scans: a step can only change the last
+ * caches of 1536 tokens and more, as many units as clusters run at once, and neither a bound so long that the few CTAs of a
+ * sequence would scan it alone nor a selection so large that the SMs the clusters leave idle are needed for it) the whole
+ * step is ONE launch, and ckv_decode is the same launch without a new token.  Otherwise it is three launches on long scans: a step can only change the last
  * block of a sequence, so a few CTAs of the scan launch write the new rows and redo that block's summary while the other
  * CTAs stream the summaries of all the other blocks; seq_lens is updated inside that launch, after every CTA has read
  * it.  (Short scans and batches above 1024 sequences take the two-call route.)  The decode arguments are

@@ -541,9 +541,10 @@ int ckv_step_host(ckv_ctx *c, const void *q_host, const void *k_new_host, const 
   };
 
   // A step that is one launch reads its inputs from the pinned buffers and writes its results there itself, completion
-  // word included: nothing is staged and there is one kernel to launch (a graph of copy-in, step and copy-out took 64 us
-  // a call at 128K where this takes 56 us).  Every CTA of a unit reads the unit's queries, so this is for steps whose CTAs
-  // read no more than kHostReadBytes over the bus; larger ones bring the inputs in with one kernel first.
+  // word included: nothing is staged and there is one kernel to launch (a graph of copy-in, step and copy-out took 76 us
+  // a call at 128K where this takes 57 to 59).  Every CTA of a unit reads the unit's queries over the bus; past kHostReadBytes
+  // a kernel brings the inputs in first, in a launch of its own.  That is the documented count of launches and not a
+  // crossover: read over the bus / copied first, 38.0 / 38.8 us a call (128 KB), 42.8 / 43.2 (256 KB), 47.3 / 50.6 (288 KB).
   if (flagged && rt.one) {
     const CkvStepPlan &plan = rt.plan;
     if (!k_pool || !v_pool || !page_table || !seq_lens) return CKV_ERR_INVALID_ARG;

@@ -412,8 +412,9 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *q, const int *seq_lens, const bf16 *k
   } else {
     // ---------------- working warps: parts of 16 blocks ----------------
     if (!RD) {
-      // w_{g,t} of Eq. 8 times the squared logit scale, summed in coordinate order as every kernel does it: scores that
-      // differ in the last bit can swap blocks at the cut.  (The first tile's data is still on its way.)
+      // w_{g,t} of Eq. 8 times the squared logit scale, summed in coordinate order as the scan kernel sums the weights it
+      // stages (those of a CTA's later units it sums in runs of eight): scores that differ in the last bit can swap blocks
+      // at the cut.  (The first tile's data is still on its way.)
       for (int i = tid; i < P.r * G; i += kWork) {
         const int g = i & (G - 1), t = i / G, gs = CKV_D / P.r, run = P.glayout == 0 ? gs : gs / 2;
         float a = 0.f;
@@ -1023,13 +1024,14 @@ cudaError_t ckv_configure_unit_step(ckv_ctx *c) {
 }
 
 // Whether a step of this size runs as one launch, and how.  Against the separate launches (us per step, back to back):
-// 14.3 / 27.4 (one head, 4K), 16.7 / 35.8 (8 units, 32K), 21.9 / 38.6 (8 units, 128K, 32-token blocks), 31.5 / 51.2 (24
-// units, 100K, bf16 summaries), 41.3 / 60.3 (16 units, 88K, r = d), 53.4 / 68.4 (32 units, 128K), 60 / 70 (64 units, 64K),
-// 61 / 81 (72 units, 58K), 95 / 147 (80 units, r = 16), 73 / 80 (88 units of 14K, r = d), 69 / 81 (128 units, 32K).
+// 12.9 / 27.4 (one head, 4K), 15.4 / 35.8 (8 units, 32K), 20.3 / 38.6 (8 units, 128K, 32-token blocks), 30.0 / 51.2 (24
+// units, 100K, bf16 summaries), 40.5 / 60.3 (16 units, 88K, r = d), 52.4 / 68.4 (32 units, 128K), 54.6 / 69.1 (72 units,
+// 64K), 56.3 / 63.8 (128 units, 32K).
 // What stays with the separate launches, and why:
 //   * fp32 pages (the attention is on bf16 tensor cores) and an explicit ckv_set_tail_mode, which asks for them;
-//   * caches under CKV_STEP_MIN_TOKENS.  Not a crossover -- one launch is the faster form there too -- but the size below
-//     which the documented two-call arrangement (append, scan, select, attention as launches of their own) is kept;
+//   * caches under CKV_STEP_MIN_TOKENS.  Not a crossover -- one launch is ahead there too (one sequence of 500 tokens 15.0 /
+//     21.1, 16 of 1000 17.5 / 26.4) -- but the size below which the documented two-call arrangement (append, scan, select,
+//     attention as launches of their own) is kept;
 //   * more units than CTAs run at once: a last wave that is nearly empty costs a whole wave (192 units: 92 / 90);
 //   * more than kOwnMost blocks a CTA where a sequence gets fewer than kSeqCtas of them.  The host knows the longest
 //     sequence only: alone among short ones, its few CTAs are all that works.  One launch / separate ones, 128 units of the

@@ -393,3 +393,11 @@ def test_host_buffer_calls_below_the_one_launch_length_are_arranged_alike():
         for x, y in zip(pinned[3:] + [a.lens], (out, ids, cnt, b.lens)):
             assert torch.equal(x.cpu(), y.cpu()), t
     assert a.ckv.read_status() == 0
+
+
+def test_the_stream_handle_read_directly_is_the_public_one():
+    """The binding reads the current stream's handle through torch's internals where they exist (3 us a call less)."""
+    side = torch.cuda.Stream()
+    assert binding._raw_stream() == binding._public_stream()
+    with torch.cuda.stream(side):
+        assert binding._raw_stream() == binding._public_stream() == binding._stream() == side.cuda_stream
