@@ -37,6 +37,8 @@ PAPER_CONTEXT = {"speedup_vs_full": 6.85, "hardware": "NVIDIA H100 80GB HBM3, CP
 # (profiles/ckv_scan_kernel_llama8b_128k_b4.md): 206.06 MB read + 10.15 MB written for the 205.5 MB of summaries the
 # step reads (mean keys hi + lo, mean values hi, variances).
 SCAN_TRAFFIC_RATIO = (206.06 + 10.15) / 205.5
+# The same for the one-launch step (profiles/ckv_unit_step_kernel_llama8b_128k_b2.md).
+STEP_TRAFFIC_RATIO = 124.5 / 119.6
 # What is stored and multiplied (the line's `dtype`): K/V pages are bf16; mean keys and mean values keep fp32
 # precision as split bf16 pairs (hi = bf16(x), lo = bf16(x - hi), relative error <= 2^-18), variances are fp32; the
 # decode step reads the mean keys as pairs and the mean values as their hi halves; the contractions run on bf16
@@ -602,6 +604,18 @@ def main():
     req = stats_b + sel_b
     step_gbs = req / (us_per_step * 1e-6) / 1e9
     scan_gbs = stats_b / (scan_us * 1e-6) / 1e9
+    # the dominant kernel of the timed step: its only launch where the step is one, else the scan
+    one = launches_per_step == 1
+    dom_gbs = req / (pipe_us * 1e-6) / 1e9 if one else scan_gbs
+    roofline = {"kernel": "ckv_unit_step_kernel" if one else "ckv_scan_kernel", "bound": "hbm", "achieved": dom_gbs,
+                "peak": peak, "peak_kind": "%s copy bandwidth" % peak_kind, "unit": "GB/s", "frac": dom_gbs / peak,
+                "frac_step": step_gbs / peak, "frac_step_of_nominal_8TBs": step_gbs / NOMINAL_HBM_GBS,
+                "frac_step_note": "the timed step (one graph replay per event pair, cold L2) on its required bytes; `frac` is "
+                                  + ("its only kernel, replayed back to back" if one else "its scan launch alone"),
+                "algorithmic_bytes": req if one else stats_b, "launch_us": pipe_us if one else scan_us,
+                "traffic": (STEP_TRAFFIC_RATIO * req if one else SCAN_TRAFFIC_RATIO * stats_b),
+                "traffic_source": "DRAM bytes per algorithmic byte in one ncu capture (profiles/ckv_unit_step_kernel_llama8b_128k_b2.md: "
+                                  "124.5 MB for 119.6 MB)" if one else "see scan_launch"}
     line = {
         "metric": METRIC if is_default else "sparse decode-attn us/step (append + decode)", "value": us_per_step, "unit": UNIT, "n_gpus": world, "steps": K, "warmup": W,
         "ms_per_step": ms_per_step, "higher_is_better": False, "scaling": "weak", "vs_baseline": None,
@@ -636,14 +650,12 @@ def main():
                               "the kernels; the timed ckv_step does the same work in one launch at this size"},
         "prefill": prefill,
         "stats_build": {"us": build_us, "gbs": build_bytes / (build_us * 1e-6) / 1e9, "bytes": build_bytes},
-        "roofline": {"kernel": "ckv_scan_kernel", "bound": "hbm", "achieved": scan_gbs, "peak": peak,
-                     "peak_kind": "%s copy bandwidth" % peak_kind, "unit": "GB/s", "frac": scan_gbs / peak,
-                     "frac_step": step_gbs / peak, "frac_step_of_nominal_8TBs": step_gbs / NOMINAL_HBM_GBS,
-                     "frac_step_note": "the whole step (scan, select, attention + merge) on its required bytes; "
-                                       "`frac` is the dominant kernel alone",
-                     "scan_form": "the launch timed here is the decode-only form (its tail CTAs redo the last "
-                                  "block's terms but append nothing); in the timed step the same launch also "
-                                  "appends the new token",
+        "roofline": roofline,
+        "scan_launch": {"kernel": "ckv_scan_kernel", "achieved": scan_gbs, "peak": peak, "unit": "GB/s",
+                     "frac": scan_gbs / peak,
+                     "note": "the summary scan as a launch of its own, decode-only form (its tail CTAs redo the last "
+                             "block's terms but append nothing); a step of separate launches runs it, one of a single "
+                             "launch does not",
                      "algorithmic_bytes": stats_b, "launch_us": scan_us,
                      "timing": "average of 16 back-to-back launches between two CUDA events on the launching stream "
                                "(median of 5 such runs); inside an eager step, between events, the same kernel "
