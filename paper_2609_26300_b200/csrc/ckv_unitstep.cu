@@ -50,7 +50,8 @@ constexpr int kThreads = (kWarps + 2) * 32;
 constexpr int kClusterCap = CKV_STEP_MAX_CLUSTER;
 constexpr int kStagesCap = 6;
 constexpr int kMinRing = 3;                     // ring stages that the score terms have to leave room for
-constexpr int kScoresCap = 9216;                // blocks of a unit whose scores every CTA can hold
+constexpr int kScoresCap = 9216;                // blocks of a unit whose scores every CTA can hold (147K tokens in 16-token blocks; the bit
+                                                // map and the memory would take 16384, longer units have not been tried)
 constexpr int kBins = 2048;                     // score histogram: 32 octaves below the largest possible score, 64 bins each
 constexpr int kBinShift = 17;                   // ... a bin is a score's bit pattern without its low 17 bits
 constexpr int kMapWords = 2 * kWork;            // selection bit map: two words per working thread, enough for kScoresCap blocks
