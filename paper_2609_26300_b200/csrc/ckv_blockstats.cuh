@@ -24,25 +24,32 @@ __device__ __forceinline__ float split_value(float x, bool lo_half) {
 // Second half of the block routine, shared by its variants: the half warps' squared deviations are combined, the
 // three summary rows are written (hw 0: mean key and variances, hw 1: mean value).  km: mean key, vs: value sums,
 // sq: this half warp's squared deviations, all for the lane's 8 coordinates.
+// KEYS / VALS: a caller that has split a block between two warps finishes the keys (mean and variances) or the values
+// alone; the warp with the keys then holds the mean key in both half warps.
+template <bool KEYS = true, bool VALS = true>
 __device__ __forceinline__ void block_stats_finish(const CkvDev &P, int b, float fc, const float (&km)[8],
                                                    const float (&vs)[8], float (&sq)[8], float *sq_smem,
                                                    __nv_bfloat16 *kmean_row, float *dbar_row,
                                                    __nv_bfloat16 *vmean_row, int lane, bool bad, BlockRow *keep = nullptr) {
   const int hw = lane >> 4, li = lane & 15;
   const float inv = 1.0f / fc;
+  if constexpr (KEYS) {
 #pragma unroll
-  for (int i = 0; i < 8; ++i) sq[i] += __shfl_xor_sync(0xffffffffu, sq[i], 16);
+    for (int i = 0; i < 8; ++i) sq[i] += __shfl_xor_sync(0xffffffffu, sq[i], 16);
+  }
   // the two mean rows leave through one store routine: half warp 0 writes the mean key, half warp 1 the mean value
   {
+    const bool key = KEYS && (!VALS || hw == 0);
     float rowv[8];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) rowv[i] = hw == 0 ? km[i] : vs[i] * inv;
-    store_split8(hw == 0 ? kmean_row : vmean_row, li, b, rowv, P.row_elems == CKV_ROW_ELEMS);
+    for (int i = 0; i < 8; ++i) rowv[i] = key ? km[i] : vs[i] * inv;
+    if ((KEYS && VALS) || hw == (KEYS ? 0 : 1)) store_split8(key ? kmean_row : vmean_row, li, b, rowv, P.row_elems == CKV_ROW_ELEMS);
     if (keep != nullptr) {
 #pragma unroll
-      for (int i = 0; i < 8; ++i) keep->x[i] = split_value(rowv[i], P.row_elems == CKV_ROW_ELEMS && !(hw == 1 && P.vhi));
+      for (int i = 0; i < 8; ++i) keep->x[i] = split_value(rowv[i], P.row_elems == CKV_ROW_ELEMS && (key || !P.vhi));
     }
   }
+  if constexpr (!KEYS) return;
   const int gs = CKV_D / P.r;
   const int run = P.glayout == 0 ? gs : gs / 2;   // consecutive coordinates of a group (two runs, 64 apart, in layout 1)
   if (P.r == CKV_D) {
@@ -128,7 +135,8 @@ __device__ __forceinline__ void combine_pages(float &na, float (&mean)[8], float
 // that has such a block's rows in registers uses this one routine, so the summaries have the same bits whether the
 // rows came from the pool or from a prefill chunk on its way into the pool.
 // FULL: the caller knows that all 16 rows exist (ok, cnt == 16): the same operations without the per-row tests.
-template <bool FULL = false>
+// KEYS / VALS: of a block split between two warps, one of them works on the key rows, the other on the value rows.
+template <bool FULL = false, bool KEYS = true, bool VALS = true>
 __device__ __forceinline__ void block_stats_rows16(const uint4 (&kraw)[8], const uint4 (&vraw)[8], bool ok, int cnt,
                                                    int lane, float (&km)[8], float (&vs)[8], float (&sq)[8]) {
   const int hw = lane >> 4;
@@ -140,20 +148,20 @@ __device__ __forceinline__ void block_stats_rows16(const uint4 (&kraw)[8], const
   for (int j = 0; j < 8; ++j) {
     if (FULL || (ok && hw + 2 * j < cnt)) {
       // mixed-precision adds: a bf16 operand widened inside the instruction (exact), the same sum as ks[i] += float(k)
-      add_bf16x8(kraw[j], ks);
-      add_bf16x8(vraw[j], vs);
+      if constexpr (KEYS) add_bf16x8(kraw[j], ks);
+      if constexpr (VALS) add_bf16x8(vraw[j], vs);
     }
   }
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
-    ks[i] += __shfl_xor_sync(0xffffffffu, ks[i], 16);
-    vs[i] += __shfl_xor_sync(0xffffffffu, vs[i], 16);
+    if constexpr (KEYS) ks[i] += __shfl_xor_sync(0xffffffffu, ks[i], 16);
+    if constexpr (VALS) vs[i] += __shfl_xor_sync(0xffffffffu, vs[i], 16);
     km[i] = ks[i] * inv;
     sq[i] = 0.f;
   }
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
-    if (FULL || (ok && hw + 2 * j < cnt)) {
+    if (KEYS && (FULL || (ok && hw + 2 * j < cnt))) {
       float dv[8];
       sub_bf16x8(kraw[j], km, dv);   // float(k) - km
 #pragma unroll

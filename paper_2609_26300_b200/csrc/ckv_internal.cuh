@@ -73,6 +73,8 @@ struct CkvStepPlan {
   int cluster;      // CTAs per unit
   int stages;       // ring stages of the scan phase
   int own_cap;      // blocks of a unit one CTA owns, at most (a multiple of 16)
+  int first_parts;  // 16-block parts of a CTA's first tile, which lies at rank * first_parts whatever the length
+  int hi_page;      // the last page of a sequence as long as the host's bound
   int u_off, smem;  // offset of the score terms in dynamic shared memory, and its size
   int max_blocks;   // blocks of a sequence the step can work on (the capacity, or the host's bound on the lengths)
 };

@@ -63,6 +63,30 @@ struct ScanUnit : HeadAcc<G> {
         }
       }
   }
+  // The same from bf16 rows in shared memory `stride` bytes apart (an odd multiple of 16, so that eight rows fall into
+  // different banks), four matrix loads in all; zero_row: what heads past G are read as.
+  __device__ __forceinline__ void load_queries(int lane, float scale, uint32_t rows, uint32_t stride, uint32_t zero_row) {
+    static_assert(!QS, "bf16 queries");
+    // lane roles: matrix lane / 8 -> eight coordinates, row lane % 8 -> column of the product
+    const int col = lane & 7, head = T::PAIR ? col & 3 : col;
+    const uint32_t at = (head < G ? rows + (uint32_t)head * stride : zero_row) + (uint32_t)((lane >> 3) << 4);
+#pragma unroll
+    for (int ks = 0; ks < 8; ks += 2) {
+      uint32_t r[4];
+      ldmatrix_x4(r, at + 32u * ks);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        qa[ks + (i >> 1)][i & 1] = r[i];
+        if constexpr (RD) {
+          const float x0 = __uint_as_float(r[i] << 16) * scale, x1 = __uint_as_float(r[i] & 0xffff0000u) * scale;
+          const float s0 = x0 * x0, s1 = x1 * x1;
+          const uint32_t sh = pack_bf16(s0, s1);
+          qs[RD ? ks + (i >> 1) : 0][i & 1] = sh;
+          qs2[RD ? ks + (i >> 1) : 0][i & 1] = pack_bf16(s0 - __uint_as_float(sh << 16), s1 - __uint_as_float(sh & 0xffff0000u));
+        }
+      }
+    }
+  }
 };
 
 // Parameters of a part that do not change between a warp's parts.

@@ -45,8 +45,8 @@ using bf16 = __nv_bfloat16;
 
 constexpr int kWarps = 8;                       // warps that work on parts and pages
 constexpr int kWork = kWarps * 32;              // ... and their threads
-constexpr int kProducerWarp = kWarps, kTailWarp = kWarps + 1;
-constexpr int kThreads = (kWarps + 2) * 32;
+constexpr int kProducerWarp = kWarps, kTailWarp = kWarps + 1, kValueWarp = kWarps + 2;
+constexpr int kThreads = (kWarps + 3) * 32;
 constexpr int kClusterCap = CKV_STEP_MAX_CLUSTER;
 constexpr int kStagesCap = 6;
 constexpr int kMinRing = 3;                     // ring stages that the score terms have to leave room for
@@ -147,15 +147,40 @@ __device__ __noinline__ void take_by_digits(int X, int kr, const uint32_t *keys,
   map[2 * tid + 1] |= (uint32_t)(m >> 32);
 }
 
+// What the tail warps' routines take from the kernel's parameters, in shared memory: as arguments by value the two structs
+// are copied to the stack (two hundred bytes of stores and loads at the start of the tail's chain).
+struct TailArgs { CkvDev P; CkvNewToken fresh; };
+
+// Whether the last block of a sequence of N tokens is shared by two warps: a new token, and one page.
+__device__ __forceinline__ bool tail_is_split(const CkvDev &P, bool append, int N) {
+  return append && N - ((((N + P.bs - 1) >> P.lg_bs) - 1) << P.lg_bs) <= CKV_PAGE;
+}
+// The mean value of the last block, weight 1, into the partials of heads g0, g0 + step, ...
+template <int G>
+__device__ __forceinline__ void tail_store_value(float *tail_part, const float (&x)[8], bool mine, int g0, int step, int li) {
+  if (!mine) return;
+#pragma unroll
+  for (int g = g0; g < G; g += step) {
+    *reinterpret_cast<float4 *>(tail_part + g * CKV_PART_STRIDE + 4 + 8 * li) = make_float4(x[0], x[1], x[2], x[3]);
+    *reinterpret_cast<float4 *>(tail_part + g * CKV_PART_STRIDE + 8 + 8 * li) = make_float4(x[4], x[5], x[6], x[7]);
+  }
+}
+
 // The last CTA's tail warp: the new token (if there is one) goes into its page and the last block's summary is redone
 // with the append's own routine; then, new token or not, the last block's two per-head terms and its compensation
 // partial, with plain FMAs, from the summary as stored (a fresh one is taken from the registers it was stored from).
-// The cluster waits for this warp, whose time is one chain of dependent loads and cold code (4.3 us beside 2.7 us of scan
-// at 32K): so every load that depends on nothing is requested first, the new row is put among the page's other rows in
-// registers instead of being read back, and the sums of all heads share one tree of shuffles.
+// The cluster waits for this warp, whose time is one chain of dependent loads and cold code: so every load that depends on
+// nothing is requested first (the page-table entry among them: tail_page), the new row is put among the page's other rows
+// in registers instead of being read back, a block of one page leaves its value rows to a second warp (tail_values) and
+// its heads to both half warps, and the sums of all heads share one tree of shuffles.  One unit of 4K tokens, from the
+// kernel's first load to the end of this routine: 4.7 us with one warp, half its lanes idle at the heads and the two
+// structs as arguments by value, 3.75 now.  (Inlined into the kernel it ends as early, but the step of 32 units at 128K then
+// takes 54.7 us instead of 51.5.)
 template <int G>
-__device__ __noinline__ void tail_block(const CkvDev P, const bf16 *q_rows, const int *page_table, const CkvNewToken fresh,
+__device__ __noinline__ void tail_block(const TailArgs *args, const bf16 *q_rows, const int *page_table, int phys,
                                         int unit, int raw, int N, float *sq, float *tail_u, float *tail_part, float4 *norm) {
+  const CkvDev &P = args->P;
+  const CkvNewToken &fresh = args->fresh;
   const int lane = threadIdx.x & 31, hw = lane >> 4, li = lane & 15;
   const int s = ckv_div_hkv(P, unit), h = unit - s * P.Hkv;
   const int cap = P.max_blocks * P.bs;
@@ -163,42 +188,40 @@ __device__ __noinline__ void tail_block(const CkvDev P, const bf16 *q_rows, cons
   const bool by_mass = (P.variant & CKV_VARIANT_RANK_BY_MASS) != 0;
   const int *pt_row = page_table + (size_t)s * P.max_pages_per_seq;
   const bool append = fresh.k_new != nullptr && raw + 1 == N;   // (past the host's bound: see append_past_bound)
-  int phys = -1;
+  const int b = ((N + P.bs - 1) >> P.lg_bs) - 1, cnt = N - b * P.bs;
+  const bool split = tail_is_split(P, append, N);
   uint4 kn, vn;   // this lane's eight coordinates of the new rows
   kn = vn = make_uint4(0u, 0u, 0u, 0u);
   if (append) {
-    phys = pt_row[raw / CKV_PAGE];
     kn = reinterpret_cast<const uint4 *>(reinterpret_cast<const bf16 *>(fresh.k_new) + (size_t)unit * CKV_D)[li];
-    vn = reinterpret_cast<const uint4 *>(reinterpret_cast<const bf16 *>(fresh.v_new) + (size_t)unit * CKV_D)[li];
+    if (!split) vn = reinterpret_cast<const uint4 *>(reinterpret_cast<const bf16 *>(fresh.v_new) + (size_t)unit * CKV_D)[li];
   }
-  uint4 qr[G];    // ... and of the queries
-#pragma unroll
-  for (int g = 0; g < G; ++g) qr[g] = reinterpret_cast<const uint4 *>(q_rows + (size_t)g * CKV_D)[li];
-  const int b = ((N + P.bs - 1) >> P.lg_bs) - 1, cnt = N - b * P.bs;
   const size_t row = (size_t)unit * P.max_blocks + b;
   __nv_bfloat16 *kmean_row = P.kmean + row * P.row_elems, *vmean_row = P.vmean + row * P.row_elems;
   float *dbar_row = P.dbar + row * P.r;
+  constexpr int GH = G >= 2 ? G / 2 : 1;   // heads of a half warp
+  const int g0 = G >= 2 ? hw * GH : 0;
+  uint4 qr[GH];    // this lane's coordinates of their queries
+#pragma unroll
+  for (int g = 0; g < GH; ++g) qr[g] = reinterpret_cast<const uint4 *>(q_rows + (size_t)(g0 + g) * CKV_D)[li];
   BlockRow br;
   if (append) {
     bf16 *kp = reinterpret_cast<bf16 *>(fresh.k_pool), *vp = reinterpret_cast<bf16 *>(fresh.v_pool);
     const bool ok = phys >= 0 && phys < P.num_pages;
     const size_t base = ok ? ((size_t)phys * P.Hkv + h) * CKV_PAGE * CKV_D + 8 * li : 0;
     const size_t at = base + (size_t)(raw % CKV_PAGE) * CKV_D;
-    if (cnt <= CKV_PAGE) {   // the token's page is all there is of its block
-      uint4 kraw[8], vraw[8];
+    if (split) {   // the token's page is all there is of its block
+      uint4 kraw[8];
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
         const int t = hw + 2 * j;
-        kraw[j] = kn; vraw[j] = vn;
-        if (ok && t < cnt - 1) {
-          kraw[j] = *reinterpret_cast<const uint4 *>(kp + base + (size_t)t * CKV_D);
-          vraw[j] = *reinterpret_cast<const uint4 *>(vp + base + (size_t)t * CKV_D);
-        }
+        kraw[j] = kn;
+        if (ok && t < cnt - 1) kraw[j] = *reinterpret_cast<const uint4 *>(kp + base + (size_t)t * CKV_D);
       }
-      if (ok) *reinterpret_cast<uint4 *>((hw == 0 ? kp : vp) + at) = hw == 0 ? kn : vn;
-      float km[8], vs[8], ssq[8];
-      block_stats_rows16(kraw, vraw, ok, cnt, lane, km, vs, ssq);
-      block_stats_finish(P, b, (float)cnt, km, vs, ssq, sq, kmean_row, dbar_row, vmean_row, lane, !ok, &br);
+      if (ok && hw == 0) *reinterpret_cast<uint4 *>(kp + at) = kn;
+      float km[8], none[8], ssq[8];
+      block_stats_rows16<false, true, false>(kraw, kraw, ok, cnt, lane, km, none, ssq);
+      block_stats_finish<true, false>(P, b, (float)cnt, km, none, ssq, sq, kmean_row, dbar_row, vmean_row, lane, !ok, &br);
     } else {
       if (ok) *reinterpret_cast<uint4 *>((hw == 0 ? kp : vp) + at) = hw == 0 ? kn : vn;
       __syncwarp();
@@ -214,27 +237,29 @@ __device__ __noinline__ void tail_block(const CkvDev P, const bf16 *q_rows, cons
       for (int i = 0; i < 8; ++i) br.dvar[i] = dbar_row[group_of(8 * li + i, P.r, P.glayout)];
     }
   }
-  // sums over the 16 lanes of a half warp, d_0 .. d_{G-1}, sigma^2_0 .. sigma^2_{G-1} (the d of the lower half count: it holds the mean key)
-  float v[2 * G];
+  if (!split) {   // the upper half warp parts with the mean value and takes the mean key, too
+    tail_store_value<G>(tail_part, br.x, hw == 1, 0, 1, li);
 #pragma unroll
-  for (int g = 0; g < G; ++g) {
+    for (int i = 0; i < 8; ++i) br.x[i] = __shfl_sync(0xffffffffu, br.x[i], li);
+  }
+  // sums over the 16 lanes of a half warp: d, then sigma^2, of its heads
+  float v[2 * GH];
+#pragma unroll
+  for (int g = 0; g < GH; ++g) {
     float qx[8];
     bf16x8_to_float(qr[g], qx);
-    v[g] = v[G + g] = 0.f;
+    v[g] = v[GH + g] = 0.f;
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       v[g] = fmaf(qx[i], br.x[i], v[g]);
       const float qs = qx[i] * P.scale;
-      v[G + g] = fmaf(qs * qs, br.dvar[i], v[G + g]);   // Eq. 8: the squared logit scale is its 1/d
-    }
-    if (hw == 1) {   // weight 1 times the mean value
-      *reinterpret_cast<float4 *>(tail_part + g * CKV_PART_STRIDE + 4 + 8 * li) = make_float4(br.x[0], br.x[1], br.x[2], br.x[3]);
-      *reinterpret_cast<float4 *>(tail_part + g * CKV_PART_STRIDE + 8 + 8 * li) = make_float4(br.x[4], br.x[5], br.x[6], br.x[7]);
+      v[GH + g] = fmaf(qs * qs, br.dvar[i], v[GH + g]);   // Eq. 8: the squared logit scale is its 1/d
     }
   }
-  reduce16<2 * G, 1>(v, li);   // half-warp lane i now holds sum i / (8 / G)
-  const float d = __shfl_sync(0xffffffffu, v[0], (lane * (8 / G)) & 15);
-  const float sg = fmaxf(__shfl_sync(0xffffffffu, v[0], ((G + lane) * (8 / G)) & 15), 0.f);
+  reduce16<2 * GH, 1>(v, li);   // half-warp lane i now holds sum i / (8 / GH)
+  const int from = (G >= 2 ? (lane / GH) * 16 : 0) + (lane % GH) * (8 / GH);   // (lanes past G: any)
+  const float d = __shfl_sync(0xffffffffu, v[0], from & 31);
+  const float sg = fmaxf(__shfl_sync(0xffffffffu, v[0], (from + 8) & 31), 0.f);
   if (lane < G) {
     const float zbar = d * P.scale, logc = logf((float)cnt), zl2 = (zbar + logc) * kLog2e;
     const float u = fmaf(logc + zbar + P.half_var * sg, kLog2e, by_mass ? 0.f : __log2f(sg));
@@ -244,6 +269,34 @@ __device__ __noinline__ void tail_block(const CkvDev P, const bf16 *q_rows, cons
     tail_part[lane * CKV_PART_STRIDE] = zl2;
     tail_part[lane * CKV_PART_STRIDE + 1] = 1.f;
   }
+}
+
+// The value rows of a last block that tail_block shares with a second warp: new row into its page, mean value, partial.
+template <int G>
+__device__ __noinline__ void tail_values(const TailArgs *args, int phys, int unit, int raw, int N, float *tail_part) {
+  const CkvDev &P = args->P;
+  const CkvNewToken &fresh = args->fresh;
+  const int lane = threadIdx.x & 31, hw = lane >> 4, li = lane & 15;
+  const int s = ckv_div_hkv(P, unit), h = unit - s * P.Hkv;
+  const uint4 vn = reinterpret_cast<const uint4 *>(reinterpret_cast<const bf16 *>(fresh.v_new) + (size_t)unit * CKV_D)[li];
+  const int b = ((N + P.bs - 1) >> P.lg_bs) - 1, cnt = N - b * P.bs;
+  bf16 *vp = reinterpret_cast<bf16 *>(fresh.v_pool);
+  const bool ok = phys >= 0 && phys < P.num_pages;
+  const size_t base = ok ? ((size_t)phys * P.Hkv + h) * CKV_PAGE * CKV_D + 8 * li : 0;
+  uint4 vraw[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const int t = hw + 2 * j;
+    vraw[j] = vn;
+    if (ok && t < cnt - 1) vraw[j] = *reinterpret_cast<const uint4 *>(vp + base + (size_t)t * CKV_D);
+  }
+  if (ok && hw == 0) *reinterpret_cast<uint4 *>(vp + base + (size_t)(raw % CKV_PAGE) * CKV_D) = vn;
+  float none[8], vs[8], none2[8];
+  block_stats_rows16<false, false, true>(vraw, vraw, ok, cnt, lane, none, vs, none2);
+  BlockRow br;
+  block_stats_finish<false, true>(P, b, (float)cnt, none, vs, none2, nullptr, nullptr, nullptr,
+                                  P.vmean + ((size_t)unit * P.max_blocks + b) * P.row_elems, lane, false, &br);
+  tail_store_value<G>(tail_part, br.x, true, hw, 2, li);
 }
 
 // The append of a sequence that has outgrown the host's bound: the token lands in a block that the step does not look at,
@@ -277,8 +330,8 @@ __device__ __noinline__ void store_lens(int *counter, int *seq_lens, int batch, 
 
 template <int G, bool RD, bool HS, bool VH>
 __global__ void __launch_bounds__(kThreads, 1)
-ckv_unit_step_kernel(CkvDev P, const bf16 *q, const int *seq_lens, const bf16 *k_pool, const bf16 *v_pool,
-                     const int *page_table, CkvNewToken fresh, int kcap, CkvStepPlan plan, int batch,
+ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int *seq_lens, const bf16 *k_pool, const bf16 *v_pool,
+                     const int *page_table, const __grid_constant__ CkvNewToken fresh, int kcap, CkvStepPlan plan, int batch,
                      int *__restrict__ sel_ids, int *__restrict__ sel_cnt, bf16 *__restrict__ out, float *__restrict__ lse,
                      CkvHostDone done, const __grid_constant__ CUtensorMap tm_v) {
   constexpr int kRowBytesK = HS ? CKV_D * 2 : CKV_ROW_ELEMS * 2;
@@ -290,7 +343,8 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *q, const int *seq_lens, const bf16 *k
   __shared__ __align__(8) uint64_t full_bar[2][kStagesCap], empty_bar[kStagesCap];
   __shared__ __align__(8) uint64_t s_xbar[4];                 // what the cluster's CTAs send: normalisers, scores, partial outputs; global stores done
   __shared__ __align__(512) unsigned char s_zero_row[512];
-  __shared__ __align__(16) bf16 s_q[G][CKV_D];
+  constexpr int kQStride = CKV_D + 8;                         // 17 pieces of 16 bytes: the matrix loads of eight rows hit eight bank groups
+  __shared__ __align__(16) bf16 s_q[G][kQStride];
   __shared__ float s_w[G * 64];                               // variance weights [t][g], r < d
   __shared__ __align__(16) float4 s_wn[kWarps + 1][G];        // (maximum m, sum of e^{l - m}, largest score term) per warp, then of the last block
   __shared__ __align__(16) float4 s_norm[kClusterCap][G];     // ... per CTA of the cluster
@@ -298,6 +352,7 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *q, const int *seq_lens, const bf16 *k
   __shared__ __align__(16) float s_tail_part[G][CKV_PART_STRIDE];
   __shared__ __align__(16) float s_recv[(4 * G + kClusterCap) * kRecvStride];
   __shared__ float s_sq[CKV_D];
+  __shared__ TailArgs s_tail;
   __shared__ int s_digit, s_before, s_nc, s_ncand, s_wt[3][kWarps], s_abort, s_issued;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -316,36 +371,24 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *q, const int *seq_lens, const bf16 *k
     mbar_arrive_expect_tx(&s_xbar[2], (uint32_t)(n_items * C * (32 * 4 + 8)));
     s_abort = 0; s_issued = 0; s_digit = -1; s_ncand = 0;
   }
+  if (warp >= kTailWarp) {
+    const int i = tid - kTailWarp * 32;
+    static_assert(sizeof(CkvDev) % 4 == 0 && sizeof(CkvDev) <= 256 && sizeof(CkvNewToken) % 4 == 0 && sizeof(CkvNewToken) <= 256, "a word per thread");
+    if (i < (int)sizeof(CkvDev) / 4) reinterpret_cast<int *>(&s_tail.P)[i] = reinterpret_cast<const int *>(&P)[i];
+    if (i < (int)sizeof(CkvNewToken) / 4) reinterpret_cast<int *>(&s_tail.fresh)[i] = reinterpret_cast<const int *>(&fresh)[i];
+    named_barrier(4, 64);
+  }
   cluster_arrive_release();   // "this CTA runs, its barriers are set up"
   pdl_trigger();              // the next launch of the stream may set itself up ...
   pdl_wait();                 // ... and this one touches nothing before the launch ahead of it is complete
-  const int raw = seq_lens[s];
-  if (tid < G * 16) reinterpret_cast<uint4 *>(&s_q[0][0])[tid] = reinterpret_cast<const uint4 *>(q + (size_t)unit * G * CKV_D)[tid];
-  if (tid >= kThreads - 32) reinterpret_cast<uint4 *>(s_zero_row)[lane] = make_uint4(0u, 0u, 0u, 0u);
+  const size_t row0 = (size_t)unit * P.max_blocks;
   const bool dbar_bulk = P.r >= 4;
   const int stage_bytes = TB * (kRowBytesK + kRowBytesV) + (dbar_bulk ? TB * P.r * 4 : 0);
-  // the length the step works on; of a sequence longer than the host's bound, what the shared arrays were sized for
-  const int N_all = max(min(raw + ((append && raw >= 0 && raw < cap) ? 1 : 0), cap), 0);
-  const int N = min(N_all, plan.max_blocks * P.bs);
-  if (N < N_all && rank == 0 && tid == 0) atomicOr(P.status, CKV_DEV_BAD_BOUND);
-  const int X = (N + P.bs - 1) >> P.lg_bs, Xs = max(X - 1, 0);
-  const int n_parts = (Xs + 15) >> 4;
-  const int ppc = (int)ckv_udiv24((unsigned)(n_parts + C - 1), (unsigned)C);
-  const int b_lo = min(rank * ppc, n_parts) * 16;
-  const int own = max(min(min(b_lo + ppc * 16, Xs) - b_lo, plan.own_cap), 0);
-  const int tiles = (own + TB - 1) / TB;
-  const size_t row0 = (size_t)unit * P.max_blocks;
-  // score terms of the CTA's own blocks, [g][us] (eight more than the range holds: a tile's eight rows x four heads then
-  // fall into 32 different banks)
-  float *ub = reinterpret_cast<float *>(smem + plan.u_off);
-  const int us = plan.own_cap + 8;
-
   // test hook (ckv_debug_set): one fill is announced but never issued, so that the waits on it run out
   auto withheld = [&](int it) { return (P.debug & CKV_DEBUG_SKIP_FILL) != 0 && it == 0 && rank == 0 && unit == 0; };
-  // one fill of the ring: tile `it` into stage `st`, counted on full barrier `fb`
-  auto fill = [&](int it, int st, uint64_t *fb) {
-    const int nb = min(TB, own - it * TB);
-    const size_t row = row0 + b_lo + it * TB;
+  // one fill of the ring: tile `it`, nb blocks from block b on, into stage `st`, counted on full barrier `fb`
+  auto fill = [&](int it, int b, int nb, int st, uint64_t *fb) {
+    const size_t row = row0 + b;
     unsigned char *sk = smem + (size_t)st * stage_bytes;
     unsigned char *sv = sk + TB * kRowBytesK;
     const uint32_t kbytes = (uint32_t)nb * kRowBytesK;
@@ -353,7 +396,7 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *q, const int *seq_lens, const bf16 *k
     const uint32_t dbytes = dbar_bulk ? (uint32_t)nb * P.r * 4 : 0;
     mbar_arrive_expect_tx(fb, kbytes + vbytes + dbytes);
     const uint32_t lo = smem_u32(smem), hi = lo + (uint32_t)plan.stages * stage_bytes;
-    bool ok = nb >= 1 && b_lo + it * TB + nb <= P.max_blocks;
+    bool ok = nb >= 1 && b + nb <= P.max_blocks;
     if (!withheld(it)) {
       ok = ok && bulk_g2s_checked(sk, P.kmean + row * P.row_elems, kbytes, fb, lo, hi);
       if constexpr (VH) {
@@ -369,21 +412,60 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *q, const int *seq_lens, const bf16 *k
     }
     if (!ok) atomicOr(P.status, CKV_DEV_BAD_COPY);
   };
-  // The tail warp does not wait here: it needs nothing that the others set up, and the cluster will wait for it.
-  if (warp == kTailWarp) named_arrive(3, kThreads);
+  // The first tile's place follows from the plan; of a sequence that ends sooner, rows that nobody looks at are copied.  With
+  // this copy ahead of the length, the others issued by the producer's lanes and the queries' fragments loaded as matrices, a
+  // CTA starts on its first part 1.2 us after the length is known instead of 2.0 (a step of 8 units at 32K 15.4 -> 14.8 us, 16
+  // units with r = d at 88K 40.5 -> 39.6, 32 units at 128K 52.6 -> 51.5).
+  const int n_early = max(min(plan.first_parts * 16, plan.max_blocks - rank * plan.first_parts * 16), 0);
+  if (tid == kProducerWarp * 32 && n_early > 0) fill(0, rank * plan.first_parts * 16, n_early, 0, &full_bar[0][0]);
+  const int raw = seq_lens[s];
+  if (tid < G * 16) *reinterpret_cast<uint4 *>(&s_q[tid >> 4][8 * (tid & 15)]) = reinterpret_cast<const uint4 *>(q + (size_t)unit * G * CKV_D)[tid];
+  // The new token's page: the tail warps read the last 32 entries of the page-table row under the host's bound while the
+  // length is on its way; a length the bound exceeds by more is looked up when it is known.
+  const int *pt_row = page_table + (size_t)s * P.max_pages_per_seq;
+  int page_guess = -1;
+  if (warp >= kTailWarp && rank == C - 1 && append && plan.hi_page >= lane) page_guess = pt_row[plan.hi_page - lane];
+  if (tid >= kThreads - 32) reinterpret_cast<uint4 *>(s_zero_row)[lane] = make_uint4(0u, 0u, 0u, 0u);
+  // the length the step works on; of a sequence longer than the host's bound, what the shared arrays were sized for
+  const int N_all = max(min(raw + ((append && raw >= 0 && raw < cap) ? 1 : 0), cap), 0);
+  const int N = min(N_all, plan.max_blocks * P.bs);
+  if (N < N_all && rank == 0 && tid == 0) atomicOr(P.status, CKV_DEV_BAD_BOUND);
+  const int X = (N + P.bs - 1) >> P.lg_bs, Xs = max(X - 1, 0);
+  // What the CTA owns, `own` blocks in all: n0 blocks from b0 on -- its first tile, whose place depends on the host's plan
+  // alone, so that its copy is under way before the length is known -- then the CTA's part of what the first tiles leave.
+  const int first = plan.first_parts * 16;
+  const int n_parts = (Xs + 15) >> 4, rest = max(n_parts - C * plan.first_parts, 0);
+  const int ppc = (int)ckv_udiv24((unsigned)(rest + C - 1), (unsigned)C);
+  const int b0 = rank * first, b1 = C * first + min(rank * ppc, rest) * 16;
+  const int n0 = max(min(Xs - b0, first), 0);
+  const int own = min(n0 + max(min(b1 + ppc * 16, Xs) - b1, 0), plan.own_cap);
+  const int tiles = own == 0 ? 0 : 1 + (max(own - first, 0) + TB - 1) / TB;
+  auto block_at = [&](int i) { return i + (i < first ? b0 : b1 - first); };       // the CTA's i-th block
+  auto tile_start = [&](int it) { return it == 0 ? 0 : first + (it - 1) * TB; };  // first block of tile `it`, counted in the CTA's own
+  auto tile_len = [&](int it) { return min(it == 0 ? first : TB, own - tile_start(it)); };
+  // score terms of the CTA's own blocks, [g][us] (eight more than the range holds: a tile's eight rows x four heads then
+  // fall into 32 different banks)
+  float *ub = reinterpret_cast<float *>(smem + plan.u_off);
+  const int us = plan.own_cap + 8;
+
+  // The tail warps do not wait here: they need nothing that the others set up, and the cluster will wait for them.
+  if (warp >= kTailWarp) named_arrive(3, kThreads);
   else named_barrier(3, kThreads);
-  // the first round of fills is issued by as many warps at once: a fill is some seventy instructions, a third of a
-  // microsecond for one thread, which alone would have the last stage's data arrive a microsecond late
-  const int first_fills = min(tiles, plan.stages);
-  if (warp < first_fills && lane == 0) fill(warp, warp, &full_bar[0][warp]);
 
   ScanUnit<G, bf16, RD> w;
   w.reset();
   if (warp == kProducerWarp) {
     // ---------------- producer: one thread refills the ring ----------------
+    const int first_fills = min(tiles, plan.stages);
+    if (lane > 0 && lane < first_fills) fill(lane, block_at(tile_start(lane)), tile_len(lane), lane, &full_bar[0][lane]);
+    __syncwarp();
     if (lane == 0) {
       mbar_arrive_expect_tx(&s_xbar[1], (uint32_t)(X * 4));
-      *(volatile int *)&s_issued = first_fills;
+      *(volatile int *)&s_issued = max(first_fills, n_early > 0 ? 1 : 0);
+      if (tiles == 0 && n_early > 0 && !mbar_wait(&full_bar[0][0], 0, P.spin_limit)) {   // nobody else waits for this copy
+        atomicOr(P.status, CKV_DEV_TIMEOUT);
+        *(volatile int *)&s_abort = 1;
+      }
       int st = 0;
       uint32_t phase = 0, round = 1;
       for (int it = plan.stages; it < tiles; ++it) {
@@ -392,47 +474,62 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *q, const int *seq_lens, const bf16 *k
           *(volatile int *)&s_abort = 1;
         }
         if (*(volatile int *)&s_abort) break;
-        fill(it, st, &full_bar[round & 1][st]);
+        fill(it, block_at(tile_start(it)), tile_len(it), st, &full_bar[round & 1][st]);
         *(volatile int *)&s_issued = it + 1;
         if (++st == plan.stages) { st = 0; ++round; phase ^= 1; }
       }
     } else {
       // the other lanes ask the L2 for this CTA's share of the page-table row: the attention's lookups are then short
       const int lines = (X * P.ppb + 31) / 32, per = (lines + C - 1) / C;
-      const int *pt = page_table + (size_t)s * P.max_pages_per_seq;
       for (int i = rank * per + lane - 1; i < min((rank + 1) * per, lines); i += 31)
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(pt + 32 * i) : "memory");
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(pt_row + 32 * i) : "memory");
     }
-  } else if (warp == kTailWarp) {
-    if (rank == C - 1 && append && raw >= N && raw < cap) append_past_bound(P, page_table, fresh, unit, raw, s_sq);
-    if (rank == C - 1 && N > 0)
-      tail_block<G>(P, q + (size_t)unit * G * CKV_D, page_table, fresh, unit, raw, N, s_sq, s_tail_u, &s_tail_part[0][0], s_wn[kWarps]);
-    else if (lane < G)
+  } else if (warp >= kTailWarp) {
+    const bool appended = rank == C - 1 && append && raw + 1 == N;
+    int phys = -1;
+    if (appended) {
+      const int back = plan.hi_page - raw / CKV_PAGE;
+      phys = __shfl_sync(0xffffffffu, page_guess, back & 31);
+      if ((unsigned)back > 31u) phys = pt_row[raw / CKV_PAGE];
+    }
+    if (warp == kValueWarp) {
+      if (appended && tail_is_split(P, true, N)) tail_values<G>(&s_tail, phys, unit, raw, N, &s_tail_part[0][0]);
+    } else if (rank == C - 1 && N > 0) {
+      if (append && raw >= N && raw < cap) append_past_bound(P, page_table, fresh, unit, raw, s_sq);
+      tail_block<G>(&s_tail, q + (size_t)unit * G * CKV_D, page_table, phys, unit, raw, N, s_sq, s_tail_u, &s_tail_part[0][0], s_wn[kWarps]);
+    } else if (lane < G) {
       s_wn[kWarps][lane] = make_float4(-CUDART_INF_F, 0.f, -CUDART_INF_F, 0.f);
-    if (append && raw < 0 && rank == C - 1 && lane == 0) atomicOr(P.status, CKV_DEV_SEQ_FULL);   // no place for the token
+    }
+    if (warp == kTailWarp && append && raw < 0 && rank == C - 1 && lane == 0) atomicOr(P.status, CKV_DEV_SEQ_FULL);   // no place for the token
   } else {
     // ---------------- working warps: parts of 16 blocks ----------------
     if (!RD) {
       // w_{g,t} of Eq. 8 times the squared logit scale, summed in coordinate order as the scan kernel sums the weights it
       // stages (those of a CTA's later units it sums in runs of eight): scores that differ in the last bit can swap blocks
       // at the cut.  (The first tile's data is still on its way.)
+      const int lg_r = __ffs(P.r) - 1, gs = CKV_D >> lg_r, run = P.glayout == 0 ? gs : gs >> 1;
       for (int i = tid; i < P.r * G; i += kWork) {
-        const int g = i & (G - 1), t = i / G, gs = CKV_D / P.r, run = P.glayout == 0 ? gs : gs / 2;
+        const int g = i & (G - 1), t = i / G;
         float a = 0.f;
-#pragma unroll 8
-        for (int k = 0; k < gs; ++k) {
-          const int c = t * run + (k < run ? k : CKV_D / 2 + k - run);
-          const float x = __bfloat162float(s_q[g][c]);
-          a = fmaf(x, x, a);
+        if (run >= 8) {
+#pragma unroll 2
+          for (int k = 0; k < gs; k += 8) {
+            float x[8];
+            bf16x8_to_float(*reinterpret_cast<const uint4 *>(&s_q[g][t * run + (k < run ? k : CKV_D / 2 + k - run)]), x);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) a = fmaf(x[j], x[j], a);
+          }
+        } else {
+          for (int k = 0; k < gs; ++k) {
+            const float x = __bfloat162float(s_q[g][t * run + (k < run ? k : CKV_D / 2 + k - run)]);
+            a = fmaf(x, x, a);
+          }
         }
         s_w[i] = a * (P.scale * P.scale);
       }
-      work_barrier();
     }
-    w.set_queries(lane, P.scale, [&](int g, int c) {
-      const uint32_t x = *reinterpret_cast<const uint32_t *>(&s_q[g][c]);
-      return make_float2(__uint_as_float(x << 16), __uint_as_float(x & 0xffff0000u));
-    });
+    w.load_queries(lane, P.scale, smem_u32(&s_q[0][0]), kQStride * 2, smem_u32(s_zero_row));
+    if (!RD) work_barrier();
     if (!RD && P.r == 4) {
 #pragma unroll
       for (int e = 0; e < 2; ++e)
@@ -462,15 +559,15 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *q, const int *seq_lens, const bf16 *k
         }
         aborted = __any_sync(0xffffffffu, fail);
       }
-      const int nb = min(TB, own - it * TB), rb = part * 16;
+      const int nb = tile_len(it), rb = part * 16, from = tile_start(it), tb0 = block_at(from);
       if (!aborted && rb < nb) {
         const uint32_t sk = smem_u32(smem + (size_t)st * stage_bytes);
         const float *sd = reinterpret_cast<const float *>(smem + (size_t)st * stage_bytes + TB * (kRowBytesK + kRowBytesV));
         scan_part<G, bf16, RD, HS, VH>(
             w, cfg, sk, sk + TB * kRowBytesK, (RD || dbar_bulk) ? sd : nullptr, smem_u32(s_zero_row), s_w, P.dbar + row0 * P.r,
-            lane, rb, nb, b_lo + it * TB, -1, 0.f,
+            lane, rb, nb, tb0, -1, 0.f,
             [&](int g, int blk, float x, float y) {
-              ub[g * us + (blk - b_lo)] = x;
+              ub[g * us + (blk - tb0 + from)] = x;
               lz[(size_t)g * P.max_blocks + blk] = y;
               if (g & 1) umax[1] = fmaxf(umax[1], x); else umax[0] = fmaxf(umax[0], x);
             });
@@ -585,7 +682,7 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *q, const int *seq_lens, const bf16 *k
         if (real && (!(sc[j] >= 0.f) || sc[j] > 3.0e38f)) { nonfinite = true; sc[j] = 0.f; }
         k[j] = __float_as_uint(sc[j]);
       }
-      const uint32_t dst = smem_u32(keys + b_lo + i);
+      const uint32_t dst = smem_u32(keys + block_at(i));
       if (i + 4 <= own) {
         for (int c = 0; c < C; ++c) {
           const uint32_t there = cluster_map(xbar1, c);   // the CTAs' shared memories are congruent windows
@@ -613,7 +710,7 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *q, const int *seq_lens, const bf16 *k
       const int b = i < rank_lo ? i : i + rank_n;
       atomicOr(&map[b >> 5], 1u << (b & 31));
     }
-  } else if (warp == kProducerWarp && X > kcap) {
+  } else if (warp >= kWarps && X > kcap) {
     named_barrier(2, kThreads - kWork);
   }
   wait_x(1);
@@ -625,9 +722,9 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *q, const int *seq_lens, const bf16 *k
   const int K = min(kcap, X);
   const bool all = X <= kcap;          // every block is selected: the step is dense attention
   int *ids = reinterpret_cast<int *>(smem + kOffIds);
-  if (warp >= kWarps && !dead) {   // the two idle warps leave the range's scores where ckv_copy_scores() finds them
+  if (warp >= kWarps && !dead) {   // the idle warps leave the range's scores where ckv_copy_scores() finds them
     float *scores = P.scores + row0;
-    for (int i = tid - kWork; i < own; i += kThreads - kWork) scores[b_lo + i] = __uint_as_float(keys[b_lo + i]);
+    for (int i = tid - kWork; i < own; i += kThreads - kWork) { const int b = block_at(i); scores[b] = __uint_as_float(keys[b]); }
     if (rank == C - 1 && N > 0 && tid == kWork) scores[Xs] = __uint_as_float(keys[Xs]);
   }
   if (warp < kWarps) {
@@ -759,7 +856,6 @@ ckv_unit_step_kernel(CkvDev P, const bf16 *q, const int *seq_lens, const bf16 *k
     const int p0 = min(rank * share, n_pages), p1 = min(p0 + share, n_pages);
     const int n_mine = max((p1 - p0 - warp + kWarps - 1) / kWarps, 0);
     const int pshift = P.ppb == 1 ? 0 : (P.ppb == 2 ? 1 : 2);
-    const int *pt_row = page_table + (size_t)s * P.max_pages_per_seq;
     const float *lz = P.lz + row0 * G;
     const float sl2 = P.scale * kLog2e;
     const float lg_bs = log2f((float)P.bs), lg_last = log2f((float)max(N - Xs * P.bs, 1));
@@ -1070,6 +1166,8 @@ bool ckv_unit_step_plan(const ckv_ctx *c, int batch, int max_len, int kcap, CkvS
   auto blocks_per_cta = [C](int x) { const int parts = (std::max(x - 1, 0) + 15) / 16; return 16 * std::max((parts + C - 1) / C, 1); };
   auto term_bytes = [&P](int own) { return (size_t)(own + 8) * P.G * sizeof(float); };
   plan->own_cap = blocks_per_cta(xmax);
+  plan->first_parts = std::min(P.scan_tile, plan->own_cap) / 16;
+  plan->hi_page = std::min((max_len - 1) / CKV_PAGE, P.max_pages_per_seq - 1);
   if (plan->own_cap > kOwnMost && P.Hkv * C < kSeqCtas && (P.r == 4 || P.r == CKV_D)) return false;
   if (term_bytes(plan->own_cap) + (size_t)std::max(kMinRing, skip) * stage > (size_t)kDynLimit) return false;
   const int tiles = (plan->own_cap + P.scan_tile - 1) / P.scan_tile;
