@@ -14,10 +14,12 @@
 //   2. every CTA sends its normaliser partials (M_g, L_g) to all, then the block scores of its own range: every CTA holds
 //      all scores of the unit.  Both exchanges are asynchronous stores counted on an mbarrier of the receiver: a cluster
 //      barrier with release semantics would wait for the scan's stores to global memory as well (1.4 us instead of 0.6).
-//   3. selection, redundantly in every CTA: a histogram over the scores' bit patterns relative to an upper bound of them
-//      (64 bins per octave, 32 octaves), the exact cut by ranking the one bin that holds it (digit by digit when that bin
-//      is crowded or the cut lies below the histogram), a bit map of the selected blocks, and their ids in position order
-//      from a prefix sum over its words.  All CTAs get the same list without another exchange.
+//   3. selection, redundantly in every CTA, a thread's scores in registers throughout: a histogram over the scores' bit
+//      patterns relative to an upper bound of them (64 bins per octave, 32 octaves), the exact cut by ranking the one bin that
+//      holds it (digit by digit when that bin is crowded or the cut lies below the histogram), a word of bits per thread for
+//      its blocks that are in, and their ids in position order from a prefix sum.  All CTAs get the same list without another
+//      exchange.  32 units of 8192 blocks: 4.2 us from the scores to the ids (6.2 with two passes over shared memory and a bit
+//      map put together by shuffles and atomics), 8 units of 2048: 2.6 (3.2).
 //   4. exact attention over the CTA's share of the list, a warp per page, into the SAME accumulators that hold the
 //      compensation sums of step 1 (both are online-softmax sums over the same heads); the selected blocks' mean terms
 //      are taken out through the tokens' weights, or with bf16 summaries as one more product over the stored rows.
@@ -54,6 +56,9 @@ constexpr int kScoresCap = 9216;                // blocks of a unit whose scores
                                                 // map and the memory would take 16384, longer units have not been tried)
 constexpr int kBins = 2048;                     // score histogram: 32 octaves below the largest possible score, 64 bins each
 constexpr int kBinShift = 17;                   // ... a bin is a score's bit pattern without its low 17 bits
+constexpr int kIdMask = (1 << (31 - kBinShift)) - 1;   // block ids beside those 17 bits in one word
+static_assert(kScoresCap <= kIdMask + 1, "block ids fit");
+constexpr int kKeyGroups = kScoresCap / 4 / kWork;   // four scores each, as a thread holds them for the selection
 constexpr int kMapWords = 2 * kWork;            // selection bit map: two words per working thread, enough for kScoresCap blocks
 constexpr int kSelCap = 512;                    // selected blocks the id list holds (unless every block is selected)
 constexpr int kOwnMost = 2800, kSeqCtas = 24;   // blocks a CTA may own where a sequence gets few CTAs (see ckv_unit_step_plan)
@@ -64,10 +69,13 @@ constexpr int kOffHist = kScoresCap * 4;
 constexpr int kOffMap = kOffHist + (kBins + 32) * 4;          // (cleared together with the histogram)
 constexpr int kOffIds = kOffMap + kMapWords * 4;
 constexpr int kOffCand = kOffIds + kSelCap * 4;
-constexpr int kOffPages = (kOffCand + kCandCap * 8 + 127) / 128 * 128;
+constexpr int kOffPages = (kOffCand + kCandCap * 4 + 127) / 128 * 128;
 constexpr int kAfterScan = kOffPages + kWarps * 2 * kPageBytes;
 constexpr int kRecvStride = 36;                 // floats of one (head, 32 coordinates) partial: values, maximum, weight sum
 constexpr int kDynLimit = 227 * 1024 - 20 * 1024;   // dynamic shared memory; the kernel's static arrays take under 20 KB
+
+// One more in a shared-memory counter.
+__device__ __forceinline__ void red_shared_inc(uint32_t addr) { asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(addr) : "memory"); }
 
 __device__ __forceinline__ void work_barrier() { named_barrier(1, kWork); }
 
@@ -660,8 +668,10 @@ ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int 
   // ---- scores of the CTA's own blocks (Eq. 10), to every CTA of the cluster ----
   const int n_recent = min(P.recent, X);
   const int rank_lo = P.sink, rank_n = max(X - n_recent - P.sink, 0);   // blocks [rank_lo, rank_lo + rank_n) are ranked, the others mandatory
-  auto ranked = [rank_lo, rank_n](int b) { return (unsigned)(b - rank_lo) < (unsigned)rank_n; };
   uint32_t *keys = reinterpret_cast<uint32_t *>(smem);   // the unit's scores; their bit patterns are ordered like the scores
+  // No score is larger, with room for the bound's and the scores' roundings; the senders hold themselves to it, too, because
+  // the histogram's addresses rely on it.
+  const uint32_t most = __float_as_uint(fminf(bound, 3.0e38f)) + (1u << 10);
   if (!normed) {
     // nothing is sent into a CTA that may not be ready for it: its wait for the scores runs out, too
   } else if (warp < kWarps) {
@@ -680,7 +690,7 @@ ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int 
       for (int j = 0; j < 4; ++j) {
         const bool real = i + j < own;
         if (real && (!(sc[j] >= 0.f) || sc[j] > 3.0e38f)) { nonfinite = true; sc[j] = 0.f; }
-        k[j] = __float_as_uint(sc[j]);
+        k[j] = min(__float_as_uint(sc[j]), most);
       }
       const uint32_t dst = smem_u32(keys + block_at(i));
       if (i + 4 <= own) {
@@ -701,18 +711,16 @@ ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int 
 #pragma unroll
     for (int g = 0; g < G; ++g) sc = fmaf(fast_exp2(s_tail_u[g] - Mg[g]), iL[g], sc);
     if (!(sc >= 0.f) || sc > 3.0e38f) { if (lane == 0) atomicOr(P.status, CKV_DEV_NONFINITE); sc = 0.f; }
-    if (lane < C) st_async_u32(cluster_map(smem_u32(keys + Xs), lane), __float_as_uint(sc), cluster_map(smem_u32(&s_xbar[1]), lane));
+    if (lane < C) st_async_u32(cluster_map(smem_u32(keys + Xs), lane), min(__float_as_uint(sc), most), cluster_map(smem_u32(&s_xbar[1]), lane));
   }
-  if (warp == kTailWarp && X > kcap) {   // the mandatory blocks are in (the other idle warp's share of the map is clear, too)
-    named_barrier(2, kThreads - kWork);
-    uint32_t *map = reinterpret_cast<uint32_t *>(smem + kOffMap);
-    for (int i = lane; i < X - rank_n; i += 32) {
-      const int b = i < rank_lo ? i : i + rank_n;
-      atomicOr(&map[b >> 5], 1u << (b & 31));
-    }
-  } else if (warp >= kWarps && X > kcap) {
-    named_barrier(2, kThreads - kWork);
-  }
+  // While the scores are on their way: a thread will keep those of 4 nj blocks in a row, s0 .. s0 + 4 nj - 1, in registers for
+  // both passes of the selection.  nj is 2 or odd, so that a warp's 16-byte reads fall into different banks (two of them,
+  // with 2), and 9 at most.  A thread's part of the selection is a word of bits; the mandatory blocks are in.
+  const int nj0 = (int)((unsigned)(X + 4 * kWork - 1) / (4 * kWork)), nj = nj0 > 2 ? nj0 | 1 : max(nj0, 1), s0 = 4 * nj * tid;
+  auto below = [](int n) { return n >= 64 ? ~0ull : (1ull << max(n, 0)) - 1ull; };   // bits 0 .. n - 1
+  unsigned long long here = below(min(4 * nj, X - s0));
+  unsigned long long rk = here & below(rank_lo + rank_n - s0) & ~below(rank_lo - s0);
+  asm volatile("" : "+l"(here), "+l"(rk));   // (here, and not where they are used)
   wait_x(1);
   // (the histogram is clear, too.)  A CTA one of whose waits ran out has scores that never came: it selects nothing and
   // contributes an empty partial, so that the others get what they wait for.
@@ -741,22 +749,35 @@ ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int 
       }
     } else {
       const int Kr = K - (X - rank_n);   // blocks to rank in (the host guarantees K >= sink + recent when K < X)
-      uint32_t *map = reinterpret_cast<uint32_t *>(smem + kOffMap);
-      auto pick = [map](int b) { atomicOr(&map[b >> 5], 1u << (b & 31)); };
+      uint32_t *map = reinterpret_cast<uint32_t *>(smem + kOffMap);   // blocks found by id (clear so far)
+      unsigned long long sel = here & ~rk;
       if (Kr > 0) {
         int *hist = reinterpret_cast<int *>(smem + kOffHist);
         const uint4 *keys4 = reinterpret_cast<const uint4 *>(keys);
-        const int groups = (X + 3) / 4;
-        const int top = (int)(__float_as_uint(fminf(bound, 3.0e38f)) >> kBinShift);
-        auto bin_of = [top](uint32_t k) { return max(top - (int)(k >> kBinShift), 0); };
-#pragma unroll 2
-        for (int i = tid; i < groups; i += kWork) {
-          const uint4 k4 = keys4[i];
-          const uint32_t k[4] = {k4.x, k4.y, k4.z, k4.w};
+        const uint32_t top = most >> kBinShift;   // bin 0
+        uint32_t key[kKeyGroups][4];
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const int d = bin_of(k[j]);
-            atomicAdd(&hist[d < kBins && ranked(4 * i + j) ? d : kBins + lane], 1);   // no branch: the rest goes aside
+        for (int j = 0; j < kKeyGroups; ++j) {
+          if (j >= nj) break;
+          const uint4 k4 = keys4[min(tid * nj + j, kScoresCap / 4 - 1)];
+          key[j][0] = k4.x; key[j][1] = k4.y; key[j][2] = k4.z; key[j][3] = k4.w;
+        }
+        {
+          // a bin's address falls with the score; what lies below the last bin or is not ranked goes aside, without a branch
+          const uint32_t h_top = smem_u32(hist) + 4 * top, aside = smem_u32(hist + kBins + lane);
+          const bool whole = __all_sync(0xffffffffu, rk == below(4 * nj));
+#pragma unroll
+          for (int j = 0; j < kKeyGroups; ++j) {
+            if (j >= nj) break;
+            uint32_t at[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) at[e] = min(h_top - (key[j][e] >> (kBinShift - 2) & ~3u), aside);
+            if (!whole) {
+#pragma unroll
+              for (int e = 0; e < 4; ++e) at[e] = (rk >> (4 * j + e) & 1) != 0 ? at[e] : aside;
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e) red_shared_inc(at[e]);
           }
         }
         work_barrier();
@@ -779,63 +800,60 @@ ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int 
         work_barrier();
         const int digit = s_digit, nc = s_nc;
         if (digit >= 0 && nc <= kCandCap) {
-          // higher bins are taken whole; the cut's bin is ranked by (score descending, id ascending)
-          int *cand = reinterpret_cast<int *>(smem + kOffCand);
-          uint32_t *candk = reinterpret_cast<uint32_t *>(smem + kOffCand) + kCandCap;
+          // higher bins are taken whole; the cut's bin is ranked by (score descending, id ascending): what tells its blocks
+          // apart, the scores' low bits and the ids, fits one word
+          uint32_t *cand = reinterpret_cast<uint32_t *>(smem + kOffCand);
           const int take = Kr - s_before;
-#pragma unroll 2
-          for (int i0 = warp * 32; i0 < groups; i0 += kWork) {   // whole warps: eight lanes make up a word of the map
-            const int i = i0 + lane;
-            uint4 k4 = make_uint4(0u, 0u, 0u, 0u);
-            if (i < groups) k4 = keys4[i];
-            const uint32_t k[4] = {k4.x, k4.y, k4.z, k4.w};
-            uint32_t above = 0, at = 0;
+          // sign bits of (threshold - 1 - score), shifted into words: 1 where the score reaches the threshold
+          const int lo1 = (int)((top - (uint32_t)digit) << kBinShift) - 1;
+          const int hi1 = digit == 0 ? 0x7fffffff : (int)((top - (uint32_t)digit + 1u) << kBinShift) - 1;
+          uint32_t ge_hi[2] = {0, 0}, ge_lo[2] = {0, 0};
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              const int d = ranked(4 * i + j) ? bin_of(k[j]) : kBins;
-              above |= d < digit ? 1u << j : 0u;
-              at |= d == digit ? 1u << j : 0u;
+          for (int j = kKeyGroups - 1; j >= 0; --j) {
+            if (j < nj) {
+#pragma unroll
+              for (int e = 3; e >= 0; --e) {
+                ge_hi[j >> 3] = __funnelshift_l((uint32_t)(hi1 - (int)key[j][e]), ge_hi[j >> 3], 1);
+                ge_lo[j >> 3] = __funnelshift_l((uint32_t)(lo1 - (int)key[j][e]), ge_lo[j >> 3], 1);
+              }
             }
-            above <<= 4 * (lane & 7);
-            above |= __shfl_xor_sync(0xffffffffu, above, 1);
-            above |= __shfl_xor_sync(0xffffffffu, above, 2);
-            above |= __shfl_xor_sync(0xffffffffu, above, 4);
-            if ((lane & 7) == 0 && above != 0) atomicOr(&map[i >> 3], above);
-            while (at != 0) {
-              const int j = __ffs(at) - 1;
-              at &= at - 1;
-              const int slot = atomicAdd(&s_ncand, 1);
-              if (slot < kCandCap) { cand[slot] = 4 * i + j; candk[slot] = k[j]; }
-            }
+          }
+          const unsigned long long above = rk & ((unsigned long long)ge_hi[1] << 32 | ge_hi[0]);
+          unsigned long long at = rk & ~above & ((unsigned long long)ge_lo[1] << 32 | ge_lo[0]);
+          sel |= above;
+          while (at != 0) {
+            const int b = s0 + __ffsll((long long)at) - 1;
+            at &= at - 1;
+            const int slot = atomicAdd(&s_ncand, 1);
+            if (slot < kCandCap) cand[slot] = keys[b] << (32 - kBinShift) >> 1 | (uint32_t)(kIdMask - b);
           }
           work_barrier();
           if (tid < nc) {
-            const int myb = cand[tid];
-            const uint32_t mk = candk[tid];
+            const uint32_t mine = cand[tid];
             int place = 0;
-#pragma unroll 4
-            for (int j = 0; j < nc; ++j) place += (candk[j] > mk || (candk[j] == mk && cand[j] < myb)) ? 1 : 0;
-            if (place < take) pick(myb);
+#pragma unroll 8
+            for (int j = 0; j < nc; ++j) place += cand[j] > mine ? 1 : 0;
+            const int b = kIdMask - (int)(mine & kIdMask);
+            if (place < take) atomicOr(&map[b >> 5], 1u << (b & 31));
           }
         } else {
           take_by_digits(X, Kr, keys, rank_lo, rank_n, hist, map, s_wt[1], s_wt[2]);
         }
       }
       work_barrier();
-      // ids in position order: two words of the map per thread
-      uint2 m2 = reinterpret_cast<const uint2 *>(map)[tid];
-      int pos = work_exclusive_scan(__popc(m2.x) + __popc(m2.y), s_wt[1]);
-#pragma unroll
-      for (int half = 0; half < 2; ++half) {
-        uint32_t bits = half == 0 ? m2.x : m2.y;
-        while (bits != 0) {
-          const int b = 64 * tid + 32 * half + __ffs(bits) - 1;
-          bits &= bits - 1;
-          if (pos < K) {
-            ids[pos] = b;
-            if (rank == 0) gids[pos] = b;
-          }
-          ++pos;
+      // ids in position order
+      {
+        const uint32_t *m = map + (s0 >> 5);
+        const uint32_t m0 = m[0], m1 = m[1], m2 = m[2];
+        sel |= here & ((unsigned long long)__funnelshift_r(m1, m2, s0 & 31) << 32 | __funnelshift_r(m0, m1, s0 & 31));
+      }
+      int pos = work_exclusive_scan(__popcll(sel), s_wt[1]);
+      for (; sel != 0; ++pos) {
+        const int b = s0 + __ffsll((long long)sel) - 1;
+        sel &= sel - 1;
+        if (pos < K) {
+          ids[pos] = b;
+          if (rank == 0) gids[pos] = b;
         }
       }
       if (rank == 0) {

@@ -325,6 +325,12 @@ def test_selected_ids_are_the_best_of_the_scores(keys, X, K):
     assert cnt.tolist() == [[K]] and ids[0, 0, :K].tolist() == sorted([0, X - 2, X - 1] + best.tolist())
 
 
+@pytest.mark.parametrize("keys,X", [("spread", n) for n in (97, 1024, 1025, 2048, 2049, 3072, 3073, 5121, 7169, 9215)] + [("alike", 1027)])
+def test_selected_ids_where_the_scores_a_thread_holds_change(keys, X):
+    """4 nj scores a thread, nj = 1, 2, 3, 5, 7, 9: full threads, one block more, and a last thread with one block."""
+    test_selected_ids_are_the_best_of_the_scores(keys, X, 64)
+
+
 def test_a_wait_that_runs_out_is_reported_and_the_context_recovers():
     w = workload(batch=1, ctx_min=None, decode_steps=0)
     d = setup(w)
