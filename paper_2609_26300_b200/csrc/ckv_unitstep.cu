@@ -163,6 +163,16 @@ struct TailArgs { CkvDev P; CkvNewToken fresh; };
 __device__ __forceinline__ bool tail_is_split(const CkvDev &P, bool append, int N) {
   return append && N - ((((N + P.bs - 1) >> P.lg_bs) - 1) << P.lg_bs) <= CKV_PAGE;
 }
+// The length a step works on, after its append: no longer than the cache, nor than the shared arrays were sized for.
+__device__ __forceinline__ int step_length(int raw, bool append, int cap, int most) {
+  return min(max(min(raw + ((append && raw >= 0 && raw < cap) ? 1 : 0), cap), 0), most);
+}
+// The page of position `raw`: lane l of `guess` holds the entry l pages before hi_page, the last one under the host's bound.
+__device__ __forceinline__ int tail_page(int guess, const int *pt_row, int hi_page, int raw) {
+  const int back = hi_page - raw / CKV_PAGE;
+  const int phys = __shfl_sync(0xffffffffu, guess, back & 31);
+  return (unsigned)back <= 31u ? phys : pt_row[raw / CKV_PAGE];
+}
 // The mean value of the last block, weight 1, into the partials of heads g0, g0 + step, ...
 template <int G>
 __device__ __forceinline__ void tail_store_value(float *tail_part, const float (&x)[8], bool mine, int g0, int step, int li) {
@@ -177,41 +187,48 @@ __device__ __forceinline__ void tail_store_value(float *tail_part, const float (
 // The last CTA's tail warp: the new token (if there is one) goes into its page and the last block's summary is redone
 // with the append's own routine; then, new token or not, the last block's two per-head terms and its compensation
 // partial, with plain FMAs, from the summary as stored (a fresh one is taken from the registers it was stored from).
-// The cluster waits for this warp, whose time is one chain of dependent loads and cold code: so every load that depends on
-// nothing is requested first (the page-table entry among them: tail_page), the new row is put among the page's other rows
-// in registers instead of being read back, a block of one page leaves its value rows to a second warp (tail_values) and
-// its heads to both half warps, and the sums of all heads share one tree of shuffles.  One unit of 4K tokens, from the
-// kernel's first load to the end of this routine: 4.7 us with one warp, half its lanes idle at the heads and the two
-// structs as arguments by value, 3.75 now.  (Inlined into the kernel it ends as early, but the step of 32 units at 128K then
-// takes 54.7 us instead of 51.5.)
+// The cluster waits for this warp, whose time is one chain of dependent loads and cold code: so the routine is entered, and
+// its addresses worked out, ahead of the wait for the launch before; every load that depends on nothing is requested first
+// (the page-table entry among them: tail_page); the new row is put among the page's other rows in registers instead of being
+// read back; a block of one page leaves its value rows to a second warp (tail_values) and its heads to both half warps; and
+// the sums of all heads share one tree of shuffles.  us a step of one unit of 4K tokens: 13.0 with one warp that starts when
+// the length is known, half its lanes idle at the heads and the two structs as arguments by value; 12.2 with two warps and
+// the structs in shared memory; 11.3 entered early.  (Inlined into the kernel the routine is no slower, but the step of 32
+// units at 128K then takes 54.7 us instead of 51.5.)
 template <int G>
-__device__ __noinline__ void tail_block(const TailArgs *args, const bf16 *q_rows, const int *page_table, int phys,
-                                        int unit, int raw, int N, float *sq, float *tail_u, float *tail_part, float4 *norm) {
-  const CkvDev &P = args->P;
-  const CkvNewToken &fresh = args->fresh;
+__device__ __noinline__ int tail_block(const TailArgs *args, const bf16 *q_rows, const int *page_table, const int *seq_lens, int unit,
+                                       int most, int hi_page, float *sq, float *tail_u, float *tail_part, float4 *norm) {
+  const CkvDev P = args->P;
+  const CkvNewToken fresh = args->fresh;
   const int lane = threadIdx.x & 31, hw = lane >> 4, li = lane & 15;
   const int s = ckv_div_hkv(P, unit), h = unit - s * P.Hkv;
   const int cap = P.max_blocks * P.bs;
   const bool lo_half = P.row_elems == CKV_ROW_ELEMS;
   const bool by_mass = (P.variant & CKV_VARIANT_RANK_BY_MASS) != 0;
   const int *pt_row = page_table + (size_t)s * P.max_pages_per_seq;
-  const bool append = fresh.k_new != nullptr && raw + 1 == N;   // (past the host's bound: see append_past_bound)
+  const bool any = fresh.k_new != nullptr;
+  const bf16 *k_new = reinterpret_cast<const bf16 *>(fresh.k_new) + (size_t)unit * CKV_D, *v_new = reinterpret_cast<const bf16 *>(fresh.v_new) + (size_t)unit * CKV_D;
+  constexpr int GH = G >= 2 ? G / 2 : 1;   // heads of a half warp
+  const int g0 = G >= 2 ? hw * GH : 0;
+  pdl_wait();
+  const int raw = seq_lens[s], page_guess = any && hi_page >= lane ? pt_row[hi_page - lane] : -1;
+  uint4 kn = make_uint4(0u, 0u, 0u, 0u), vn;   // this lane's eight coordinates of the new rows
+  if (any) kn = reinterpret_cast<const uint4 *>(k_new)[li];
+  uint4 qr[GH];    // ... and of the queries
+#pragma unroll
+  for (int g = 0; g < GH; ++g) qr[g] = reinterpret_cast<const uint4 *>(q_rows + (size_t)(g0 + g) * CKV_D)[li];
+  named_arrive(3, kThreads);   // nothing here needs what the others set up, and the cluster will wait for this warp
+  const int N = step_length(raw, any, cap, most);
+  if (N == 0) return raw;
+  const bool append = any && raw + 1 == N;   // (past the host's bound: see append_past_bound)
+  const int phys = append ? tail_page(page_guess, pt_row, hi_page, raw) : -1;
   const int b = ((N + P.bs - 1) >> P.lg_bs) - 1, cnt = N - b * P.bs;
   const bool split = tail_is_split(P, append, N);
-  uint4 kn, vn;   // this lane's eight coordinates of the new rows
-  kn = vn = make_uint4(0u, 0u, 0u, 0u);
-  if (append) {
-    kn = reinterpret_cast<const uint4 *>(reinterpret_cast<const bf16 *>(fresh.k_new) + (size_t)unit * CKV_D)[li];
-    if (!split) vn = reinterpret_cast<const uint4 *>(reinterpret_cast<const bf16 *>(fresh.v_new) + (size_t)unit * CKV_D)[li];
-  }
+  vn = kn;
+  if (append && !split) vn = reinterpret_cast<const uint4 *>(v_new)[li];
   const size_t row = (size_t)unit * P.max_blocks + b;
   __nv_bfloat16 *kmean_row = P.kmean + row * P.row_elems, *vmean_row = P.vmean + row * P.row_elems;
   float *dbar_row = P.dbar + row * P.r;
-  constexpr int GH = G >= 2 ? G / 2 : 1;   // heads of a half warp
-  const int g0 = G >= 2 ? hw * GH : 0;
-  uint4 qr[GH];    // this lane's coordinates of their queries
-#pragma unroll
-  for (int g = 0; g < GH; ++g) qr[g] = reinterpret_cast<const uint4 *>(q_rows + (size_t)(g0 + g) * CKV_D)[li];
   BlockRow br;
   if (append) {
     bf16 *kp = reinterpret_cast<bf16 *>(fresh.k_pool), *vp = reinterpret_cast<bf16 *>(fresh.v_pool);
@@ -277,16 +294,26 @@ __device__ __noinline__ void tail_block(const TailArgs *args, const bf16 *q_rows
     tail_part[lane * CKV_PART_STRIDE] = zl2;
     tail_part[lane * CKV_PART_STRIDE + 1] = 1.f;
   }
+  return raw;
 }
 
 // The value rows of a last block that tail_block shares with a second warp: new row into its page, mean value, partial.
 template <int G>
-__device__ __noinline__ void tail_values(const TailArgs *args, int phys, int unit, int raw, int N, float *tail_part) {
-  const CkvDev &P = args->P;
-  const CkvNewToken &fresh = args->fresh;
+__device__ __noinline__ int tail_values(const TailArgs *args, const int *page_table, const int *seq_lens, int unit, int most, int hi_page, float *tail_part) {
+  const CkvDev P = args->P;
+  const CkvNewToken fresh = args->fresh;
   const int lane = threadIdx.x & 31, hw = lane >> 4, li = lane & 15;
   const int s = ckv_div_hkv(P, unit), h = unit - s * P.Hkv;
-  const uint4 vn = reinterpret_cast<const uint4 *>(reinterpret_cast<const bf16 *>(fresh.v_new) + (size_t)unit * CKV_D)[li];
+  const int *pt_row = page_table + (size_t)s * P.max_pages_per_seq;
+  const bool any = fresh.k_new != nullptr;
+  pdl_wait();
+  const int raw = seq_lens[s], page_guess = any && hi_page >= lane ? pt_row[hi_page - lane] : -1;
+  uint4 vn = make_uint4(0u, 0u, 0u, 0u);
+  if (any) vn = reinterpret_cast<const uint4 *>(reinterpret_cast<const bf16 *>(fresh.v_new) + (size_t)unit * CKV_D)[li];
+  named_arrive(3, kThreads);
+  const int N = step_length(raw, any, P.max_blocks * P.bs, most);
+  if (!any || N == 0 || raw + 1 != N || !tail_is_split(P, true, N)) return raw;
+  const int phys = tail_page(page_guess, pt_row, hi_page, raw);
   const int b = ((N + P.bs - 1) >> P.lg_bs) - 1, cnt = N - b * P.bs;
   bf16 *vp = reinterpret_cast<bf16 *>(fresh.v_pool);
   const bool ok = phys >= 0 && phys < P.num_pages;
@@ -305,6 +332,7 @@ __device__ __noinline__ void tail_values(const TailArgs *args, int phys, int uni
   block_stats_finish<false, true>(P, b, (float)cnt, none, vs, none2, nullptr, nullptr, nullptr,
                                   P.vmean + ((size_t)unit * P.max_blocks + b) * P.row_elems, lane, false, &br);
   tail_store_value<G>(tail_part, br.x, true, hw, 2, li);
+  return raw;
 }
 
 // The append of a sequence that has outgrown the host's bound: the token lands in a block that the step does not look at,
@@ -386,9 +414,9 @@ ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int 
     if (i < (int)sizeof(CkvNewToken) / 4) reinterpret_cast<int *>(&s_tail.fresh)[i] = reinterpret_cast<const int *>(&fresh)[i];
     named_barrier(4, 64);
   }
+  if (warp == kValueWarp) reinterpret_cast<uint4 *>(s_zero_row)[lane] = make_uint4(0u, 0u, 0u, 0u);
   cluster_arrive_release();   // "this CTA runs, its barriers are set up"
   pdl_trigger();              // the next launch of the stream may set itself up ...
-  pdl_wait();                 // ... and this one touches nothing before the launch ahead of it is complete
   const size_t row0 = (size_t)unit * P.max_blocks;
   const bool dbar_bulk = P.r >= 4;
   const int stage_bytes = TB * (kRowBytesK + kRowBytesV) + (dbar_bulk ? TB * P.r * 4 : 0);
@@ -425,18 +453,27 @@ ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int 
   // CTA starts on its first part 1.2 us after the length is known instead of 2.0 (a step of 8 units at 32K 15.4 -> 14.8 us, 16
   // units with r = d at 88K 40.5 -> 39.6, 32 units at 128K 52.6 -> 51.5).
   const int n_early = max(min(plan.first_parts * 16, plan.max_blocks - rank * plan.first_parts * 16), 0);
-  if (tid == kProducerWarp * 32 && n_early > 0) fill(0, rank * plan.first_parts * 16, n_early, 0, &full_bar[0][0]);
-  const int raw = seq_lens[s];
-  if (tid < G * 16) *reinterpret_cast<uint4 *>(&s_q[tid >> 4][8 * (tid & 15)]) = reinterpret_cast<const uint4 *>(q + (size_t)unit * G * CKV_D)[tid];
-  // The new token's page: the tail warps read the last 32 entries of the page-table row under the host's bound while the
-  // length is on its way; a length the bound exceeds by more is looked up when it is known.
+  // The launch ahead of this one is waited for in each of the three branches: nobody touches anything before that.  The tail
+  // routines set up all they can ahead of it.  Only the working warps wait for the queries' staging: the producer wants the
+  // length alone (queries in host memory take 3 us to arrive).
   const int *pt_row = page_table + (size_t)s * P.max_pages_per_seq;
-  int page_guess = -1;
-  if (warp >= kTailWarp && rank == C - 1 && append && plan.hi_page >= lane) page_guess = pt_row[plan.hi_page - lane];
-  if (tid >= kThreads - 32) reinterpret_cast<uint4 *>(s_zero_row)[lane] = make_uint4(0u, 0u, 0u, 0u);
+  const int most_len = plan.max_blocks * P.bs;
+  int raw;
+  if (warp >= kTailWarp && rank == C - 1) {
+    raw = warp == kTailWarp ? tail_block<G>(&s_tail, q + (size_t)unit * G * CKV_D, page_table, seq_lens, unit, most_len, plan.hi_page, s_sq,
+                                            s_tail_u, &s_tail_part[0][0], s_wn[kWarps])
+                            : tail_values<G>(&s_tail, page_table, seq_lens, unit, most_len, plan.hi_page, &s_tail_part[0][0]);
+  } else {
+    pdl_wait();
+    if (tid == kProducerWarp * 32 && n_early > 0) fill(0, rank * plan.first_parts * 16, n_early, 0, &full_bar[0][0]);
+    raw = seq_lens[s];
+    if (tid < G * 16) *reinterpret_cast<uint4 *>(&s_q[tid >> 4][8 * (tid & 15)]) = reinterpret_cast<const uint4 *>(q + (size_t)unit * G * CKV_D)[tid];
+    if (warp < kWarps) named_barrier(3, kThreads);
+    else named_arrive(3, kThreads);
+  }
   // the length the step works on; of a sequence longer than the host's bound, what the shared arrays were sized for
   const int N_all = max(min(raw + ((append && raw >= 0 && raw < cap) ? 1 : 0), cap), 0);
-  const int N = min(N_all, plan.max_blocks * P.bs);
+  const int N = min(N_all, most_len);
   if (N < N_all && rank == 0 && tid == 0) atomicOr(P.status, CKV_DEV_BAD_BOUND);
   const int X = (N + P.bs - 1) >> P.lg_bs, Xs = max(X - 1, 0);
   // What the CTA owns, `own` blocks in all: n0 blocks from b0 on -- its first tile, whose place depends on the host's plan
@@ -455,10 +492,6 @@ ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int 
   // fall into 32 different banks)
   float *ub = reinterpret_cast<float *>(smem + plan.u_off);
   const int us = plan.own_cap + 8;
-
-  // The tail warps do not wait here: they need nothing that the others set up, and the cluster will wait for them.
-  if (warp >= kTailWarp) named_arrive(3, kThreads);
-  else named_barrier(3, kThreads);
 
   ScanUnit<G, bf16, RD> w;
   w.reset();
@@ -493,21 +526,8 @@ ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int 
         asm volatile("prefetch.global.L2 [%0];" ::"l"(pt_row + 32 * i) : "memory");
     }
   } else if (warp >= kTailWarp) {
-    const bool appended = rank == C - 1 && append && raw + 1 == N;
-    int phys = -1;
-    if (appended) {
-      const int back = plan.hi_page - raw / CKV_PAGE;
-      phys = __shfl_sync(0xffffffffu, page_guess, back & 31);
-      if ((unsigned)back > 31u) phys = pt_row[raw / CKV_PAGE];
-    }
-    if (warp == kValueWarp) {
-      if (appended && tail_is_split(P, true, N)) tail_values<G>(&s_tail, phys, unit, raw, N, &s_tail_part[0][0]);
-    } else if (rank == C - 1 && N > 0) {
-      if (append && raw >= N && raw < cap) append_past_bound(P, page_table, fresh, unit, raw, s_sq);
-      tail_block<G>(&s_tail, q + (size_t)unit * G * CKV_D, page_table, phys, unit, raw, N, s_sq, s_tail_u, &s_tail_part[0][0], s_wn[kWarps]);
-    } else if (lane < G) {
-      s_wn[kWarps][lane] = make_float4(-CUDART_INF_F, 0.f, -CUDART_INF_F, 0.f);
-    }
+    if (warp == kTailWarp && rank == C - 1 && append && raw >= N && raw < cap) append_past_bound(P, page_table, fresh, unit, raw, s_sq);
+    if (warp == kTailWarp && (rank != C - 1 || N == 0) && lane < G) s_wn[kWarps][lane] = make_float4(-CUDART_INF_F, 0.f, -CUDART_INF_F, 0.f);
     if (warp == kTailWarp && append && raw < 0 && rank == C - 1 && lane == 0) atomicOr(P.status, CKV_DEV_SEQ_FULL);   // no place for the token
   } else {
     // ---------------- working warps: parts of 16 blocks ----------------
