@@ -74,6 +74,8 @@ constexpr int kAfterScan = kOffPages + kWarps * 2 * kPageBytes;
 constexpr int kRecvStride = 36;                 // floats of one (head, 32 coordinates) partial: values, maximum, weight sum
 constexpr int kDynLimit = 227 * 1024 - 20 * 1024;   // dynamic shared memory; the kernel's static arrays take under 20 KB
 
+// 2^(a - b) of two running maxima, 0 where a is -inf (as b may be, too).
+__device__ __forceinline__ float part_scale(float a, float b) { return a == -CUDART_INF_F ? 0.f : fast_exp2(a - b); }
 // One more in a shared-memory counter.
 __device__ __forceinline__ void red_shared_inc(uint32_t addr) { asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(addr) : "memory"); }
 
@@ -629,7 +631,7 @@ ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int 
 #pragma unroll
     for (int i = 1; i <= kWarps; ++i) { m = fmaxf(m, e[i].x); u = fmaxf(u, e[i].z); }
 #pragma unroll
-    for (int i = 0; i <= kWarps; ++i) l = fmaf(e[i].y, exp2_diff(e[i].x, m), l);
+    for (int i = 0; i <= kWarps; ++i) l = fmaf(e[i].y, part_scale(e[i].x, m), l);
     if (lane < C) {
       const uint32_t x0 = smem_u32(&s_xbar[0]), there = cluster_map(x0, lane);   // the CTAs' shared memories are congruent windows
       st_async_u32x4(there + (smem_u32(&s_norm[rank][warp]) - x0), __float_as_uint(m), __float_as_uint(l), __float_as_uint(u), 0u, there);
@@ -673,7 +675,7 @@ ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int 
       u = fmaxf(u, __shfl_xor_sync(0xffffffffu, u, o));
     }
 #pragma unroll
-    for (int i = 0; i < EPL; ++i) l = fmaf(e[i].y, exp2_diff(e[i].x, m), l);
+    for (int i = 0; i < EPL; ++i) l = fmaf(e[i].y, part_scale(e[i].x, m), l);
 #pragma unroll
     for (int o = LPH / 2; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
     const float il = 1.0f / l, b = fast_exp2(u - m) * il;
@@ -1043,7 +1045,7 @@ ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int 
       float4 num = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
       for (int e = 0; e <= kWarps; ++e) {
-        const float sc = exp2_diff(ml[e].x, M);
+        const float sc = part_scale(ml[e].x, M);
         if (sc != 0.f) {   // an entry that holds nothing may hold any bits
           den = fmaf(ml[e].y, sc, den);
           num.x = fmaf(x[e].x, sc, num.x); num.y = fmaf(x[e].y, sc, num.y);
@@ -1068,7 +1070,7 @@ ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int 
       for (int e = 0; e < C; ++e) M = fmaxf(M, e0[e * kRecvStride + 32]);
 #pragma unroll 4
       for (int e = 0; e < C; ++e) {
-        const float sc = exp2_diff(e0[e * kRecvStride + 32], M);
+        const float sc = part_scale(e0[e * kRecvStride + 32], M);
         den = fmaf(e0[e * kRecvStride + 33], sc, den);
         o = fmaf(e0[e * kRecvStride + lane], sc, o);
       }
