@@ -71,6 +71,7 @@ struct CkvHostDone { int *flag, *count, *ctas; };
 // How a step runs as one launch (ckv_unit_step_plan).
 struct CkvStepPlan {
   int cluster;      // CTAs per unit
+  unsigned c_magic; // floor(2^32 / cluster) + 1: x / cluster = umulhi(x, c_magic) (cluster > 1)
   int stages;       // ring stages of the scan phase
   int own_cap;      // blocks of a unit one CTA owns, at most (a multiple of 16)
   int first_parts;  // 16-block parts of a CTA's first tile, which lies at rank * first_parts whatever the length

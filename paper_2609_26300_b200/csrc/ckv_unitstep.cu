@@ -399,6 +399,9 @@ ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int 
   const int unit = blockIdx.y, s = ckv_div_hkv(P, unit), h = unit - s * P.Hkv;
   const bool append = fresh.k_new != nullptr;
   const int cap = P.max_blocks * P.bs;
+  auto div_c = [&](int x) { return C == 1 ? x : (int)__umulhi((unsigned)x, plan.c_magic); };   // x / C, 0 <= x < 2^32 / C
+  float log_bs = logf((float)P.bs);
+  asm volatile("" : "+f"(log_bs));   // (here, ahead of the wait for the launch before, and not where it is used)
   if (tid == kProducerWarp * 32) {
     for (int st = 0; st < plan.stages; ++st) { mbar_init(&full_bar[0][st], 1); mbar_init(&full_bar[1][st], 1); mbar_init(&empty_bar[st], kParts); }
     for (int i = 0; i < 3; ++i) mbar_init(&s_xbar[i], 1);
@@ -482,7 +485,7 @@ ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int 
   // alone, so that its copy is under way before the length is known -- then the CTA's part of what the first tiles leave.
   const int first = plan.first_parts * 16;
   const int n_parts = (Xs + 15) >> 4, rest = max(n_parts - C * plan.first_parts, 0);
-  const int ppc = (int)ckv_udiv24((unsigned)(rest + C - 1), (unsigned)C);
+  const int ppc = div_c(rest + C - 1);
   const int b0 = rank * first, b1 = C * first + min(rank * ppc, rest) * 16;
   const int n0 = max(min(Xs - b0, first), 0);
   const int own = min(n0 + max(min(b1 + ppc * 16, Xs) - b1, 0), plan.own_cap);
@@ -566,7 +569,7 @@ ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int 
 #pragma unroll
         for (int t = 0; t < 4; ++t) w.wown[e][t] = T::head(lane, e) < G ? s_w[t * G + T::head(lane, e)] : 0.f;
     }
-    const ScanPartCfg cfg{P.scale, P.half_var, logf((float)P.bs), P.r, P.max_blocks, (P.variant & CKV_VARIANT_RANK_BY_MASS) != 0, P.r == 4};
+    const ScanPartCfg cfg{P.scale, P.half_var, log_bs, P.r, P.max_blocks, (P.variant & CKV_VARIANT_RANK_BY_MASS) != 0, P.r == 4};
     float *lz = P.lz + row0 * G;
     const int part = warp % kParts;
     // A warp visits every kSkip-th tile.  A fill is only issued once the one plan.stages before it was released, and
@@ -742,7 +745,8 @@ ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int 
   auto below = [](int n) { return n >= 64 ? ~0ull : (1ull << max(n, 0)) - 1ull; };   // bits 0 .. n - 1
   unsigned long long here = below(min(4 * nj, X - s0));
   unsigned long long rk = here & below(rank_lo + rank_n - s0) & ~below(rank_lo - s0);
-  asm volatile("" : "+l"(here), "+l"(rk));   // (here, and not where they are used)
+  float lg_bs = log2f((float)P.bs), lg_last = log2f((float)max(N - Xs * P.bs, 1));   // the attention's
+  asm volatile("" : "+l"(here), "+l"(rk), "+f"(lg_bs), "+f"(lg_last));   // (here, and not where they are used)
   wait_x(1);
   // (the histogram is clear, too.)  A CTA one of whose waits ran out has scores that never came: it selects nothing and
   // contributes an empty partial, so that the others get what they wait for.
@@ -892,13 +896,12 @@ ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int 
     const bool comp = nsel < X && !dead && !(P.variant & CKV_VARIANT_DROP);
     if (!comp) w.reset();   // nothing is compensated: the scan's sums are not wanted
     const int n_pages = dead ? 0 : (all ? (N + CKV_PAGE - 1) / CKV_PAGE : nsel * P.ppb);
-    const int share = (int)ckv_udiv24((unsigned)(n_pages + C - 1), (unsigned)C);
+    const int share = div_c(n_pages + C - 1);
     const int p0 = min(rank * share, n_pages), p1 = min(p0 + share, n_pages);
     const int n_mine = max((p1 - p0 - warp + kWarps - 1) / kWarps, 0);
     const int pshift = P.ppb == 1 ? 0 : (P.ppb == 2 ? 1 : 2);
     const float *lz = P.lz + row0 * G;
     const float sl2 = P.scale * kLog2e;
-    const float lg_bs = log2f((float)P.bs), lg_last = log2f((float)max(N - Xs * P.bs, 1));
     const uint32_t buf0 = smem_u32(smem + kOffPages) + warp * 2 * kPageBytes;
     const bool rows_rm = HS && comp;   // one more item per 16 pages: the mean-value rows of their blocks
     bool bad = false;
@@ -1052,7 +1055,7 @@ ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int 
           num.z = fmaf(x[e].z, sc, num.z); num.w = fmaf(x[e].w, sc, num.w);
         }
       }
-      const int item = 4 * g + (c >> 5), slot = (int)ckv_udiv24((unsigned)item, (unsigned)C);
+      const int item = 4 * g + (c >> 5), slot = div_c(item);
       const uint32_t to = (uint32_t)(item - slot * C);
       const uint32_t ent = smem_u32(s_recv) + (uint32_t)((slot * C + rank) * kRecvStride) * 4u;
       const uint32_t bar = cluster_map(smem_u32(&s_xbar[2]), to);
@@ -1223,6 +1226,7 @@ bool ckv_unit_step_plan(const ckv_ctx *c, int batch, int max_len, int kcap, CkvS
   }
   plan->smem = (int)std::max(plan->u_off + term_bytes(plan->own_cap), (size_t)kAfterScan);
   plan->cluster = C;
+  plan->c_magic = C > 1 ? (unsigned)(0x100000000ull / (unsigned)C) + 1u : 0u;
   return true;
 }
 
