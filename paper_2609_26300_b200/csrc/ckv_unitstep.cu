@@ -58,7 +58,8 @@ constexpr int kBins = 2048;                     // score histogram: 32 octaves b
 constexpr int kBinShift = 17;                   // ... a bin is a score's bit pattern without its low 17 bits
 constexpr int kIdMask = (1 << (31 - kBinShift)) - 1;   // block ids beside those 17 bits in one word
 static_assert(kScoresCap <= kIdMask + 1, "block ids fit");
-constexpr int kKeyGroups = kScoresCap / 4 / kWork;   // four scores each, as a thread holds them for the selection
+constexpr int kKeyGroups = kScoresCap / 4 / kWork;   // four scores each, as a thread holds them for the selection (a whole number: none of a thread's lies past the array)
+static_assert(kKeyGroups * 4 * kWork == kScoresCap && kKeyGroups % 2 == 1, "see the selection");
 constexpr int kMapWords = 2 * kWork;            // selection bit map: two words per working thread, enough for kScoresCap blocks
 constexpr int kSelCap = 512;                    // selected blocks the id list holds (unless every block is selected)
 constexpr int kOwnMost = 2800, kSeqCtas = 24;   // blocks a CTA may own where a sequence gets few CTAs (see ckv_unit_step_plan)
@@ -746,15 +747,18 @@ ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int 
   unsigned long long here = below(min(4 * nj, X - s0));
   unsigned long long rk = here & below(rank_lo + rank_n - s0) & ~below(rank_lo - s0);
   float lg_bs = log2f((float)P.bs), lg_last = log2f((float)max(N - Xs * P.bs, 1));   // the attention's
-  asm volatile("" : "+l"(here), "+l"(rk), "+f"(lg_bs), "+f"(lg_last));   // (here, and not where they are used)
+  const int K = min(kcap, X);
+  const bool all = X <= kcap;          // every block is selected: the step is dense attention
+  // ... and the attention's share of the selected pages
+  const int n_pages = all ? (N + CKV_PAGE - 1) / CKV_PAGE : K * P.ppb, share = div_c(n_pages + C - 1);
+  int p0 = min(rank * share, n_pages), n_mine = max((min(p0 + share, n_pages) - p0 - warp + kWarps - 1) / kWarps, 0);
+  asm volatile("" : "+l"(here), "+l"(rk), "+f"(lg_bs), "+f"(lg_last), "+r"(p0), "+r"(n_mine));   // (here, and not where they are used)
   wait_x(1);
   // (the histogram is clear, too.)  A CTA one of whose waits ran out has scores that never came: it selects nothing and
   // contributes an empty partial, so that the others get what they wait for.
   const bool dead = __syncthreads_or(*(volatile int *)&s_abort) != 0;
 
   // ---- selection (Eq. 11), the same in every CTA ----
-  const int K = min(kcap, X);
-  const bool all = X <= kcap;          // every block is selected: the step is dense attention
   int *ids = reinterpret_cast<int *>(smem + kOffIds);
   if (warp >= kWarps && !dead) {   // the idle warps leave the range's scores where ckv_copy_scores() finds them
     float *scores = P.scores + row0;
@@ -785,7 +789,7 @@ ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int 
 #pragma unroll
         for (int j = 0; j < kKeyGroups; ++j) {
           if (j >= nj) break;
-          const uint4 k4 = keys4[min(tid * nj + j, kScoresCap / 4 - 1)];
+          const uint4 k4 = keys4[tid * nj + j];
           key[j][0] = k4.x; key[j][1] = k4.y; key[j][2] = k4.z; key[j][3] = k4.w;
         }
         {
@@ -847,6 +851,7 @@ ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int 
           const unsigned long long above = rk & ((unsigned long long)ge_hi[1] << 32 | ge_hi[0]);
           unsigned long long at = rk & ~above & ((unsigned long long)ge_lo[1] << 32 | ge_lo[0]);
           sel |= above;
+          if (tid >= nc && tid < nc + 3) cand[tid] = 0;   // the last group of four is filled up
           while (at != 0) {
             const int b = s0 + __ffsll((long long)at) - 1;
             at &= at - 1;
@@ -857,8 +862,11 @@ ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int 
           if (tid < nc) {
             const uint32_t mine = cand[tid];
             int place = 0;
-#pragma unroll 8
-            for (int j = 0; j < nc; ++j) place += cand[j] > mine ? 1 : 0;
+#pragma unroll 2
+            for (int j = 0; j < nc; j += 4) {
+              const uint4 k = *reinterpret_cast<const uint4 *>(cand + j);
+              place += (k.x > mine ? 1 : 0) + (k.y > mine ? 1 : 0) + (k.z > mine ? 1 : 0) + (k.w > mine ? 1 : 0);
+            }
             const int b = kIdMask - (int)(mine & kIdMask);
             if (place < take) atomicOr(&map[b >> 5], 1u << (b & 31));
           }
@@ -895,10 +903,7 @@ ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int 
     // ---- exact attention over the CTA's share of the selected pages ----
     const bool comp = nsel < X && !dead && !(P.variant & CKV_VARIANT_DROP);
     if (!comp) w.reset();   // nothing is compensated: the scan's sums are not wanted
-    const int n_pages = dead ? 0 : (all ? (N + CKV_PAGE - 1) / CKV_PAGE : nsel * P.ppb);
-    const int share = div_c(n_pages + C - 1);
-    const int p0 = min(rank * share, n_pages), p1 = min(p0 + share, n_pages);
-    const int n_mine = max((p1 - p0 - warp + kWarps - 1) / kWarps, 0);
+    if (dead) n_mine = 0;
     const int pshift = P.ppb == 1 ? 0 : (P.ppb == 2 ? 1 : 2);
     const float *lz = P.lz + row0 * G;
     const float sl2 = P.scale * kLog2e;
