@@ -27,8 +27,8 @@ constexpr int kBins = 4096;
 constexpr int kFineShift = 17;                  // the first histogram: 64 bins an octave ...
 constexpr int kFineBase = (127 - 54) << 6;      // ... from 2^-54 to 2^10; what lies outside goes into the end bins
 
-// Exclusive prefix sum of one int per thread over the CTA; *total (if given) receives the sum.  A caller's next use of
-// the same warp_tot lies behind a barrier of its own.
+// Exclusive prefix sum of one int per thread over the CTA (one barrier); *total (if given; the caller's own) receives the
+// sum.  A caller's next use of the same warp_tot lies behind a barrier of its own.
 __device__ __forceinline__ int block_exclusive_scan(int v, int *warp_tot, int *total) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int inc = v;
@@ -39,19 +39,9 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int *warp_tot, int *t
   }
   if (lane == 31) warp_tot[warp] = inc;
   __syncthreads();
-  if (warp == 0) {
-    const int w = warp_tot[lane];
-    int winc = w;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int t = __shfl_up_sync(0xffffffffu, winc, o);
-      if (lane >= o) winc += t;
-    }
-    warp_tot[lane] = winc - w;
-    if (total != nullptr && lane == 31) *total = winc;
-  }
-  __syncthreads();
-  return warp_tot[warp] + inc - v;
+  const int w = warp_tot[lane];   // every warp adds up the totals it needs: no second barrier
+  if (total != nullptr) *total = __reduce_add_sync(0xffffffffu, w);
+  return __reduce_add_sync(0xffffffffu, lane < warp ? w : 0) + inc - v;
 }
 
 template <int G>
@@ -203,9 +193,12 @@ __global__ void __launch_bounds__(kThreads) ckv_select_kernel(CkvDev P, const in
     direct = cached && s_total <= kThreads;
     if (direct) {   // rank the bin's blocks by (score descending, id ascending) and mark the first `take`
       const int digit = s_digit, take = s_remaining, nc = s_total;
+      // the bin's keys (the end bins take what lies outside the histogram)
+      const uint32_t from = digit == 0 ? 0u : (uint32_t)(kFineBase + digit) << kFineShift;
+      const uint32_t past = digit == kBins - 1 ? 0x80000000u : (uint32_t)(kFineBase + digit + 1) << kFineShift;
       for (int b = tid; b < X; b += kThreads) {
         const uint32_t k = skeys[b];
-        if (bin0(k) == digit && !mandatory(b)) s_cand[atomicAdd(&s_ncand, 1)] = (uint64_t)k << 32 | (uint32_t)~b;
+        if (k - from < past - from && !mandatory(b)) s_cand[atomicAdd(&s_ncand, 1)] = (uint64_t)k << 32 | (uint32_t)~b;
       }
       __syncthreads();
       if (tid < nc) {
@@ -288,8 +281,8 @@ __global__ void __launch_bounds__(kThreads) ckv_select_kernel(CkvDev P, const in
   } else {
     walk([&](int b) { ++c_sel; if (masked) picked |= 1u << (b - b0); });
   }
-  int pos = block_exclusive_scan(c_sel, s_wtot[2], &s_total);
-  const int total = s_total;
+  int total;
+  int pos = block_exclusive_scan(c_sel, s_wtot[2], &total);
   if (masked) {
     while (picked != 0) {
       const int j = __ffs(picked) - 1;
