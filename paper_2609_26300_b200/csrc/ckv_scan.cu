@@ -278,7 +278,8 @@ ckv_scan_kernel(CkvDev P, const QT *q, const int *seq_lens, int units, int stage
   // spans more than two), staged by the consumer warps while the first fills are on their way: a warp that moves
   // on to another unit then sets up from shared memory instead of paying a round trip to global memory.
   constexpr int kStagedUnits = 4;
-  __shared__ __align__(16) __nv_bfloat16 s_q[kStagedUnits][G][CKV_D];
+  constexpr int kQStride = CKV_D + 8;   // (eight rows' matrix loads hit eight bank groups)
+  __shared__ __align__(16) __nv_bfloat16 s_q[kStagedUnits][G][kQStride];
   __shared__ float s_w[kStagedUnits][G][4];
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -419,7 +420,7 @@ ckv_scan_kernel(CkvDev P, const QT *q, const int *seq_lens, int units, int stage
         if (uu <= s_ulast && uu < units) {
           const int s2 = ckv_div_hkv(P, uu), h2 = uu - s2 * P.Hkv;
           const uint4 *src = reinterpret_cast<const uint4 *>(q + ((size_t)s2 * P.Hq + h2 * G) * CKV_D);
-          reinterpret_cast<uint4 *>(&s_q[k][0][0])[pc] = src[pc];
+          *reinterpret_cast<uint4 *>(&s_q[k][pc >> 4][8 * (pc & 15)]) = src[pc];
         }
       }
       named_barrier(1, kConsumerWarps * 32);
@@ -428,10 +429,13 @@ ckv_scan_kernel(CkvDev P, const QT *q, const int *seq_lens, int units, int stage
         const int k = idx / (G * 4), g = (idx / 4) % G, t = idx % 4;
         if (s_u0 + k <= s_ulast) {
           float w = 0.f;
-          for (int i = 0; i < CKV_D / 4; ++i) {   // the group's 32 coordinates: one run, or two runs of 16
+#pragma unroll
+          for (int i = 0; i < CKV_D / 4; i += 8) {   // the group's 32 coordinates: one run, or two runs of 16
             const int c = P.glayout == 0 ? 32 * t + i : (i < 16 ? 16 * t + i : CKV_D / 2 + 16 * t + (i - 16));
-            const float x = __bfloat162float(s_q[k][g][c]);
-            w = fmaf(x, x, w);
+            float x[8];
+            load8<false>(&s_q[k][g][c], x);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) w = fmaf(x[j], x[j], w);
           }
           s_w[k][g][t] = w * (P.scale * P.scale);
         }
@@ -518,10 +522,7 @@ ckv_scan_kernel(CkvDev P, const QT *q, const int *seq_lens, int units, int stage
         const int uk = u - s_u0;
         const bool from_smem = staged && uk < kStagedUnits;
         if (from_smem) {
-          w.set_queries(lane, P.scale, [&](int g, int c) {
-            const uint32_t x = *reinterpret_cast<const uint32_t *>(&s_q[uk][g][c]);
-            return make_float2(__uint_as_float(x << 16), __uint_as_float(x & 0xffff0000u));
-          });
+          if constexpr (!QS) w.load_queries(lane, P.scale, smem_u32(&s_q[uk][0][0]), kQStride * 2, smem_u32(s_zero_row));
 #pragma unroll
           for (int e = 0; e < 2; ++e)
 #pragma unroll
@@ -620,8 +621,8 @@ ScanCfg scan_cfg(const CkvDev &P, int G) {
   const size_t stage_bytes = TB * (krow + vrow) + (P.r >= 4 ? TB * P.r * 4 : 0);
   const size_t sw_bytes = (P.r == 4 || P.r == CKV_D) ? 0 : (size_t)kConsumerWarps * P.r * G * 4;   // weight table of the generic path
   // 227 KB per CTA, less the kernel's static shared memory (lengths, barriers, the row of zeros: under 6 KB; staged
-  // query rows and variance weights: 4 units x G x 272 bytes) and a reserve
-  const size_t stat = 6 * 1024 + (size_t)4 * G * (CKV_D * 2 + 16);
+  // query rows and variance weights: 4 units x G x 288 bytes) and a reserve
+  const size_t stat = 6 * 1024 + (size_t)4 * G * (CKV_D * 2 + 32);
   const size_t budget = 227 * 1024 - stat - 1024 - sw_bytes;
   int stages = (int)(budget / stage_bytes);
   if (stages > kMaxStages) stages = kMaxStages;
