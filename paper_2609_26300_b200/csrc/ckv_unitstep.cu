@@ -1169,13 +1169,13 @@ cudaError_t ckv_configure_unit_step(ckv_ctx *c) {
 }
 
 // Whether a step of this size runs as one launch, and how.  Against the separate launches (us per step, back to back):
-// 12.9 / 27.4 (one head, 4K), 15.4 / 35.8 (8 units, 32K), 20.3 / 38.6 (8 units, 128K, 32-token blocks), 30.0 / 51.2 (24
-// units, 100K, bf16 summaries), 40.5 / 60.3 (16 units, 88K, r = d), 52.4 / 68.4 (32 units, 128K), 54.6 / 69.1 (72 units,
-// 64K), 56.3 / 63.8 (128 units, 32K).
+// 11.0 / 19.3 (one head, 4K), 13.0 / 24.9 (8 units, 32K), 17.2 / 29.4 (8 units, 128K, 32-token blocks), 29.0 / 38.8 (24 units,
+// 100K, bf16 summaries), 36.7 / 47.5 (16 units, 88K, r = d), 48.2 / 61.2 (32 units, 128K), 57.7 / 77.1 (72 units, 64K), 64.6 /
+// 74.2 (128 units, 32K).
 // What stays with the separate launches, and why:
 //   * fp32 pages (the attention is on bf16 tensor cores) and an explicit ckv_set_tail_mode, which asks for them;
-//   * caches under CKV_STEP_MIN_TOKENS.  Not a crossover -- one launch is ahead there too (one sequence of 500 tokens 15.0 /
-//     21.1, 16 of 1000 17.5 / 26.4) -- but the size below which the documented two-call arrangement (append, scan, select,
+//   * caches under CKV_STEP_MIN_TOKENS.  Not a crossover -- one launch is ahead there too (one sequence of 1600 tokens 11.5 /
+//     19.5, 16 of them 17.2 / 27.1) -- but the size below which the documented two-call arrangement (append, scan, select,
 //     attention as launches of their own) is kept;
 //   * more units than CTAs run at once: a last wave that is nearly empty costs a whole wave (192 units: 92 / 90);
 //   * more than kOwnMost blocks a CTA where a sequence gets fewer than kSeqCtas of them.  The host knows the longest
