@@ -73,7 +73,7 @@ constexpr int kOffCand = kOffIds + kSelCap * 4;
 constexpr int kOffPages = (kOffCand + kCandCap * 4 + 127) / 128 * 128;
 constexpr int kAfterScan = kOffPages + kWarps * 2 * kPageBytes;
 constexpr int kRecvStride = 36;                 // floats of one (head, 32 coordinates) partial: values, maximum, weight sum
-constexpr int kDynLimit = 227 * 1024 - 20 * 1024;   // dynamic shared memory; the kernel's static arrays take under 20 KB
+constexpr int kDynLimit = 227 * 1024 - 20 * 1024;   // dynamic shared memory; the kernel's static arrays take 20 KB at most
 
 // 2^(a - b) of two running maxima, 0 where a is -inf (as b may be, too).
 __device__ __forceinline__ float part_scale(float a, float b) { return a == -CUDART_INF_F ? 0.f : fast_exp2(a - b); }
