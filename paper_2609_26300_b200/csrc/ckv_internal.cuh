@@ -74,7 +74,7 @@ struct CkvStepPlan {
   unsigned c_magic; // floor(2^32 / cluster) + 1: x / cluster = umulhi(x, c_magic) (cluster > 1)
   int stages;       // ring stages of the scan phase
   int own_cap;      // blocks of a unit one CTA owns, at most (a multiple of 16)
-  int first_parts;  // 16-block parts of a CTA's first tile, which lies at rank * first_parts whatever the length
+  int early_parts;  // 16-block parts a CTA owns of a sequence as long as the host's bound
   int hi_page;      // the last page of a sequence as long as the host's bound
   int u_off, smem;  // offset of the score terms in dynamic shared memory, and its size
   int max_blocks;   // blocks of a sequence the step can work on (the capacity, or the host's bound on the lengths)

@@ -427,9 +427,9 @@ ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int 
   const bool dbar_bulk = P.r >= 4;
   const int stage_bytes = TB * (kRowBytesK + kRowBytesV) + (dbar_bulk ? TB * P.r * 4 : 0);
   // test hook (ckv_debug_set): one fill is announced but never issued, so that the waits on it run out
-  auto withheld = [&](int it) { return (P.debug & CKV_DEBUG_SKIP_FILL) != 0 && it == 0 && rank == 0 && unit == 0; };
-  // one fill of the ring: tile `it`, nb blocks from block b on, into stage `st`, counted on full barrier `fb`
-  auto fill = [&](int it, int b, int nb, int st, uint64_t *fb) {
+  auto withheld = [&](int f) { return (P.debug & CKV_DEBUG_SKIP_FILL) != 0 && f == 0 && rank == 0 && unit == 0; };
+  // fill `f` of the ring: nb blocks from block b on into stage `st`, counted on full barrier `fb`
+  auto fill = [&](int f, int b, int nb, int st, uint64_t *fb) {
     const size_t row = row0 + b;
     unsigned char *sk = smem + (size_t)st * stage_bytes;
     unsigned char *sv = sk + TB * kRowBytesK;
@@ -439,7 +439,7 @@ ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int 
     mbar_arrive_expect_tx(fb, kbytes + vbytes + dbytes);
     const uint32_t lo = smem_u32(smem), hi = lo + (uint32_t)plan.stages * stage_bytes;
     bool ok = nb >= 1 && b + nb <= P.max_blocks;
-    if (!withheld(it)) {
+    if (!withheld(f)) {
       ok = ok && bulk_g2s_checked(sk, P.kmean + row * P.row_elems, kbytes, fb, lo, hi);
       if constexpr (VH) {
         // rows [row, row + TB) of the mean-values region, first 256 bytes of each (rows past the range are never read)
@@ -454,11 +454,15 @@ ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int 
     }
     if (!ok) atomicOr(P.status, CKV_DEV_BAD_COPY);
   };
-  // The first tile's place follows from the plan; of a sequence that ends sooner, rows that nobody looks at are copied.  With
-  // this copy ahead of the length, the others issued by the producer's lanes and the queries' fragments loaded as matrices, a
-  // CTA starts on its first part 1.2 us after the length is known instead of 2.0 (a step of 8 units at 32K 15.4 -> 14.8 us, 16
-  // units with r = d at 88K 40.5 -> 39.6, 32 units at 128K 52.6 -> 51.5).
-  const int n_early = max(min(plan.first_parts * 16, plan.max_blocks - rank * plan.first_parts * 16), 0);
+  // Ahead of the length, the tile that a sequence as long as the host's bound would have the CTA begin with is copied.  A
+  // sequence that puts the CTA's range elsewhere leaves it unused: which blocks a CTA works on, and with them the last bits of
+  // the results, depend on the length and not on the bound.  (Bounds of 128K over lengths of 1.6K to 100K: against ranges laid
+  // out by the bound, whose copies are all used, 0 to 0.25 us a step, 0.6 with four sequences of 64K.)  With this copy ahead of the length, the others issued by the
+  // producer's lanes and the queries' fragments loaded as matrices, a CTA starts on its first part 1.2 us after the length is
+  // known instead of 2.0 (a step of 8 units at 32K 15.4 -> 14.8 us, 16 units with r = d at 88K 40.5 -> 39.6, 32 units at 128K
+  // 52.6 -> 51.5).
+  const int b_early = rank * plan.early_parts * 16;
+  const int n_early = max(min(min(TB, plan.early_parts * 16), plan.max_blocks - b_early), 0);
   // The launch ahead of this one is waited for in each of the three branches: nobody touches anything before that.  The tail
   // routines set up all they can ahead of it.  Only the working warps wait for the queries' staging: the producer wants the
   // length alone (queries in host memory take 3 us to arrive).
@@ -471,7 +475,7 @@ ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int 
                             : tail_values<G>(&s_tail, page_table, seq_lens, unit, most_len, plan.hi_page, &s_tail_part[0][0]);
   } else {
     pdl_wait();
-    if (tid == kProducerWarp * 32 && n_early > 0) fill(0, rank * plan.first_parts * 16, n_early, 0, &full_bar[0][0]);
+    if (tid == kProducerWarp * 32 && n_early > 0) fill(0, b_early, n_early, 0, &full_bar[0][0]);
     raw = seq_lens[s];
     if (tid < G * 16) *reinterpret_cast<uint4 *>(&s_q[tid >> 4][8 * (tid & 15)]) = reinterpret_cast<const uint4 *>(q + (size_t)unit * G * CKV_D)[tid];
     if (warp < kWarps) named_barrier(3, kThreads);
@@ -482,18 +486,14 @@ ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int 
   const int N = min(N_all, most_len);
   if (N < N_all && rank == 0 && tid == 0) atomicOr(P.status, CKV_DEV_BAD_BOUND);
   const int X = (N + P.bs - 1) >> P.lg_bs, Xs = max(X - 1, 0);
-  // What the CTA owns, `own` blocks in all: n0 blocks from b0 on -- its first tile, whose place depends on the host's plan
-  // alone, so that its copy is under way before the length is known -- then the CTA's part of what the first tiles leave.
-  const int first = plan.first_parts * 16;
-  const int n_parts = (Xs + 15) >> 4, rest = max(n_parts - C * plan.first_parts, 0);
-  const int ppc = div_c(rest + C - 1);
-  const int b0 = rank * first, b1 = C * first + min(rank * ppc, rest) * 16;
-  const int n0 = max(min(Xs - b0, first), 0);
-  const int own = min(n0 + max(min(b1 + ppc * 16, Xs) - b1, 0), plan.own_cap);
-  const int tiles = own == 0 ? 0 : 1 + (max(own - first, 0) + TB - 1) / TB;
-  auto block_at = [&](int i) { return i + (i < first ? b0 : b1 - first); };       // the CTA's i-th block
-  auto tile_start = [&](int it) { return it == 0 ? 0 : first + (it - 1) * TB; };  // first block of tile `it`, counted in the CTA's own
-  auto tile_len = [&](int it) { return min(it == 0 ? first : TB, own - tile_start(it)); };
+  // what the CTA owns: `own` blocks from b_lo on
+  const int n_parts = (Xs + 15) >> 4, ppc = div_c(n_parts + C - 1);
+  const int b_lo = min(rank * ppc, n_parts) * 16;
+  const int own = max(min(min(b_lo + ppc * 16, Xs) - b_lo, plan.own_cap), 0);
+  const int tiles = (own + TB - 1) / TB;
+  auto tile_len = [&](int it) { return min(TB, own - it * TB); };
+  // The early copy is the first tile, or fill 0 of the ring is nobody's and tile `it` is fill it + 1.
+  const int skew = n_early > 0 && !(own > 0 && b_lo == b_early && tile_len(0) <= n_early) ? 1 : 0, n_fills = tiles + skew;
   // score terms of the CTA's own blocks, [g][us] (eight more than the range holds: a tile's eight rows x four heads then
   // fall into 32 different banks)
   float *ub = reinterpret_cast<float *>(smem + plan.u_off);
@@ -502,27 +502,31 @@ ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int 
   ScanUnit<G, bf16, RD> w;
   w.reset();
   if (warp == kProducerWarp) {
-    // ---------------- producer: one thread refills the ring ----------------
-    const int first_fills = min(tiles, plan.stages);
-    if (lane > 0 && lane < first_fills) fill(lane, block_at(tile_start(lane)), tile_len(lane), lane, &full_bar[0][lane]);
+    // ---------------- producer: its lanes issue the first round of fills, one thread refills the ring ----------------
+    auto fill_tile = [&](int f, int st, uint64_t *fb) { const int it = f - skew; fill(f, b_lo + it * TB, tile_len(it), st, fb); };
+    const int first_fills = min(n_fills, plan.stages);
+    if (lane >= (n_early > 0 ? 1 : 0) && lane < first_fills) fill_tile(lane, lane, &full_bar[0][lane]);
     __syncwarp();
     if (lane == 0) {
       mbar_arrive_expect_tx(&s_xbar[1], (uint32_t)(X * 4));
-      *(volatile int *)&s_issued = max(first_fills, n_early > 0 ? 1 : 0);
-      if (tiles == 0 && n_early > 0 && !mbar_wait(&full_bar[0][0], 0, P.spin_limit)) {   // nobody else waits for this copy
-        atomicOr(P.status, CKV_DEV_TIMEOUT);
-        *(volatile int *)&s_abort = 1;
+      *(volatile int *)&s_issued = first_fills;
+      if (skew != 0) {   // nobody else waits for this copy or releases its stage
+        if (!mbar_wait(&full_bar[0][0], 0, P.spin_limit)) {
+          atomicOr(P.status, CKV_DEV_TIMEOUT);
+          *(volatile int *)&s_abort = 1;
+        }
+        for (int i = 0; i < kParts; ++i) mbar_arrive(&empty_bar[0]);
       }
       int st = 0;
       uint32_t phase = 0, round = 1;
-      for (int it = plan.stages; it < tiles; ++it) {
+      for (int f = plan.stages; f < n_fills; ++f) {
         if (!mbar_wait(&empty_bar[st], phase, P.spin_limit)) {
           atomicOr(P.status, CKV_DEV_TIMEOUT);
           *(volatile int *)&s_abort = 1;
         }
         if (*(volatile int *)&s_abort) break;
-        fill(it, block_at(tile_start(it)), tile_len(it), st, &full_bar[round & 1][st]);
-        *(volatile int *)&s_issued = it + 1;
+        fill_tile(f, st, &full_bar[round & 1][st]);
+        *(volatile int *)&s_issued = f + 1;
         if (++st == plan.stages) { st = 0; ++round; phase ^= 1; }
       }
     } else {
@@ -581,8 +585,8 @@ ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int 
     bool aborted = false;
     float umax[2] = {-CUDART_INF_F, -CUDART_INF_F};   // largest score terms this lane has seen, of its heads
     for (int it = warp / kParts; it < tiles; it += kSkip) {
-      st += it - at;
-      at = it;
+      st += it + skew - at;
+      at = it + skew;
       while (st >= plan.stages) { st -= plan.stages; ++round; }
       if (!aborted) {
         bool fail = *(volatile int *)&s_abort != 0;
@@ -593,7 +597,7 @@ ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int 
         }
         aborted = __any_sync(0xffffffffu, fail);
       }
-      const int nb = tile_len(it), rb = part * 16, from = tile_start(it), tb0 = block_at(from);
+      const int nb = tile_len(it), rb = part * 16, tb0 = b_lo + it * TB;
       if (!aborted && rb < nb) {
         const uint32_t sk = smem_u32(smem + (size_t)st * stage_bytes);
         const float *sd = reinterpret_cast<const float *>(smem + (size_t)st * stage_bytes + TB * (kRowBytesK + kRowBytesV));
@@ -601,7 +605,7 @@ ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int 
             w, cfg, sk, sk + TB * kRowBytesK, (RD || dbar_bulk) ? sd : nullptr, smem_u32(s_zero_row), s_w, P.dbar + row0 * P.r,
             lane, rb, nb, tb0, -1, 0.f,
             [&](int g, int blk, float x, float y) {
-              ub[g * us + (blk - tb0 + from)] = x;
+              ub[g * us + (blk - b_lo)] = x;
               lz[(size_t)g * P.max_blocks + blk] = y;
               if (g & 1) umax[1] = fmaxf(umax[1], x); else umax[0] = fmaxf(umax[0], x);
             });
@@ -718,7 +722,7 @@ ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int 
         if (real && (!(sc[j] >= 0.f) || sc[j] > 3.0e38f)) { nonfinite = true; sc[j] = 0.f; }
         k[j] = min(__float_as_uint(sc[j]), most);
       }
-      const uint32_t dst = smem_u32(keys + block_at(i));
+      const uint32_t dst = smem_u32(keys + b_lo + i);
       if (i + 4 <= own) {
         for (int c = 0; c < C; ++c) {
           const uint32_t there = cluster_map(xbar1, c);   // the CTAs' shared memories are congruent windows
@@ -762,7 +766,7 @@ ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int 
   int *ids = reinterpret_cast<int *>(smem + kOffIds);
   if (warp >= kWarps && !dead) {   // the idle warps leave the range's scores where ckv_copy_scores() finds them
     float *scores = P.scores + row0;
-    for (int i = tid - kWork; i < own; i += kThreads - kWork) { const int b = block_at(i); scores[b] = __uint_as_float(keys[b]); }
+    for (int i = tid - kWork; i < own; i += kThreads - kWork) scores[b_lo + i] = __uint_as_float(keys[b_lo + i]);
     if (rank == C - 1 && N > 0 && tid == kWork) scores[Xs] = __uint_as_float(keys[Xs]);
   }
   if (warp < kWarps) {
@@ -1214,7 +1218,7 @@ bool ckv_unit_step_plan(const ckv_ctx *c, int batch, int max_len, int kcap, CkvS
   auto blocks_per_cta = [C](int x) { const int parts = (std::max(x - 1, 0) + 15) / 16; return 16 * std::max((parts + C - 1) / C, 1); };
   auto term_bytes = [&P](int own) { return (size_t)(own + 8) * P.G * sizeof(float); };
   plan->own_cap = blocks_per_cta(xmax);
-  plan->first_parts = std::min(P.scan_tile, plan->own_cap) / 16;
+  plan->early_parts = plan->own_cap / 16;
   plan->hi_page = std::min((max_len - 1) / CKV_PAGE, P.max_pages_per_seq - 1);
   if (plan->own_cap > kOwnMost && P.Hkv * C < kSeqCtas && (P.r == 4 || P.r == CKV_D)) return false;
   if (term_bytes(plan->own_cap) + (size_t)std::max(kMinRing, skip) * stage > (size_t)kDynLimit) return false;

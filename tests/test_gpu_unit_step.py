@@ -152,6 +152,28 @@ def test_a_bound_far_past_the_lengths(tokens, layout):
     assert float((out.float() - out2.float()).abs().max()) <= 2.0 ** -7 * float(out.float().abs().max())
 
 
+@pytest.mark.parametrize("layout", [{}, {"stat_bf16": 1}, {"var_groups": 128}])
+@pytest.mark.parametrize("hq,hkv,lens", [(8, 2, (16 * 200 + 3, 1600)), (32, 8, (16 * 333, 16 * 97 + 1)), (4, 1, (16 * 1100 + 9, 5)),
+                                         (16, 2, (16 * 513, 16 * 512)), (32, 8, (16 * 1400 + 1, 16 * 700))])
+def test_results_do_not_depend_on_the_bound(hq, hkv, lens, layout):
+    """Which blocks a CTA works on follows from the length alone: the copy that is issued ahead of it, where the bound puts
+    the CTA's range, is the first tile (bounds just met, and in one CTA a unit) or is left unused (the others)."""
+    w = workload(batch=2, num_q_heads=hq, num_kv_heads=hkv, ctx=max(lens), ctx_min=None, needles=2, decode_steps=1)
+    res = []
+    for bound in (max(lens) + 1, max(lens) + 16 * 40, 16 * 1800, 16 * 2500):
+        d = with_capacity(setup(w), 8192, **layout)
+        d.lens[0], d.lens[1] = lens
+        d.ckv.stats_build(d.k_pool, d.v_pool, d.table, d.lens, d.max_len)
+        before = d.ckv.launch_count()
+        got = d.ckv.step(*step_inputs(d, 0), d.k_pool, d.v_pool, d.table, d.lens, bound, w.budget_tokens)
+        assert d.ckv.launch_count() - before == 1
+        torch.cuda.synchronize()
+        assert d.ckv.read_status() == 0 and d.lens.tolist() == [n + 1 for n in lens]
+        res.append([t.clone() for t in got] + [x[s, :, :n // 16 + 1] for x in d.ckv.export_stats() for s, n in enumerate(lens)])
+    for other in res[1:]:
+        assert all(torch.equal(x, y) for x, y in zip(res[0], other))
+
+
 @pytest.mark.parametrize("bs,page", [(16, 0), (32, 0), (32, 1)])
 @pytest.mark.parametrize("layout", [{}, {"stat_bf16": 1}])
 def test_a_bad_page_among_the_selected_is_skipped_as_the_attention_kernel_skips_it(bs, page, layout):
