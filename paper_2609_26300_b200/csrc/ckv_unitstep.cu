@@ -75,8 +75,6 @@ constexpr int kAfterScan = kOffPages + kWarps * 2 * kPageBytes;
 constexpr int kRecvStride = 36;                 // floats of one (head, 32 coordinates) partial: values, maximum, weight sum
 constexpr int kDynLimit = 227 * 1024 - 20 * 1024;   // dynamic shared memory; the kernel's static arrays take 20 KB at most
 
-// 2^(a - b) of two running maxima, 0 where a is -inf (as b may be, too).
-__device__ __forceinline__ float part_scale(float a, float b) { return a == -CUDART_INF_F ? 0.f : fast_exp2(a - b); }
 // One more in a shared-memory counter.
 __device__ __forceinline__ void red_shared_inc(uint32_t addr) { asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(addr) : "memory"); }
 
@@ -635,11 +633,17 @@ ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int 
     float4 e[kWarps + 1];
 #pragma unroll
     for (int i = 0; i <= kWarps; ++i) e[i] = s_wn[i][warp];
+    const float mine = s_wn[min(lane, kWarps)][warp].x;
     float m = e[0].x, l = 0.f, u = e[0].z;
 #pragma unroll
     for (int i = 1; i <= kWarps; ++i) { m = fmaxf(m, e[i].x); u = fmaxf(u, e[i].z); }
+    // One weight a lane, handed round, here and in the merges below: what is weighted may be as large as fp32 allows, so a
+    // weight below 2^-126 counts, and exp2f with its steps for such results is a few instructions once instead of per entry.
+    // The code between the phases is run once a launch and its length is its time (us a step of one unit of 4K tokens, of 8 of
+    // 32K, of 32 of 128K: 10.7, 12.9, 47.9 this way; 11.1, 13.3, 48.2 with exp2f for every entry).
+    const float sc = exp2_diff(mine, m);
 #pragma unroll
-    for (int i = 0; i <= kWarps; ++i) l = fmaf(e[i].y, part_scale(e[i].x, m), l);
+    for (int i = 0; i <= kWarps; ++i) l = fmaf(e[i].y, __shfl_sync(0xffffffffu, sc, i), l);
     if (lane < C) {
       const uint32_t x0 = smem_u32(&s_xbar[0]), there = cluster_map(x0, lane);   // the CTAs' shared memories are congruent windows
       st_async_u32x4(there + (smem_u32(&s_norm[rank][warp]) - x0), __float_as_uint(m), __float_as_uint(l), __float_as_uint(u), 0u, there);
@@ -683,7 +687,7 @@ ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int 
       u = fmaxf(u, __shfl_xor_sync(0xffffffffu, u, o));
     }
 #pragma unroll
-    for (int i = 0; i < EPL; ++i) l = fmaf(e[i].y, part_scale(e[i].x, m), l);
+    for (int i = 0; i < EPL; ++i) l = fmaf(e[i].y, exp2_diff(e[i].x, m), l);
 #pragma unroll
     for (int o = LPH / 2; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
     const float il = 1.0f / l, b = fast_exp2(u - m) * il;
@@ -1043,21 +1047,26 @@ ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int 
       const int g = idx / (CKV_D / 4), c = 4 * (idx % (CKV_D / 4));
       float2 ml[kWarps + 1];
       float4 x[kWarps + 1];
+      float mine = *(entry(min(lane, kWarps)) + g * CKV_PART_STRIDE);   // a warp works on one head
 #pragma unroll
       for (int e = 0; e <= kWarps; ++e) {
         const float *p = entry(e) + g * CKV_PART_STRIDE;
         ml[e] = *reinterpret_cast<const float2 *>(p);
         x[e] = *reinterpret_cast<const float4 *>(p + 4 + c);
       }
-      if (!with_tail) ml[kWarps].x = -CUDART_INF_F;
+      if (!with_tail) {
+        ml[kWarps].x = -CUDART_INF_F;
+        if (lane >= kWarps) mine = -CUDART_INF_F;
+      }
       float M = ml[0].x;
 #pragma unroll
       for (int e = 1; e <= kWarps; ++e) M = fmaxf(M, ml[e].x);
+      const float sc_mine = exp2_diff(mine, M);
       float den = 0.f;
       float4 num = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
       for (int e = 0; e <= kWarps; ++e) {
-        const float sc = part_scale(ml[e].x, M);
+        const float sc = __shfl_sync(0xffffffffu, sc_mine, e);
         if (sc != 0.f) {   // an entry that holds nothing may hold any bits
           den = fmaf(ml[e].y, sc, den);
           num.x = fmaf(x[e].x, sc, num.x); num.y = fmaf(x[e].y, sc, num.y);
@@ -1077,12 +1086,13 @@ ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int 
     for (int slot = warp; slot * C + rank < 4 * G; slot += kWarps) {
       const int item = slot * C + rank, g = item >> 2, c = (item & 3) * 32 + lane;
       const float *e0 = s_recv + (size_t)slot * C * kRecvStride;
-      float M = -CUDART_INF_F, den = 0.f, o = 0.f;
-#pragma unroll 4
-      for (int e = 0; e < C; ++e) M = fmaxf(M, e0[e * kRecvStride + 32]);
-#pragma unroll 4
+      const float mine = e0[min(lane, C - 1) * kRecvStride + 32];
+      const float M = warp_max(mine);
+      float den = 0.f, o = 0.f;
+      const float sc_mine = exp2_diff(mine, M);
+#pragma unroll 8
       for (int e = 0; e < C; ++e) {
-        const float sc = part_scale(e0[e * kRecvStride + 32], M);
+        const float sc = __shfl_sync(0xffffffffu, sc_mine, e);
         den = fmaf(e0[e * kRecvStride + 33], sc, den);
         o = fmaf(e0[e * kRecvStride + lane], sc, o);
       }

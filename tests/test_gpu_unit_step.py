@@ -4,8 +4,9 @@ and summary layout, ties at the cut.  Oracle and tolerances are those of helpers
 import pytest
 import torch
 
+from oracle import compkv_oracle as O
 from paper_2609_26300_b200 import binding, synth
-from helpers import check_unit_decode, setup
+from helpers import OUT_TOL, check_scores, check_unit_decode, rel_inf, setup
 
 pytestmark = pytest.mark.gpu
 
@@ -200,6 +201,61 @@ def test_a_bad_page_among_the_selected_is_skipped_as_the_attention_kernel_skips_
     # log-sum-exps as close as the two arrangements are on good pages (fp32 sums in another order), rows to bf16 rounding
     assert float((res[0][1] - res[1][1]).abs().max()) <= 1e-4 and float((res[0][1] - good[1]).abs().max()) > 1e-2
     assert float((res[0][0].float() - res[1][0].float()).abs().max()) <= 2.0 ** -7 * float(res[1][0].float().abs().max())
+
+
+def blocks_of(means, devs, values, g):
+    """One KV head: block b's keys are means[b] +- devs[b] in every coordinate (half of its tokens each), its values values[b]."""
+    sign = torch.tensor([1.0, -1.0]).repeat(8)
+    k = (means[:, None] + devs[:, None] * sign)[:, None, :, None].expand(-1, 1, 16, 128)
+    v = values[:, None, None, None].expand(-1, 1, 16, 128) * (1.0 + torch.randint(0, 2, (len(means), 1, 1, 128), generator=g) / 2)
+    return k.contiguous().bfloat16(), v.contiguous().bfloat16()
+
+
+def small_weights_case(means, devs, values, budget):
+    X = len(means)
+    k, v = blocks_of(means, devs, values, torch.Generator().manual_seed(3))
+    q = torch.full((1, 4, 128), 4.0).bfloat16()   # 45.25 units of logit per unit of a key's coordinates
+    ckv = binding.CompKV(4, 1, max_batch=1, max_blocks_per_seq=256, num_pages=X)
+    table = torch.full((1, 256), -1, dtype=torch.int32)
+    table[0, :X] = torch.arange(X, dtype=torch.int32)
+    args = [t.cuda() for t in (q, k, v, table, torch.tensor([16 * X], dtype=torch.int32))]
+    ckv.stats_build(*args[1:], 16 * X)
+    res = []
+    for tail, launches in ((binding.CKV_TAIL_AUTO, 1), (binding.CKV_TAIL_ON, 3)):
+        ckv.set_tail_mode(tail)
+        before = ckv.launch_count()
+        out, lse, ids, cnt = ckv.decode(*args, 16 * X, budget)
+        assert ckv.launch_count() - before == launches
+        res.append((out.double().cpu().numpy()[0], ckv.copy_scores(1).double().cpu().numpy()[0, 0, :X]))
+    torch.cuda.synchronize()
+    assert ckv.read_status() == 0
+    K, V = (t.float().numpy().reshape(16 * X, 128) for t in (k, v))
+    return res, q[0].float().numpy(), K, V
+
+
+def test_normalisers_count_parts_whose_mean_terms_are_below_2_to_the_minus_126():
+    """Eq. 9's sum has e^{zbar + sigma^2 / 2}: 112 blocks whose mean terms lie 2^-128 below the largest and whose variance
+    terms are 2^122 make up half of it.  They are other CTAs' (other warps', in the separate launches) than the largest is."""
+    means, devs = torch.full((129,), -2.0), torch.full((129,), 0.0625)
+    means[0] = 1.03125
+    means[16:128], devs[16:128] = -0.9375, 3.25
+    res, q, K, V = small_weights_case(means, devs, torch.ones(129), 16 * 12)
+    st = O.stats(K, V, 16, 4, 1)
+    sc = O.scores(q, st)
+    for _, scores in res:
+        check_scores(scores, sc)
+
+
+@pytest.mark.parametrize("where,value", [(slice(1, 8), 2.0 ** 122), (slice(16, 128), 2.0 ** 120)])   # other warps of the largest weight's CTA; other CTAs
+def test_outputs_count_partials_whose_weights_are_below_2_to_the_minus_126(where, value):
+    """Every block selected; tokens of weight 2^-128 beside the largest have values that make up for it (a page's sum is still
+    an fp32 number)."""
+    means, values = torch.full((129,), -2.0), torch.ones(129)
+    means[0], means[where], values[where] = 1.03125, -0.9375, value
+    res, q, K, V = small_weights_case(means, torch.full((129,), 0.0625), values, 16 * 140)
+    ref = O.dense(q, K, V)[0]
+    assert abs(ref).min() > 1.05
+    assert rel_inf(res[0][0], ref) <= OUT_TOL[torch.bfloat16]
 
 
 def with_capacity(d, max_blocks, **layout):
