@@ -411,6 +411,7 @@ ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int 
     mbar_arrive_expect_tx(&s_xbar[2], (uint32_t)(n_items * C * (32 * 4 + 8)));
     s_abort = 0; s_issued = 0; s_digit = -1; s_ncand = 0;
   }
+  if (warp == kProducerWarp) __syncwarp();   // its other lanes arm these barriers, too
   if (warp >= kTailWarp) {
     const int i = tid - kTailWarp * 32;
     static_assert(sizeof(CkvDev) % 4 == 0 && sizeof(CkvDev) <= 256 && sizeof(CkvNewToken) % 4 == 0 && sizeof(CkvNewToken) <= 256, "a word per thread");

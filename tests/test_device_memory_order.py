@@ -20,6 +20,15 @@ def test_completion_word_is_stored_behind_what_the_counter_showed():
     assert "__threadfence_system()" in src[count:store]
 
 
+def test_barriers_are_set_up_before_other_lanes_of_the_producer_warp_use_them():
+    """One lane initialises the ring's barriers, its neighbours issue fills on them, and no barrier that waits lies between the
+    two: the warp is synchronised right behind the initialisation."""
+    src = code("ckv_unitstep.cu")
+    init = src.index("fence_barrier_init()")
+    assert init < src.index("if (warp == kProducerWarp) __syncwarp()", init) < src.index("cluster_arrive_release()", init)
+    assert src.index("cluster_arrive_release()", init) < src.index("fill_tile(lane, lane", init)
+
+
 def test_kernels_that_start_early_do_not_call_their_inputs_constant():
     """A programmatic dependent launch runs while the launch ahead of it still writes: `__ldg` and `const __restrict__`
     would let the compiler move loads up past griddepcontrol.wait."""
