@@ -844,16 +844,17 @@ ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int 
           uint32_t *cand = reinterpret_cast<uint32_t *>(smem + kOffCand);
           const int take = Kr - s_before;
           // sign bits of (threshold - 1 - score), shifted into words: 1 where the score reaches the threshold
-          const int lo1 = (int)((top - (uint32_t)digit) << kBinShift) - 1;
-          const int hi1 = digit == 0 ? 0x7fffffff : (int)((top - (uint32_t)digit + 1u) << kBinShift) - 1;
+          // (unsigned: words past the unit's scores hold anything, their bits are masked)
+          const uint32_t lo1 = ((top - (uint32_t)digit) << kBinShift) - 1u;
+          const uint32_t hi1 = digit == 0 ? 0x7fffffffu : ((top - (uint32_t)digit + 1u) << kBinShift) - 1u;
           uint32_t ge_hi[2] = {0, 0}, ge_lo[2] = {0, 0};
 #pragma unroll
           for (int j = kKeyGroups - 1; j >= 0; --j) {
             if (j < nj) {
 #pragma unroll
               for (int e = 3; e >= 0; --e) {
-                ge_hi[j >> 3] = __funnelshift_l((uint32_t)(hi1 - (int)key[j][e]), ge_hi[j >> 3], 1);
-                ge_lo[j >> 3] = __funnelshift_l((uint32_t)(lo1 - (int)key[j][e]), ge_lo[j >> 3], 1);
+                ge_hi[j >> 3] = __funnelshift_l(hi1 - key[j][e], ge_hi[j >> 3], 1);
+                ge_lo[j >> 3] = __funnelshift_l(lo1 - key[j][e], ge_lo[j >> 3], 1);
               }
             }
           }

@@ -20,6 +20,14 @@ def test_completion_word_is_stored_behind_what_the_counter_showed():
     assert "__threadfence_system()" in src[count:store]
 
 
+def test_words_of_any_content_are_subtracted_as_unsigned_numbers():
+    """The selection compares by the sign of a difference, also for words past the unit's scores, which hold what the ring left
+    (negative numbers among them) and whose bits are masked: as signed numbers that would overflow."""
+    src = code("ckv_unitstep.cu")
+    assert src.count("- key[j][e]") == 2 and "(int)key[j][e]" not in src
+    assert re.search(r"const uint32_t lo1 = ", src) and re.search(r"const uint32_t hi1 = ", src)
+
+
 def test_barriers_are_set_up_before_other_lanes_of_the_producer_warp_use_them():
     """One lane initialises the ring's barriers, its neighbours issue fills on them, and no barrier that waits lies between the
     two: the warp is synchronised right behind the initialisation."""
