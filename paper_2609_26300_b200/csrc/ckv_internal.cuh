@@ -91,6 +91,7 @@ struct ckv_ctx {
   int sm_count;
   int tail_mode;   // ckv_tail_mode
   int step_clusters[CKV_STEP_MAX_CLUSTER + 1];   // clusters of each size the device holds at once (one-launch step)
+  int step_smem;   // dynamic shared memory that step can take
   CUtensorMap tm_vhi;   // vhi: the mean-values region as rows of 128 bf16 (the hi halves) 512 bytes apart, boxes of 64 rows
   volatile int *host_flag;   // pinned word ckv_step_host waits on (null: stream synchronisation instead)
   int *host_flag_dev;        // the same word as the device sees it

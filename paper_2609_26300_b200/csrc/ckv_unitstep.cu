@@ -73,7 +73,8 @@ constexpr int kOffCand = kOffIds + kSelCap * 4;
 constexpr int kOffPages = (kOffCand + kCandCap * 4 + 127) / 128 * 128;
 constexpr int kAfterScan = kOffPages + kWarps * 2 * kPageBytes;
 constexpr int kRecvStride = 36;                 // floats of one (head, 32 coordinates) partial: values, maximum, weight sum
-constexpr int kDynLimit = 227 * 1024 - 20 * 1024;   // dynamic shared memory; the kernel's static arrays take 20 KB at most
+constexpr int kSmemCta = 227 * 1024;            // shared memory a CTA can have, static and dynamic
+constexpr int kDynMost = kSmemCta - 20 * 1024;  // dynamic shared memory, at most (see ckv_configure_unit_step)
 
 // One more in a shared-memory counter.
 __device__ __forceinline__ void red_shared_inc(uint32_t addr) { asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(addr) : "memory"); }
@@ -1159,7 +1160,14 @@ cudaError_t ckv_configure_unit_step(ckv_ctx *c) {
   if (c->layout.kv_dtype != CKV_BF16) return cudaSuccess;
   const void *k = kernel_of(c->dev);
   if (k == nullptr) return cudaErrorInvalidValue;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynLimit);
+  // What the static arrays leave: all of kDynMost today, with groups of eight to the byte; a field more in the structs that
+  // are copied into shared memory makes the ring a little smaller, and no context fails.
+  cudaFuncAttributes fa = {};
+  cudaError_t e = cudaFuncGetAttributes(&fa, k);
+  if (e != cudaSuccess) return e;
+  c->step_smem = std::min(kDynMost, (kSmemCta - (int)fa.sharedSizeBytes) / 1024 * 1024);
+  if (c->step_smem < kAfterScan) return cudaSuccess;   // the step stays with its separate launches
+  e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, c->step_smem);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   int dev = 0;
   if (e == cudaSuccess) e = cudaGetDevice(&dev);
@@ -1233,15 +1241,15 @@ bool ckv_unit_step_plan(const ckv_ctx *c, int batch, int max_len, int kcap, CkvS
   plan->early_parts = plan->own_cap / 16;
   plan->hi_page = std::min((max_len - 1) / CKV_PAGE, P.max_pages_per_seq - 1);
   if (plan->own_cap > kOwnMost && P.Hkv * C < kSeqCtas && (P.r == 4 || P.r == CKV_D)) return false;
-  if (term_bytes(plan->own_cap) + (size_t)std::max(kMinRing, skip) * stage > (size_t)kDynLimit) return false;
+  if (term_bytes(plan->own_cap) + (size_t)std::max(kMinRing, skip) * stage > (size_t)c->step_smem) return false;
   const int tiles = (plan->own_cap + P.scan_tile - 1) / P.scan_tile;
-  plan->stages = std::min({kStagesCap, (int)(((size_t)kDynLimit - term_bytes(plan->own_cap)) / stage), std::max(tiles, skip)});
+  plan->stages = std::min({kStagesCap, (int)(((size_t)c->step_smem - term_bytes(plan->own_cap)) / stage), std::max(tiles, skip)});
   plan->u_off = (int)(plan->stages * stage);
   plan->max_blocks = xmax;
   // Where the arrays can be sized for the cache's capacity beside the same ring, they are: a bound that turns out too small
   // (a captured step replayed once too often) then costs nothing.
   const int full = blocks_per_cta(P.max_blocks);
-  if (P.max_blocks <= kScoresCap && (kcap >= P.max_blocks || kcap <= kSelCap) && plan->u_off + term_bytes(full) <= (size_t)kDynLimit) {
+  if (P.max_blocks <= kScoresCap && (kcap >= P.max_blocks || kcap <= kSelCap) && plan->u_off + term_bytes(full) <= (size_t)c->step_smem) {
     plan->own_cap = full;
     plan->max_blocks = P.max_blocks;
   }
