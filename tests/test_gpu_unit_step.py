@@ -130,22 +130,22 @@ def test_a_negative_length_drops_the_token_in_every_arrangement(tail):
 @pytest.mark.parametrize("layout", [{}, {"stat_bf16": 1}, {"var_groups": 128}])
 @pytest.mark.parametrize("tokens", [1, 16 * 33, 16 * 64, 16 * 64 + 1, 16 * 65 + 1, 16 * 640, 16 * 641 + 9, 16 * 1000 + 3])
 def test_a_bound_far_past_the_lengths(tokens, layout):
-    """A CTA's first tile lies where the bound puts it (blocks 64 r .. 64 r + 63 here, 32 of them with r = d), whatever the
-    length; the new token's page is then not among the 32 last ones under the bound.  Lengths at the edges of tiles, with
-    CTAs that own nothing, beside one as long as the bound: results and summaries against a bound that is just met."""
+    """A sequence far shorter than the bound beside one as long as it: its CTAs' ranges are not where the early copies are, some
+    own nothing, and the new token's page is not among the 32 last ones under the bound.  Lengths at the edges of tiles (64
+    blocks here, 32 with r = d): results and summaries of both sequences against the separate launches."""
     w = workload(batch=2, ctx=16 * 1500, ctx_min=None, needles=2, decode_steps=2)
     res = []
-    for bound in (16 * 1500 + 1, None):
+    for tail, launches in ((binding.CKV_TAIL_AUTO, 1), (binding.CKV_TAIL_ON, 3)):
         d = setup(w, **layout)
         d.lens[1] = tokens
-        if bound is None:
-            d.lens[0] = 1
-            bound = max(tokens + 1, 1537)
+        d.ckv.set_tail_mode(tail)
         d.ckv.stats_build(d.k_pool, d.v_pool, d.table, d.lens, d.max_len)
-        got = d.ckv.step(*step_inputs(d, 0), d.k_pool, d.v_pool, d.table, d.lens, bound, w.budget_tokens)
+        before = d.ckv.launch_count()
+        got = d.ckv.step(*step_inputs(d, 0), d.k_pool, d.v_pool, d.table, d.lens, 16 * 1500 + 1, w.budget_tokens)
+        assert d.ckv.launch_count() - before == launches
         torch.cuda.synchronize()
-        assert d.ckv.read_status() == 0 and int(d.lens[1]) == tokens + 1
-        res.append([t[1].clone() for t in got] + [x[1, :, :tokens // 16 + 1] for x in d.ckv.export_stats()])
+        assert d.ckv.read_status() == 0 and d.lens.tolist() == [16 * 1500 + 1, tokens + 1]
+        res.append([t.clone() for t in got] + [x[s, :, :n // 16 + 1] for x in d.ckv.export_stats() for s, n in ((0, 16 * 1500), (1, tokens))])
     (out, lse, ids, cnt, *st), (out2, lse2, ids2, cnt2, *st2) = res
     assert torch.equal(ids, ids2) and torch.equal(cnt, cnt2) and all(torch.equal(x, y) for x, y in zip(st, st2))
     # the same fp32 terms in another order: the log-sum-exp to a few 2^-24 of its terms, the rows to one bf16 rounding
