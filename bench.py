@@ -37,8 +37,8 @@ PAPER_CONTEXT = {"speedup_vs_full": 6.85, "hardware": "NVIDIA H100 80GB HBM3, CP
 # (profiles/ckv_scan_kernel_llama8b_128k_b4.md): 206.06 MB read + 10.15 MB written for the 205.5 MB of summaries the
 # step reads (mean keys hi + lo, mean values hi, variances).
 SCAN_TRAFFIC_RATIO = (206.06 + 10.15) / 205.5
-# The same for the one-launch step (profiles/ckv_unit_step_kernel_llama8b_128k_b2.md).
-STEP_TRAFFIC_RATIO = 124.5 / 119.6
+# The same for the one-launch step (profiles/ckv_unit_step_kernel_llama8b_128k_b2.md): 120.5 MB read + 5.3 MB written.
+STEP_TRAFFIC_RATIO = 125.8 / 119.6
 # What is stored and multiplied (the line's `dtype`): K/V pages are bf16; mean keys and mean values keep fp32
 # precision as split bf16 pairs (hi = bf16(x), lo = bf16(x - hi), relative error <= 2^-18), variances are fp32; the
 # decode step reads the mean keys as pairs and the mean values as their hi halves; the contractions run on bf16
@@ -615,7 +615,7 @@ def main():
                 "algorithmic_bytes": req if one else stats_b, "launch_us": pipe_us if one else scan_us,
                 "traffic": (STEP_TRAFFIC_RATIO * req if one else SCAN_TRAFFIC_RATIO * stats_b),
                 "traffic_source": "DRAM bytes per algorithmic byte in one ncu capture (profiles/ckv_unit_step_kernel_llama8b_128k_b2.md: "
-                                  "124.5 MB for 119.6 MB)" if one else "see scan_launch"}
+                                  "125.8 MB for 119.6 MB)" if one else "see scan_launch"}
     line = {
         "metric": METRIC if is_default else "sparse decode-attn us/step (append + decode)", "value": us_per_step, "unit": UNIT, "n_gpus": world, "steps": K, "warmup": W,
         "ms_per_step": ms_per_step, "higher_is_better": False, "scaling": "weak", "vs_baseline": None,
