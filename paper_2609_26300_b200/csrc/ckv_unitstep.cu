@@ -1092,13 +1092,17 @@ ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int 
       const float mine = e0[min(lane, C - 1) * kRecvStride + 32];
       const float M = warp_max(mine);
       float den = 0.f, o = 0.f;
-      const float sc_mine = exp2_diff(mine, M);
-#pragma unroll 8
-      for (int e = 0; e < C; ++e) {
-        const float sc = __shfl_sync(0xffffffffu, sc_mine, e);
-        den = fmaf(e0[e * kRecvStride + 33], sc, den);
-        o = fmaf(e0[e * kRecvStride + lane], sc, o);
-      }
+      // eight entries at a time, those past the last with a weight of zero: a loop with a remainder, like any other code here,
+      // costs its length (24 units of 100K with bf16 summaries 27.2 us a step that way, 26.7 this way)
+      const float sc_mine = lane < C ? exp2_diff(mine, M) : 0.f;
+      for (int e = 0; e < C; e += 8)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const float *p = e0 + min(e + j, C - 1) * kRecvStride;
+          const float sc = __shfl_sync(0xffffffffu, sc_mine, e + j);
+          den = fmaf(p[33], sc, den);
+          o = fmaf(p[lane], sc, o);
+        }
       out[((size_t)unit * G + g) * CKV_D + c] = __float2bfloat16_rn(N > 0 ? o / den : 0.f);   // an empty sequence: zero
       if (lse != nullptr && (item & 3) == 0 && lane == 0) lse[(size_t)unit * G + g] = N > 0 ? (M + log2f(den)) * kLn2 : -CUDART_INF_F;
     }
