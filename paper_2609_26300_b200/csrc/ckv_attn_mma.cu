@@ -440,8 +440,8 @@ ckv_attn_mma_kernel(CkvDev P, const __nv_bfloat16 *q, const __nv_bfloat16 *k_poo
     __syncthreads();
 #pragma unroll
     for (int it = 0; it < NI; ++it) num[it] = 0.f;
-    // every entry is read (a slot that holds nothing is multiplied by a zero that replaces its value, not by
-    // its bits), so the loads of all entries are independent and in flight together
+    // every entry up to the last filled slot is read, whatever its weight (where that is zero, a zero replaces the value,
+    // which may be any bits), so the loads are independent and in flight together
 #pragma unroll 4
     for (int e = 0; e < W + min(kSlots, max(my_cnt - base, 0)); ++e) {
       const float *ep = sf + s_ent[e] + 4;

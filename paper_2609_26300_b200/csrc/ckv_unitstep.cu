@@ -8,9 +8,10 @@
 // nothing waits for another unit.  A cluster barrier costs 0.1 us here, a launch about 2 us.
 //
 // CTA `rank` of the cluster owns a contiguous range of the unit's blocks (all but the last one), in 16-block parts:
-//   1. scan: a producer thread streams the range's summaries into a ring of shared-memory stages, eight warps work on
-//      parts (scan_part, shared with the persistent scan kernel); the score terms stay in shared memory.  Meanwhile one
-//      warp of the last CTA appends the new token, redoes the last block's summary and computes its terms.
+//   1. scan: a producer warp streams the range's summaries into a ring of shared-memory stages (its lanes issue the first
+//      round, one of them the rest, and the first tile, at a guess, before the length is known), eight warps work on
+//      parts (scan_part, shared with the persistent scan kernel); the score terms stay in shared memory.  Meanwhile two
+//      warps of the last CTA append the new token, redo the last block's summary and compute its terms.
 //   2. every CTA sends its normaliser partials (M_g, L_g) to all, then the block scores of its own range: every CTA holds
 //      all scores of the unit.  Both exchanges are asynchronous stores counted on an mbarrier of the receiver: a cluster
 //      barrier with release semantics would wait for the scan's stores to global memory as well (1.4 us instead of 0.6).
@@ -457,10 +458,11 @@ ckv_unit_step_kernel(const __grid_constant__ CkvDev P, const bf16 *q, const int 
   // Ahead of the length, the tile that a sequence as long as the host's bound would have the CTA begin with is copied.  A
   // sequence that puts the CTA's range elsewhere leaves it unused: which blocks a CTA works on, and with them the last bits of
   // the results, depend on the length and not on the bound.  (Bounds of 128K over lengths of 1.6K to 100K: against ranges laid
-  // out by the bound, whose copies are all used, 0 to 0.25 us a step, 0.6 with four sequences of 64K.)  With this copy ahead of the length, the others issued by the
-  // producer's lanes and the queries' fragments loaded as matrices, a CTA starts on its first part 1.2 us after the length is
-  // known instead of 2.0 (a step of 8 units at 32K 15.4 -> 14.8 us, 16 units with r = d at 88K 40.5 -> 39.6, 32 units at 128K
-  // 52.6 -> 51.5).
+  // out by the bound, whose copies are all used, 0 to 0.25 us a step, 0.6 with four sequences of 64K; 72 units of 8.4K to 9.2K
+  // tokens with r = d, where every second CTA's copy goes unused, 20.3 -> 20.6.)  With this copy ahead
+  // of the length, the others issued by the producer's lanes and the queries' fragments loaded as matrices, a CTA starts on
+  // its first part 1.2 us after the length is known instead of 2.0 (a step of 8 units at 32K 15.4 -> 14.8 us, 16 units with
+  // r = d at 88K 40.5 -> 39.6, 32 units at 128K 52.6 -> 51.5).
   const int b_early = rank * plan.early_parts * 16;
   const int n_early = max(min(min(TB, plan.early_parts * 16), plan.max_blocks - b_early), 0);
   // The launch ahead of this one is waited for in each of the three branches: nobody touches anything before that.  The tail
@@ -1196,29 +1198,32 @@ cudaError_t ckv_configure_unit_step(ckv_ctx *c) {
   return cudaSuccess;
 }
 
-// Whether a step of this size runs as one launch, and how.  Against the separate launches (us per step, back to back):
-// 11.0 / 19.3 (one head, 4K), 13.0 / 24.9 (8 units, 32K), 17.2 / 29.4 (8 units, 128K, 32-token blocks), 29.0 / 38.8 (24 units,
-// 100K, bf16 summaries), 36.7 / 47.5 (16 units, 88K, r = d), 48.2 / 61.2 (32 units, 128K), 57.7 / 77.1 (72 units, 64K), 64.6 /
-// 74.2 (128 units, 32K).
+// Whether a step of this size runs as one launch, and how.  All figures: one launch / the faster form of the separate
+// launches, us per step, sixteen steps replayed back to back, pages in random order, budgets of 2K tokens where nothing is
+// said.  11.3 / 20.1 (one head, 4K, 256 tokens), 12.3 / 25.3 (8 units, 32K, 1K tokens), 16.4 / 29.4 (8 units, 128K, 32-token
+// blocks, 4K tokens), 29.5 / 39.0 (24 units, 100K, bf16 summaries), 36.4 / 47.7 (16 units, 88K, r = d), 47.6 / 64.1 (32 units,
+// 128K), 56.8 / 77.3 (72 units, 64K), 63.7 / 74.6 (128 units, 32K).
 // What stays with the separate launches, and why:
 //   * fp32 pages (the attention is on bf16 tensor cores) and an explicit ckv_set_tail_mode, which asks for them;
-//   * caches under CKV_STEP_MIN_TOKENS.  Not a crossover -- one launch is ahead there too (one sequence of 1600 tokens 11.5 /
-//     19.5, 16 of them 17.2 / 27.1) -- but the size below which the documented two-call arrangement (append, scan, select,
+//   * caches under CKV_STEP_MIN_TOKENS.  Not a crossover -- one launch is ahead there too (one sequence of 1600 tokens 11.8 /
+//     21.4, 16 of them 21.1 / 30.4) -- but the size below which the documented two-call arrangement (append, scan, select,
 //     attention as launches of their own) is kept;
-//   * more units than CTAs run at once: a last wave that is nearly empty costs a whole wave (192 units: 92 / 90);
+//   * more units than CTAs run at once: a last wave that is nearly empty costs a whole wave (192 units, one CTA each: 8K 73.8 /
+//     76.1, 16K 89.7 / 89.7, 32K 117.6 / 113.5; 256 units, whose last wave is not, 16K 96.3 / 108.0);
 //   * more than kOwnMost blocks a CTA where a sequence gets fewer than kSeqCtas of them.  The host knows the longest
-//     sequence only: alone among short ones, its few CTAs are all that works.  One launch / separate ones, 128 units of the
-//     default layout, all long, then lengths of a quarter and up, then one long and 15 of 1K: 32K 56.3 / 63.8, 49.5 / 55.3,
-//     42.2 / 34.5; 40K 66.3 / 73.0, 58.9 / 64.2, 47.6 / 35.9; 56K 84.1 / 89.8, 72.4 / 72.2, 58.7 / 39.7; one head a group,
-//     130K 147 / 161, 127 / 121, 106 / 49.  At 45K a CTA the last of the usual spread's gain goes, and the uneven batch loses a
-//     quarter.  (24 CTAs a sequence, 128K: 59.2 / 71.1, 54.8 / 63.3, 44.0 / 40.5: no line.  Groups other than 4 and 128: one
-//     launch is ahead either way, 75.0 / 143, 70.9 / 162, 68.3 / 101 at 32K with 16 of them.);
+//     sequence only: alone among short ones, its few CTAs are all that works.  128 units of the default layout, all
+//     long, then lengths of a quarter and up, then one long and 15 of 1K: 32K 63.5 / 74.7, 55.7 / 66.7, 48.4 / 40.0; 40K 71.3 /
+//     84.1, 62.6 / 71.3, 54.0 / 41.1; 56K 86.8 / 101.1, 77.3 / 84.9, 66.2 / 43.8; one head a group, 130K 152 / 172, 133 / 131,
+//     114 / 51.  From 45K a CTA on the uneven batch loses a third and more, against a gain of a tenth that is gone at 130K.
+//     (24 CTAs a sequence, 128K: 57.7 / 76.7, 52.0 / 66.3, 44.6 / 38.4: no line.  Groups other than 4 and 128: one launch is
+//     ahead either way, 77.6 / 148, 68.4 / 196, 66.6 / 102 at 32K with 16 of them.);
 //   * large selections where the clusters leave SMs idle (selected bytes x idle share from kIdleMost on): the attention is most
-//     of such a step, and a launch of its own keeps the whole chip at it.  One launch / separate ones / the product: 80 units
-//     (68 SMs idle) 4K tokens of 32K 73.8 / 68.3 / 77 MB, 8K of 16K 95.8 / 81.7 / 154, 32K of 40K 290 / 216 / 616; 104 units
-//     8K of 16K 103.3 / 99.5 / 130; 128 units 8K of 16K 104.6 / 104.7 / 72, 16K of 40K 189 / 184 / 145.  Not where the
+//     of such a step, and a launch of its own keeps the whole chip at it.  64-token blocks, with the product: 80 units (68
+//     SMs idle) 4K tokens of 32K 51.6 / 56.7 / 77 MB, 8K of 16K 82.4 / 76.0 / 154, 32K of 40K 286 / 221 / 616; 104 units 8K of
+//     16K 90.7 / 93.3 / 130; 128 units 8K of 16K 98.5 / 107.0 / 72, 16K of 40K 184.7 / 192.9 / 145.  (The line is from before
+//     the step got faster; by these figures it costs 3 to 4 % between 80 MB and 150.)  Not where the
 //     attention's own clusters fill more than nine tenths of their places, two a SM, and no longer pack: 72 units in
-//     clusters of 4 (288 CTAs), 32K of 40K 205 / 256;
+//     clusters of 4 (288 CTAs), 32K of 40K 193 / 259;
 //   * more selected blocks or scores than the shared arrays hold, or score terms that leave no room for the ring: one CTA
 //     per unit with eight heads beyond about 30K tokens.  There the persistent scan's even split of the tiles is worth
 //     more (a long sequence of a ragged batch is one CTA's work here), and its three launches are kept.
