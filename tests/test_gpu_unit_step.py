@@ -425,6 +425,25 @@ def test_a_wait_that_runs_out_is_reported_and_the_context_recovers():
     assert d.ckv.read_status() == 0 and all(torch.equal(x, y) for x, y in zip(good, again))
 
 
+def test_an_early_copy_that_is_nobodys_and_never_comes_is_reported():
+    """Five tokens under a bound of 4800: no CTA owns a block, and only the producer waits for what was copied ahead."""
+    w = workload(batch=1, ctx=16 * 300, ctx_min=None, decode_steps=0)
+    d = setup(w)
+    d.lens[0] = 5
+    d.ckv.stats_build(d.k_pool, d.v_pool, d.table, d.lens, d.max_len)
+    q = torch.from_numpy(synth.queries(w, 0)).to(d.dtype).cuda()
+    call = (q, d.k_pool, d.v_pool, d.table, d.lens, d.max_len, w.budget_tokens)
+    good = [t.clone() for t in d.ckv.decode(*call)]
+    d.ckv.debug_set(1 << 10, binding.CKV_DEBUG_SKIP_FILL)
+    d.ckv.decode(*call)
+    torch.cuda.synchronize()
+    assert d.ckv.read_status() & binding.CKV_DEV_TIMEOUT
+    d.ckv.debug_set(0, 0)
+    again = d.ckv.decode(*call)
+    torch.cuda.synchronize()
+    assert d.ckv.read_status() == 0 and all(torch.equal(x, y) for x, y in zip(good, again))
+
+
 @pytest.mark.parametrize("polls", [1, 64])
 @pytest.mark.parametrize("batch", [1, 9])
 def test_waits_that_run_out_in_the_exchanges(polls, batch):
