@@ -37,7 +37,7 @@ PAPER_CONTEXT = {"speedup_vs_full": 6.85, "hardware": "NVIDIA H100 80GB HBM3, CP
 # (profiles/ckv_scan_kernel_llama8b_128k_b4.md): 206.06 MB read + 10.15 MB written for the 205.5 MB of summaries the
 # step reads (mean keys hi + lo, mean values hi, variances).
 SCAN_TRAFFIC_RATIO = (206.06 + 10.15) / 205.5
-# The same for the one-launch step (profiles/ckv_unit_step_kernel_llama8b_128k_b2.md): 120.5 MB read + 5.3 MB written.
+# The same for the one-launch step (profiles/ckv_unit_step_kernel_llama8b_128k_b2.md): 120.5 MB read + 5.3 MB written (mean of two).
 STEP_TRAFFIC_RATIO = 125.8 / 119.6
 # What is stored and multiplied (the line's `dtype`): K/V pages are bf16; mean keys and mean values keep fp32
 # precision as split bf16 pairs (hi = bf16(x), lo = bf16(x - hi), relative error <= 2^-18), variances are fp32; the
