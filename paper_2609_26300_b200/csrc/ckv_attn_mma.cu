@@ -48,13 +48,15 @@ constexpr int kAuxBytes = kLsOff + 256;
 constexpr int kMaxEntries = 32;                       // partials a CTA folds per round: one per lane
 constexpr int kPartBytes = CKV_PART_STRIDE * 4;       // one head's partial
 
-// Scan partials that a warp of the sparse form brings in besides those that fit its idle page buffer.  A split of a ragged
+// Scan partials that a warp of the clustered form brings in besides those that fit its idle page buffer.  A split of a ragged
 // batch has up to a dozen: with eight heads (4.2 KB a partial, one a buffer) that was three rounds of copy, reduction and
 // three barriers; two CTAs still fit an SM.  128 units of eight heads, 16K to 64K: 80.0 us a step, 78.0 now (this launch
-// 23.1 -> 21.0 us under the profiler).
-template <int G, bool DENSE> constexpr int kExtraSlots = DENSE ? 0 : (G == 8 ? 2 : (G == 4 ? 4 : 0));
-template <int G, bool DENSE, int W> constexpr size_t dyn_smem() {
-  return (size_t)W * (2 * kPageBytes + kAuxBytes + kExtraSlots<G, DENSE> * G * kPartBytes);
+// 23.1 -> 21.0 us under the profiler).  Not where a unit has more splits than a cluster takes: a split then has a handful of
+// them, and the larger CTAs (two to an SM either way) made that launch 12.0 -> 13.6 us under the profiler (8 units of 300K / 400K
+// / 500K 53.3 / 80.5 / 98.7 us a step, 54.8 / 81.9 / 100.5 with the slots).
+template <int G, bool CL> constexpr int kExtraSlots = CL ? (G == 8 ? 2 : (G == 4 ? 4 : 0)) : 0;
+template <int G, bool CL, int W> constexpr size_t dyn_smem() {
+  return (size_t)W * (2 * kPageBytes + kAuxBytes + kExtraSlots<G, CL> * G * kPartBytes);
 }
 
 constexpr int kMaxCluster = 8;    // splits of a unit that can be one cluster (the portable size; 13 measured far slower)
@@ -188,7 +190,7 @@ ckv_attn_mma_kernel(CkvDev P, const __nv_bfloat16 *q, const __nv_bfloat16 *k_poo
   // the scan partials this CTA folds in: partial j of the unit goes to split j % n_active
   constexpr int kBufSlots = (kPageBytes / (G * kPartBytes)) < ((kMaxEntries - W) / W) ? (kPageBytes / (G * kPartBytes))
                                                                                       : ((kMaxEntries - W) / W);
-  constexpr int kSlotsPerWarp = kBufSlots + kExtraSlots<G, DENSE>;
+  constexpr int kSlotsPerWarp = kBufSlots + kExtraSlots<G, CL>;
   constexpr int kSlots = W * kSlotsPerWarp;
   static_assert(W + kSlots <= kMaxEntries, "a lane per entry");
   constexpr uint32_t kExtraOff = (uint32_t)W * (2 * kPageBytes + kAuxBytes);   // [warp][slot][G] partials
@@ -203,7 +205,7 @@ ckv_attn_mma_kernel(CkvDev P, const __nv_bfloat16 *q, const __nv_bfloat16 *k_poo
       if (idx < my_cnt) {
         const float *src = cp0 + (size_t)(blockIdx.x + (size_t)idx * n_active) * step;
         const uint32_t dst = k < kBufSlots ? wtiles_u32 + bufsel * kPageBytes + k * (G * kPartBytes)
-                                           : (uint32_t)__cvta_generic_to_shared(smem) + kExtraOff + (uint32_t)(warp * kExtraSlots<G, DENSE> + k - kBufSlots) * (G * kPartBytes);
+                                           : (uint32_t)__cvta_generic_to_shared(smem) + kExtraOff + (uint32_t)(warp * kExtraSlots<G, CL> + k - kBufSlots) * (G * kPartBytes);
         for (int c = lane; c < G * (kPartBytes / 16); c += 32) cp_async16(dst + 16 * c, src + 4 * c, true);
       }
     }
@@ -419,7 +421,7 @@ ckv_attn_mma_kernel(CkvDev P, const __nv_bfloat16 *q, const __nv_bfloat16 *k_poo
     } else {
       const int c = tid - W, we = c / kSlotsPerWarp, k = c % kSlotsPerWarp;
       off = k < kBufSlots ? region(we, red_buf(we) ^ 1) + k * G * CKV_PART_STRIDE
-                          : (int)(kExtraOff / 4) + (we * kExtraSlots<G, DENSE> + k - kBufSlots) * G * CKV_PART_STRIDE;
+                          : (int)(kExtraOff / 4) + (we * kExtraSlots<G, CL> + k - kBufSlots) * G * CKV_PART_STRIDE;
     }
     s_ent[tid] = off;
   }
@@ -552,7 +554,7 @@ bool cluster_fits(int n_splits, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(n_splits, 1, 1);
   cfg.blockDim = dim3(kSparseWarps * 32);
-  cfg.dynamicSmemBytes = dyn_smem<G, false, kSparseWarps>();
+  cfg.dynamicSmemBytes = dyn_smem<G, true, kSparseWarps>();
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -572,25 +574,25 @@ cudaError_t launch_g(ckv_ctx *c, bool dense, const void *q, const void *k_pool, 
   const int units = (int)grid.y;
   const __nv_bfloat16 *qp = (const __nv_bfloat16 *)q, *kp = (const __nv_bfloat16 *)k_pool, *vp = (const __nv_bfloat16 *)v_pool;
   if (dense)
-    return ckv_launch_pdl(ckv_attn_mma_kernel<G, true, kDenseWarps, false, false>, grid, dim3(kDenseWarps * 32), dyn_smem<G, true, kDenseWarps>(), st, 0,
+    return ckv_launch_pdl(ckv_attn_mma_kernel<G, true, kDenseWarps, false, false>, grid, dim3(kDenseWarps * 32), dyn_smem<G, false, kDenseWarps>(), st, 0,
                           c->dev, qp, kp, vp, page_table, seq_lens, sel_ids, sel_cnt, kcap, pps, scan_grid, units, (__nv_bfloat16 *)out, lse);
   const bool rm = c->dev.row_elems == CKV_D;   // bf16 summaries: removal with the stored mean-value rows
   const bool cl = cluster_fits<G>((int)grid.x, st);   // the unit's splits as one cluster: partials never leave the SMs
   auto kernel = cl ? (rm ? ckv_attn_mma_kernel<G, false, kSparseWarps, true, true> : ckv_attn_mma_kernel<G, false, kSparseWarps, true, false>)
                    : (rm ? ckv_attn_mma_kernel<G, false, kSparseWarps, false, true> : ckv_attn_mma_kernel<G, false, kSparseWarps, false, false>);
-  return ckv_launch_pdl(kernel, grid, dim3(kSparseWarps * 32), dyn_smem<G, false, kSparseWarps>(), st, cl ? (int)grid.x : 0,
+  return ckv_launch_pdl(kernel, grid, dim3(kSparseWarps * 32), cl ? dyn_smem<G, true, kSparseWarps>() : dyn_smem<G, false, kSparseWarps>(), st, cl ? (int)grid.x : 0,
                         c->dev, qp, kp, vp, page_table, seq_lens, sel_ids, sel_cnt, kcap, pps, scan_grid, units, (__nv_bfloat16 *)out, lse);
 }
 
 template <int G>
 cudaError_t configure_g() {
   cudaError_t e = cudaFuncSetAttribute(ckv_attn_mma_kernel<G, true, kDenseWarps, false, false>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn_smem<G, true, kDenseWarps>());
-  const int sm = (int)dyn_smem<G, false, kSparseWarps>();
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn_smem<G, false, kDenseWarps>());
+  const int sm = (int)dyn_smem<G, false, kSparseWarps>(), sm_cl = (int)dyn_smem<G, true, kSparseWarps>();
   if (e == cudaSuccess) e = cudaFuncSetAttribute(ckv_attn_mma_kernel<G, false, kSparseWarps, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(ckv_attn_mma_kernel<G, false, kSparseWarps, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(ckv_attn_mma_kernel<G, false, kSparseWarps, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(ckv_attn_mma_kernel<G, false, kSparseWarps, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(ckv_attn_mma_kernel<G, false, kSparseWarps, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm_cl);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(ckv_attn_mma_kernel<G, false, kSparseWarps, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm_cl);
   return e;
 }
 

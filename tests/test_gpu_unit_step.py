@@ -409,6 +409,15 @@ def test_selected_ids_where_the_scores_a_thread_holds_change(keys, X):
     test_selected_ids_are_the_best_of_the_scores(keys, X, 64)
 
 
+@pytest.mark.parametrize("hq", [2, 8, 16])
+@pytest.mark.parametrize("layout", [{}, {"stat_bf16": 1}])
+def test_more_splits_than_a_cluster_takes(hq, layout):
+    """Two units with 600 selected pages: 65 attention splits each, merged through global memory, and more scan partials a split
+    than a round takes with eight heads."""
+    run(workload(batch=1, num_q_heads=hq, num_kv_heads=2, ctx=16 * 1100 + 5, ctx_min=None, budget_tokens=16 * 600, decode_steps=1),
+        1, launches=3, tail=binding.CKV_TAIL_ON, **layout)
+
+
 def test_a_wait_that_runs_out_is_reported_and_the_context_recovers():
     w = workload(batch=1, ctx_min=None, decode_steps=0)
     d = setup(w)
