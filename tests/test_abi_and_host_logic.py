@@ -119,3 +119,12 @@ def test_missing_library_fails_loudly(monkeypatch, tmp_path):
     monkeypatch.setattr(binding, "LIB_PATH", str(tmp_path / "nope.so"))
     with pytest.raises(RuntimeError, match="not built"):
         binding.load()
+
+
+def test_the_one_launch_steps_shared_memory_is_what_its_static_arrays_leave():
+    """A constant beside static arrays that fill the rest to the byte would refuse every context of eight heads a group as soon
+    as a struct that is copied into shared memory grows: the plan takes the limit that was worked out from the kernel."""
+    with open(os.path.join(ROOT, "paper_2609_26300_b200", "csrc", "ckv_unitstep.cu")) as f:
+        src = re.sub(r"//[^\n]*", "", f.read())
+    assert re.search(r"c->step_smem = std::min\(kDynMost, \(kSmemCta - \(int\)fa\.sharedSizeBytes\)", src)
+    assert src.count("kDynMost") == 2 and src.count("(size_t)c->step_smem") == 3
